@@ -26,7 +26,7 @@ __global__ void __launch_bounds__(B, 1024 / B) batch_kernel(const CaseDev* __res
                                                   const int32_t* __restrict__ job_start, BatchHeader* hdr,
                                                   int32_t* __restrict__ case_step,
                                                   const int32_t* __restrict__ case_cap, Launch L, int n_steps) {
-  __shared__ TeamShared sh;
+  __shared__ TeamShared<B> sh;
   __shared__ CaseDev s_cs;
   __shared__ int s_job[4];
   const int n_jobs = hdr->n_jobs, n_tickets = hdr->n_tickets;
@@ -77,6 +77,7 @@ __global__ void __launch_bounds__(B, 1024 / B) batch_kernel(const CaseDev* __res
       }
     }
     __syncthreads();
+    if (run > 0) team_leave(tm, sh);
     if (run > 0 && tm.rank == 0 && threadIdx.x == 0) case_step[c] = base + run;
     __syncthreads();
   }
@@ -88,6 +89,7 @@ __global__ void batch_prepare_kernel(const CaseDev* __restrict__ cases, int n_ca
   if (i < n_cases) {
     SyncWords* sw = cases[i].sync;
     sw->count = 0;
+    sw->gen = 0;
     sw->status = 0;
     case_step[i] = 0;
     // forms that update the FP64 field directly leave the triple-float one stale
@@ -152,7 +154,7 @@ int max_coresident_batch_ctas(int threads, int W, int form, int device) {
     return 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
   const int n = per_sm * sms;
-  return n < kMaxCtas ? n : kMaxCtas;
+  return n < kMaxCtas / 2 ? n : kMaxCtas / 2;  // the partial sums' table holds two buffers
 }
 
 cudaError_t launch_batch_prepare(const CaseDev* cases, int n_cases, int32_t* case_step, cudaStream_t s) {

@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(B, 1024 / B) dd_step_kernel(CaseDev cs, const 
                                                               const int32_t* __restrict__ cta_part,
                                                               const int32_t* __restrict__ cta_rank, Launch L,
                                                               int n_steps) {
-  __shared__ TeamShared sh;
+  __shared__ TeamShared<B> sh;
   __shared__ DdPart me;
   if (threadIdx.x == 0) me = parts[cta_part[blockIdx.x]];
   __syncthreads();
@@ -203,8 +203,11 @@ __global__ void __launch_bounds__(B, 1024 / B) dd_step_kernel(CaseDev cs, const 
     double v[1] = {0.0};
     for (int c = c0 + tid; c < c1; c += B) v[0] += me.x[c];
     dd_push(parts, me, e0, e1, true, B);
-    if (!team_allreduce<1>(tm, v, sh)) return;
-    const double xRef = v[0] / (double)cs.N;
+    if (!team_allreduce<1, B>(tm, v, sh, [&](int, double t, int lane) {
+          if (lane == 0) sh.xref = t / (double)cs.N;
+        }))
+      return;
+    const double xRef = sh.xref;
     // ---- rows, initial residual, normFactor, first direction (p = w, exchanged) ---------
     double u[3] = {0.0, 0.0, 0.0};
     for (int c = c0 + tid; c < c1; c += B) {
@@ -221,15 +224,23 @@ __global__ void __launch_bounds__(B, 1024 / B) dd_step_kernel(CaseDev cs, const 
       me.p[c] = wc;
     }
     dd_push(parts, me, e0, e1, false, B);
-    if (!team_allreduce<3>(tm, u, sh)) return;
-    const double nf = u[0] + kSmall;
-    const double init_res = u[1] / nf;
-    double res = init_res, rho = u[2], beta = 0.0;
+    if (!team_allreduce<3, B>(tm, u, sh, [&](int k, double t, int lane) {
+          if (lane == 0) sh.out[k] = t;
+        }))
+      return;
+    if (tid == 0) {
+      sh.nf = sh.out[0] + kSmall;
+      sh.init_res = sh.res = sh.out[1] / sh.nf;
+      sh.rho = sh.out[2];
+      sh.conv = converged(sh.res, sh.init_res, cs.tol, cs.rel_tol) ? 1 : 0;
+      sh.code = cs.min_iter > 0 || !sh.conv ? kGo : kStop;
+    }
+    __syncthreads();
     int iters = 0, status = 0;
-    bool conv = converged(res, init_res, cs.tol, cs.rel_tol);
-    if (cs.min_iter > 0 || !conv) {
-      for (;;) {
+    {  // the iterations
+      while (sh.code == kGo) {
         if (iters > 0) {
+          const double beta = sh.beta;
           int c = c0 + tid;
           for (; c + B < c1; c += 2 * B) {  // two cells per trip, the next trip prefetched
             pf_next<B>(me.p, c, c1);
@@ -240,7 +251,7 @@ __global__ void __launch_bounds__(B, 1024 / B) dd_step_kernel(CaseDev cs, const 
           }
           if (c < c1) me.p[c] = fma(beta, me.p[c], me.w[c]);
           dd_push(parts, me, e0, e1, false, B);
-          if (!team_barrier(tm, sh)) return;
+          if (!team_barrier<B>(tm, sh)) return;
         }
         // q = A p over the owned rows (ghost columns from the exchange), sigma = p.q; with a
         // fixed slot width two rows per trip, all their loads issued first, the matrix with
@@ -284,13 +295,9 @@ __global__ void __launch_bounds__(B, 1024 / B) dd_step_kernel(CaseDev cs, const 
           me.q[c] = acc;
           s1[0] = fma(acc, pc, s1[0]);
         }
-        if (!team_allreduce<1>(tm, s1, sh)) return;
-        const double sigma = s1[0];
-        if (fabs(sigma) / nf < kVSmall) {
-          status = LFM_ESINGULAR;
-          break;
-        }
-        const double alpha = rho / sigma;
+        if (!team_allreduce<1, B>(tm, s1, sh, [&](int, double t, int lane) { fin_sigma(sh, t, lane); })) return;
+        if (sh.code != kGo) break;
+        const double alpha = sh.alpha;
         double s2[2] = {0.0, 0.0};
         for (int c = c0 + tid; c < c1; c += B) {
           if (c + B < c1) {  // the next trip's cell, into L2
@@ -308,21 +315,16 @@ __global__ void __launch_bounds__(B, 1024 / B) dd_step_kernel(CaseDev cs, const 
           s2[0] += fabs(rn);
           s2[1] = fma(wn, rn, s2[1]);
         }
-        if (!team_allreduce<2>(tm, s2, sh)) return;
-        res = s2[0] / nf;
-        beta = s2[1] / rho;
-        rho = s2[1];
         ++iters;
-        if (!isfinite(res)) {
-          status = LFM_ENONFINITE;
-          break;
-        }
-        conv = converged(res, init_res, cs.tol, cs.rel_tol);
-        if (!((iters < cs.max_iter && !conv) || iters < cs.min_iter)) break;
+        if (!team_allreduce<2, B>(tm, s2, sh, [&](int k, double t, int lane) {
+              fin_update(sh, k, t, lane, cs.tol, cs.rel_tol, iters, cs.max_iter, cs.min_iter);
+            }))
+          return;
       }
     }
-    conv = converged(res, init_res, cs.tol, cs.rel_tol);
-    write_stats(cs, tm, step, iters, conv ? 1 : 0, iters > 0 ? 1 : 0, status, init_res, res, nf);
+    if (sh.code == kSingular) status = LFM_ESINGULAR;
+    if (sh.code == kNonFinite) status = LFM_ENONFINITE;
+    write_stats(cs, tm, step, iters, sh.conv, iters > 0 ? 1 : 0, status, sh.init_res, sh.res, sh.nf);
     if (status != 0) {
       if (tm.rank == 0 && tid == 0) set_status(cs.sync, status);
       return;
@@ -344,7 +346,7 @@ int dd_max_ctas(int threads, int W, int device) {
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, 0) != cudaSuccess) return 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
   const int n = per_sm * sms;
-  return n < kMaxCtas ? n : kMaxCtas;
+  return n < kMaxCtas / 2 ? n : kMaxCtas / 2;  // the partial sums' table holds two buffers
 }
 
 cudaError_t launch_dd_steps(const CaseDev& cs, const DdPart* parts, const int32_t* cta_part, const int32_t* cta_rank,

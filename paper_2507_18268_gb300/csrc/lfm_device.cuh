@@ -1,21 +1,24 @@
 // Device primitives: bounded team barriers with deterministic reductions.
 //
 // A "team" is a set of co-resident CTAs (a cooperative launch guarantees co-residency)
-// working on one case. Each barrier may carry up to kMaxSums FP64 sums: every CTA reduces
-// its threads' values with a fixed warp-shuffle / shared-memory tree, writes the CTA total
-// to its slot of a partial table, and arrives on a counter. The last CTA to arrive adds the
-// slots in rank order (lane l takes ranks l, l+32, ...; then a fixed xor tree), publishes
-// the sums and releases the barrier by bumping a generation word. The result depends only
-// on the team size, never on arrival order, so repeated runs are bitwise identical. The
-// barrier is a chain of L2 round trips, so it is built to keep that chain short: arrival is
-// one acquire-release atomic, the release one release store, and no fence sits on the
-// critical path (about 5.4 us with one sum for 304 CTAs on GB300, 7.7 us with a fence before
-// the arrival and around the last arriver's reduction). Each further sum costs more than a
-// round trip does: the CTA's own reduction adds in FP64, which GB300 issues slowly, so
-// block_reduce keeps its FP64 adds few.
+// working on one case. Each barrier may carry up to kMaxSums FP64 sums: every CTA reduces its
+// threads' values in a fixed order (block_sums), publishes its partial sums and arrives on a
+// counter that only grows; every CTA waits for the counter itself, then adds all CTAs' partial
+// sums in rank order. The result depends only on the block and team size, never on arrival
+// order, so repeated runs are bitwise identical.
 //
-// Every wait is bounded: a waiter that sees no release within the launch's time limit (or
-// sees another CTA's error) records an error status and the caller leaves the kernel.
+// What bounds a barrier on GB300 (304 CTAs of 512 threads): the chain release - counter -
+// acquire takes 1.6 us; the rest is FP64. A scheduler's FP64 unit takes about 64 clocks per
+// warp instruction (half a lane per clock), dependent or not, so a sum costs what its longest
+// chain of warp-wide adds on one scheduler does, and a value computed by every thread costs
+// thousands of clocks: an FP64 division by all threads of 304 x 512 takes 2.8 us, by one warp
+// 0.4. Hence (i) block_sums spreads each sum over warps of four schedulers with no lane idle
+// until the last tree; (ii) the scalars that follow from the totals (alpha, beta, the scaled
+// residual and the stopping decision) are formed by one lane of the warp that holds the total
+// (`fin`) and handed to the CTA through shared memory.
+//
+// Every wait is bounded: a waiter that sees too few arrivals within the launch's time limit
+// (or sees another CTA's error) records an error status and the caller leaves the kernel.
 #pragma once
 
 #include <cstdint>
@@ -36,8 +39,10 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
   return v;
 }
 
-__device__ __forceinline__ void st_release_u32(unsigned* p, unsigned v) {
-  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+__device__ __forceinline__ unsigned ld_relaxed_u32(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
 }
 
 __device__ __forceinline__ int ld_volatile_i32(const int32_t* p) {
@@ -75,6 +80,7 @@ __device__ __forceinline__ int checked_index(int i, int n, int fallback, int sit
 #define LFM_IDX(i, n, fallback, site) (i)
 #endif
 
+// Launch-wide team: CTAs of a cooperative launch, meeting through global memory.
 struct Team {
   int size;
   int rank;
@@ -83,202 +89,195 @@ struct Team {
   uint64_t timeout_ns;
 };
 
-// Shared scratch a CTA needs for team_allreduce.
-constexpr int kRedSlots = 256;  // block_reduce's shared partial sums (all NS sums together)
+constexpr int kTeamCap = kMaxCtas / 2;  // partials: two buffers (barrier parity) of kMaxSums rows
 
+// What the iteration decides after a pass (TeamShared::code).
+enum StepCode { kGo = 0, kStop = 1, kSingular = 2, kNonFinite = 3 };
+
+// Shared scratch of a CTA in a team, and the scalars of the solve it is in: written by one
+// lane inside a barrier (or by thread 0 between two __syncthreads), read by all threads.
+template <int B>
 struct TeamShared {
-  double red[kRedSlots];
-  double out[kMaxSums];
-  int flag[4];
-  unsigned gen;  // thread 0: the team's generation before this CTA's next arrival
+  double red[B];            // block_sums
+  double out[kMaxSums];     // team totals, where a barrier has no fin of its own
+  double alpha, beta, rho;  // rho: w.r of the current residual
+  double nf, init_res, res; // normFactor, the solve's first and latest scaled residual
+  double nf0, init0;        // those of the step's first solve
+  double xref;
+  double inner_tol;         // mixed form: the inner solve's tolerance
+  double seed[3];           // mixed form: the next step's normFactor sum, sum|r|, rho
+  float2 alpha2, beta2, xref2;  // double-float copies (hi, lo)
+  float alpha32, beta32;
+  int code, conv;
+  int ok;                   // 0: a wait ran out or another CTA failed
+  int par;                  // parity of the next barrier
+  unsigned target;          // the counter's value after the last barrier passed
+  unsigned long long phase[kPhases], phase_t;
 };
 
-// Thread 0 of a CTA, when the CTA joins a team (before its first arrival): the team's
-// generation word, which no barrier can move before this CTA has arrived. team_allreduce
-// then tracks the generation itself (one more per barrier passed), so that no load of it
-// sits before an arrival.
-__device__ __forceinline__ void team_join(const Team& tm, TeamShared& sh) {
-  sh.gen = *reinterpret_cast<volatile unsigned*>(&tm.sw->gen);
+// Thread 0 of a CTA, when the CTA joins a team (before its first arrival): the counter's value
+// before the team's first barrier, which team_leave or the host left in gen. A CTA that joins
+// a team whose wait has already run out leaves at its first barrier.
+template <int B>
+__device__ __forceinline__ void team_join(const Team& tm, TeamShared<B>& sh) {
+  sh.target = *reinterpret_cast<volatile unsigned*>(&tm.sw->gen);
+  sh.par = 0;
+  sh.ok = ld_volatile_i32(&tm.sw->status) != LFM_ETIMEOUT;
 }
 
-// Spins until *gen != g. False (with the error recorded) when the time limit runs out or
-// another CTA has recorded an error. The load is an acquire: what the releasing CTA wrote
-// before its release is visible to this thread afterwards, without a further fence.
-__device__ __forceinline__ bool wait_generation(unsigned* gen, unsigned g, int32_t* status,
-                                                uint64_t timeout_ns) {
-  uint64_t t0 = global_timer_ns();
+// After a team's last barrier of a run: where its next run's counter starts (every CTA of the
+// team has joined by then). Only launches without a host reset in between need it.
+template <int B>
+__device__ __forceinline__ void team_leave(const Team& tm, TeamShared<B>& sh) {
+  if (tm.rank == 0 && threadIdx.x == 0 && sh.ok) *reinterpret_cast<volatile unsigned*>(&tm.sw->gen) = sh.target;
+}
+
+// Spins until *count has reached target (modulo 2^32). False (with the error recorded) when
+// the time limit runs out or another CTA has recorded an error. It polls with relaxed loads and
+// acquires once at the end (what the arriving CTAs wrote before their arrival is visible to this
+// thread afterwards): an acquire drops the SM's L1 lines, which a CTA of the team that is still
+// in its gathers on the same SM would miss at every poll.
+__device__ __forceinline__ bool wait_count(unsigned* count, unsigned target, int32_t* status, uint64_t timeout_ns) {
+  uint64_t t0 = 0;
   unsigned spins = 0;
-  while (ld_acquire_u32(gen) == g) {
+  while ((int)(ld_relaxed_u32(count) - target) < 0) {
     ++spins;
-    if (spins > 16) __nanosleep(32);
+    if (spins > 64) __nanosleep(20);
     if ((spins & 31u) == 0) {
-      if (ld_volatile_i32(status) != 0) return false;
-      if (global_timer_ns() - t0 > timeout_ns) {
+      if (ld_volatile_i32(status) != 0) return (int)(ld_acquire_u32(count) - target) >= 0;
+      const uint64_t now = global_timer_ns();
+      if (t0 == 0) t0 = now;
+      if (now - t0 > timeout_ns) {
         atomicCAS(status, 0, (int32_t)LFM_ETIMEOUT);
         return false;
       }
     }
   }
+  ld_acquire_u32(count);
   return true;
 }
 
-// Arrival at a team barrier: one acquire-release add on the arrival counter (the release
-// orders this CTA's partial sums before it, the acquire makes every earlier arrival's
-// partial sums visible to the last arriver).
-__device__ __forceinline__ unsigned arrive_acq_rel(unsigned* count) {
-  unsigned old;
-  asm volatile("atom.add.acq_rel.gpu.u32 %0, [%1], 1;" : "=r"(old) : "l"(count) : "memory");
-  return old;
+// Arrival at a team barrier: a release add without a return value (it orders this CTA's phase
+// and partial sum before it).
+__device__ __forceinline__ void arrive_release(unsigned* count) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
 }
 
-// Fixed-pattern reduction of NS values over the CTA: each warp folds its lanes by an xor tree
-// down to vpw partial sums (lanes 0 .. vpw - 1; vpw the largest of 8, 4, 2, 1 whose partials
-// of 32 warps and all sums fit kRedSlots), the partials go through shared memory, and warp 0
-// sums them: lane l takes partials l, l + 32, ... in index order, then a five-level xor
-// tree. Totals land in sh.out (visible after the caller's next __syncthreads). The order
-// depends only on the block size. The FP64 pipe issues about two operations per clock per
-// SM on GB300, so the fewer FP64 adds matter: against a full xor tree in every warp this
-// measured 5.95 -> 5.45, 9.34 -> 7.63 and 15.17 -> 12.90 us per barrier with 1, 2 and 4
-// sums over 304 CTAs.
-template <int NS>
-__host__ __device__ constexpr int partials_per_warp() {  // sized for the largest block, 32 warps
-  return 32 * 8 * NS <= kRedSlots ? 8 : 32 * 4 * NS <= kRedSlots ? 4 : 32 * 2 * NS <= kRedSlots ? 2 : 1;
-}
-
-template <int NS>
-__device__ __forceinline__ void block_reduce(double* v, TeamShared& sh) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  constexpr int vpw = partials_per_warp<NS>();
+// Fixed-order sums of NS values over the CTA. The values of one sum at a time go through
+// shared memory to G warps, one per scheduler, whose lanes add B / (32 G) of them each; the
+// lane sums go through shared memory once more to warp k (sum k), which adds G per lane and
+// then its lanes (xor tree). Returns the total of sum k in every lane of warp k < NS. Chain of
+// FP64 adds at 512 threads: 3 + 3 + 5 for each sum, the sums on different schedulers. (Each
+// warp folding its own lanes first took 2 to 4 adds on each of a scheduler's four warps and
+// sum, and one warp then added all sums: a barrier of 304 CTAs of 512 with 0 / 1 / 2 / 4 sums
+// took 2.06 / 5.25 / 8.6 / 15.0 us and takes 1.56 / 4.41 / 4.88 / 7.87.) The order depends only
+// on the block size.
+template <int NS, int B>
+__device__ __forceinline__ double block_sums(const double* v, TeamShared<B>& sh) {
+  constexpr int nw = B / 32, kRows = NS <= 1 ? 1 : NS == 2 ? 2 : 4;
+  constexpr int G = nw / kRows < 4 ? nw / kRows : 4;  // warps per sum
+  constexpr int kPer = B / (32 * G);                  // values per lane
+  constexpr int kStride = NS == 1 ? kPer * 32 : 32;   // lane sums: NS = 1 in the warp's own range
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  double q[kPer];
 #pragma unroll
   for (int k = 0; k < NS; ++k) {
+    if (k > 0) __syncthreads();
+    sh.red[tid] = v[k];
+    __syncthreads();
+    if (warp / G == k) {
+      const double* from = sh.red + (warp % G) * (kPer * 32) + lane;
 #pragma unroll
-    for (int o = 16; o >= vpw; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-  }
-  const int nv = nw * vpw;
-  if (lane < vpw) {
-#pragma unroll
-    for (int k = 0; k < NS; ++k) sh.red[k * nv + warp * vpw + lane] = v[k];
-  }
-  __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int k = 0; k < NS; ++k) {
-      double t = 0.0;
-      for (int i = lane; i < nv; i += 32) t += sh.red[k * nv + i];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-      if (lane == 0) sh.out[k] = t;
+      for (int i = 0; i < kPer; ++i) q[i] = from[32 * i];
     }
   }
+  if (NS > 1) __syncthreads();
+  if (warp < NS * G) {
+    double t = q[0];
+#pragma unroll
+    for (int i = 1; i < kPer; ++i) t += q[i];
+    sh.red[warp * kStride + lane] = t;
+  }
+  __syncthreads();
+  double t = 0.0;
+  if (warp < NS) {
+    const double* from = sh.red + warp * G * kStride + lane;
+    t = from[0];
+#pragma unroll
+    for (int g = 1; g < G; ++g) t += from[g * kStride];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  }
+  return t;
 }
 
-// Team-wide barrier carrying NS sums. On return (true) v[k] holds the team totals in every
-// thread. False: a wait ran out or another CTA failed; the caller must leave the kernel.
-// Protocol: thread 0 stores the CTA's partial sums and arrives (one acquire-release add;
-// the generation it waits on is its own count, see team_join); the CTA that finds size - 1 arrivals before its own is the last:
-// warp 0 loads all partial sums at once, adds them in rank order (lane l takes ranks l,
-// l + 32, ..., then a fixed xor tree), publishes the totals, clears the counter and releases
-// the generation with a release store (which orders the totals and the cleared counter
-// before it). The others wait for the generation with acquire loads and then read the
-// totals. The sums depend only on the team size, never on arrival order. (Detecting the
-// last arrival by a remainder modulo the team size, with a counter never cleared, measured
-// 10 % slower in the mixed form's A p: the division's code sits in its inner loop.)
-template <int NS>
-__device__ bool team_allreduce(const Team& tm, double* v, TeamShared& sh) {
-  // Every thread's global writes of the phase must be ordered before thread 0 signals
-  // arrival: block_reduce synchronises the CTA itself; a barrier without sums needs its own.
+// Team-wide barrier carrying NS sums. fin(k, total, lane) runs in all lanes of warp k < NS with
+// the team total of sum k and may write scalars of sh, which every thread may read on return.
+// False: a wait ran out or another CTA failed; the caller must leave the kernel.
+// Protocol: warp k stores the CTA's partial of sum k and arrives; it waits until all CTAs have
+// arrived for every sum and adds the partials in rank order (lane l takes ranks l, l + 32, ...,
+// all loaded first; then a fixed xor tree). The partials are double-buffered by the barrier's
+// parity: a CTA can overwrite one only two barriers later, when every CTA has arrived at the
+// barrier between and so has read it. (With a last arriver that adds the partials, publishes
+// the totals and releases a generation word, three more L2 round trips sit in the chain:
+// 2.06 us without sums against 1.60.)
+template <int NS, int B, class Fin>
+__device__ bool team_allreduce(const Team& tm, const double* v, TeamShared<B>& sh, Fin&& fin) {
+  constexpr int kArrivals = NS > 0 ? NS : 1;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double tot = 0.0;
+  // every thread's global writes of the phase are ordered before the arrivals below by the
+  // CTA synchronisation inside block_sums, or by this one
   if constexpr (NS > 0) {
-    block_reduce<NS>(v, sh);
+    tot = block_sums<NS, B>(v, sh);
   } else {
     __syncthreads();
   }
-  if (tm.size == 1) {
-    __syncthreads();
-    if constexpr (NS > 0) {
-#pragma unroll
-      for (int k = 0; k < NS; ++k) v[k] = sh.out[k];
-    }
-    return true;
-  }
-  if (threadIdx.x == 0) {
-    if constexpr (NS > 0) {
-#pragma unroll
-      for (int k = 0; k < NS; ++k) __stcg(&tm.partials[tm.rank * kMaxSums + k], sh.out[k]);
-    }
-    const unsigned g = sh.gen;
-    const unsigned prev = arrive_acq_rel(&tm.sw->count);
-    const int last = prev == (unsigned)(tm.size - 1);
-    int ok = 1;
-    if (!last) {
-      ok = wait_generation(&tm.sw->gen, g, &tm.sw->status, tm.timeout_ns);
-      if constexpr (NS > 0) {
-        if (ok) {
-#pragma unroll
-          for (int k = 0; k < NS; ++k) sh.out[k] = __ldcg(&tm.sw->scalars[k]);
-        }
+  if (warp < kArrivals) {
+    if (tm.size > 1) {
+      double* pt = tm.partials + (size_t)(sh.par * kMaxSums + warp) * kTeamCap;
+      if (lane == 0) {
+        if constexpr (NS > 0) __stcg(pt + tm.rank, tot);
+        arrive_release(&tm.sw->count);
+        if (sh.ok && !wait_count(&tm.sw->count, sh.target + (unsigned)(kArrivals * tm.size), &tm.sw->status,
+                                 tm.timeout_ns))
+          sh.ok = 0;
       }
-    }
-    sh.flag[0] = last;
-    sh.flag[1] = ok;
-    sh.flag[2] = (int)g;
-    sh.gen = g + 1u;
-  }
-  __syncthreads();
-  if (!sh.flag[1]) return false;
-  if (sh.flag[0]) {
-    if (threadIdx.x < 32) {
-      const int lane = threadIdx.x;
+      __syncwarp();
       if constexpr (NS > 0) {
-        // loads first, 16 values per lane in flight (lane l takes ranks l, l + 32, ...), then
-        // the adds; 16 doubles per lane keep within the kernels' 64-register budget
-        constexpr int kBatch = 16 / NS;
-        double t[NS];
-#pragma unroll
-        for (int k = 0; k < NS; ++k) t[k] = 0.0;
+        constexpr int kBatch = 10;
+        tot = 0.0;
         for (int r0 = 0; r0 < tm.size; r0 += 32 * kBatch) {
-          double buf[kBatch][NS];
+          double buf[kBatch];
 #pragma unroll
           for (int i = 0; i < kBatch; ++i) {
             const int r = r0 + lane + 32 * i;
-#pragma unroll
-            for (int k = 0; k < NS; ++k) buf[i][k] = r < tm.size ? __ldcg(&tm.partials[r * kMaxSums + k]) : 0.0;
+            buf[i] = r < tm.size ? __ldcg(pt + r) : 0.0;
           }
 #pragma unroll
           for (int i = 0; i < kBatch; ++i)
-#pragma unroll
-            for (int k = 0; k < NS; ++k) t[k] += buf[i][k];
+            if (r0 + 32 * i < tm.size) tot += buf[i];
         }
 #pragma unroll
-        for (int k = 0; k < NS; ++k) {
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) t[k] += __shfl_xor_sync(0xffffffffu, t[k], o);
-        }
-        if (lane == 0) {
-#pragma unroll
-          for (int k = 0; k < NS; ++k) {
-            sh.out[k] = t[k];
-            __stcg(&tm.sw->scalars[k], t[k]);
-          }
-        }
-      }
-      __syncwarp();
-      if (lane == 0) {
-        tm.sw->count = 0u;  // ordered before the release below; no CTA arrives again before it
-        st_release_u32(&tm.sw->gen, (unsigned)sh.flag[2] + 1u);
+        for (int o = 16; o > 0; o >>= 1)
+          if (tm.size > o) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+        tot = __shfl_sync(0xffffffffu, tot, 0);
       }
     }
-    __syncthreads();
+    if constexpr (NS > 0) fin(warp, tot, lane);
   }
-  if constexpr (NS > 0) {
-#pragma unroll
-    for (int k = 0; k < NS; ++k) v[k] = sh.out[k];
+  __syncthreads();
+  if (threadIdx.x == 0 && tm.size > 1) {  // read again only after the next barrier's first synchronisation
+    sh.target += (unsigned)(kArrivals * tm.size);
+    sh.par ^= 1;
   }
-  return true;
+  return sh.ok != 0;
 }
 
 // Team-wide barrier without sums.
-__device__ __forceinline__ bool team_barrier(const Team& tm, TeamShared& sh) {
-  return team_allreduce<0>(tm, nullptr, sh);
+template <int B>
+__device__ __forceinline__ bool team_barrier(const Team& tm, TeamShared<B>& sh) {
+  return team_allreduce<0, B>(tm, nullptr, sh, [](int, double, int) {});
 }
 
 // ---- bulk copies global -> shared, completed on an mbarrier ------------------------------
@@ -383,8 +382,8 @@ __device__ __forceinline__ void mbar_drain(uint64_t* bar, unsigned parity, uint6
 // issued as soon as every thread is done with tile t. False when a wait ran out or another CTA
 // failed (status recorded): the CTA then lets its copies in flight land (bounded) before the
 // caller leaves.
-template <int TC, unsigned kStage, typename Issue, typename Body>
-__device__ __forceinline__ bool staged_tiles(int c0, int c1, const Team& tm, Issue&& issue, Body&& body) {
+template <int TC, unsigned kStage, class TM, typename Issue, typename Body>
+__device__ __forceinline__ bool staged_tiles(int c0, int c1, const TM& tm, Issue&& issue, Body&& body) {
   unsigned char* sm = lfm_dyn_smem;
   uint64_t* bar = reinterpret_cast<uint64_t*>(sm + 2 * kStage);
   const int tid = threadIdx.x;

@@ -22,12 +22,11 @@ constexpr int kStaticMaxFaces = 1 << 18;
 
 // Barrier words of one team of CTAs; each field sits on its own 128-byte line.
 struct alignas(128) SyncWords {
-  unsigned int count;                // arrivals at the current barrier
+  unsigned int count;                // arrivals, one per CTA and sum of every barrier (only grows)
   unsigned int pad0[31];
-  unsigned int gen;                  // barrier generation (released by the last arrival)
+  unsigned int gen;                  // count before the team's next run (see team_leave)
   unsigned int pad1[31];
-  double scalars[kMaxSums];          // reduced values published by the last arrival
-  double pad2[16 - kMaxSums];
+  unsigned int pad2[32];
   int32_t status;                    // first error of the launch (0 = none)
   int32_t pad3[31];
   unsigned long long phase_ns[8];    // time per phase kind, accumulated by the team's rank 0
@@ -152,7 +151,7 @@ struct CaseDev {
 
   // team state
   SyncWords* sync;
-  double* partials;          // [kMaxCtas * kMaxSums]
+  double* partials;          // [2][kMaxSums][kMaxCtas / 2] per-CTA partial sums by barrier parity
   lfm_step_stats* stats;     // [kStatsCap]
 };
 

@@ -507,9 +507,9 @@ __device__ __forceinline__ bool use_bulk_f32(const Slots<float>& A) {
   return W > 0 && (A.N & 3) == 0 && dyn_smem_bytes() >= stage_bytes_f32<B, W>();
 }
 
-template <int B, int W>
+template <int B, int W, class TM>
 __device__ __noinline__ double pass_amul_dot_f32_bulk(Slots<float> A, int c0, int c1, const float* __restrict__ p,
-                                                   float* __restrict__ q, const Team& tm, bool& ok) {
+                                                   float* __restrict__ q, const TM& tm, bool& ok) {
   constexpr int TC = 2 * B;
   constexpr int kW = W > 0 ? W : 1;
   constexpr unsigned kPlane = TC * 4u;
@@ -571,9 +571,9 @@ __device__ __noinline__ double pass_amul_dot_f32_bulk(Slots<float> A, int c0, in
 
 // M (FP32) over the bulk-staged rows where the launch gave the shared memory for them, else
 // the register form.
-template <int B, int W>
+template <int B, int W, class TM>
 __device__ __forceinline__ double amul_dot_f32(Slots<float> A, int c0, int c1, const float* __restrict__ p,
-                                               float* __restrict__ q, const Team& tm, bool& ok) {
+                                               float* __restrict__ q, const TM& tm, bool& ok) {
   ok = true;
   if constexpr (W > 0) {
     if (use_bulk_f32<B, W>(A)) return pass_amul_dot_f32_bulk<B, W>(A, c0, c1, p, q, tm, ok);
@@ -741,27 +741,42 @@ __device__ __forceinline__ void pass_correct(int c0, int c1, double* __restrict_
 }
 
 // Wall time per phase kind, measured by the team's rank-0 thread between barrier exits
-// (so each phase's share includes its barrier wait: the team's critical path).
+// (so each phase's share includes its barrier wait: the team's critical path). The times are
+// kept in shared memory and added to the launch's once per step, by adds that nothing waits
+// for: a load-add-store to global memory here stalled the rank-0 CTA, and with it the team,
+// for an L2 round trip per phase.
+template <int B, class TM>
 struct PhaseClock {
-  bool on;
-  unsigned long long t;
-  unsigned long long* acc;
-  __device__ __forceinline__ PhaseClock(const CaseDev& cs, const Team& tm)
-      : on(tm.rank == 0 && threadIdx.x == 0), t(0), acc(cs.sync->phase_ns) {
-    if (on) t = global_timer_ns();
+  const CaseDev& cs;
+  const TM& tm;
+  TeamShared<B>& sh;
+  __device__ __forceinline__ bool on() const { return tm.rank == 0 && threadIdx.x == 0; }
+  __device__ __forceinline__ PhaseClock(const CaseDev& c, const TM& t, TeamShared<B>& s) : cs(c), tm(t), sh(s) {
+    if (on()) {
+      for (int k = 0; k < kPhases; ++k) sh.phase[k] = 0;
+      sh.phase_t = global_timer_ns();
+    }
   }
   __device__ __forceinline__ void lap(int phase) {
-    if (on) {
+    if (on()) {
       const unsigned long long now = global_timer_ns();
-      acc[phase] += now - t;
-      t = now;
+      sh.phase[phase] += now - sh.phase_t;
+      sh.phase_t = now;
+    }
+  }
+  __device__ __forceinline__ void flush() {
+    if (on()) {
+      for (int k = 0; k < kPhases; ++k) {
+        if (sh.phase[k]) atomicAdd(&cs.sync->phase_ns[k], sh.phase[k]);
+        sh.phase[k] = 0;
+      }
     }
   }
 };
 
-__device__ __forceinline__ void write_stats(const CaseDev& cs, const Team& tm, int slot, int iters,
-                                            int conv, int sweeps, int status, double init_res,
-                                            double final_res, double nf) {
+template <class TM>
+__device__ __forceinline__ void write_stats(const CaseDev& cs, const TM& tm, int slot, int iters, int conv, int sweeps,
+                                            int status, double init_res, double final_res, double nf) {
   if (tm.rank == 0 && threadIdx.x == 0) {
     lfm_step_stats st;
     st.iters = iters;
@@ -775,28 +790,60 @@ __device__ __forceinline__ void write_stats(const CaseDev& cs, const Team& tm, i
   }
 }
 
+// ---- the scalars of a solve, formed inside the barriers by one lane (see lfm_device.cuh) ---
+// After M (one sum, sigma = p.Ap): lane 0 alpha = rho / sigma, lane 1 the singularity test; the
+// two divisions are one instruction sequence on two lanes.
+template <int B>
+__device__ __forceinline__ void fin_sigma(TeamShared<B>& sh, double sigma, int lane) {
+  const double q = (lane == 0 ? sh.rho : fabs(sigma)) / (lane == 0 ? sigma : sh.nf);
+  if (lane == 0) {
+    sh.alpha = q;
+    sh.alpha32 = (float)q;
+  }
+  if (lane == 1) sh.code = q < kVSmall ? kSingular : kGo;
+}
+
+// After U (sum 0 = sum|r|, sum 1 = w.r, in two warps): the scaled residual and whether to go
+// on after `iters` iterations (tol < 0: no absolute test), and beta = rho' / rho.
+template <int B>
+__device__ __forceinline__ void fin_update(TeamShared<B>& sh, int k, double t, int lane, double tol, double rel_tol,
+                                           int iters, int max_iter, int min_iter) {
+  if (lane != 0) return;
+  if (k == 0) {
+    const double res = t / sh.nf;
+    const bool conv = converged(res, sh.init_res, tol, rel_tol);
+    sh.res = res;
+    sh.conv = conv ? 1 : 0;
+    sh.code = !isfinite(res) ? kNonFinite : ((iters < max_iter && !conv) || iters < min_iter) ? kGo : kStop;
+  } else {
+    const double beta = t / sh.rho;
+    sh.beta = beta;
+    sh.beta32 = (float)beta;
+    sh.rho = t;
+  }
+}
+
 // Start of an assembly: the per-thread sums of T (with the faces for matrix read-back, the
 // copy of T at the start of the step when save_old, and with general geometry the Gauss
-// gradient in the same phase) and their team sum for xRef. False when a barrier failed (the
+// gradient in the same phase) and xRef, their team mean. False when a barrier failed (the
 // caller leaves the kernel).
-template <int B, int W, bool kMixed>
-__device__ __forceinline__ bool assemble_prologue(const CaseDev& cs, const CaseDev& cref, const Team& tm, int c0,
+template <int B, int W, bool kMixed, class TM>
+__device__ __forceinline__ bool assemble_prologue(const CaseDev& cs, const CaseDev& cref, const TM& tm, int c0,
                                                   int c1, int f0, int f1, bool write_upper, bool save_old,
-                                                  double& sum_x, TeamShared& sh) {
+                                                  TeamShared<B>& sh) {
   double v[1] = {pass_faces<B, kMixed>(cref, f0, f1, c0, c1, write_upper, save_old)};
   if (cs.Sf) pass_grad<B, W>(cref, c0, c1);
-  if (!team_allreduce<1>(tm, v, sh)) return false;
-  sum_x = v[0];
-  return true;
+  return team_allreduce<1, B>(tm, v, sh, [&](int, double t, int lane) {
+    if (lane == 0) sh.xref = t / (double)cs.N;
+  });
 }
 
 // =======================================================================================
 // FP64 steps (1 + n_corr assemble-and-solve passes per step)
 // =======================================================================================
-template <int B, int W>
-__device__ void run_steps_f64(const CaseDev& cs, const CaseDev& cref, const Team& tm, int n_steps, int mode,
-                              TeamShared& sh,
-                              int stats_base = 0) {
+template <int B, int W, class TM>
+__device__ void run_steps_f64(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps, int mode,
+                              TeamShared<B>& sh, int stats_base = 0) {
   int c0, c1, f0, f1;
   cta_range(cs.N, tm.size, tm.rank, c0, c1);
   cta_range(cs.F, tm.size, tm.rank, f0, f1);
@@ -808,17 +855,14 @@ __device__ void run_steps_f64(const CaseDev& cs, const CaseDev& cref, const Team
   double* __restrict__ q = cs.q;
   const double* __restrict__ rD = cs.rD;
 
-  PhaseClock clk(cs, tm);
+  PhaseClock<B, TM> clk(cs, tm, sh);
   const bool corr_mode = cs.n_corr > 0 || cs.Sf != nullptr || cs.vSu != nullptr || cs.vSp != nullptr;
   for (int step = 0; step < n_steps; ++step) {
     int iters_tot = 0, solves = 0, status = 0;
-    double nf0 = 0.0, init0 = 0.0, res = 0.0;
-    bool conv = false;
     for (int pass = 0; pass <= cs.n_corr; ++pass) {
       // ---- A1: face coefficients, sum of T (and the gradient / correction fluxes) --------
-      double sum_x = 0.0;
       if (!assemble_prologue<B, W, false>(cs, cref, tm, c0, c1, f0, f1, mode == kModeAssembleOnly,
-                                       pass == 0 && cs.n_corr > 0, sum_x, sh))
+                                          pass == 0 && cs.n_corr > 0, sh))
         return;
       clk.lap(kPhAssembly);
       if (mode == kModeAssembleOnly) {
@@ -826,63 +870,58 @@ __device__ void run_steps_f64(const CaseDev& cs, const CaseDev& cref, const Team
         return;
       }
       // ---- A2 + I: rows of the matrix, initial residual, normFactor, first direction -----
-      const double xRef = sum_x / (double)cs.N;
+      const double xRef = sh.xref;
       const Sums3 ui = corr_mode ? pass_rows_init_f64<B, W, true>(cref, c0, c1, xRef)
                                  : pass_rows_init_f64<B, W, false>(cref, c0, c1, xRef);
-      double u[3] = {ui.a, ui.b, ui.c};  // normFactor sum, sum|r|, rho
-      if (!team_allreduce<3>(tm, u, sh)) return;
+      const double u[3] = {ui.a, ui.b, ui.c};  // normFactor sum, sum|r|, rho
+      if (!team_allreduce<3, B>(tm, u, sh, [&](int k, double t, int lane) {
+            if (lane == 0) sh.out[k] = t;
+          }))
+        return;
       clk.lap(kPhInit);
-      const double nf = u[0] + kSmall;
-      const double init_res = u[1] / nf;
-      res = init_res;
-      double rho = u[2], beta = 0.0;
-      int iters = 0;
-      conv = converged(res, init_res, cs.tol, cs.rel_tol);
-      if (cs.min_iter > 0 || !conv) {
-        for (;;) {
-          if (iters > 0) {
-            // ---- P: search direction -----------------------------------------------
-            pass_direction<B, double>(c0, c1, beta, p, w);
-            if (!team_barrier(tm, sh)) return;
-            clk.lap(kPhP);
-          }
-          // ---- M: q = A p, sigma = p.q --------------------------------------------
-          double s1[1] = {pass_amul_dot_f64<B, W>(slots64(cs), c0, c1, p, q)};
-          if (!team_allreduce<1>(tm, s1, sh)) return;
-          clk.lap(kPhM);
-          const double sigma = s1[0];
-          if (fabs(sigma) / nf < kVSmall) {
-            status = LFM_ESINGULAR;
-            break;
-          }
-          const double alpha = rho / sigma;
-          // ---- U: update, residual, preconditioned residual, next rho --------------
-          const double2 su = pass_update_f64<B>(c0, c1, alpha, x, r, w, p, q, rD);
-          double s2[2] = {su.x, su.y};
-          if (!team_allreduce<2>(tm, s2, sh)) return;
-          clk.lap(kPhU);
-          res = s2[0] / nf;
-          beta = s2[1] / rho;
-          rho = s2[1];
-          ++iters;
-          if (!isfinite(res)) {
-            status = LFM_ENONFINITE;
-            break;
-          }
-          conv = converged(res, init_res, cs.tol, cs.rel_tol);
-          if (!((iters < cs.max_iter && !conv) || iters < cs.min_iter)) break;
+      if (tid == 0) {
+        sh.nf = sh.out[0] + kSmall;
+        sh.init_res = sh.res = sh.out[1] / sh.nf;
+        sh.rho = sh.out[2];
+        sh.conv = converged(sh.res, sh.init_res, cs.tol, cs.rel_tol) ? 1 : 0;
+        sh.code = cs.min_iter > 0 || !sh.conv ? kGo : kStop;
+        if (pass == 0) {
+          sh.nf0 = sh.nf;
+          sh.init0 = sh.init_res;
         }
       }
-      conv = converged(res, init_res, cs.tol, cs.rel_tol);
-      if (pass == 0) {
-        nf0 = nf;
-        init0 = init_res;
+      __syncthreads();
+      int iters = 0;
+      while (sh.code == kGo) {
+        if (iters > 0) {
+          // ---- P: search direction -----------------------------------------------
+          pass_direction<B, double>(c0, c1, sh.beta, p, w);
+          if (!team_barrier<B>(tm, sh)) return;
+          clk.lap(kPhP);
+        }
+        // ---- M: q = A p, sigma = p.q -> alpha ------------------------------------
+        const double s1[1] = {pass_amul_dot_f64<B, W>(slots64(cs), c0, c1, p, q)};
+        if (!team_allreduce<1, B>(tm, s1, sh, [&](int, double t, int lane) { fin_sigma(sh, t, lane); })) return;
+        clk.lap(kPhM);
+        if (sh.code != kGo) break;
+        // ---- U: update, residual, preconditioned residual, next rho -> beta ------
+        const double2 su = pass_update_f64<B>(c0, c1, sh.alpha, x, r, w, p, q, rD);
+        const double s2[2] = {su.x, su.y};
+        ++iters;
+        if (!team_allreduce<2, B>(tm, s2, sh, [&](int k, double t, int lane) {
+              fin_update(sh, k, t, lane, cs.tol, cs.rel_tol, iters, cs.max_iter, cs.min_iter);
+            }))
+          return;
+        clk.lap(kPhU);
       }
+      if (sh.code == kSingular) status = LFM_ESINGULAR;
+      if (sh.code == kNonFinite) status = LFM_ENONFINITE;
       iters_tot += iters;
       solves += iters > 0 ? 1 : 0;
       if (status != 0) break;
     }
-    write_stats(cs, tm, stats_base + step, iters_tot, conv ? 1 : 0, solves, status, init0, res, nf0);
+    write_stats(cs, tm, stats_base + step, iters_tot, sh.conv, solves, status, sh.init0, sh.res, sh.nf0);
+    clk.flush();
     if (status != 0) {
       if (tm.rank == 0 && tid == 0) set_status(cs.sync, status);
       return;
@@ -893,10 +932,74 @@ __device__ void run_steps_f64(const CaseDev& cs, const CaseDev& cref, const Team
 // =======================================================================================
 // Mixed-precision steps (FP32 inner CG inside FP64 defect correction)
 // =======================================================================================
-template <int B, int W>
-__device__ void run_steps_mixed(const CaseDev& cs, const CaseDev& cref, const Team& tm, int n_steps, int mode,
-                              TeamShared& sh,
-                                int stats_base = 0) {
+// Thread 0, with the totals of a true residual (normFactor with the small constant added, sum|r|,
+// rho): the outer residual, and whether another sweep of the inner solve follows.
+template <int B>
+__device__ __forceinline__ void mixed_outer(TeamShared<B>& sh, const CaseDev& cs, int pass, int sweeps, int iters,
+                                            double nf, double sum_r, double rho) {
+  if (sweeps == 0) {
+    sh.nf = nf;
+    sh.init_res = sum_r / nf;
+    if (pass == 0) {
+      sh.nf0 = nf;
+      sh.init0 = sh.init_res;
+    }
+  }
+  const double res = sum_r / sh.nf;
+  const bool ok = converged(res, sh.init_res, cs.tol, cs.rel_tol);
+  sh.res = res;
+  sh.conv = ok ? 1 : 0;
+  sh.rho = rho;
+  sh.inner_tol = fmax(cs.tol, kInnerRel * res);
+  sh.code = !isfinite(res) ? kNonFinite
+            : (ok && !(sweeps == 0 && cs.min_iter > 0)) || sweeps == kMaxSweeps || iters >= cs.max_iter ? kStop : kGo;
+}
+
+// The inner FP32 CG on A dx = r from its seed (r, p = w; sh.rho, sh.inner_tol): sh.code tells how
+// it ended. False when a barrier failed (the caller leaves).
+template <int B, int W, class TM>
+__device__ __forceinline__ bool inner_cg_f32(const CaseDev& cs, const TM& tm, TeamShared<B>& sh, PhaseClock<B, TM>& clk,
+                                             int c0, int c1, int min_inner, int& iters, float* __restrict__ dx,
+                                             float* __restrict__ r, float* __restrict__ w, float* __restrict__ p,
+                                             float* __restrict__ q, const float* __restrict__ rD) {
+  for (int k = 0;;) {
+    if (k > 0) {
+      pass_direction<B, float>(c0, c1, sh.beta32, p, w);
+      if (!team_barrier<B>(tm, sh)) return false;
+      clk.lap(kPhP);
+    }
+    bool m_ok;
+    const double s1[1] = {amul_dot_f32<B, W>(slots32(cs), c0, c1, p, q, tm, m_ok)};
+    if (!m_ok) return false;
+    if (!team_allreduce<1, B>(tm, s1, sh, [&](int, double t, int lane) { fin_sigma(sh, t, lane); })) return false;
+    clk.lap(kPhM);
+    if (sh.code != kGo) return true;
+    const double2 su = k == 0 ? pass_update_f32<B, true>(c0, c1, sh.alpha32, dx, r, w, p, q, rD)
+                              : pass_update_f32<B, false>(c0, c1, sh.alpha32, dx, r, w, p, q, rD);
+    const double s2[2] = {su.x, su.y};
+    ++k;
+    ++iters;
+    if (!team_allreduce<2, B>(tm, s2, sh, [&](int i, double t, int lane) {
+          if (lane != 0) return;
+          if (i == 0) {
+            const double res = t / sh.nf;
+            sh.code = !isfinite(res)                                                        ? kNonFinite
+                      : (iters < cs.max_iter && !(res < sh.inner_tol)) || k < min_inner ? kGo
+                                                                                            : kStop;
+          } else {
+            sh.beta32 = (float)(t / sh.rho);
+            sh.rho = t;
+          }
+        }))
+      return false;
+    clk.lap(kPhU);
+    if (sh.code != kGo) return true;
+  }
+}
+
+template <int B, int W, class TM>
+__device__ void run_steps_mixed(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps, int mode,
+                                TeamShared<B>& sh, int stats_base = 0) {
   int c0, c1, f0, f1;
   cta_range(cs.N, tm.size, tm.rank, c0, c1);
   cta_range(cs.F, tm.size, tm.rank, f0, f1);
@@ -909,25 +1012,21 @@ __device__ void run_steps_mixed(const CaseDev& cs, const CaseDev& cref, const Te
   float* __restrict__ q = cs.q32;
   const float* __restrict__ rD = cs.rD32;
 
-  PhaseClock clk(cs, tm);
+  PhaseClock<B, TM> clk(cs, tm, sh);
   const bool corr_mode = cs.n_corr > 0 || cs.Sf != nullptr || cs.vSu != nullptr || cs.vSp != nullptr;
   for (int step = 0; step < n_steps; ++step) {
     int iters_tot = 0, sweeps_tot = 0, status = 0;
-    double nf0 = 0.0, init0 = 0.0, res = 0.0;
-    bool conv = false;
     for (int pass = 0; pass <= cs.n_corr; ++pass) {
-      double sum_x = 0.0;
       if (!assemble_prologue<B, W, true>(cs, cref, tm, c0, c1, f0, f1, mode == kModeAssembleOnly,
-                                      pass == 0 && cs.n_corr > 0, sum_x, sh))
+                                         pass == 0 && cs.n_corr > 0, sh))
         return;
       clk.lap(kPhAssembly);
       if (mode == kModeAssembleOnly) {
         pass_rows_only<B, W, true>(cref, c0, c1);
         return;
       }
-      const double xRef = sum_x / (double)cs.N;
+      const double xRef = sh.xref;
 
-      double nf = 0.0, init_res = 0.0;
       int iters = 0, sweeps = 0;
       for (;;) {
         // ---- T: FP64 true residual r = b - A x, seeded into the FP32 inner solve; on the
@@ -939,76 +1038,35 @@ __device__ void run_steps_mixed(const CaseDev& cs, const CaseDev& cref, const Te
           ui = pass_true_residual<B, W, true, true>(cref, c0, c1, xRef);
         else
           ui = pass_true_residual<B, W, true, false>(cref, c0, c1, xRef);
-        double u[3] = {ui.a, ui.b, ui.c};  // normFactor sum (first sweep), sum|r|, rho
-        if (!team_allreduce<3>(tm, u, sh)) return;
+        const double u[3] = {ui.a, ui.b, ui.c};  // normFactor sum (first sweep), sum|r|, rho
+        if (!team_allreduce<3, B>(tm, u, sh, [&](int k, double t, int lane) {
+              if (lane == 0) sh.out[k] = t;
+            }))
+          return;
         clk.lap(kPhInit);
-        if (sweeps == 0) {
-          nf = u[0] + kSmall;
-          init_res = u[1] / nf;
-        }
-        res = u[1] / nf;
-        if (!isfinite(res)) {
-          status = LFM_ENONFINITE;
+        if (tid == 0) mixed_outer(sh, cs, pass, sweeps, iters, sh.out[0] + kSmall, sh.out[1], sh.out[2]);
+        __syncthreads();
+        if (sh.code != kGo) {
+          if (sh.code == kNonFinite) status = LFM_ENONFINITE;
           break;
         }
-        const bool c_ok = converged(res, init_res, cs.tol, cs.rel_tol);
-        if ((c_ok && !(sweeps == 0 && cs.min_iter > 0)) || sweeps == kMaxSweeps || iters >= cs.max_iter) break;
-
-        // ---- inner FP32 CG on A dx = r ------------------------------------------------
-        const double inner_tol = fmax(cs.tol, kInnerRel * res);
-        const int min_inner = sweeps == 0 ? cs.min_iter : 0;
-        double rho = u[2], beta = 0.0;
-        int k = 0;
-        for (;;) {
-          if (k > 0) {
-            pass_direction<B, float>(c0, c1, (float)beta, p, w);
-            if (!team_barrier(tm, sh)) return;
-            clk.lap(kPhP);
-          }
-          bool m_ok;
-          double s1[1] = {amul_dot_f32<B, W>(slots32(cs), c0, c1, p, q, tm, m_ok)};
-          if (!m_ok) return;
-          if (!team_allreduce<1>(tm, s1, sh)) return;
-          clk.lap(kPhM);
-          const double sigma = s1[0];
-          if (fabs(sigma) / nf < kVSmall) {
-            status = LFM_ESINGULAR;
-            break;
-          }
-          const double2 su = k == 0 ? pass_update_f32<B, true>(c0, c1, (float)(rho / sigma), dx, r, w, p, q, rD)
-                                    : pass_update_f32<B, false>(c0, c1, (float)(rho / sigma), dx, r, w, p, q, rD);
-          double s2[2] = {su.x, su.y};
-          if (!team_allreduce<2>(tm, s2, sh)) return;
-          clk.lap(kPhU);
-          const double inner_res = s2[0] / nf;
-          beta = s2[1] / rho;
-          rho = s2[1];
-          ++k;
-          ++iters;
-          if (!isfinite(inner_res)) {
-            status = LFM_ENONFINITE;
-            break;
-          }
-          const bool inner_conv = inner_res < inner_tol;
-          if (!((iters < cs.max_iter && !inner_conv) || k < min_inner)) break;
-        }
+        if (!inner_cg_f32<B, W>(cs, tm, sh, clk, c0, c1, sweeps == 0 ? cs.min_iter : 0, iters, dx, r, w, p, q, rD))
+          return;
+        if (sh.code == kSingular) status = LFM_ESINGULAR;
+        if (sh.code == kNonFinite) status = LFM_ENONFINITE;
         if (status != 0) break;
         // ---- x += dx (FP64) ----------------------------------------------------------
         pass_correct<B>(c0, c1, x, dx);
-        if (!team_barrier(tm, sh)) return;
+        if (!team_barrier<B>(tm, sh)) return;
         clk.lap(kPhCorrect);
         ++sweeps;
-      }
-      conv = converged(res, init_res, cs.tol, cs.rel_tol);
-      if (pass == 0) {
-        nf0 = nf;
-        init0 = init_res;
       }
       iters_tot += iters;
       sweeps_tot += sweeps;
       if (status != 0) break;
     }
-    write_stats(cs, tm, stats_base + step, iters_tot, conv ? 1 : 0, sweeps_tot, status, init0, res, nf0);
+    write_stats(cs, tm, stats_base + step, iters_tot, sh.conv, sweeps_tot, status, sh.init0, sh.res, sh.nf0);
+    clk.flush();
     if (status != 0) {
       if (tm.rank == 0 && tid == 0) set_status(cs.sync, status);
       return;

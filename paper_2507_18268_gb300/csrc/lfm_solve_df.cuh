@@ -52,7 +52,17 @@
 namespace lfm {
 namespace {
 
-__device__ __forceinline__ df df_from_scalar(double v) { return df_from_double(v); }
+__device__ __forceinline__ float2 pair_of(double v) {
+  const df d = df_from_double(v);
+  return make_float2(d.hi, d.lo);
+}
+__device__ __forceinline__ df df_of(float2 v) { return mkdf(v.x, v.y); }
+
+// The team mean of the field as a pair (xRef), formed in the barrier that carries its sum.
+template <int B>
+__device__ __forceinline__ void fin_mean_df(TeamShared<B>& sh, const CaseDev& cs, double t, int lane) {
+  if (lane == 0) sh.xref2 = pair_of(t / (double)cs.N);
+}
 
 // S: this thread's sum of x over [c0, c1) (per-thread df64 sum, converted once). `convert`:
 // first pass of the launch, the triple-float field is split from the FP64 field x. `fold`:
@@ -101,7 +111,8 @@ __device__ __noinline__ double pass_sum_df(const CaseDev& cs, int c0, int c1, bo
 // After the first barrier of a launch that split the FP64 field: every CTA has read the flag,
 // so the team's rank 0 marks the triple-float field current (it persists across launches:
 // the FP64 field is only its rounding, rewritten at the end of every launch).
-__device__ __forceinline__ void mark_split(const CaseDev& cs, const Team& tm, bool& convert) {
+template <class TM>
+__device__ __forceinline__ void mark_split(const CaseDev& cs, const TM& tm, bool& convert) {
   if (convert && tm.rank == 0 && threadIdx.x == 0) *reinterpret_cast<volatile int32_t*>(cs.flags) = 1;
   convert = false;
 }
@@ -254,14 +265,13 @@ __device__ __forceinline__ void prefetch_row_df(const CaseDev& cs, int c) {
 // differences of nearby values here are almost exact, so r keeps the format's relative
 // accuracy. A x for the normFactor terms is then b - r.
 template <int B, int W, bool kSrc>
-__device__ __noinline__ Sums3 pass_rows_init_df(const CaseDev& cs, int c0, int c1, double xRef) {
+__device__ __noinline__ Sums3 pass_rows_init_df(const CaseDev& cs, int c0, int c1, df xr) {
   const float2* __restrict__ x2 = cs.x2;
   const float* __restrict__ xl = cs.xlo;
   const float2* __restrict__ g2 = cs.g2;
   float2* __restrict__ r2 = reinterpret_cast<float2*>(cs.r);
   float2* __restrict__ p2 = reinterpret_cast<float2*>(cs.p);
   const size_t N = (size_t)cs.N;
-  const df xr = df_from_scalar(xRef);
   DfAcc a_nf, a_r, a_rho;
   for (int c = c0 + (int)threadIdx.x; c < c1; c += B) {
     if (c + B < c1) prefetch_row_df<W>(cs, c + B);
@@ -358,11 +368,15 @@ __device__ __forceinline__ void rows2_df(const CaseDev& cs, int c, int c2, const
       g[k] = df{a.x, a.y};
       h[k] = df{b.x, b.y};
     }
+    df xo[W], xo2[W];
 #pragma unroll
-    for (int k = 0; k < W; ++k) {
-      acc = df_fma(df_neg(g[k]), ld_df(v + o[k]), acc);
-      acc2 = df_fma(df_neg(h[k]), ld_df(v + o2[k]), acc2);
-    }
+    for (int k = 0; k < W; ++k) xo[k] = ld_df(v + o[k]);
+#pragma unroll
+    for (int k = 0; k < W; ++k) xo2[k] = ld_df(v + o2[k]);
+#pragma unroll
+    for (int k = 0; k < W; ++k) acc = df_fma(df_neg(g[k]), xo[k], acc);
+#pragma unroll
+    for (int k = 0; k < W; ++k) acc2 = df_fma(df_neg(h[k]), xo2[k], acc2);
   } else {
     for (int k = 0; k < cs.W; ++k) {
       const size_t at = (size_t)k * N;
@@ -479,8 +493,8 @@ __device__ __forceinline__ double2 pass_update_df(int c0, int c1, df alpha, floa
 // The steps of one launch. Returns false when a barrier failed (the caller leaves).
 // `pending` tracks whether e holds a correction not yet added to the field (the same in every
 // CTA: it follows the team-wide iteration counts).
-template <int B, int W, bool kGeom>
-__device__ bool steps_df64(const CaseDev& cs, const CaseDev& cref, const Team& tm, int n_steps, TeamShared& sh,
+template <int B, int W, bool kGeom, class TM>
+__device__ bool steps_df64(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps, TeamShared<B>& sh,
                            int stats_base, int c0, int c1, bool& pending) {
   const int tid = threadIdx.x;
   float2* __restrict__ e = cs.e2;
@@ -489,85 +503,81 @@ __device__ bool steps_df64(const CaseDev& cs, const CaseDev& cref, const Team& t
   float2* __restrict__ p = reinterpret_cast<float2*>(cs.p);
   float2* __restrict__ q = reinterpret_cast<float2*>(cs.q);
   const float2* __restrict__ rD = cs.rD2;
-  const double inv_scale = 1.0 / cs.df_scale;  // a power of two: exact
 
-  PhaseClock clk(cs, tm);
+  PhaseClock<B, TM> clk(cs, tm, sh);
   const bool src_mode = cs.n_corr > 0 || cs.vSu != nullptr || cs.vSp != nullptr || (kGeom && cs.Sf != nullptr);
   bool convert = ld_volatile_i32(cs.flags) == 0;  // read by every CTA before the first barrier
   for (int step = 0; step < n_steps; ++step) {
     int iters_tot = 0, solves = 0, status = 0;
-    double nf0 = 0.0, init0 = 0.0, res = 0.0;
-    bool conv = false;
     for (int pass = 0; pass <= cs.n_corr; ++pass) {
       // ---- S: sum of x (first pass of the launch: split the FP64 field; otherwise the last
       //      solve's correction is added first) ---------------------------------------------
-      double v[1] = {pass_sum_df<B>(cref, c0, c1, convert, pending, pass == 0 && cs.n_corr > 0)};
+      const double v[1] = {pass_sum_df<B>(cref, c0, c1, convert, pending, pass == 0 && cs.n_corr > 0)};
       pending = false;
-      if (!team_allreduce<1>(tm, v, sh)) return false;
+      if (!team_allreduce<1, B>(tm, v, sh, [&](int, double t, int lane) { fin_mean_df(sh, cs, t, lane); })) return false;
       mark_split(cs, tm, convert);
       if constexpr (kGeom) {
         if (cs.Sf) {  // ---- G: the gradient of the (folded) field, for the correction --------
           pass_grad_df<B, W>(cref, c0, c1);
-          if (!team_barrier(tm, sh)) return false;
+          if (!team_barrier<B>(tm, sh)) return false;
         }
       }
       clk.lap(kPhAssembly);
       // ---- R: rows, initial residual, normFactor, first direction ----------------------
-      const double xRef = v[0] / (double)cs.N;
-      const Sums3 ui = src_mode ? pass_rows_init_df<B, W, true>(cref, c0, c1, xRef)
-                                : pass_rows_init_df<B, W, false>(cref, c0, c1, xRef);
-      double u[3] = {ui.a, ui.b, ui.c};
-      if (!team_allreduce<3>(tm, u, sh)) return false;
+      const Sums3 ui = src_mode ? pass_rows_init_df<B, W, true>(cref, c0, c1, df_of(sh.xref2))
+                                : pass_rows_init_df<B, W, false>(cref, c0, c1, df_of(sh.xref2));
+      const double u[3] = {ui.a, ui.b, ui.c};
+      if (!team_allreduce<3, B>(tm, u, sh, [&](int k, double t, int lane) {
+            if (lane == 0) sh.out[k] = t;
+          }))
+        return false;
       clk.lap(kPhInit);
-      const double nf = u[0] + kSmall * cs.df_scale;
-      const double init_res = u[1] / nf;
-      res = init_res;
-      double rho = u[2], beta = 0.0;
-      int iters = 0;
-      conv = converged(res, init_res, cs.tol, cs.rel_tol);
-      if (cs.min_iter > 0 || !conv) {
-        for (;;) {
-          if (iters > 0) {
-            pass_direction_df<B>(c0, c1, df_from_scalar(beta), p, w);
-            if (!team_barrier(tm, sh)) return false;
-            clk.lap(kPhP);
-          }
-          double s1[1] = {pass_amul_dot_df<B, W>(cs, c0, c1, p, q)};
-          if (!team_allreduce<1>(tm, s1, sh)) return false;
-          clk.lap(kPhM);
-          const double sigma = s1[0];
-          if (fabs(sigma) / nf < kVSmall) {
-            status = LFM_ESINGULAR;
-            break;
-          }
-          const double alpha = rho / sigma;
-          const double2 su = pass_update_df<B>(c0, c1, df_from_scalar(alpha), e, iters == 0, r, w, p, q, rD);
-          pending = true;
-          double s2[2] = {su.x, su.y};
-          if (!team_allreduce<2>(tm, s2, sh)) return false;
-          clk.lap(kPhU);
-          res = s2[0] / nf;
-          beta = s2[1] / rho;
-          rho = s2[1];
-          ++iters;
-          if (!isfinite(res)) {
-            status = LFM_ENONFINITE;
-            break;
-          }
-          conv = converged(res, init_res, cs.tol, cs.rel_tol);
-          if (!((iters < cs.max_iter && !conv) || iters < cs.min_iter)) break;
+      if (tid == 0) {
+        sh.nf = sh.out[0] + kSmall * cs.df_scale;
+        sh.init_res = sh.res = sh.out[1] / sh.nf;
+        sh.rho = sh.out[2];
+        sh.conv = converged(sh.res, sh.init_res, cs.tol, cs.rel_tol) ? 1 : 0;
+        sh.code = cs.min_iter > 0 || !sh.conv ? kGo : kStop;
+        if (pass == 0) {
+          sh.nf0 = sh.nf * (1.0 / cs.df_scale);  // a power of two: exact
+          sh.init0 = sh.init_res;
         }
       }
-      conv = converged(res, init_res, cs.tol, cs.rel_tol);
-      if (pass == 0) {
-        nf0 = nf * inv_scale;
-        init0 = init_res;
+      __syncthreads();
+      int iters = 0;
+      while (sh.code == kGo) {
+        if (iters > 0) {
+          pass_direction_df<B>(c0, c1, df_of(sh.beta2), p, w);
+          if (!team_barrier<B>(tm, sh)) return false;
+          clk.lap(kPhP);
+        }
+        const double s1[1] = {pass_amul_dot_df<B, W>(cs, c0, c1, p, q)};
+        if (!team_allreduce<1, B>(tm, s1, sh, [&](int, double t, int lane) {
+              fin_sigma(sh, t, lane);
+              if (lane == 0) sh.alpha2 = pair_of(sh.alpha);
+            }))
+          return false;
+        clk.lap(kPhM);
+        if (sh.code != kGo) break;
+        const double2 su = pass_update_df<B>(c0, c1, df_of(sh.alpha2), e, iters == 0, r, w, p, q, rD);
+        pending = true;
+        const double s2[2] = {su.x, su.y};
+        ++iters;
+        if (!team_allreduce<2, B>(tm, s2, sh, [&](int k, double t, int lane) {
+              fin_update(sh, k, t, lane, cs.tol, cs.rel_tol, iters, cs.max_iter, cs.min_iter);
+              if (k == 1 && lane == 0) sh.beta2 = pair_of(sh.beta);
+            }))
+          return false;
+        clk.lap(kPhU);
       }
+      if (sh.code == kSingular) status = LFM_ESINGULAR;
+      if (sh.code == kNonFinite) status = LFM_ENONFINITE;
       iters_tot += iters;
       solves += iters > 0 ? 1 : 0;
       if (status != 0) break;
     }
-    write_stats(cs, tm, stats_base + step, iters_tot, conv ? 1 : 0, solves, status, init0, res, nf0);
+    write_stats(cs, tm, stats_base + step, iters_tot, sh.conv, solves, status, sh.init0, sh.res, sh.nf0);
+    clk.flush();
     if (status != 0) {
       if (tm.rank == 0 && tid == 0) set_status(cs.sync, status);
       return true;
@@ -577,8 +587,8 @@ __device__ bool steps_df64(const CaseDev& cs, const CaseDev& cref, const Team& t
 }
 
 // kGeom: the kernel serves general geometry (the gradient phase is compiled in).
-template <int B, int W, bool kGeom = false>
-__device__ void run_steps_df64(const CaseDev& cs, const CaseDev& cref, const Team& tm, int n_steps, TeamShared& sh,
+template <int B, int W, bool kGeom = false, class TM>
+__device__ void run_steps_df64(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps, TeamShared<B>& sh,
                                int stats_base = 0) {
   if (n_steps <= 0) return;
   int c0, c1;

@@ -107,9 +107,8 @@ __device__ __forceinline__ void seed_row_df(const CaseDev& cs, int c, df d, df s
 // the caller unscales) and the seed of the inner solve. kSrc: correctors (ddt source from
 // x_old) or volumetric sources present.
 template <int B, int W, bool kSrc>
-__device__ __noinline__ Sums3 pass_rows_init_mixed_df(const CaseDev& cs, int c0, int c1, double xRef, float s32,
+__device__ __noinline__ Sums3 pass_rows_init_mixed_df(const CaseDev& cs, int c0, int c1, df xr, float s32,
                                                       float inv_s32) {
-  const df xr = df_from_scalar(xRef);
   DfAcc a_nf, a_r;
   Acc2f a_rho;
   for (int c = c0 + (int)threadIdx.x; c < c1; c += B) {
@@ -177,12 +176,11 @@ struct Sums4 {
 };
 
 // V: the step's verification residual and the next step's T0 in one pass over the rows (no
-// sources, no correctors; see the head of this file). xRef_next: mean of the corrected x.
+// sources, no correctors; see the head of this file). xr: mean of the corrected x.
 // Returns sum|r_v| (scaled), then the next step's normFactor sum, sum|r'| and rho.
 template <int B, int W>
-__device__ __noinline__ Sums4 pass_verify_next_df(const CaseDev& cs, int c0, int c1, double xRef_next, float s32,
+__device__ __noinline__ Sums4 pass_verify_next_df(const CaseDev& cs, int c0, int c1, df xr, float s32,
                                                     float inv_s32) {
-  const df xr = df_from_scalar(xRef_next);
   DfAcc a_v, a_nf, a_r;
   Acc2f a_rho;
   for (int c = c0 + (int)threadIdx.x; c < c1; c += B) {
@@ -255,8 +253,8 @@ __device__ __forceinline__ bool mixed_uses_df(const CaseDev& cs) {
   return cs.x2 != nullptr && cs.Sf == nullptr && cs.df_scale >= 0x1p-100 && cs.df_scale <= 0x1p100;
 }
 
-template <int B, int W>
-__device__ bool steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const Team& tm, int n_steps, TeamShared& sh,
+template <int B, int W, class TM>
+__device__ bool steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps, TeamShared<B>& sh,
                                int stats_base, int c0, int c1) {
   const int tid = threadIdx.x;
   float* __restrict__ dx = cs.dx32;
@@ -265,53 +263,43 @@ __device__ bool steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const Tea
   float* __restrict__ p = cs.p32;
   float* __restrict__ q = cs.q32;
   const float* __restrict__ rD = cs.rD32;
-  const double inv_scale = 1.0 / cs.df_scale;  // a power of two: exact
-  const float s32 = (float)cs.df_scale, inv_s32 = (float)inv_scale;
+  const float s32 = (float)cs.df_scale, inv_s32 = (float)(1.0 / cs.df_scale);  // powers of two: exact
 
-  PhaseClock clk(cs, tm);
+  PhaseClock<B, TM> clk(cs, tm, sh);
   const bool src_mode = cs.n_corr > 0 || cs.vSu != nullptr || cs.vSp != nullptr;
   const bool fuse = !src_mode;  // verification fused with the next step's T0 (pass V)
   // this step's rows and seed come from the last V pass: of this launch, or of the last
   // launch when it ended with them in place and nothing changed since (flags[1], cleared by
   // the host with every change to the case; read by every CTA before the first barrier)
   bool seeded = fuse && ld_volatile_i32(cs.flags + 1) != 0 && ld_volatile_i32(cs.flags) != 0;
-  double seed[3] = {0.0, 0.0, 0.0};  // their team totals: normFactor sum, sum|r|, rho
-  if (seeded) {
-    seed[0] = __ldcg(cs.seed_sums);
-    seed[1] = __ldcg(cs.seed_sums + 1);
-    seed[2] = __ldcg(cs.seed_sums + 2);
-  }
+  if (seeded && tid == 0)
+    for (int k = 0; k < 3; ++k) sh.seed[k] = __ldcg(cs.seed_sums + k);  // normFactor sum, sum|r|, rho
   bool convert = ld_volatile_i32(cs.flags) == 0;  // read by every CTA before the first barrier
   for (int step = 0; step < n_steps; ++step) {
     int iters_tot = 0, sweeps_tot = 0, status = 0;
-    double nf0 = 0.0, init0 = 0.0, res = 0.0;
-    bool conv = false;
     for (int pass = 0; pass <= cs.n_corr; ++pass) {
-      double xRef = 0.0;
       // x_old holds the step's starting field once S ran (pass 0 saves it, later passes keep
       // it); a seeded step saves it at its first correction
       bool old_saved = !seeded;
       bool have_u = seeded;
-      double u[3] = {seed[0], seed[1], seed[2]};
       seeded = false;
-      // consumed: constants from here on, so that no register holds them through the sweeps
-      seed[0] = seed[1] = seed[2] = 0.0;
-      if (have_u == false) {
+      if (!have_u) {
         // ---- S: sum of x; the step's starting field (T1's ddt term) ------------------
-        double v[1] = {pass_sum_df<B>(cref, c0, c1, convert, false, pass == 0)};
-        if (!team_allreduce<1>(tm, v, sh)) return false;
+        const double v[1] = {pass_sum_df<B>(cref, c0, c1, convert, false, pass == 0)};
+        if (!team_allreduce<1, B>(tm, v, sh, [&](int, double t, int lane) { fin_mean_df(sh, cs, t, lane); }))
+          return false;
         mark_split(cs, tm, convert);
         clk.lap(kPhAssembly);
-        xRef = v[0] / (double)cs.N;
       }
-      double nf = 0.0, init_res = 0.0;
       int iters = 0, sweeps = 0;
       for (;;) {
         // ---- T0 (rows + true residual) or T1 (true residual after a correction) ----------
         if (!have_u) {
+          double u[3];
           if (sweeps == 0) {
-            const Sums3 ui = src_mode ? pass_rows_init_mixed_df<B, W, true>(cref, c0, c1, xRef, s32, inv_s32)
-                                      : pass_rows_init_mixed_df<B, W, false>(cref, c0, c1, xRef, s32, inv_s32);
+            const Sums3 ui = src_mode
+                                 ? pass_rows_init_mixed_df<B, W, true>(cref, c0, c1, df_of(sh.xref2), s32, inv_s32)
+                                 : pass_rows_init_mixed_df<B, W, false>(cref, c0, c1, df_of(sh.xref2), s32, inv_s32);
             u[0] = ui.a;
             u[1] = ui.b;
             u[2] = ui.c;
@@ -322,98 +310,72 @@ __device__ bool steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const Tea
             u[1] = ut.x;
             u[2] = ut.y;
           }
-          if (!team_allreduce<3>(tm, u, sh)) return false;
+          if (!team_allreduce<3, B>(tm, u, sh, [&](int k, double t, int lane) {
+                if (lane == 0) sh.seed[k] = t;
+              }))
+            return false;
           clk.lap(kPhInit);
         }
         have_u = false;
-        if (sweeps == 0) {
-          nf = (u[0] + kSmall * cs.df_scale) * inv_scale;
-          init_res = u[1] * inv_scale / nf;
+        if (tid == 0) {
+          const double inv_scale = 1.0 / cs.df_scale;
+          mixed_outer(sh, cs, pass, sweeps, iters, (sh.seed[0] + kSmall * cs.df_scale) * inv_scale,
+                      sh.seed[1] * inv_scale, sh.seed[2]);
         }
-        res = u[1] * inv_scale / nf;
-        if (!isfinite(res)) {
-          status = LFM_ENONFINITE;
+        __syncthreads();
+        if (sh.code != kGo) {
+          if (sh.code == kNonFinite) status = LFM_ENONFINITE;
           break;
         }
-        const bool c_ok = converged(res, init_res, cs.tol, cs.rel_tol);
-        if ((c_ok && !(sweeps == 0 && cs.min_iter > 0)) || sweeps == kMaxSweeps || iters >= cs.max_iter) break;
-
         // ---- inner FP32 CG on A dx = r (unscaled) -----------------------------------------
-        const double inner_tol = fmax(cs.tol, kInnerRel * res);
-        const int min_inner = sweeps == 0 ? cs.min_iter : 0;
-        double rho = u[2], beta = 0.0;
-        int k = 0;
-        for (;;) {
-          if (k > 0) {
-            pass_direction<B, float>(c0, c1, (float)beta, p, w);
-            if (!team_barrier(tm, sh)) return false;
-            clk.lap(kPhP);
-          }
-          bool m_ok;
-          double s1[1] = {amul_dot_f32<B, W>(slots32(cs), c0, c1, p, q, tm, m_ok)};
-          if (!m_ok) return false;
-          if (!team_allreduce<1>(tm, s1, sh)) return false;
-          clk.lap(kPhM);
-          const double sigma = s1[0];
-          if (fabs(sigma) / nf < kVSmall) {
-            status = LFM_ESINGULAR;
-            break;
-          }
-          const double2 su = k == 0 ? pass_update_f32<B, true>(c0, c1, (float)(rho / sigma), dx, r, w, p, q, rD)
-                                    : pass_update_f32<B, false>(c0, c1, (float)(rho / sigma), dx, r, w, p, q, rD);
-          double s2[2] = {su.x, su.y};
-          if (!team_allreduce<2>(tm, s2, sh)) return false;
-          clk.lap(kPhU);
-          const double inner_res = s2[0] / nf;
-          beta = s2[1] / rho;
-          rho = s2[1];
-          ++k;
-          ++iters;
-          if (!isfinite(inner_res)) {
-            status = LFM_ENONFINITE;
-            break;
-          }
-          const bool inner_conv = inner_res < inner_tol;
-          if (!((iters < cs.max_iter && !inner_conv) || k < min_inner)) break;
-        }
+        if (!inner_cg_f32<B, W>(cs, tm, sh, clk, c0, c1, sweeps == 0 ? cs.min_iter : 0, iters, dx, r, w, p, q, rD))
+          return false;
+        if (sh.code == kSingular) status = LFM_ESINGULAR;
+        if (sh.code == kNonFinite) status = LFM_ENONFINITE;
         if (status != 0) break;
         // ---- C: x += dx --------------------------------------------------------------------
-        double sx[1] = {pass_correct_df<B>(cref, c0, c1, !old_saved)};
-        if (!team_allreduce<1>(tm, sx, sh)) return false;
+        const double sx[1] = {pass_correct_df<B>(cref, c0, c1, !old_saved)};
+        if (!team_allreduce<1, B>(tm, sx, sh, [&](int, double t, int lane) { fin_mean_df(sh, cs, t, lane); }))
+          return false;
         old_saved = true;
         clk.lap(kPhCorrect);
         ++sweeps;
         if (fuse) {
           // ---- V: the verification residual and the next step's T0 -----------------------
-          const Sums4 uv = pass_verify_next_df<B, W>(cref, c0, c1, sx[0] / (double)cs.N, s32, inv_s32);
-          double v4[4] = {uv.a, uv.b, uv.c, uv.d};
-          if (!team_allreduce<4>(tm, v4, sh)) return false;
+          const Sums4 uv = pass_verify_next_df<B, W>(cref, c0, c1, df_of(sh.xref2), s32, inv_s32);
+          const double v4[4] = {uv.a, uv.b, uv.c, uv.d};
+          if (!team_allreduce<4, B>(tm, v4, sh, [&](int k, double t, int lane) {
+                if (lane != 0) return;
+                if (k > 0) {
+                  sh.seed[k - 1] = t;
+                  return;
+                }
+                const double res = t * (1.0 / cs.df_scale) / sh.nf;
+                const bool ok = converged(res, sh.init_res, cs.tol, cs.rel_tol);
+                sh.res = res;
+                sh.conv = ok ? 1 : 0;
+                sh.code = !isfinite(res) ? kNonFinite
+                          : ok || sweeps == kMaxSweeps || iters >= cs.max_iter ? kStop : kGo;
+              }))
+            return false;
           clk.lap(kPhInit);
-          res = v4[0] * inv_scale / nf;
-          if (!isfinite(res)) {
+          if (sh.code == kNonFinite) {
             status = LFM_ENONFINITE;
             break;
           }
-          if (converged(res, init_res, cs.tol, cs.rel_tol) || sweeps == kMaxSweeps || iters >= cs.max_iter) {
+          if (sh.code == kStop) {
             seeded = true;  // the step ends with this x: the next one starts from V's rows
-            seed[0] = v4[1];
-            seed[1] = v4[2];
-            seed[2] = v4[3];
             break;
           }
           // another sweep: T1 re-seeds the inner solve from the verification residual
         }
       }
-      conv = converged(res, init_res, cs.tol, cs.rel_tol);
-      if (pass == 0) {
-        nf0 = nf;
-        init0 = init_res;
-      }
       iters_tot += iters;
       sweeps_tot += sweeps;
       if (status != 0) break;
     }
-    write_stats(cs, tm, stats_base + step, iters_tot, conv ? 1 : 0, sweeps_tot, status, init0, res, nf0);
+    write_stats(cs, tm, stats_base + step, iters_tot, sh.conv, sweeps_tot, status, sh.init0, sh.res, sh.nf0);
+    clk.flush();
     if (status != 0) {
       if (tm.rank == 0 && tid == 0) set_status(cs.sync, status);
       return true;
@@ -422,20 +384,17 @@ __device__ bool steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const Tea
   // the launch ends: whether the next step's rows and seed are in place, for the next launch
   // (every CTA read flags[1] before the first barrier of this launch)
   if (tm.rank == 0 && tid == 0) {
-    if (seeded) {
-      cs.seed_sums[0] = seed[0];
-      cs.seed_sums[1] = seed[1];
-      cs.seed_sums[2] = seed[2];
-    }
+    if (seeded)
+      for (int k = 0; k < 3; ++k) cs.seed_sums[k] = sh.seed[k];
     *reinterpret_cast<volatile int32_t*>(cs.flags + 1) = seeded ? 1 : 0;
   }
   return true;
 }
 
 // The mixed form with df64 outer passes (the case must satisfy mixed_uses_df).
-template <int B, int W>
-__device__ void run_steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const Team& tm, int n_steps,
-                                   TeamShared& sh, int stats_base = 0) {
+template <int B, int W, class TM>
+__device__ void run_steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps,
+                                   TeamShared<B>& sh, int stats_base = 0) {
   if (n_steps <= 0) return;
   int c0, c1;
   cta_range(cs.N, tm.size, tm.rank, c0, c1);
@@ -444,9 +403,9 @@ __device__ void run_steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const
 }
 
 // The mixed form: df64 outer passes where mixed_uses_df, else FP64 ones (lfm_solve.cuh).
-template <int B, int W>
-__device__ void run_steps_mixed_any(const CaseDev& cs, const CaseDev& cref, const Team& tm, int n_steps, int mode,
-                                    TeamShared& sh, int stats_base = 0) {
+template <int B, int W, class TM>
+__device__ void run_steps_mixed_any(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps, int mode,
+                                    TeamShared<B>& sh, int stats_base = 0) {
   if (mode != kModeSteps || !mixed_uses_df(cs))
     run_steps_mixed<B, W>(cs, cref, tm, n_steps, mode, sh, stats_base);
   else

@@ -18,7 +18,7 @@ namespace {
 // ---- kernels ---------------------------------------------------------------------------
 template <int B, int W>
 __global__ void __launch_bounds__(B, 1024 / B) step_kernel_f64(CaseDev cs, Launch L, int n_steps, int mode) {
-  __shared__ TeamShared sh;
+  __shared__ TeamShared<B> sh;
   __shared__ CaseDev s_cs;  // addressable copy for the per-step passes
   if ((int)blockIdx.x == L.skip_cta) return;  // test hook: never arrive
   if (threadIdx.x == 0) s_cs = cs;
@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(B, 1024 / B) step_kernel_f64(CaseDev cs, Launc
 
 template <int B, int W>
 __global__ void __launch_bounds__(B, 1024 / B) step_kernel_mixed(CaseDev cs, Launch L, int n_steps, int mode) {
-  __shared__ TeamShared sh;
+  __shared__ TeamShared<B> sh;
   __shared__ CaseDev s_cs;  // addressable copy for the per-step passes
   if ((int)blockIdx.x == L.skip_cta) return;
   if (threadIdx.x == 0) s_cs = cs;
@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(B, 1024 / B) step_kernel_mixed(CaseDev cs, Lau
 // The mixed form with df64 outer passes (orthogonal meshes; the host chooses it).
 template <int B, int W>
 __global__ void __launch_bounds__(B, 1024 / B) step_kernel_mixed_df(CaseDev cs, Launch L, int n_steps, int mode) {
-  __shared__ TeamShared sh;
+  __shared__ TeamShared<B> sh;
   __shared__ CaseDev s_cs;
   if ((int)blockIdx.x == L.skip_cta) return;
   if (threadIdx.x == 0) s_cs = cs;
@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(B, 1024 / B) step_kernel_mixed_df(CaseDev cs, 
 
 template <int B, int W, bool kGeom>
 __global__ void __launch_bounds__(B, 1024 / B) step_kernel_df64(CaseDev cs, Launch L, int n_steps, int mode) {
-  __shared__ TeamShared sh;
+  __shared__ TeamShared<B> sh;
   __shared__ CaseDev s_cs;  // addressable copy for the per-step passes
   if ((int)blockIdx.x == L.skip_cta) return;
   if (threadIdx.x == 0) s_cs = cs;
@@ -380,7 +380,7 @@ int max_coresident_ctas(int precision, int threads, int W, int device) {
   if (per_sm <= 0) return 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
   int n = per_sm * sms;
-  return n < kMaxCtas ? n : kMaxCtas;
+  return n < kMaxCtas / 2 ? n : kMaxCtas / 2;  // the partial sums' table holds two buffers
 }
 
 cudaError_t launch_steps(const CaseDev& cs, const Launch& L, int n_steps, int mode,
