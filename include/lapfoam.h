@@ -371,6 +371,13 @@ int lfm_debug_staged_passes(lfm_ctx *ctx, int64_t *n);
  * that. */
 int lfm_debug_stage_rows(lfm_ctx *ctx, int32_t on);
 
+/* Test switch: on != 0 (the default) lets the kernels read a six-slot mesh's neighbours from
+ * packed codes where its neighbour distances are few enough (a naturally numbered box), on == 0
+ * from the slot rows, with bitwise the same results. n (may be NULL) receives the number of
+ * distinct distances, 0 where the mesh does not pack. LFM_ESTATE before a mesh is uploaded or
+ * while an advance is pending. */
+int lfm_debug_pack_slots(lfm_ctx *ctx, int32_t on, int32_t *n);
+
 /* 1 when this library is the checked build (compiled with LFM_CHECKED, liblapfoam_checked.so),
  * else 0. In the checked build every kernel tests each index it reads from the mesh's
  * addressing before using it as an address: a slot's neighbour cell (< n_cells), a face's

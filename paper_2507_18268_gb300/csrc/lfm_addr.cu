@@ -12,6 +12,7 @@
 //   - boundary faces of each cell the same way (b_start, b_face);
 //   - the slot-major rows (slot_other, slot_face: neighbour-side faces, owned faces, padding)
 //     and each face's two slot positions (face_slots).
+#include <algorithm>
 #include <cstdint>
 #include <vector>
 
@@ -225,6 +226,86 @@ cudaError_t build_addressing(int32_t N, int32_t F, int32_t NB, int32_t W, const 
   } while (false);
   cudaError_t e2 = cudaFreeAsync(buf, s);
   return e != cudaSuccess ? e : e2;
+}
+
+namespace {
+
+constexpr int32_t kNoDelta = (int32_t)0x80808080;  // no distance: six slots bound N below 2^32 / 6
+
+// Adds d to a table of kMaxDeltas entries (empty: kNoDelta); false when it is full.
+__device__ __forceinline__ bool table_add(int32_t* t, int32_t d) {
+  for (int i = 0; i < kMaxDeltas; ++i) {
+    int32_t v = *reinterpret_cast<volatile int32_t*>(t + i);
+    if (v == kNoDelta) v = atomicCAS(t + i, kNoDelta, d);
+    if (v == kNoDelta || v == d) return true;
+  }
+  return false;
+}
+
+// The distinct neighbour distances of a mesh: per block in shared memory, merged into out
+// (out[kMaxDeltas] != 0: more than fit; blocks that see it stop).
+__global__ void delta_find_kernel(int32_t N, int32_t W, const int32_t* __restrict__ other, int32_t* __restrict__ out) {
+  __shared__ int32_t t[kMaxDeltas];
+  if (threadIdx.x < kMaxDeltas) t[threadIdx.x] = kNoDelta;
+  __syncthreads();
+  bool fits = true;
+  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < N && fits; c += (int64_t)gridDim.x * blockDim.x) {
+    if (*reinterpret_cast<volatile int32_t*>(out + kMaxDeltas) != 0) break;
+    for (int k = 0; k < W && fits; ++k) fits = table_add(t, other[(size_t)k * N + c] - (int32_t)c);
+  }
+  if (!fits) atomicExch(out + kMaxDeltas, 1);
+  __syncthreads();
+  if (threadIdx.x < kMaxDeltas && t[threadIdx.x] != kNoDelta && !table_add(out, t[threadIdx.x]))
+    atomicExch(out + kMaxDeltas, 1);
+}
+
+struct DeltaTable {
+  int32_t d[kMaxDeltas];
+};
+
+__global__ void slot_code_kernel(int32_t N, int32_t W, const int32_t* __restrict__ other,
+                                 const int32_t* __restrict__ b_start, DeltaTable t, uint32_t* __restrict__ code) {
+  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (c >= N) return;
+  uint32_t w = b_start[c + 1] != b_start[c] ? 0x80000000u : 0u;
+  for (int k = 0; k < W; ++k) {
+    const int32_t d = other[(size_t)k * N + c] - (int32_t)c;
+    uint32_t at = 0;
+#pragma unroll
+    for (int i = 0; i < kMaxDeltas; ++i)
+      if (t.d[i] == d) at = (uint32_t)i;
+    w |= at << (4 * k);
+  }
+  code[c] = w;
+}
+
+}  // namespace
+
+cudaError_t build_slot_codes(int32_t N, int32_t W, const int32_t* slot_other, const int32_t* b_start, uint32_t* code,
+                             int32_t* scratch, int32_t* delta, int* n, cudaStream_t s) {
+  *n = 0;
+  if (N <= 0 || W * 4 > 28) return cudaSuccess;
+  int32_t found[kMaxDeltas + 1];
+  cudaError_t e;
+  if ((e = cudaMemsetAsync(scratch, 0x80, sizeof(int32_t) * kMaxDeltas, s)) != cudaSuccess ||
+      (e = cudaMemsetAsync(scratch + kMaxDeltas, 0, sizeof(int32_t), s)) != cudaSuccess)
+    return e;
+  const int64_t blocks = ((int64_t)N + 255) / 256;
+  delta_find_kernel<<<(unsigned)(blocks < 1216 ? blocks : 1216), 256, 0, s>>>(N, W, slot_other, scratch);
+  if ((e = cudaGetLastError()) != cudaSuccess ||
+      (e = cudaMemcpyAsync(found, scratch, sizeof found, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+      (e = cudaStreamSynchronize(s)) != cudaSuccess)
+    return e;
+  if (found[kMaxDeltas] != 0) return cudaSuccess;
+  const int m = (int)(std::remove(found, found + kMaxDeltas, kNoDelta) - found);
+  std::sort(found, found + m);
+  DeltaTable t;
+  for (int i = 0; i < kMaxDeltas; ++i) t.d[i] = delta[i] = i < m ? found[i] : kNoDelta;
+  slot_code_kernel<<<(unsigned)blocks, 256, 0, s>>>(N, W, slot_other, b_start, t, code);
+  if ((e = cudaGetLastError()) != cudaSuccess || (e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
+  for (int i = m; i < kMaxDeltas; ++i) delta[i] = 0;  // never named by a code
+  *n = m;
+  return cudaSuccess;
 }
 
 }  // namespace lfm

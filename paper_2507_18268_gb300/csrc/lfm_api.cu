@@ -34,7 +34,7 @@ size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 // Byte layout of a case's workspace. Offsets are relative to the workspace base.
 struct Layout {
   size_t sync, partials, stats;
-  size_t slot_other, slot_face, face_slots, b_start, b_face, bcell, btype;
+  size_t slot_other, slot_code, slot_face, face_slots, b_start, b_face, bcell, btype;
   size_t V, magSf, delta, DT, bmagSf, bdelta, bDT, bval;
   size_t diag, upper, slot_coef, src, rD, vdt, x, x_old, vSu, vSp, r, w, p, q, Tb;
   size_t Sf, fw, corr, bSf, gE, gD, gH, cK, cL, grad;  // general geometry (0 when absent)
@@ -75,6 +75,7 @@ Layout make_layout(int64_t N, int64_t F, int64_t NB, int64_t W, int kind, bool s
   L.flags = take(256);
   if (!shared_mesh) {
     L.slot_other = take(4 * W * N);
+    L.slot_code = take(W == 6 ? 4 * N : 0);
     L.slot_face = take(4 * W * N);
     L.face_slots = take(8 * F);
     L.b_start = take(4 * (N + 1));
@@ -211,6 +212,8 @@ struct lfm_ctx {
   bool coef_dirty = true;             // FP64 / FP32 slot coefficients to rebuild before the next launch
   double mean_V = 1.0;                // mean cell volume (sets the df64 scale with dt)
   bool has_geom = false;              // general geometry uploaded (corrected laplacian)
+  int packed = 0;                     // distinct neighbour distances where the slots are packed (own mesh)
+  bool pack_on = true;                // test switch: kernels read the packed slots
   bool ops_dirty = false;             // operator weights to rebuild before the next launch
   bool has_Su = false, has_Sp = false;  // volumetric source set (lfm_set_source)
   int32_t n_corr = 0;                 // non-orthogonal corrector passes per step
@@ -373,7 +376,7 @@ int h2d(lfm_ctx* c, size_t off, const T* src, size_t n) {
 // per CTA (the best shape in launch-shape sweeps on the 200^3 graded box).
 int choose_launch(lfm_ctx* c) {
   const int threads = 512;
-  int maxc = max_coresident_ctas(c->opts.precision, threads, c->W, c->device);
+  int maxc = max_coresident_ctas(c->opts.precision, threads, kernel_width(c->W, c->cs.slot_code != nullptr, threads), c->device);
   if (maxc <= 0) return fail(c, LFM_ECUDA, "cannot size the cooperative launch");
   int64_t want = ((int64_t)c->N + 4095) / 4096;
   if (want < 1) want = 1;
@@ -386,7 +389,7 @@ int choose_launch(lfm_ctx* c) {
 Launch current_launch(lfm_ctx* c, int& err) {
   Launch L{};
   L.threads = c->threads > 0 ? c->threads : c->tuned_threads;
-  int maxc = max_coresident_ctas(c->opts.precision, L.threads, c->W, c->device);
+  int maxc = max_coresident_ctas(c->opts.precision, L.threads, kernel_width(c->W, c->cs.slot_code != nullptr, L.threads), c->device);
   L.ctas = c->ctas > 0 ? c->ctas : c->tuned_ctas;
   if (L.ctas > maxc) L.ctas = maxc;
   err = L.ctas <= 0 ? 1 : 0;
@@ -438,6 +441,10 @@ void bind_pointers(lfm_ctx* c) {
   if (c->mesh_src) {
     const CaseDev& m = c->mesh_src->cs;
     cs.slot_other = m.slot_other;
+    cs.slot_code = c->pack_on && c->mesh_src->packed
+                       ? reinterpret_cast<const uint32_t*>(c->mesh_src->ws + c->mesh_src->lay.slot_code)
+                       : nullptr;
+    std::copy(m.slot_delta, m.slot_delta + kMaxDeltas, cs.slot_delta);
     cs.slot_face = m.slot_face;
     cs.face_slots = m.face_slots;
     cs.b_start = m.b_start;
@@ -455,6 +462,7 @@ void bind_pointers(lfm_ctx* c) {
     cs.gE = m.gE;
   } else {
     cs.slot_other = reinterpret_cast<const int32_t*>(b + L.slot_other);
+    cs.slot_code = c->pack_on && c->packed ? reinterpret_cast<const uint32_t*>(b + L.slot_code) : nullptr;
     cs.slot_face = reinterpret_cast<const int32_t*>(b + L.slot_face);
     cs.face_slots = reinterpret_cast<const uint32_t*>(b + L.face_slots);
     cs.b_start = reinterpret_cast<const int32_t*>(b + L.b_start);
@@ -517,6 +525,19 @@ void bind_pointers(lfm_ctx* c) {
   cs.vdt2 = f ? reinterpret_cast<const float2*>(b + L.vdt2) : nullptr;
   cs.g2 = f ? reinterpret_cast<const float2*>(b + L.g2) : nullptr;
   cs.df_scale = df_scale_for(c->mean_V, c->dt);
+}
+
+// Packs the neighbours of a six-slot mesh whose neighbour distances are few (see
+// CaseDev::slot_code). The partial-sum table, not yet in use, holds the search's result.
+int pack_slots(lfm_ctx* c) {
+  if (c->W != 6) return LFM_OK;
+  uint32_t* code = reinterpret_cast<uint32_t*>(c->ws + c->lay.slot_code);
+  int n = 0;
+  CK(c, build_slot_codes(c->N, c->W, c->cs.slot_other, c->cs.b_start, code, reinterpret_cast<int32_t*>(c->cs.partials),
+                         c->cs.slot_delta, &n, c->stream));
+  c->packed = n;
+  if (c->packed && c->pack_on) c->cs.slot_code = code;
+  return LFM_OK;
 }
 
 // V/dt per cell, recomputed when dt or the mesh changes (the assembly reads it every step).
@@ -606,7 +627,7 @@ int enqueue_chunk(lfm_ctx* c, int steps, int mode) {
   Launch L = current_launch(c, e);
   if (e) return fail(c, LFM_ECUDA, "no co-resident CTA fits the step kernel");
   if (mode == kModeAssembleOnly && c->opts.precision == LFM_DF64) {  // read-back runs the FP64 assembly
-    const int m = max_coresident_ctas(LFM_FP64, L.threads, c->W, c->device);
+    const int m = max_coresident_ctas(LFM_FP64, L.threads, kernel_width(c->W, c->cs.slot_code != nullptr, L.threads), c->device);
     if (L.ctas > m) L.ctas = m;
     if (L.ctas <= 0) return fail(c, LFM_ECUDA, "no co-resident CTA fits the assembly kernel");
   }
@@ -767,6 +788,7 @@ static int upload_mesh_impl(lfm_ctx* c, const lfm_mesh* m, const lfm_geometry* g
   c->F = m->n_faces;
   c->NB = m->n_bfaces;
   c->W = W;
+  c->packed = 0;
   c->has64 = has64;
   c->has32 = has32;
   c->hasdf = hasdf;
@@ -809,6 +831,7 @@ static int upload_mesh_impl(lfm_ctx* c, const lfm_mesh* m, const lfm_geometry* g
     cudaFree(on);
     if (e != cudaSuccess) return cuda_fail(c, e, "device face addressing");
   }
+  if ((rc = pack_slots(c))) return rc;
   if ((rc = h2d(c, Y.btype, btype.data(), NB)) || (rc = h2d(c, Y.V, m->V, N)) ||
       (rc = h2d(c, Y.magSf, m->magSf, F)) || (rc = h2d(c, Y.delta, m->deltaCoeffs, F)) ||
       (rc = h2d(c, Y.bmagSf, m->bmagSf, NB)) || (rc = h2d(c, Y.bdelta, m->bdeltaCoeffs, NB)) ||
@@ -935,6 +958,7 @@ int lfm_upload_box(lfm_ctx* c, int32_t nx, int32_t ny, int32_t nz, const double*
   c->F = F;
   c->NB = NB;
   c->W = W;
+  c->packed = 0;
   c->has64 = has64;
   c->has32 = has32;
   c->hasdf = hasdf;
@@ -960,6 +984,7 @@ int lfm_upload_box(lfm_ctx* c, int32_t nx, int32_t ny, int32_t nz, const double*
   CK(c, launch_box(nx, ny, nz, W, coords, coords + nx + 1, coords + nx + ny + 2, c->cs, c->stream));
   std::vector<int32_t> btype(NB, LFM_ZERO_GRADIENT);
   int rc;
+  if ((rc = pack_slots(c))) return rc;
   if ((rc = h2d(c, Y.btype, btype.data(), NB))) return rc;
   CK(c, cudaMemsetAsync(c->ws + Y.bDT, 0, sizeof(double) * NB, c->stream));
   CK(c, cudaMemsetAsync(c->ws + Y.bval, 0, sizeof(double) * NB, c->stream));
@@ -1470,6 +1495,17 @@ int lfm_debug_staged_passes(lfm_ctx* c, int64_t* n) {
   return LFM_OK;
 }
 
+int lfm_debug_pack_slots(lfm_ctx* c, int32_t on, int32_t* n) {
+  int rc = need_uploaded(c);
+  if (rc) return rc;
+  if (c->pending_steps > 0 || ctx_batch_pending(c)) return fail(c, LFM_ESTATE, "an advance is pending");
+  if ((rc = invalidate_seed(c))) return rc;
+  c->pack_on = on != 0;
+  bind_pointers(c);
+  if (n) *n = (c->mesh_src ? c->mesh_src : c)->packed;
+  return choose_launch(c);
+}
+
 int lfm_debug_stage_rows(lfm_ctx* c, int32_t on) {
   if (!c) return fail_free(LFM_EINVAL, "context is NULL");
   c->stage_rows = on != 0 ? 1 : 0;
@@ -1774,6 +1810,7 @@ int lfm_batch_advance_capped_async(lfm_batch* b, int32_t n_steps, int32_t use_gr
   int rc = ensure_capacity(b, n);
   if (rc) return rc;
   int W = 6, form = kBatchAny;
+  bool coded = true;
   for (int i = 0; i < n; ++i) {
     lfm_ctx* c = b->slots[b->order[i]];
     if (c->pending_steps) return bfail(b, LFM_ESTATE, "case %d has a pending advance of its own", b->order[i]);
@@ -1786,10 +1823,12 @@ int lfm_batch_advance_capped_async(lfm_batch* b, int32_t n_steps, int32_t use_gr
       return bfail(b, LFM_ECUDA, "case %d: coefficient set-up failed", b->order[i]);
     b->h_cases[i] = c->cs;
     if (c->W != 6) W = 0;
+    if (c->cs.slot_code == nullptr) coded = false;
     const int p = c->opts.precision;
     const int f = p == LFM_FP64 ? kBatchFp64 : p == LFM_DF64 ? kBatchDf64 : kBatchAny;
     form = i == 0 ? f : (form == f ? form : kBatchAny);
   }
+  W = kernel_width(W, coded, b->threads);
   const int ctas = max_coresident_batch_ctas(b->threads, W, form, b->device);
   if (ctas <= 0) return bfail(b, LFM_ECUDA, "no co-resident CTA fits the batch kernel");
   // jobs: team sizes from the size classes, longest (estimated) job first

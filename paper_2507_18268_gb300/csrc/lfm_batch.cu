@@ -115,12 +115,17 @@ __global__ void batch_collect_kernel(const CaseDev* __restrict__ cases, int n_ca
   }
 }
 
+template <int B, int W>
+void* batch_fn_of(int form) {
+  if (form == kBatchFp64) return (void*)batch_kernel<B, W, kBatchFp64>;
+  if (form == kBatchDf64) return (void*)batch_kernel<B, W, kBatchDf64>;
+  return (void*)batch_kernel<B, W, kBatchAny>;
+}
+
 template <int B>
 void* batch_fn_w(int W, int form) {
-  if (W != 6) return (void*)batch_kernel<B, 0, kBatchAny>;
-  if (form == kBatchFp64) return (void*)batch_kernel<B, 6, kBatchFp64>;
-  if (form == kBatchDf64) return (void*)batch_kernel<B, 6, kBatchDf64>;
-  return (void*)batch_kernel<B, 6, kBatchAny>;
+  if (W == (6 | kCodedBit)) return batch_fn_of<B, (6 | kCodedBit)>(form);
+  return W == 6 ? batch_fn_of<B, 6>(form) : (void*)batch_kernel<B, 0, kBatchAny>;
 }
 
 void* batch_fn(int threads, int W, int form) {
@@ -134,7 +139,15 @@ void* batch_fn(int threads, int W, int form) {
 // Dynamic shared memory of a batched kernel: the stages of the bulk-staged FP32 A p, for the
 // kernel that runs mixed cases (six slots).
 unsigned batch_dyn_smem(int threads, int W, int form) {
-  if (W != 6 || form != kBatchAny) return 0;
+  if (form != kBatchAny) return 0;
+  if (W == (6 | kCodedBit)) {
+    switch (threads) {
+      case 256: return stage_bytes_f32<256, (6 | kCodedBit)>();
+      case 512: return stage_bytes_f32<512, (6 | kCodedBit)>();
+      default: return 0;
+    }
+  }
+  if (W != 6) return 0;
   switch (threads) {
     case 256: return stage_bytes_f32<256, 6>();
     case 512: return stage_bytes_f32<512, 6>();

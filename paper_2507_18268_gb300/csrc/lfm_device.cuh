@@ -280,6 +280,16 @@ __device__ __forceinline__ bool team_barrier(const Team& tm, TeamShared<B>& sh) 
   return team_allreduce<0, B>(tm, nullptr, sh, [](int, double, int) {});
 }
 
+// Slot k's neighbour distance of a packed slot word (CaseDev::slot_code), from the table at
+// shared-memory address dl. The lanes of a warp mostly hold the same word, and sixteen words
+// sit in different banks, so the lookup never serialises.
+__device__ __forceinline__ int code_delta(uint32_t dl, uint32_t word, int k) {
+  const uint32_t at = (k == 0 ? word << 2 : word >> (4 * k - 2)) & 60u;
+  int d;
+  asm("ld.shared.s32 %0, [%1];" : "=r"(d) : "r"(dl + at));
+  return d;
+}
+
 // ---- bulk copies global -> shared, completed on an mbarrier ------------------------------
 // One thread arms a stage's mbarrier with the byte count it expects and issues the bulk
 // copies (cp.async.bulk: the copy engine moves the bytes, no thread registers hold them);

@@ -17,6 +17,15 @@ constexpr int kMaxCtas = 8192;       // capacity of the per-CTA partial-sum tabl
 constexpr int kStatsCap = 1024;      // per-launch statistics records
 constexpr int kMaxSweeps = 5;        // mixed precision: defect-correction sweeps per step
 constexpr int kMaxSlots = 32;        // largest number of internal faces per cell
+constexpr int kMaxDeltas = 16;       // distinct neighbour distances a coded slot row can name
+
+// Slot width a kernel is compiled for: 0 (the case's, read at run time), 6 (neighbours read
+// from slot_other) or 6 | kCodedBit (neighbours from the packed codes, see CaseDev::slot_code).
+constexpr int kCodedBit = 16;
+template <int W>
+constexpr int kSlots = W & (kCodedBit - 1);
+template <int W>
+constexpr bool kCoded = (W & kCodedBit) != 0;
 constexpr int kStaticMaxCells = 1 << 16;   // allocation-free solve: largest system
 constexpr int kStaticMaxFaces = 1 << 18;
 
@@ -50,6 +59,12 @@ struct CaseDev {
   // owned faces (ascending), then padding (other = c, face = -1, coefficient 0).
   int32_t W;
   const int32_t* slot_other; // [W*N] the other cell of the slot's face
+  // Packed form of slot_other for six-slot meshes whose neighbour distances other - c take at
+  // most kMaxDeltas values (a naturally numbered box has seven): bits 4k .. 4k + 3 of a cell's
+  // word name slot k's entry of slot_delta, bit 31 says whether the cell has boundary faces. Null
+  // where the mesh does not pack. One word per cell instead of six.
+  const uint32_t* slot_code; // [N]
+  int32_t slot_delta[kMaxDeltas];
   const int32_t* slot_face;  // [W*N] face id, -1 for padding
   const uint32_t* face_slots; // [2F] face f sits at slot face_slots[2f] (= k*N + owner) of
                               // its owner's row and at face_slots[2f+1] of its neighbour's
@@ -198,6 +213,8 @@ cudaError_t launch_steps(const CaseDev& cs, const Launch& L, int n_steps, int mo
 // Opts a kernel into more than 48 KB of dynamic shared memory (once per kernel and device).
 cudaError_t allow_dyn_smem(void* fn, unsigned bytes);
 int max_coresident_ctas(int precision, int threads, int W, int device);
+// Slot width (template argument) of the step kernel a case runs at `threads` per CTA.
+int kernel_width(int W, bool coded, int threads);
 cudaError_t launch_boundary_values(const CaseDev& cs, double* Tb, cudaStream_t stream);
 // Gauss linear gradient of the current T: cells into cs.grad, and (bgrad non-null) the
 // corrected boundary values [3NB] (x,y,z per face).
@@ -226,6 +243,13 @@ cudaError_t build_addressing(int32_t N, int32_t F, int32_t NB, int32_t W, const 
                              const int32_t* neighbour, const int32_t* bface_cell, int32_t* slot_other,
                              int32_t* slot_face, uint32_t* face_slots, int32_t* b_start, int32_t* b_face,
                              cudaStream_t stream);
+
+// Packs slot_other into codes (see CaseDev::slot_code) where the mesh allows: delta receives
+// the distinct neighbour distances in ascending order, *n their number, 0 where there are more
+// than kMaxDeltas (code is then not written). scratch: kMaxDeltas + 1 ints of device memory.
+// Synchronises the stream.
+cudaError_t build_slot_codes(int32_t N, int32_t W, const int32_t* slot_other, const int32_t* b_start, uint32_t* code,
+                             int32_t* scratch, int32_t* delta, int* n, cudaStream_t stream);
 
 // Box meshes built from closed forms (lfm_box.cu).
 int box_slot_width(long long nx, long long ny, long long nz);

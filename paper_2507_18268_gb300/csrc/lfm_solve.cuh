@@ -73,7 +73,38 @@ __device__ __forceinline__ void cta_range(int N, int size, int rank, int& c0, in
 // Slot count: the compile-time width when the kernel is specialised, else the case's.
 template <int W>
 __device__ __forceinline__ int nslots(const CaseDev& cs) {
-  return W > 0 ? W : cs.W;
+  return W > 0 ? kSlots<W> : cs.W;
+}
+
+// The neighbours of row c in slot order, for a kernel specialised for six slots: from the packed
+// codes (one word and six lookups in the delta table at shared address dl) or from slot_other.
+// Returns the code word (all ones when not coded: the row may have boundary faces). kStream:
+// evict-first loads, for passes that gather. Packed, a row of the FP32 A p reads 4 bytes of
+// indices instead of 24 (60 -> 40 bytes per cell), holds one register for them instead of six,
+// and needs no dependent global load before its gathers but the word.
+template <int W, bool kStream>
+__device__ __forceinline__ uint32_t neighbours(const int32_t* __restrict__ other, const uint32_t* __restrict__ code,
+                                               int N, uint32_t dl, int c, int (&o)[kSlots<W>], int site) {
+  if constexpr (kCoded<W>) {
+    const uint32_t word = kStream ? __ldcs(code + c) : __ldg(code + c);
+#pragma unroll
+    for (int k = 0; k < kSlots<W>; ++k) o[k] = LFM_IDX(c + code_delta(dl, word, k), N, c, site);
+    return word;
+  } else {
+#pragma unroll
+    for (int k = 0; k < kSlots<W>; ++k) {
+      const int32_t* at = other + (size_t)k * N + c;
+      o[k] = LFM_IDX(kStream ? __ldcs(at) : __ldg(at), N, c, site);
+    }
+    return 0xffffffffu;
+  }
+}
+
+// Shared-memory address of the delta table in the CTA's copy of the case descriptor.
+template <int W>
+__device__ __forceinline__ uint32_t delta_table(const CaseDev& shared_cs) {
+  if constexpr (kCoded<W>) return smem_addr(shared_cs.slot_delta);
+  return 0;
 }
 
 // ---- FP64-accurate accumulation of FP32 terms without FP64 instructions -----------------
@@ -141,8 +172,13 @@ __device__ __forceinline__ double plus_zero(double v) {
 }
 
 // xo: T of the cell at the start of the step (the ddt source).
-__device__ __forceinline__ void row_boundary(const CaseDev& cs, int c, double xo, Row& o) {
-  const int b0 = __ldg(cs.b_start + c), b1 = __ldg(cs.b_start + c + 1);
+// word: the row's slot code (bit 31 clear: no boundary faces, nothing to look up).
+__device__ __forceinline__ void row_boundary(const CaseDev& cs, int c, double xo, Row& o, uint32_t word = 0xffffffffu) {
+  int b0 = 0, b1 = 0;
+  if (word >> 31) {
+    b0 = __ldg(cs.b_start + c);
+    b1 = __ldg(cs.b_start + c + 1);
+  }
   const double vdt = cs.vdt[c];  // V/dt, formed once per (mesh, dt): the same IEEE quotient
   const double sv = __dmul_rn(vdt, xo);
   if (b0 == b1) {  // no boundary face: the sums below start from zero
@@ -172,17 +208,19 @@ __device__ __forceinline__ void row_boundary(const CaseDev& cs, int c, double xo
 template <int W>
 __device__ __forceinline__ void op_grad(const CaseDev& cs, int c, const double* __restrict__ x, double* g) {
   const size_t N = (size_t)cs.N;
-  const int ns = W > 0 ? W : cs.W;
+  const int ns = nslots<W>(cs);
   const size_t WN = (size_t)ns * N;
+  int o[W > 0 ? kSlots<W> : 1];
+  if constexpr (W > 0) neighbours<W, false>(cs.slot_other, cs.slot_code, cs.N, delta_table<W>(cs), c, o, kChkSlotCell);
   const double xc = x[c];
   double g0 = fma(__ldg(cs.gD + c), xc, __ldg(cs.gH + c));
   double g1 = fma(__ldg(cs.gD + N + c), xc, __ldg(cs.gH + N + c));
   double g2 = fma(__ldg(cs.gD + 2 * N + c), xc, __ldg(cs.gH + 2 * N + c));
 #pragma unroll
-  for (int k = 0; k < (W > 0 ? W : kMaxSlots); ++k) {
+  for (int k = 0; k < (W > 0 ? kSlots<W> : kMaxSlots); ++k) {
     if (W == 0 && k >= ns) break;
     const size_t at = (size_t)k * N + c;
-    const double xo = x[LFM_IDX(__ldg(cs.slot_other + at), cs.N, c, kChkSlotCell)];
+    const double xo = x[W > 0 ? o[W > 0 ? k : 0] : LFM_IDX(__ldg(cs.slot_other + at), cs.N, c, kChkSlotCell)];
     g0 = fma(__ldg(cs.gE + at), xo, g0);
     g1 = fma(__ldg(cs.gE + WN + at), xo, g1);
     g2 = fma(__ldg(cs.gE + 2 * WN + at), xo, g2);
@@ -197,17 +235,19 @@ __device__ __forceinline__ void op_grad(const CaseDev& cs, int c, const double* 
 template <int W>
 __device__ __forceinline__ double op_corr_source(const CaseDev& cs, int c) {
   const size_t N = (size_t)cs.N;
-  const int ns = W > 0 ? W : cs.W;
+  const int ns = nslots<W>(cs);
   const size_t WN = (size_t)ns * N;
+  int oc[W > 0 ? kSlots<W> : 1];
+  if constexpr (W > 0) neighbours<W, false>(cs.slot_other, cs.slot_code, cs.N, delta_table<W>(cs), c, oc, kChkSlotCell);
   const double* G = cs.grad;
   double v = __ldg(cs.cK + c) * G[c];
   v = fma(__ldg(cs.cK + N + c), G[N + c], v);
   v = fma(__ldg(cs.cK + 2 * N + c), G[2 * N + c], v);
 #pragma unroll
-  for (int k = 0; k < (W > 0 ? W : kMaxSlots); ++k) {
+  for (int k = 0; k < (W > 0 ? kSlots<W> : kMaxSlots); ++k) {
     if (W == 0 && k >= ns) break;
     const size_t at = (size_t)k * N + c;
-    const int o = LFM_IDX(__ldg(cs.slot_other + at), cs.N, c, kChkSlotCell);
+    const int o = W > 0 ? oc[W > 0 ? k : 0] : LFM_IDX(__ldg(cs.slot_other + at), cs.N, c, kChkSlotCell);
     v = fma(__ldg(cs.cL + at), G[o], v);
     v = fma(__ldg(cs.cL + WN + at), G[N + o], v);
     v = fma(__ldg(cs.cL + 2 * WN + at), G[2 * N + o], v);
@@ -226,20 +266,20 @@ __device__ __forceinline__ Row assemble_row(const CaseDev& cs, int c, const doub
   o.xc = x[c];
   o.d = 0.0;
   double off = 0.0;  // sum of the off-diagonal products, slot order
+  uint32_t word = 0xffffffffu;
   if constexpr (W > 0) {
-    int oc[W];
-    double u[W];
+    constexpr int S = kSlots<W>;
+    int oc[S];
+    double u[S];
+    word = neighbours<W, false>(cs.slot_other, cs.slot_code, cs.N, delta_table<W>(cs), c, oc, kChkSlotCell);
 #pragma unroll
-    for (int k = 0; k < W; ++k) {
-      oc[k] = LFM_IDX(__ldg(cs.slot_other + (size_t)k * N + c), cs.N, c, kChkSlotCell);
-      u[k] = cs.slot_coef[(size_t)k * N + c];
-    }
+    for (int k = 0; k < S; ++k) u[k] = cs.slot_coef[(size_t)k * N + c];
     // 0 + g_0 = g_0 exactly; the sign of a zero cannot reach d, which ends above V/dt > 0
     o.d = -u[0];
 #pragma unroll
-    for (int k = 1; k < W; ++k) o.d = __dadd_rn(o.d, -u[k]);  // padding slots hold 0
+    for (int k = 1; k < S; ++k) o.d = __dadd_rn(o.d, -u[k]);  // padding slots hold 0
 #pragma unroll
-    for (int k = 0; k < W; ++k) off = fma(u[k], x[oc[k]], off);
+    for (int k = 0; k < S; ++k) off = fma(u[k], x[oc[k]], off);
   } else {
     const int ns = cs.W;
     for (int k = 0; k < ns; ++k) {
@@ -249,7 +289,7 @@ __device__ __forceinline__ Row assemble_row(const CaseDev& cs, int c, const doub
       off = fma(u, x[LFM_IDX(__ldg(cs.slot_other + at), cs.N, c, kChkSlotCell)], off);
     }
   }
-  row_boundary(cs, c, kCorr && cs.n_corr > 0 ? cs.x_old[c] : o.xc, o);
+  row_boundary(cs, c, kCorr && cs.n_corr > 0 ? cs.x_old[c] : o.xc, o, word);
   if (kCorr && cs.vSp) {  // implicit part of the source S_T = Su + Sp T
     const double v = cs.vSp[c];
     o.d = __dsub_rn(o.d, v);
@@ -356,13 +396,18 @@ struct Slots {
   const int32_t* other;  // [W*N] neighbour cell per slot (padding: the cell itself)
   const T* coef;         // [W*N] off-diagonal per slot (padding: 0)
   const T* diag;         // [N]
+  const uint32_t* code;  // [N] packed neighbours (coded kernels)
+  uint32_t dl;           // shared address of their delta table
 };
 
-__device__ __forceinline__ Slots<double> slots64(const CaseDev& cs) {
-  return Slots<double>{cs.N, cs.W, cs.slot_other, cs.slot_coef, cs.diag};
+// cref: the CTA's copy of the case descriptor in shared memory.
+template <int W>
+__device__ __forceinline__ Slots<double> slots64(const CaseDev& cs, const CaseDev& cref) {
+  return Slots<double>{cs.N, cs.W, cs.slot_other, cs.slot_coef, cs.diag, cs.slot_code, delta_table<W>(cref)};
 }
-__device__ __forceinline__ Slots<float> slots32(const CaseDev& cs) {
-  return Slots<float>{cs.N, cs.W, cs.slot_other, cs.slot_coef32, cs.diag32};
+template <int W>
+__device__ __forceinline__ Slots<float> slots32(const CaseDev& cs, const CaseDev& cref) {
+  return Slots<float>{cs.N, cs.W, cs.slot_other, cs.slot_coef32, cs.diag32, cs.slot_code, delta_table<W>(cref)};
 }
 
 __device__ __forceinline__ double fmadd(double a, double b, double c) { return fma(a, b, c); }
@@ -379,7 +424,23 @@ __device__ __forceinline__ void rows2(const Slots<T>& A, int c, int c2, const T*
   vc = v[c];
   vc2 = v[c2];
   T acc = __ldcs(A.diag + c) * vc, acc2 = __ldcs(A.diag + c2) * vc2;
-  if constexpr (W > 0) {
+  if constexpr (kCoded<W>) {
+    constexpr int S = kSlots<W>;
+    int o[S], o2[S];
+    T u[S], u2[S];
+    neighbours<W, true>(A.other, A.code, A.N, A.dl, c, o, kChkSlotCell);
+    neighbours<W, true>(A.other, A.code, A.N, A.dl, c2, o2, kChkSlotCell);
+#pragma unroll
+    for (int k = 0; k < S; ++k) {
+      u[k] = __ldcs(A.coef + (size_t)k * N + c);
+      u2[k] = __ldcs(A.coef + (size_t)k * N + c2);
+    }
+#pragma unroll
+    for (int k = 0; k < S; ++k) {
+      acc = fmadd(u[k], v[o[k]], acc);
+      acc2 = fmadd(u2[k], v[o2[k]], acc2);
+    }
+  } else if constexpr (W > 0) {
     int o[W], o2[W];
     T u[W], u2[W];
 #pragma unroll
@@ -408,14 +469,18 @@ __device__ __forceinline__ void rows2(const Slots<T>& A, int c, int c2, const T*
 template <int W, typename T>
 __device__ __forceinline__ T row1(const Slots<T>& A, int c, const T* __restrict__ v, T& vc) {
   const size_t N = (size_t)A.N;
-  const int ns = W > 0 ? W : A.W;
   vc = v[c];
   T acc = A.diag[c] * vc;
+  if constexpr (W > 0) {
+    int o[kSlots<W>];
+    neighbours<W, false>(A.other, A.code, A.N, A.dl, c, o, kChkSlotCell);
 #pragma unroll
-  for (int k = 0; k < (W > 0 ? W : kMaxSlots); ++k) {
-    if (W == 0 && k >= ns) break;
-    const size_t at = (size_t)k * N + c;
-    acc = fmadd(A.coef[at], v[LFM_IDX(__ldg(A.other + at), A.N, c, kChkSlotCell)], acc);
+    for (int k = 0; k < kSlots<W>; ++k) acc = fmadd(A.coef[(size_t)k * N + c], v[o[k]], acc);
+  } else {
+    for (int k = 0; k < A.W; ++k) {
+      const size_t at = (size_t)k * N + c;
+      acc = fmadd(A.coef[at], v[LFM_IDX(__ldg(A.other + at), A.N, c, kChkSlotCell)], acc);
+    }
   }
   return acc;
 }
@@ -497,9 +562,13 @@ __device__ __forceinline__ double pass_amul_dot_f32(Slots<float> A, int c0, int 
 // wait ran out (status recorded; the caller leaves). (The FP64 A p measured slower staged:
 // its 8-byte coefficients leave room for one row per thread per tile, or only the indices
 // can be staged, and that pass is bound by FP64 issue and the gathers, not by its loads.)
+template <int W>
+__host__ __device__ constexpr unsigned stage_planes() {  // index planes (or the code words), coefficients, diagonal
+  return (kCoded<W> ? 1u : (unsigned)kSlots<W>) + kSlots<W> + 1u;
+}
 template <int B, int W>
 __host__ __device__ constexpr unsigned stage_bytes_f32() {
-  return W > 0 ? 2u * (2u * B) * (4u * W + 4u * (W + 1u)) + 16u : 0u;
+  return W > 0 ? 2u * (2u * B) * 4u * stage_planes<W>() + 16u : 0u;
 }
 
 template <int B, int W>
@@ -511,43 +580,59 @@ template <int B, int W, class TM>
 __device__ __noinline__ double pass_amul_dot_f32_bulk(Slots<float> A, int c0, int c1, const float* __restrict__ p,
                                                    float* __restrict__ q, const TM& tm, bool& ok) {
   constexpr int TC = 2 * B;
-  constexpr int kW = W > 0 ? W : 1;
+  constexpr int S = W > 0 ? kSlots<W> : 1;
+  constexpr int kIdx = kCoded<W> ? 1 : S;  // index planes
   constexpr unsigned kPlane = TC * 4u;
-  constexpr unsigned kStage = (2u * kW + 1u) * kPlane;
+  constexpr unsigned kPlanes = kIdx + S + 1u;
+  constexpr unsigned kStage = kPlanes * kPlane;
   const size_t N = (size_t)A.N;
   const int tid = threadIdx.x;
   Acc2f sig;
   auto issue = [&](unsigned char* st, int t0, int n, uint64_t* bar, uint64_t pol) {
     const unsigned bytes = (unsigned)n * 4u;
-    mbar_arrive_expect_tx(bar, (2u * kW + 1u) * bytes);
+    mbar_arrive_expect_tx(bar, kPlanes * bytes);
+    if constexpr (kCoded<W>) {
+      bulk_g2s(st, A.code + t0, bytes, bar, pol);
+    } else {
 #pragma unroll
-    for (int k = 0; k < kW; ++k) {
-      bulk_g2s(st + k * kPlane, A.other + (size_t)k * N + t0, bytes, bar, pol);
-      bulk_g2s(st + (kW + k) * kPlane, A.coef + (size_t)k * N + t0, bytes, bar, pol);
+      for (int k = 0; k < S; ++k) bulk_g2s(st + k * kPlane, A.other + (size_t)k * N + t0, bytes, bar, pol);
     }
-    bulk_g2s(st + 2 * kW * kPlane, A.diag + t0, bytes, bar, pol);
+#pragma unroll
+    for (int k = 0; k < S; ++k) bulk_g2s(st + (kIdx + k) * kPlane, A.coef + (size_t)k * N + t0, bytes, bar, pol);
+    bulk_g2s(st + (kIdx + S) * kPlane, A.diag + t0, bytes, bar, pol);
+  };
+  // slot k's neighbour of the tile's cell j (label c)
+  auto cols = [&](const int32_t* so, int j, int c, int (&o)[S]) {
+    if constexpr (kCoded<W>) {
+      const uint32_t word = (uint32_t)so[j];
+#pragma unroll
+      for (int k = 0; k < S; ++k) o[k] = LFM_IDX(c + code_delta(A.dl, word, k), A.N, c, kChkSlotCell);
+    } else {
+#pragma unroll
+      for (int k = 0; k < S; ++k) o[k] = LFM_IDX(so[k * TC + j], A.N, c, kChkSlotCell);
+    }
   };
   auto body = [&](const unsigned char* st, int t0, int nt) {
     const int32_t* so = reinterpret_cast<const int32_t*>(st);
-    const float* sc = reinterpret_cast<const float*>(st + kW * kPlane);
-    const float* sd = reinterpret_cast<const float*>(st + 2 * kW * kPlane);
+    const float* sc = reinterpret_cast<const float*>(st + kIdx * kPlane);
+    const float* sd = reinterpret_cast<const float*>(st + (kIdx + S) * kPlane);
     const int j = tid;
     if (j + B < nt) {
       // both rows' loads issued before either is used (as in rows2)
       const int j2 = j + B, c = t0 + j, c2 = t0 + j2;
       const float vc = p[c], vc2 = p[c2];
       float acc = sd[j] * vc, acc2 = sd[j2] * vc2;
-      int o[kW], o2[kW];
-      float u[kW], u2[kW];
+      int o[S], o2[S];
+      float u[S], u2[S];
+      cols(so, j, c, o);
+      cols(so, j2, c2, o2);
 #pragma unroll
-      for (int k = 0; k < kW; ++k) {
-        o[k] = LFM_IDX(so[k * TC + j], A.N, c, kChkSlotCell);
-        o2[k] = LFM_IDX(so[k * TC + j2], A.N, c2, kChkSlotCell);
+      for (int k = 0; k < S; ++k) {
         u[k] = sc[k * TC + j];
         u2[k] = sc[k * TC + j2];
       }
 #pragma unroll
-      for (int k = 0; k < kW; ++k) {
+      for (int k = 0; k < S; ++k) {
         acc = fmaf(u[k], p[o[k]], acc);
         acc2 = fmaf(u2[k], p[o2[k]], acc2);
       }
@@ -559,8 +644,10 @@ __device__ __noinline__ double pass_amul_dot_f32_bulk(Slots<float> A, int c0, in
       const int c = t0 + j;
       const float vc = p[c];
       float y = sd[j] * vc;
+      int o[S];
+      cols(so, j, c, o);
 #pragma unroll
-      for (int k = 0; k < kW; ++k) y = fmaf(sc[k * TC + j], p[LFM_IDX(so[k * TC + j], A.N, c, kChkSlotCell)], y);
+      for (int k = 0; k < S; ++k) y = fmaf(sc[k * TC + j], p[o[k]], y);
       q[c] = y;
       sig.add_prod(y, vc);
     }
@@ -720,7 +807,7 @@ __device__ __noinline__ Sums3 pass_true_residual(const CaseDev& cs, int c0, int 
       rc = o.s - o.ax;
     } else {
       double xc;
-      rc = cs.src[c] - row1<W>(slots64(cs), c, x, xc);
+      rc = cs.src[c] - row1<W>(slots64<W>(cs, cs), c, x, xc);
       rd32 = cs.rD32[c];
     }
     u1 += fabs(rc);
@@ -900,7 +987,7 @@ __device__ void run_steps_f64(const CaseDev& cs, const CaseDev& cref, const TM& 
           clk.lap(kPhP);
         }
         // ---- M: q = A p, sigma = p.q -> alpha ------------------------------------
-        const double s1[1] = {pass_amul_dot_f64<B, W>(slots64(cs), c0, c1, p, q)};
+        const double s1[1] = {pass_amul_dot_f64<B, W>(slots64<W>(cs, cref), c0, c1, p, q)};
         if (!team_allreduce<1, B>(tm, s1, sh, [&](int, double t, int lane) { fin_sigma(sh, t, lane); })) return;
         clk.lap(kPhM);
         if (sh.code != kGo) break;
@@ -958,7 +1045,7 @@ __device__ __forceinline__ void mixed_outer(TeamShared<B>& sh, const CaseDev& cs
 // The inner FP32 CG on A dx = r from its seed (r, p = w; sh.rho, sh.inner_tol): sh.code tells how
 // it ended. False when a barrier failed (the caller leaves).
 template <int B, int W, class TM>
-__device__ __forceinline__ bool inner_cg_f32(const CaseDev& cs, const TM& tm, TeamShared<B>& sh, PhaseClock<B, TM>& clk,
+__device__ __forceinline__ bool inner_cg_f32(const CaseDev& cs, const CaseDev& cref, const TM& tm, TeamShared<B>& sh, PhaseClock<B, TM>& clk,
                                              int c0, int c1, int min_inner, int& iters, float* __restrict__ dx,
                                              float* __restrict__ r, float* __restrict__ w, float* __restrict__ p,
                                              float* __restrict__ q, const float* __restrict__ rD) {
@@ -969,7 +1056,7 @@ __device__ __forceinline__ bool inner_cg_f32(const CaseDev& cs, const TM& tm, Te
       clk.lap(kPhP);
     }
     bool m_ok;
-    const double s1[1] = {amul_dot_f32<B, W>(slots32(cs), c0, c1, p, q, tm, m_ok)};
+    const double s1[1] = {amul_dot_f32<B, W>(slots32<W>(cs, cref), c0, c1, p, q, tm, m_ok)};
     if (!m_ok) return false;
     if (!team_allreduce<1, B>(tm, s1, sh, [&](int, double t, int lane) { fin_sigma(sh, t, lane); })) return false;
     clk.lap(kPhM);
@@ -1050,7 +1137,7 @@ __device__ void run_steps_mixed(const CaseDev& cs, const CaseDev& cref, const TM
           if (sh.code == kNonFinite) status = LFM_ENONFINITE;
           break;
         }
-        if (!inner_cg_f32<B, W>(cs, tm, sh, clk, c0, c1, sweeps == 0 ? cs.min_iter : 0, iters, dx, r, w, p, q, rD))
+        if (!inner_cg_f32<B, W>(cs, cref, tm, sh, clk, c0, c1, sweeps == 0 ? cs.min_iter : 0, iters, dx, r, w, p, q, rD))
           return;
         if (sh.code == kSingular) status = LFM_ESINGULAR;
         if (sh.code == kNonFinite) status = LFM_ENONFINITE;

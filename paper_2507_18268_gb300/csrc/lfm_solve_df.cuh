@@ -136,8 +136,13 @@ __device__ __noinline__ void pass_store_x(const CaseDev& cs, int c0, int c1, boo
 
 // Boundary conductance, source and flux g_b (T_b - x_c) of row c (fixedValue faces;
 // zeroGradient adds nothing), in FP64 with the case scale, in ascending face order.
-__device__ __forceinline__ void row_boundary_df(const CaseDev& cs, int c, tf xc, df& gsum, df& ssum, df& flux) {
-  const int b0 = __ldg(cs.b_start + c), b1 = __ldg(cs.b_start + c + 1);
+__device__ __forceinline__ void row_boundary_df(const CaseDev& cs, int c, tf xc, df& gsum, df& ssum, df& flux,
+                                                uint32_t word = 0xffffffffu) {
+  int b0 = 0, b1 = 0;
+  if (word >> 31) {  // the slot code says whether there are any (all ones when not coded)
+    b0 = __ldg(cs.b_start + c);
+    b1 = __ldg(cs.b_start + c + 1);
+  }
   gsum = mkdf(0.0f, 0.0f);
   ssum = mkdf(0.0f, 0.0f);
   flux = mkdf(0.0f, 0.0f);
@@ -171,16 +176,19 @@ __device__ __noinline__ void pass_grad_df(const CaseDev& cs, int c0, int c1) {
   const float2* __restrict__ x2 = cs.x2;
   const float* __restrict__ xl = cs.xlo;
   const size_t N = (size_t)cs.N;
-  const int ns = W > 0 ? W : cs.W;
+  const int ns = nslots<W>(cs);
   const size_t WN = (size_t)ns * N;
   for (int c = c0 + (int)threadIdx.x; c < c1; c += B) {
     const tf xc = ld_tf(x2, xl, c);
     df g0 = mkdf(0.0f, 0.0f), g1 = g0, g2 = g0;
+    int o[W > 0 ? kSlots<W> : 1];
+    if constexpr (W > 0) neighbours<W, false>(cs.slot_other, cs.slot_code, cs.N, delta_table<W>(cs), c, o, kChkSlotCellDf);
 #pragma unroll
-    for (int k = 0; k < (W > 0 ? W : kMaxSlots); ++k) {
+    for (int k = 0; k < (W > 0 ? kSlots<W> : kMaxSlots); ++k) {
       if (W == 0 && k >= ns) break;
       const size_t at = (size_t)k * N + c;
-      const df d = tf_diff(ld_tf(x2, xl, LFM_IDX(__ldg(cs.slot_other + at), cs.N, c, kChkSlotCellDf)), xc);
+      const int oc = W > 0 ? o[W > 0 ? k : 0] : LFM_IDX(__ldg(cs.slot_other + at), cs.N, c, kChkSlotCellDf);
+      const df d = tf_diff(ld_tf(x2, xl, oc), xc);
       g0 = df_fma(ldg_df(cs.gE2 + at), d, g0);
       g1 = df_fma(ldg_df(cs.gE2 + WN + at), d, g1);
       g2 = df_fma(ldg_df(cs.gE2 + 2 * WN + at), d, g2);
@@ -217,17 +225,19 @@ __device__ __noinline__ void pass_grad_df(const CaseDev& cs, int c0, int c1) {
 template <int W>
 __device__ __forceinline__ df op_corr_df(const CaseDev& cs, int c) {
   const size_t N = (size_t)cs.N;
-  const int ns = W > 0 ? W : cs.W;
+  const int ns = nslots<W>(cs);
   const size_t WN = (size_t)ns * N;
+  int oc[W > 0 ? kSlots<W> : 1];
+  if constexpr (W > 0) neighbours<W, false>(cs.slot_other, cs.slot_code, cs.N, delta_table<W>(cs), c, oc, kChkSlotCellDf);
   const float2* __restrict__ G = cs.grad2;
   df v = df_mul(ldg_df(cs.cK2 + c), ld_df(G + c));
   v = df_fma(ldg_df(cs.cK2 + N + c), ld_df(G + N + c), v);
   v = df_fma(ldg_df(cs.cK2 + 2 * N + c), ld_df(G + 2 * N + c), v);
 #pragma unroll
-  for (int k = 0; k < (W > 0 ? W : kMaxSlots); ++k) {
+  for (int k = 0; k < (W > 0 ? kSlots<W> : kMaxSlots); ++k) {
     if (W == 0 && k >= ns) break;
     const size_t at = (size_t)k * N + c;
-    const int o = LFM_IDX(__ldg(cs.slot_other + at), cs.N, c, kChkSlotCellDf);
+    const int o = W > 0 ? oc[W > 0 ? k : 0] : LFM_IDX(__ldg(cs.slot_other + at), cs.N, c, kChkSlotCellDf);
     v = df_fma(ldg_df(cs.cL2 + at), ld_df(G + o), v);
     v = df_fma(ldg_df(cs.cL2 + WN + at), ld_df(G + N + o), v);
     v = df_fma(ldg_df(cs.cL2 + 2 * WN + at), ld_df(G + 2 * N + o), v);
@@ -242,10 +252,11 @@ __device__ __forceinline__ df op_corr_df(const CaseDev& cs, int c) {
 template <int W>
 __device__ __forceinline__ void prefetch_row_df(const CaseDev& cs, int c) {
   const size_t N = (size_t)cs.N;
-  const int ns = W > 0 ? W : cs.W;
-  for (int k = 0; k < (W > 0 ? W : kMaxSlots); ++k) {
+  const int ns = nslots<W>(cs);
+  if (kCoded<W>) prefetch_l2(cs.slot_code + c);
+  for (int k = 0; k < (W > 0 ? kSlots<W> : kMaxSlots); ++k) {
     if (W == 0 && k >= ns) break;
-    prefetch_l2(cs.slot_other + (size_t)k * N + c);
+    if (!kCoded<W>) prefetch_l2(cs.slot_other + (size_t)k * N + c);
     prefetch_l2(cs.g2 + (size_t)k * N + c);
   }
   prefetch_l2(cs.x2 + c);
@@ -277,23 +288,23 @@ __device__ __noinline__ Sums3 pass_rows_init_df(const CaseDev& cs, int c0, int c
     if (c + B < c1) prefetch_row_df<W>(cs, c + B);
     const tf xc = ld_tf(x2, xl, c);
     df d, flux;
+    uint32_t word = 0xffffffffu;
     if constexpr (W > 0) {
-      int o[W];
-      df g[W];
+      constexpr int S = kSlots<W>;
+      int o[S];
+      df g[S];
+      word = neighbours<W, false>(cs.slot_other, cs.slot_code, cs.N, delta_table<W>(cs), c, o, kChkSlotCellDf);
 #pragma unroll
-      for (int k = 0; k < W; ++k) {
-        o[k] = LFM_IDX(__ldg(cs.slot_other + (size_t)k * N + c), cs.N, c, kChkSlotCellDf);
-        g[k] = ldg_df(g2 + (size_t)k * N + c);
-      }
-      tf xo_[W];
+      for (int k = 0; k < S; ++k) g[k] = ldg_df(g2 + (size_t)k * N + c);
+      tf xo_[S];
 #pragma unroll
-      for (int k = 0; k < W; ++k) xo_[k] = ld_tf(x2, xl, o[k]);
+      for (int k = 0; k < S; ++k) xo_[k] = ld_tf(x2, xl, o[k]);
       d = g[0];
 #pragma unroll
-      for (int k = 1; k < W; ++k) d = df_add(d, g[k]);  // padding slots hold 0
+      for (int k = 1; k < S; ++k) d = df_add(d, g[k]);  // padding slots hold 0
       flux = df_mul(g[0], tf_diff(xo_[0], xc));
 #pragma unroll
-      for (int k = 1; k < W; ++k) flux = df_fma(g[k], tf_diff(xo_[k], xc), flux);
+      for (int k = 1; k < S; ++k) flux = df_fma(g[k], tf_diff(xo_[k], xc), flux);
     } else {
       d = mkdf(0.0f, 0.0f);
       flux = mkdf(0.0f, 0.0f);
@@ -305,7 +316,7 @@ __device__ __noinline__ Sums3 pass_rows_init_df(const CaseDev& cs, int c0, int c
       }
     }
     df gb, sb, fb;
-    row_boundary_df(cs, c, xc, gb, sb, fb);
+    row_boundary_df(cs, c, xc, gb, sb, fb, word);
     const df vdt = ldg_df(cs.vdt2 + c);
     const df xcd = tf_to_df(xc);
     const bool has_old = kSrc && cs.n_corr > 0;
@@ -349,15 +360,36 @@ __device__ __noinline__ Sums3 pass_rows_init_df(const CaseDev& cs, int c0, int c
 // Rows c and c2 of A v, all loads of both rows issued before any is used; the matrix arrays
 // with evict-first (streaming) loads, so that they do not displace the gathered vector.
 template <int W>
-__device__ __forceinline__ void rows2_df(const CaseDev& cs, int c, int c2, const float2* __restrict__ v, df& y,
-                                         df& y2, df& vc, df& vc2) {
+__device__ __forceinline__ void rows2_df(const CaseDev& cs, uint32_t dl, int c, int c2,
+                                         const float2* __restrict__ v, df& y, df& y2, df& vc, df& vc2) {
   const size_t N = (size_t)cs.N;
   const float2* __restrict__ g2 = cs.g2;
   vc = ld_df(v + c);
   vc2 = ld_df(v + c2);
   const float2 dd1 = __ldcs(cs.diag2 + c), dd2 = __ldcs(cs.diag2 + c2);
   df acc = df_mul(df{dd1.x, dd1.y}, vc), acc2 = df_mul(df{dd2.x, dd2.y}, vc2);
-  if constexpr (W > 0) {
+  if constexpr (kCoded<W>) {
+    constexpr int S = kSlots<W>;
+    int o[S], o2[S];
+    df g[S], h[S];
+    neighbours<W, true>(cs.slot_other, cs.slot_code, cs.N, dl, c, o, kChkSlotCellDf);
+    neighbours<W, true>(cs.slot_other, cs.slot_code, cs.N, dl, c2, o2, kChkSlotCellDf);
+#pragma unroll
+    for (int k = 0; k < S; ++k) {
+      const float2 a = __ldcs(g2 + (size_t)k * N + c), b = __ldcs(g2 + (size_t)k * N + c2);
+      g[k] = df{a.x, a.y};
+      h[k] = df{b.x, b.y};
+    }
+    df xo[S], xo2[S];
+#pragma unroll
+    for (int k = 0; k < S; ++k) xo[k] = ld_df(v + o[k]);
+#pragma unroll
+    for (int k = 0; k < S; ++k) xo2[k] = ld_df(v + o2[k]);
+#pragma unroll
+    for (int k = 0; k < S; ++k) acc = df_fma(df_neg(g[k]), xo[k], acc);
+#pragma unroll
+    for (int k = 0; k < S; ++k) acc2 = df_fma(df_neg(h[k]), xo2[k], acc2);
+  } else if constexpr (W > 0) {
     int o[W], o2[W];
     df g[W], h[W];
 #pragma unroll
@@ -389,16 +421,21 @@ __device__ __forceinline__ void rows2_df(const CaseDev& cs, int c, int c2, const
 }
 
 template <int W>
-__device__ __forceinline__ df row1_df(const CaseDev& cs, int c, const float2* __restrict__ v, df& vc) {
+__device__ __forceinline__ df row1_df(const CaseDev& cs, uint32_t dl, int c, const float2* __restrict__ v, df& vc) {
   const size_t N = (size_t)cs.N;
-  const int ns = W > 0 ? W : cs.W;
   vc = ld_df(v + c);
   df acc = df_mul(ld_df(cs.diag2 + c), vc);
+  if constexpr (W > 0) {
+    int o[kSlots<W>];
+    neighbours<W, false>(cs.slot_other, cs.slot_code, cs.N, dl, c, o, kChkSlotCellDf);
 #pragma unroll
-  for (int k = 0; k < (W > 0 ? W : kMaxSlots); ++k) {
-    if (W == 0 && k >= ns) break;
-    const size_t at = (size_t)k * N + c;
-    acc = df_fma(df_neg(ldg_df(cs.g2 + at)), ld_df(v + LFM_IDX(__ldg(cs.slot_other + at), cs.N, c, kChkSlotCellDf)), acc);
+    for (int k = 0; k < kSlots<W>; ++k)
+      acc = df_fma(df_neg(ldg_df(cs.g2 + (size_t)k * N + c)), ld_df(v + o[k]), acc);
+  } else {
+    for (int k = 0; k < cs.W; ++k) {
+      const size_t at = (size_t)k * N + c;
+      acc = df_fma(df_neg(ldg_df(cs.g2 + at)), ld_df(v + LFM_IDX(__ldg(cs.slot_other + at), cs.N, c, kChkSlotCellDf)), acc);
+    }
   }
   return acc;
 }
@@ -420,13 +457,13 @@ __device__ __forceinline__ void pass_direction_df(int c0, int c1, df beta, float
 
 // M: q = A p; returns this thread's share of p.q.
 template <int B, int W>
-__device__ __forceinline__ double pass_amul_dot_df(const CaseDev& cs, int c0, int c1, const float2* __restrict__ p,
+__device__ __forceinline__ double pass_amul_dot_df(const CaseDev& cs, uint32_t dl, int c0, int c1, const float2* __restrict__ p,
                                                    float2* __restrict__ q) {
   DfAcc s;
   int c = c0 + (int)threadIdx.x;
   for (; c + B < c1; c += 2 * B) {
     df y1, y2, pc1, pc2;
-    rows2_df<W>(cs, c, c + B, p, y1, y2, pc1, pc2);
+    rows2_df<W>(cs, dl, c, c + B, p, y1, y2, pc1, pc2);
     st_df(q + c, y1);
     st_df(q + c + B, y2);
     s.add(df_mul(y1, pc1));
@@ -434,7 +471,7 @@ __device__ __forceinline__ double pass_amul_dot_df(const CaseDev& cs, int c0, in
   }
   if (c < c1) {
     df pc;
-    const df y = row1_df<W>(cs, c, p, pc);
+    const df y = row1_df<W>(cs, dl, c, p, pc);
     st_df(q + c, y);
     s.add(df_mul(y, pc));
   }
@@ -551,7 +588,7 @@ __device__ bool steps_df64(const CaseDev& cs, const CaseDev& cref, const TM& tm,
           if (!team_barrier<B>(tm, sh)) return false;
           clk.lap(kPhP);
         }
-        const double s1[1] = {pass_amul_dot_df<B, W>(cs, c0, c1, p, q)};
+        const double s1[1] = {pass_amul_dot_df<B, W>(cs, delta_table<W>(cref), c0, c1, p, q)};
         if (!team_allreduce<1, B>(tm, s1, sh, [&](int, double t, int lane) {
               fin_sigma(sh, t, lane);
               if (lane == 0) sh.alpha2 = pair_of(sh.alpha);

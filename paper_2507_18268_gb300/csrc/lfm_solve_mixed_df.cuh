@@ -43,30 +43,30 @@ namespace {
 // Row c's face part in flux form over the slots (slot order): flux = sum_k g_k (x_other(k) -
 // x_c) and, with kDiag, the sum d of the slot conductances (the diagonal's face part).
 template <int W, bool kDiag>
-__device__ __forceinline__ void row_flux_df(const CaseDev& cs, int c, const tf& xc, df& d, df& flux) {
+__device__ __forceinline__ void row_flux_df(const CaseDev& cs, int c, const tf& xc, df& d, df& flux, uint32_t& word) {
   const float2* __restrict__ x2 = cs.x2;
   const float* __restrict__ xl = cs.xlo;
   const float2* __restrict__ g2 = cs.g2;
   const size_t N = (size_t)cs.N;
+  word = 0xffffffffu;
   if constexpr (W > 0) {
-    int o[W];
-    df g[W];
+    constexpr int S = kSlots<W>;
+    int o[S];
+    df g[S];
+    word = neighbours<W, false>(cs.slot_other, cs.slot_code, cs.N, delta_table<W>(cs), c, o, kChkSlotCellDf);
 #pragma unroll
-    for (int k = 0; k < W; ++k) {
-      o[k] = LFM_IDX(__ldg(cs.slot_other + (size_t)k * N + c), cs.N, c, kChkSlotCellDf);
-      g[k] = ldg_df(g2 + (size_t)k * N + c);
-    }
-    tf xo[W];
+    for (int k = 0; k < S; ++k) g[k] = ldg_df(g2 + (size_t)k * N + c);
+    tf xo[S];
 #pragma unroll
-    for (int k = 0; k < W; ++k) xo[k] = ld_tf(x2, xl, o[k]);
+    for (int k = 0; k < S; ++k) xo[k] = ld_tf(x2, xl, o[k]);
     if constexpr (kDiag) {
       d = g[0];
 #pragma unroll
-      for (int k = 1; k < W; ++k) d = df_add(d, g[k]);  // padding slots hold 0
+      for (int k = 1; k < S; ++k) d = df_add(d, g[k]);  // padding slots hold 0
     }
     flux = df_mul(g[0], tf_diff(xo[0], xc));
 #pragma unroll
-    for (int k = 1; k < W; ++k) flux = df_fma(g[k], tf_diff(xo[k], xc), flux);
+    for (int k = 1; k < S; ++k) flux = df_fma(g[k], tf_diff(xo[k], xc), flux);
   } else {
     d = mkdf(0.0f, 0.0f);
     flux = mkdf(0.0f, 0.0f);
@@ -115,9 +115,10 @@ __device__ __noinline__ Sums3 pass_rows_init_mixed_df(const CaseDev& cs, int c0,
     if (c + B < c1) prefetch_row_df<W>(cs, c + B);
     const tf xc = ld_tf(cs.x2, cs.xlo, c);
     df d, flux;
-    row_flux_df<W, true>(cs, c, xc, d, flux);
+    uint32_t word;
+    row_flux_df<W, true>(cs, c, xc, d, flux, word);
     df gb, sb, fb;
-    row_boundary_df(cs, c, xc, gb, sb, fb);
+    row_boundary_df(cs, c, xc, gb, sb, fb, word);
     const df vdt = ldg_df(cs.vdt2 + c);
     const bool has_old = kSrc && cs.n_corr > 0;
     const tf xo = has_old ? ld_tf(reinterpret_cast<const float2*>(cs.x_old), cs.xolo, c) : xc;
@@ -149,9 +150,10 @@ __device__ __noinline__ double2 pass_true_residual_df(const CaseDev& cs, int c0,
   for (int c = c0 + (int)threadIdx.x; c < c1; c += B) {
     const tf xc = ld_tf(cs.x2, cs.xlo, c);
     df d, flux;
-    row_flux_df<W, false>(cs, c, xc, d, flux);
+    uint32_t word;
+    row_flux_df<W, false>(cs, c, xc, d, flux, word);
     df gb, sb, fb;
-    row_boundary_df(cs, c, xc, gb, sb, fb);
+    row_boundary_df(cs, c, xc, gb, sb, fb, word);
     const tf xo = ld_tf(reinterpret_cast<const float2*>(cs.x_old), cs.xolo, c);
     df rc = df_fma(ldg_df(cs.vdt2 + c), tf_diff(xo, xc), df_add(flux, fb));
     if (kSrc && (cs.vSp || cs.vSu)) {
@@ -189,13 +191,14 @@ __device__ __noinline__ Sums4 pass_verify_next_df(const CaseDev& cs, int c0, int
       // and the next row's per-cell values only this pass reads
       prefetch_l2(cs.x_old + c + B);
       prefetch_l2(cs.xolo + c + B);
-      prefetch_l2(cs.b_start + c + B);
+      if (!kCoded<W>) prefetch_l2(cs.b_start + c + B);
     }
     const tf xc = ld_tf(cs.x2, cs.xlo, c);
     df d, flux;
-    row_flux_df<W, true>(cs, c, xc, d, flux);
+    uint32_t word;
+    row_flux_df<W, true>(cs, c, xc, d, flux, word);
     df gb, sb, fb;
-    row_boundary_df(cs, c, xc, gb, sb, fb);
+    row_boundary_df(cs, c, xc, gb, sb, fb, word);
     const df vdt = ldg_df(cs.vdt2 + c);
     const tf xo = ld_tf(reinterpret_cast<const float2*>(cs.x_old), cs.xolo, c);
     const df rn = df_add(flux, fb);  // the next step's first residual
@@ -328,7 +331,7 @@ __device__ bool steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const TM&
           break;
         }
         // ---- inner FP32 CG on A dx = r (unscaled) -----------------------------------------
-        if (!inner_cg_f32<B, W>(cs, tm, sh, clk, c0, c1, sweeps == 0 ? cs.min_iter : 0, iters, dx, r, w, p, q, rD))
+        if (!inner_cg_f32<B, W>(cs, cref, tm, sh, clk, c0, c1, sweeps == 0 ? cs.min_iter : 0, iters, dx, r, w, p, q, rD))
           return false;
         if (sh.code == kSingular) status = LFM_ESINGULAR;
         if (sh.code == kNonFinite) status = LFM_ENONFINITE;

@@ -297,21 +297,24 @@ __global__ void fill_kernel(double* a, size_t n, double v) {
 // and the df64 form on general geometry (the orthogonal df64 kernel carries no gradient phase).
 constexpr int kMixedDf = 100;
 constexpr int kDf64Geom = 101;
+// Kernels for packed slot codes are compiled for up to this many threads per CTA; a larger CTA,
+// which no default shape uses, reads slot_other.
+constexpr int kMaxCodedThreads = 512;
+
+template <int B, int W>
+void* step_fn_of(int precision) {
+  if (precision == kMixedDf) return (void*)step_kernel_mixed_df<B, W>;
+  if (precision == LFM_MIXED) return (void*)step_kernel_mixed<B, W>;
+  if (precision == kDf64Geom) return (void*)step_kernel_df64<B, W, true>;
+  if (precision == LFM_DF64) return (void*)step_kernel_df64<B, W, false>;
+  return (void*)step_kernel_f64<B, W>;
+}
 
 template <int B>
 void* step_fn_w(int precision, int W) {
-  if (W == 6) {
-    if (precision == kMixedDf) return (void*)step_kernel_mixed_df<B, 6>;
-    if (precision == LFM_MIXED) return (void*)step_kernel_mixed<B, 6>;
-    if (precision == kDf64Geom) return (void*)step_kernel_df64<B, 6, true>;
-    if (precision == LFM_DF64) return (void*)step_kernel_df64<B, 6, false>;
-    return (void*)step_kernel_f64<B, 6>;
-  }
-  if (precision == kMixedDf) return (void*)step_kernel_mixed_df<B, 0>;
-  if (precision == LFM_MIXED) return (void*)step_kernel_mixed<B, 0>;
-  if (precision == kDf64Geom) return (void*)step_kernel_df64<B, 0, true>;
-  if (precision == LFM_DF64) return (void*)step_kernel_df64<B, 0, false>;
-  return (void*)step_kernel_f64<B, 0>;
+  if constexpr (B <= kMaxCodedThreads)
+    if (W == (6 | kCodedBit)) return step_fn_of<B, (6 | kCodedBit)>(precision);
+  return W == 6 ? step_fn_of<B, 6>(precision) : step_fn_of<B, 0>(precision);
 }
 
 void* step_fn_for(int precision, int threads, int W) {
@@ -330,6 +333,13 @@ void* step_fn_for(int precision, int threads, int W) {
 // through L1, lost more (skewed200: 0.71 -> 0.86 and 1.97 -> 2.01 ms per step) than its A p
 // gained (0.655 -> 0.638).
 unsigned step_dyn_smem(int precision, int threads, int W) {
+  if (precision == kMixedDf && W == (6 | kCodedBit)) {
+    switch (threads) {
+      case 256: return stage_bytes_f32<256, (6 | kCodedBit)>();
+      case 512: return stage_bytes_f32<512, (6 | kCodedBit)>();
+      default: return 0;
+    }
+  }
   if (precision == kMixedDf && W == 6) {
     switch (threads) {
       case 256: return stage_bytes_f32<256, 6>();
@@ -370,6 +380,10 @@ cudaError_t allow_dyn_smem(void* fn, unsigned bytes) {
   return e;
 }
 
+int kernel_width(int W, bool coded, int threads) {
+  return W == 6 ? (coded && threads <= kMaxCodedThreads ? (6 | kCodedBit) : 6) : 0;
+}
+
 int max_coresident_ctas(int precision, int threads, int W, int device) {
   int sms = 0;
   int per_sm = per_sm_ctas(precision, threads, W);
@@ -391,9 +405,10 @@ cudaError_t launch_steps(const CaseDev& cs, const Launch& L, int n_steps, int mo
   const bool mixed_df = prec == LFM_MIXED && mode == kModeSteps && mixed_runs_df(cs);
   const bool df_geom = prec == LFM_DF64 && cs.Sf != nullptr;
   const int kind = mixed_df ? kMixedDf : (df_geom ? kDf64Geom : prec);
-  void* fn = step_fn_for(kind, L.threads, cs.W);
+  const int W = kernel_width(cs.W, cs.slot_code != nullptr, L.threads);
+  void* fn = step_fn_for(kind, L.threads, W);
   if (!fn) return cudaErrorInvalidValue;
-  const unsigned dyn = L.stage_rows ? step_dyn_smem(kind, L.threads, cs.W) : 0u;
+  const unsigned dyn = L.stage_rows ? step_dyn_smem(kind, L.threads, W) : 0u;
   const cudaError_t e = allow_dyn_smem(fn, dyn);
   if (e != cudaSuccess) return e;
   CaseDev a0 = cs;
