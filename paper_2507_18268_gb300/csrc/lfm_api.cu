@@ -41,6 +41,7 @@ struct Layout {
   size_t diag32, slot_coef32, rD32, dx32, r32, w32, p32, q32;
   size_t x2, xlo, xolo, e2, diag2, rD2, vdt2, g2;  // df64 form (0 when absent)
   size_t gE2, cK2, cL2, gZ, grad2;                  // df64 form on general geometry
+  size_t bg, bT, bgT, bsum2;                        // boundary faces' row terms
   size_t flags;
   size_t total;
 };
@@ -105,6 +106,10 @@ Layout make_layout(int64_t N, int64_t F, int64_t NB, int64_t W, int kind, bool s
   L.DT = take(8 * F);
   L.bDT = take(8 * NB);
   L.bval = take(8 * NB);
+  L.bg = take(8 * NB);
+  L.bT = take(8 * NB);
+  L.bgT = take(8 * NB);
+  L.bsum2 = take(16 * NB);
   L.diag = take(8 * N);
   L.upper = take(8 * F);
   L.slot_coef = take(8 * W * N);
@@ -209,6 +214,7 @@ struct lfm_ctx {
   bool has64 = false, has32 = false;  // solver blocks present in the workspace
   bool hasdf = false;                 // df64 block present
   bool df_dirty = true;               // df64 conductances / V/dt to rebuild before the next df64 launch
+  bool bnd_dirty = true;              // boundary faces' row terms to rebuild before the next launch
   bool coef_dirty = true;             // FP64 / FP32 slot coefficients to rebuild before the next launch
   double mean_V = 1.0;                // mean cell volume (sets the df64 scale with dt)
   bool has_geom = false;              // general geometry uploaded (corrected laplacian)
@@ -438,6 +444,10 @@ void bind_pointers(lfm_ctx* c) {
   cs.DT = reinterpret_cast<const double*>(b + L.DT);
   cs.bDT = reinterpret_cast<const double*>(b + L.bDT);
   cs.bval = reinterpret_cast<const double*>(b + L.bval);
+  cs.bg = reinterpret_cast<const double*>(b + L.bg);
+  cs.bT = reinterpret_cast<const double*>(b + L.bT);
+  cs.bgT = reinterpret_cast<const double*>(b + L.bgT);
+  cs.bsum2 = reinterpret_cast<const float4*>(b + L.bsum2);
   if (c->mesh_src) {
     const CaseDev& m = c->mesh_src->cs;
     cs.slot_other = m.slot_other;
@@ -548,6 +558,7 @@ int refresh_vdt(lfm_ctx* c) {
   CK(c, cudaStreamSynchronize(c->stream));
   c->cs.df_scale = df_scale_for(c->mean_V, c->dt);
   c->df_dirty = true;
+  c->bnd_dirty = true;  // its df64 pairs carry the scale
   return LFM_OK;
 }
 
@@ -570,6 +581,16 @@ int refresh_df(lfm_ctx* c) {
   CK(c, launch_df_setup(c->cs, c->stream));
   CK(c, cudaStreamSynchronize(c->stream));  // batches launch on their own stream
   c->df_dirty = false;
+  return LFM_OK;
+}
+
+// Rebuilds the boundary faces' row terms when the patches, their values, DT, dt or the mesh
+// changed since the last launch (every form's rows read them, matrix read-back too).
+int refresh_bnd(lfm_ctx* c) {
+  if (!c->bnd_dirty) return LFM_OK;
+  CK(c, launch_boundary_terms(c->cs, c->stream));
+  CK(c, cudaStreamSynchronize(c->stream));  // batches launch on their own stream
+  c->bnd_dirty = false;
   return LFM_OK;
 }
 
@@ -613,6 +634,7 @@ int need_uploaded(lfm_ctx* c) {
 int enqueue_chunk(lfm_ctx* c, int steps, int mode) {
   refresh_case(c);
   if (int rc = refresh_ops(c)) return rc;
+  if (int rc = refresh_bnd(c)) return rc;
   if (mode == kModeSteps) {
     if (int rc = refresh_coef(c)) return rc;
     if (int rc = refresh_df(c)) return rc;
@@ -793,6 +815,7 @@ static int upload_mesh_impl(lfm_ctx* c, const lfm_mesh* m, const lfm_geometry* g
   c->has32 = has32;
   c->hasdf = hasdf;
   c->df_dirty = true;
+  c->bnd_dirty = true;
   c->coef_dirty = true;
   c->has_geom = geo != nullptr;
   c->n_corr = 0;
@@ -963,6 +986,7 @@ int lfm_upload_box(lfm_ctx* c, int32_t nx, int32_t ny, int32_t nz, const double*
   c->has32 = has32;
   c->hasdf = hasdf;
   c->df_dirty = true;
+  c->bnd_dirty = true;
   c->coef_dirty = true;
   c->has_geom = false;
   c->n_corr = 0;
@@ -1053,6 +1077,7 @@ int lfm_upload_mesh_shared(lfm_ctx* c, lfm_ctx* src) {
   c->has32 = has32;
   c->hasdf = hasdf;
   c->df_dirty = true;
+  c->bnd_dirty = true;
   c->coef_dirty = true;
   c->has_geom = root->has_geom;
   c->ops_dirty = root->has_geom;
@@ -1126,6 +1151,7 @@ int lfm_set_diffusivity(lfm_ctx* c, double uniform, const double* DT_faces, cons
   CK(c, cudaStreamSynchronize(c->stream));
   c->ops_dirty = true;
   c->df_dirty = true;
+  c->bnd_dirty = true;
   c->coef_dirty = true;
   return LFM_OK;
 }
@@ -1158,6 +1184,7 @@ int lfm_set_diffusivity_cells(lfm_ctx* c, const double* DT_cells, const double* 
   c->cs.DT_is_uniform = 0;
   c->ops_dirty = true;
   c->df_dirty = true;
+  c->bnd_dirty = true;
   c->coef_dirty = true;
   return LFM_OK;
 }
@@ -1214,6 +1241,7 @@ int lfm_set_patch(lfm_ctx* c, int32_t patch, int32_t type, const double* values,
   CK(c, cudaStreamSynchronize(c->stream));
   c->patch_type[patch] = type;
   c->ops_dirty = true;
+  c->bnd_dirty = true;
   return LFM_OK;
 }
 
@@ -1819,7 +1847,7 @@ int lfm_batch_advance_capped_async(lfm_batch* b, int32_t n_steps, int32_t use_gr
     if ((c->opts.precision == LFM_FP64 && !c->has64) || (c->opts.precision == LFM_MIXED && !c->has32) ||
         (c->opts.precision == LFM_DF64 && !(c->hasdf && c->has64)))
       return bfail(b, LFM_ENOMEM, "case %d has no buffers for its precision", b->order[i]);
-    if (refresh_coef(c) != LFM_OK || refresh_df(c) != LFM_OK)
+    if (refresh_coef(c) != LFM_OK || refresh_bnd(c) != LFM_OK || refresh_df(c) != LFM_OK)
       return bfail(b, LFM_ECUDA, "case %d: coefficient set-up failed", b->order[i]);
     b->h_cases[i] = c->cs;
     if (c->W != 6) W = 0;
@@ -2243,7 +2271,7 @@ int lfm_dd_advance(lfm_dd* d, int32_t n_steps, lfm_step_stats* out) {
   if (n_steps == 0) return LFM_OK;
   DeviceGuard g(c->device);
   refresh_case(c);
-  if ((rc = refresh_coef(c))) return ddfail(d, rc, "coefficient set-up of the case failed");
+  if ((rc = refresh_coef(c)) || (rc = refresh_bnd(c))) return ddfail(d, rc, "coefficient set-up of the case failed");
   CaseDev cs = c->cs;  // the case's rows, with the decomposition's own barrier words and records
   cs.sync = d->sync;
   cs.partials = d->partials;

@@ -85,6 +85,14 @@ struct CaseDev {
   const double* bDT;         // [NB]
   const double* bval;        // [NB]  fixedValue values
   const int32_t* btype;      // [NB]  LFM_FIXED_VALUE / LFM_ZERO_GRADIENT
+  // what a row adds for each of its boundary faces, in the order of b_face (rebuilt when the
+  // patches, DT, dt or the mesh change): the conductance g_b = (DT |Sf|) deltaCoeff, zero for
+  // zeroGradient, T_b and g_b T_b; and at the first face of each cell the cell's sums of g_b and
+  // g_b T_b, times df_scale, as double-float pairs (x, y and z, w)
+  const double* bg;          // [NB]
+  const double* bT;          // [NB]
+  const double* bgT;         // [NB]
+  const float4* bsum2;       // [NB]
 
   // general (non-orthogonal) geometry; null for orthogonal meshes. With it, delta holds the
   // implicit (nonOrthDeltaCoeffs) coefficients and the corrected laplacian adds an explicit
@@ -236,6 +244,8 @@ bool mixed_runs_df(const CaseDev& cs);
 // df64 form set-up: the per-slot conductances g2 and V/dt (vdt2), both times cs.df_scale,
 // and on general geometry the operator weights gE2, cK2, cL2 and gZ (see CaseDev).
 cudaError_t launch_df_setup(const CaseDev& cs, cudaStream_t stream);
+// Set-up of the boundary faces' row terms (bg, bT, bgT, bsum2).
+cudaError_t launch_boundary_terms(const CaseDev& cs, cudaStream_t stream);
 
 // Face-to-cell addressing of a general mesh built on the device (lfm_addr.cu): owner,
 // neighbour, bface_cell are device arrays; W the largest internal-face count of a cell.

@@ -171,8 +171,11 @@ __device__ __forceinline__ double plus_zero(double v) {
   return (bits << 1) == 0 ? 0.0 : v;
 }
 
-// xo: T of the cell at the start of the step (the ddt source).
-// word: the row's slot code (bit 31 clear: no boundary faces, nothing to look up).
+// xo: T of the cell at the start of the step (the ddt source). kDiag: the diagonal is summed too.
+// word: the row's slot code (bit 31 clear: no boundary faces, nothing to look up). The faces'
+// conductances lie in list order (CaseDev::bg): one level of loads after b_start, where walking
+// face id -> type, DT, |Sf|, deltaCoeff, value took three, in a third of all warps of a box.
+template <bool kDiag = true>
 __device__ __forceinline__ void row_boundary(const CaseDev& cs, int c, double xo, Row& o, uint32_t word = 0xffffffffu) {
   int b0 = 0, b1 = 0;
   if (word >> 31) {
@@ -182,22 +185,20 @@ __device__ __forceinline__ void row_boundary(const CaseDev& cs, int c, double xo
   const double vdt = cs.vdt[c];  // V/dt, formed once per (mesh, dt): the same IEEE quotient
   const double sv = __dmul_rn(vdt, xo);
   if (b0 == b1) {  // no boundary face: the sums below start from zero
-    o.d = __dadd_rn(o.d, vdt);
+    if constexpr (kDiag) o.d = __dadd_rn(o.d, vdt);
     o.s = plus_zero(sv);
     o.sa = vdt;
     return;
   }
   double s = 0.0, gsum = 0.0;  // source, boundary conductance of the row
   for (int k = b0; k < b1; ++k) {
-    const int bf = LFM_IDX(__ldg(cs.b_face + k), cs.NB, 0, kChkBFace);
-    if (__ldg(cs.btype + bf) == LFM_FIXED_VALUE) {
-      const double gb = __dmul_rn(__dmul_rn(__ldg(cs.bDT + bf), __ldg(cs.bmagSf + bf)), __ldg(cs.bdelta + bf));
-      o.d = __dadd_rn(o.d, gb);
-      s = __dadd_rn(s, __dmul_rn(gb, __ldg(cs.bval + bf)));
-      gsum = __dadd_rn(gsum, gb);
-    }
+    const double gb = __ldg(cs.bg + k);
+    if (__double_as_longlong(gb) == 0) continue;  // zeroGradient (or no conductance): adds nothing
+    if constexpr (kDiag) o.d = __dadd_rn(o.d, gb);
+    s = __dadd_rn(s, __ldg(cs.bgT + k));
+    gsum = __dadd_rn(gsum, gb);
   }
-  o.d = __dadd_rn(o.d, vdt);
+  if constexpr (kDiag) o.d = __dadd_rn(o.d, vdt);
   o.s = __dadd_rn(s, sv);
   o.sa = gsum + vdt;
 }
@@ -259,7 +260,11 @@ __device__ __forceinline__ double op_corr_source(const CaseDev& cs, int c) {
 // source: the ddt source comes from x_old (with correctors), the source S_T = Su + Sp T
 // enters (V Su to the source, -V Sp to the diagonal), and the explicit correction of the
 // row's faces is added to the source.
-template <int W, bool kCorr = false>
+// kRows: the diagonal is assembled; false: it is read back. The matrix does not depend on T, so
+// a launch assembles it in its first pass over the rows, every launch anew, and the later steps
+// and corrector passes form the source and the residual only: of a row's 32 FP64 instructions,
+// which bound this pass, 16 remain.
+template <int W, bool kCorr = false, bool kRows = true>
 __device__ __forceinline__ Row assemble_row(const CaseDev& cs, int c, const double* __restrict__ x) {
   const size_t N = (size_t)cs.N;
   Row o;
@@ -274,10 +279,12 @@ __device__ __forceinline__ Row assemble_row(const CaseDev& cs, int c, const doub
     word = neighbours<W, false>(cs.slot_other, cs.slot_code, cs.N, delta_table<W>(cs), c, oc, kChkSlotCell);
 #pragma unroll
     for (int k = 0; k < S; ++k) u[k] = cs.slot_coef[(size_t)k * N + c];
-    // 0 + g_0 = g_0 exactly; the sign of a zero cannot reach d, which ends above V/dt > 0
-    o.d = -u[0];
+    if constexpr (kRows) {
+      // 0 + g_0 = g_0 exactly; the sign of a zero cannot reach d, which ends above V/dt > 0
+      o.d = -u[0];
 #pragma unroll
-    for (int k = 1; k < S; ++k) o.d = __dadd_rn(o.d, -u[k]);  // padding slots hold 0
+      for (int k = 1; k < S; ++k) o.d = __dadd_rn(o.d, -u[k]);  // padding slots hold 0
+    }
 #pragma unroll
     for (int k = 0; k < S; ++k) off = fma(u[k], x[oc[k]], off);
   } else {
@@ -285,14 +292,15 @@ __device__ __forceinline__ Row assemble_row(const CaseDev& cs, int c, const doub
     for (int k = 0; k < ns; ++k) {
       const size_t at = (size_t)k * N + c;
       const double u = cs.slot_coef[at];
-      o.d = __dadd_rn(o.d, -u);
+      if constexpr (kRows) o.d = __dadd_rn(o.d, -u);
       off = fma(u, x[LFM_IDX(__ldg(cs.slot_other + at), cs.N, c, kChkSlotCell)], off);
     }
   }
-  row_boundary(cs, c, kCorr && cs.n_corr > 0 ? cs.x_old[c] : o.xc, o, word);
+  row_boundary<kRows>(cs, c, kCorr && cs.n_corr > 0 ? cs.x_old[c] : o.xc, o, word);
+  if constexpr (!kRows) o.d = cs.diag[c];
   if (kCorr && cs.vSp) {  // implicit part of the source S_T = Su + Sp T
     const double v = cs.vSp[c];
-    o.d = __dsub_rn(o.d, v);
+    if constexpr (kRows) o.d = __dsub_rn(o.d, v);
     o.sa = o.sa - v;
   }
   if (kCorr && cs.vSu) o.s = __dadd_rn(o.s, cs.vSu[c]);
@@ -761,18 +769,23 @@ struct Sums3 {
   double a, b, c;
 };
 
-// A2 + I (FP64 step): the rows of the matrix and, from the same loaded row, r = b - A x,
+// A2 + I (FP64 step): the rows of the matrix (kRows) and, from the same loaded row, r = b - A x,
 // the normFactor terms, sum|r|, w = rD r and rho; p = w. Returns this thread's normFactor
 // sum, sum|r| and rho.
-template <int B, int W, bool kCorr>
+template <int B, int W, bool kCorr, bool kRows>
 __device__ __noinline__ Sums3 pass_rows_init_f64(const CaseDev& cs, int c0, int c1, double xRef) {
   double* __restrict__ r = cs.r;
   double* __restrict__ p = cs.p;
   const double* __restrict__ x = cs.x;
   double u0 = 0.0, u1 = 0.0, u2 = 0.0;
   for (int c = c0 + (int)threadIdx.x; c < c1; c += B) {
-    const Row o = assemble_row<W, kCorr>(cs, c, x);
-    const double rd = store_row<false>(cs, c, o, false);
+    const Row o = assemble_row<W, kCorr, kRows>(cs, c, x);
+    double rd;
+    if constexpr (kRows) {
+      rd = store_row<false>(cs, c, o, false);
+    } else {
+      rd = cs.rD[c];
+    }
     const double rc = o.s - o.ax;
     u0 += fabs(fma(-o.sa, xRef, o.ax)) + fabs(fma(-o.sa, xRef, o.s));
     u1 += fabs(rc);
@@ -789,7 +802,7 @@ __device__ __noinline__ Sums3 pass_rows_init_f64(const CaseDev& cs, int c0, int 
 // With kFirst it is computed together with the rows of
 // the matrix (A2) and the normFactor terms. Returns this thread's normFactor sum (kFirst),
 // sum|r| and rho (FP32 terms accumulated exactly as FP32 pairs).
-template <int B, int W, bool kFirst, bool kCorr>
+template <int B, int W, bool kFirst, bool kCorr, bool kRows = true>
 __device__ __noinline__ Sums3 pass_true_residual(const CaseDev& cs, int c0, int c1, double xRef) {
   float* __restrict__ r = cs.r32;
   float* __restrict__ w = cs.w32;
@@ -801,8 +814,13 @@ __device__ __noinline__ Sums3 pass_true_residual(const CaseDev& cs, int c0, int 
     double rc;
     float rd32;
     if (kFirst) {
-      const Row o = assemble_row<W, kCorr>(cs, c, x);
-      rd32 = (float)store_row<true>(cs, c, o, true);
+      const Row o = assemble_row<W, kCorr, kRows>(cs, c, x);
+      if constexpr (kRows) {
+        rd32 = (float)store_row<true>(cs, c, o, true);
+      } else {
+        cs.src[c] = o.s;
+        rd32 = cs.rD32[c];
+      }
       u0 += fabs(fma(-o.sa, xRef, o.ax)) + fabs(fma(-o.sa, xRef, o.s));
       rc = o.s - o.ax;
     } else {
@@ -958,8 +976,11 @@ __device__ void run_steps_f64(const CaseDev& cs, const CaseDev& cref, const TM& 
       }
       // ---- A2 + I: rows of the matrix, initial residual, normFactor, first direction -----
       const double xRef = sh.xref;
-      const Sums3 ui = corr_mode ? pass_rows_init_f64<B, W, true>(cref, c0, c1, xRef)
-                                 : pass_rows_init_f64<B, W, false>(cref, c0, c1, xRef);
+      const bool rows = step == 0 && pass == 0;  // the matrix is assembled in the launch's first pass
+      const Sums3 ui = corr_mode ? (rows ? pass_rows_init_f64<B, W, true, true>(cref, c0, c1, xRef)
+                                         : pass_rows_init_f64<B, W, true, false>(cref, c0, c1, xRef))
+                                 : (rows ? pass_rows_init_f64<B, W, false, true>(cref, c0, c1, xRef)
+                                         : pass_rows_init_f64<B, W, false, false>(cref, c0, c1, xRef));
       const double u[3] = {ui.a, ui.b, ui.c};  // normFactor sum, sum|r|, rho
       if (!team_allreduce<3, B>(tm, u, sh, [&](int k, double t, int lane) {
             if (lane == 0) sh.out[k] = t;
@@ -1121,10 +1142,12 @@ __device__ void run_steps_mixed(const CaseDev& cs, const CaseDev& cref, const TM
         Sums3 ui;
         if (sweeps > 0)
           ui = pass_true_residual<B, W, false, false>(cref, c0, c1, xRef);
-        else if (corr_mode)
-          ui = pass_true_residual<B, W, true, true>(cref, c0, c1, xRef);
-        else
-          ui = pass_true_residual<B, W, true, false>(cref, c0, c1, xRef);
+        else if (step == 0 && pass == 0)
+          ui = corr_mode ? pass_true_residual<B, W, true, true>(cref, c0, c1, xRef)
+                         : pass_true_residual<B, W, true, false>(cref, c0, c1, xRef);
+        else  // the launch's first pass assembled the matrix
+          ui = corr_mode ? pass_true_residual<B, W, true, true, false>(cref, c0, c1, xRef)
+                         : pass_true_residual<B, W, true, false, false>(cref, c0, c1, xRef);
         const double u[3] = {ui.a, ui.b, ui.c};  // normFactor sum (first sweep), sum|r|, rho
         if (!team_allreduce<3, B>(tm, u, sh, [&](int k, double t, int lane) {
               if (lane == 0) sh.out[k] = t;

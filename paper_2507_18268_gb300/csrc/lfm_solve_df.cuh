@@ -134,33 +134,29 @@ __device__ __noinline__ void pass_store_x(const CaseDev& cs, int c0, int c1, boo
   }
 }
 
-// Boundary conductance, source and flux g_b (T_b - x_c) of row c (fixedValue faces;
-// zeroGradient adds nothing), in FP64 with the case scale, in ascending face order.
+// Boundary conductance, source and flux g_b (T_b - x_c) of row c (fixedValue faces; zeroGradient
+// adds nothing), in FP64 with the case scale, in ascending face order. The first two do not depend
+// on the field and come as pairs from set-up; the flux is formed here, two FP64 operations per
+// face beside the conversions (a third of a box's warps hold a boundary cell, and each spent some 25
+// warp instructions of 64 clocks on the three sums).
 __device__ __forceinline__ void row_boundary_df(const CaseDev& cs, int c, tf xc, df& gsum, df& ssum, df& flux,
                                                 uint32_t word = 0xffffffffu) {
-  int b0 = 0, b1 = 0;
-  if (word >> 31) {  // the slot code says whether there are any (all ones when not coded)
-    b0 = __ldg(cs.b_start + c);
-    b1 = __ldg(cs.b_start + c + 1);
-  }
   gsum = mkdf(0.0f, 0.0f);
   ssum = mkdf(0.0f, 0.0f);
   flux = mkdf(0.0f, 0.0f);
+  if (!(word >> 31)) return;  // the slot code says whether there are any (all ones when not coded)
+  const int b0 = __ldg(cs.b_start + c), b1 = __ldg(cs.b_start + c + 1);
   if (b0 == b1) return;
+  const float4 sums = __ldg(cs.bsum2 + b0);
+  if (sums.x == 0.0f) return;  // no fixedValue face (or no conductance)
+  gsum = mkdf(sums.x, sums.y);
+  ssum = mkdf(sums.z, sums.w);
   const double x = tf_to_double(xc);
-  double g = 0.0, s = 0.0, fl = 0.0;
+  double fl = 0.0;
   for (int k = b0; k < b1; ++k) {
-    const int bf = LFM_IDX(__ldg(cs.b_face + k), cs.NB, 0, kChkBFace);
-    if (__ldg(cs.btype + bf) == LFM_FIXED_VALUE) {
-      const double gb = __ldg(cs.bDT + bf) * __ldg(cs.bmagSf + bf) * __ldg(cs.bdelta + bf) * cs.df_scale;
-      const double tb = __ldg(cs.bval + bf);
-      g += gb;
-      s += gb * tb;
-      fl += gb * (tb - x);
-    }
+    const double gb = __ldg(cs.bg + k) * cs.df_scale;  // a power of two: exact
+    if (__double_as_longlong(gb) != 0) fl += gb * (__ldg(cs.bT + k) - x);
   }
-  gsum = df_from_double(g);
-  ssum = df_from_double(s);
   flux = df_from_double(fl);
 }
 
@@ -275,7 +271,9 @@ __device__ __forceinline__ void prefetch_row_df(const CaseDev& cs, int c) {
 // |b| / |r| (about 1e6 for a time step that changes T by one part in a million); the
 // differences of nearby values here are almost exact, so r keeps the format's relative
 // accuracy. A x for the normFactor terms is then b - r.
-template <int B, int W, bool kSrc>
+// kRows: the diagonal and its reciprocal are formed (the first pass of a launch); false: the
+// reciprocal is read back, the diagonal is not needed.
+template <int B, int W, bool kSrc, bool kRows>
 __device__ __noinline__ Sums3 pass_rows_init_df(const CaseDev& cs, int c0, int c1, df xr) {
   const float2* __restrict__ x2 = cs.x2;
   const float* __restrict__ xl = cs.xlo;
@@ -299,9 +297,11 @@ __device__ __noinline__ Sums3 pass_rows_init_df(const CaseDev& cs, int c0, int c
       tf xo_[S];
 #pragma unroll
       for (int k = 0; k < S; ++k) xo_[k] = ld_tf(x2, xl, o[k]);
-      d = g[0];
+      if constexpr (kRows) {
+        d = g[0];
 #pragma unroll
-      for (int k = 1; k < S; ++k) d = df_add(d, g[k]);  // padding slots hold 0
+        for (int k = 1; k < S; ++k) d = df_add(d, g[k]);  // padding slots hold 0
+      }
       flux = df_mul(g[0], tf_diff(xo_[0], xc));
 #pragma unroll
       for (int k = 1; k < S; ++k) flux = df_fma(g[k], tf_diff(xo_[k], xc), flux);
@@ -311,7 +311,7 @@ __device__ __noinline__ Sums3 pass_rows_init_df(const CaseDev& cs, int c0, int c
       for (int k = 0; k < cs.W; ++k) {
         const size_t at = (size_t)k * N + c;
         const df gk = ldg_df(g2 + at);
-        d = df_add(d, gk);
+        if constexpr (kRows) d = df_add(d, gk);
         flux = df_fma(gk, tf_diff(ld_tf(x2, xl, LFM_IDX(__ldg(cs.slot_other + at), cs.N, c, kChkSlotCellDf)), xc), flux);
       }
     }
@@ -321,7 +321,7 @@ __device__ __noinline__ Sums3 pass_rows_init_df(const CaseDev& cs, int c0, int c
     const df xcd = tf_to_df(xc);
     const bool has_old = kSrc && cs.n_corr > 0;
     const tf xo = has_old ? ld_tf(reinterpret_cast<const float2*>(cs.x_old), cs.xolo, c) : xc;
-    d = df_add(df_add(d, gb), vdt);
+    if constexpr (kRows) d = df_add(df_add(d, gb), vdt);
     df src = df_fma(vdt, has_old ? tf_to_df(xo) : xcd, sb);
     df sa = df_add(vdt, gb);
     df rc = df_add(flux, fb);
@@ -331,7 +331,7 @@ __device__ __noinline__ Sums3 pass_rows_init_df(const CaseDev& cs, int c0, int c
       const double sp = cs.vSp ? cs.vSp[c] * cs.df_scale : 0.0;
       const double su = cs.vSu ? cs.vSu[c] * cs.df_scale : 0.0;
       const df vsp = df_from_double(sp);
-      d = df_sub(d, vsp);
+      if constexpr (kRows) d = df_sub(d, vsp);
       sa = df_sub(sa, vsp);
       src = df_add(src, df_from_double(su));
       rc = df_add(rc, df_from_double(fma(sp, tf_to_double(xc), su)));
@@ -342,15 +342,17 @@ __device__ __noinline__ Sums3 pass_rows_init_df(const CaseDev& cs, int c0, int c
       rc = df_add(rc, corr);
     }
     const df ax = df_sub(src, rc);
-    const df rd = df_rcp(d);
+    const df rd = kRows ? df_rcp(d) : ld_df(cs.rD2 + c);
     const df sx = df_mul(sa, xr);
     a_nf.add(df_abs(df_sub(ax, sx)));
     a_nf.add(df_abs(df_sub(src, sx)));
     a_r.add(df_abs(rc));
     const df wc = df_mul(rd, rc);
     a_rho.add(df_mul(wc, rc));
-    st_df(cs.diag2 + c, d);
-    st_df(cs.rD2 + c, rd);
+    if constexpr (kRows) {
+      st_df(cs.diag2 + c, d);
+      st_df(cs.rD2 + c, rd);
+    }
     st_df(r2 + c, rc);
     st_df(p2 + c, wc);
   }
@@ -561,8 +563,12 @@ __device__ bool steps_df64(const CaseDev& cs, const CaseDev& cref, const TM& tm,
       }
       clk.lap(kPhAssembly);
       // ---- R: rows, initial residual, normFactor, first direction ----------------------
-      const Sums3 ui = src_mode ? pass_rows_init_df<B, W, true>(cref, c0, c1, df_of(sh.xref2))
-                                : pass_rows_init_df<B, W, false>(cref, c0, c1, df_of(sh.xref2));
+      const bool rows = step == 0 && pass == 0;  // the matrix is assembled in the launch's first pass
+      const df xr = df_of(sh.xref2);
+      const Sums3 ui = src_mode ? (rows ? pass_rows_init_df<B, W, true, true>(cref, c0, c1, xr)
+                                        : pass_rows_init_df<B, W, true, false>(cref, c0, c1, xr))
+                                : (rows ? pass_rows_init_df<B, W, false, true>(cref, c0, c1, xr)
+                                        : pass_rows_init_df<B, W, false, false>(cref, c0, c1, xr));
       const double u[3] = {ui.a, ui.b, ui.c};
       if (!team_allreduce<3, B>(tm, u, sh, [&](int k, double t, int lane) {
             if (lane == 0) sh.out[k] = t;

@@ -79,25 +79,32 @@ __device__ __forceinline__ void row_flux_df(const CaseDev& cs, int c, const tf& 
   }
 }
 
-// The rest of a step's first row pass once the row is assembled (diag d, source src, row sum
-// sa, residual rc; all scaled): A x = src - rc and the normFactor terms against xRef (xr),
+// The rest of a step's first row pass once the row is assembled (kRows: diag d; source src, row
+// sum sa, residual rc; all scaled): A x = src - rc and the normFactor terms against xRef (xr),
 // sum|r|, and the inner solve's seed r32 = r / s, w32 = rD32 r32, p32 = w32 (dx32 starts at zero
 // implicitly: the solve's first update writes it),
-// rho = w32.r32 (FP32 pairs), with the FP32 copies of diag / s and s / diag.
+// rho = w32.r32 (FP32 pairs), with the FP32 copies of diag / s and s / diag (kRows; otherwise the
+// latter is read back: the matrix does not change within a launch, or since the last launch when
+// that left the seed).
+template <bool kRows>
 __device__ __forceinline__ void seed_row_df(const CaseDev& cs, int c, df d, df src, df sa, df rc, df xr, float s32,
                                             float inv_s32, DfAcc& a_nf, DfAcc& a_r, Acc2f& a_rho) {
   const df ax = df_sub(src, rc);
-  const df rd = df_rcp(d);
   const df sx = df_mul(sa, xr);
   a_nf.add(df_abs(df_sub(ax, sx)));
   a_nf.add(df_abs(df_sub(src, sx)));
   a_r.add(df_abs(rc));
-  const float rd32 = __fmul_rn(rd.hi, s32);
+  float rd32;
+  if constexpr (kRows) {
+    rd32 = __fmul_rn(df_rcp(d).hi, s32);
+    cs.diag32[c] = __fmul_rn(d.hi, inv_s32);
+    cs.rD32[c] = rd32;
+  } else {
+    rd32 = cs.rD32[c];
+  }
   const float r32 = __fmul_rn(rc.hi, inv_s32);
   const float w32 = __fmul_rn(rd32, r32);
   a_rho.add_prod(w32, r32);
-  cs.diag32[c] = __fmul_rn(d.hi, inv_s32);
-  cs.rD32[c] = rd32;
   cs.r32[c] = r32;
   cs.w32[c] = w32;
   cs.p32[c] = w32;
@@ -106,7 +113,7 @@ __device__ __forceinline__ void seed_row_df(const CaseDev& cs, int c, df d, df s
 // T0: rows of the matrix, the true residual (flux form), normFactor terms, sum|r| (scaled;
 // the caller unscales) and the seed of the inner solve. kSrc: correctors (ddt source from
 // x_old) or volumetric sources present.
-template <int B, int W, bool kSrc>
+template <int B, int W, bool kSrc, bool kRows>
 __device__ __noinline__ Sums3 pass_rows_init_mixed_df(const CaseDev& cs, int c0, int c1, df xr, float s32,
                                                       float inv_s32) {
   DfAcc a_nf, a_r;
@@ -116,13 +123,13 @@ __device__ __noinline__ Sums3 pass_rows_init_mixed_df(const CaseDev& cs, int c0,
     const tf xc = ld_tf(cs.x2, cs.xlo, c);
     df d, flux;
     uint32_t word;
-    row_flux_df<W, true>(cs, c, xc, d, flux, word);
+    row_flux_df<W, kRows>(cs, c, xc, d, flux, word);
     df gb, sb, fb;
     row_boundary_df(cs, c, xc, gb, sb, fb, word);
     const df vdt = ldg_df(cs.vdt2 + c);
     const bool has_old = kSrc && cs.n_corr > 0;
     const tf xo = has_old ? ld_tf(reinterpret_cast<const float2*>(cs.x_old), cs.xolo, c) : xc;
-    d = df_add(df_add(d, gb), vdt);
+    if constexpr (kRows) d = df_add(df_add(d, gb), vdt);
     df src = df_fma(vdt, tf_to_df(xo), sb);
     df sa = df_add(vdt, gb);
     df rc = df_add(flux, fb);
@@ -131,12 +138,12 @@ __device__ __noinline__ Sums3 pass_rows_init_mixed_df(const CaseDev& cs, int c0,
       const double sp = cs.vSp ? cs.vSp[c] * cs.df_scale : 0.0;
       const double su = cs.vSu ? cs.vSu[c] * cs.df_scale : 0.0;
       const df vsp = df_from_double(sp);
-      d = df_sub(d, vsp);
+      if constexpr (kRows) d = df_sub(d, vsp);
       sa = df_sub(sa, vsp);
       src = df_add(src, df_from_double(su));
       rc = df_add(rc, df_from_double(fma(sp, tf_to_double(xc), su)));
     }
-    seed_row_df(cs, c, d, src, sa, rc, xr, s32, inv_s32, a_nf, a_r, a_rho);
+    seed_row_df<kRows>(cs, c, d, src, sa, rc, xr, s32, inv_s32, a_nf, a_r, a_rho);
   }
   return Sums3{a_nf.value(), a_r.value(), a_rho.value()};
 }
@@ -196,15 +203,14 @@ __device__ __noinline__ Sums4 pass_verify_next_df(const CaseDev& cs, int c0, int
     const tf xc = ld_tf(cs.x2, cs.xlo, c);
     df d, flux;
     uint32_t word;
-    row_flux_df<W, true>(cs, c, xc, d, flux, word);
+    row_flux_df<W, false>(cs, c, xc, d, flux, word);
     df gb, sb, fb;
     row_boundary_df(cs, c, xc, gb, sb, fb, word);
     const df vdt = ldg_df(cs.vdt2 + c);
     const tf xo = ld_tf(reinterpret_cast<const float2*>(cs.x_old), cs.xolo, c);
     const df rn = df_add(flux, fb);  // the next step's first residual
     a_v.add(df_abs(df_fma(vdt, tf_diff(xo, xc), rn)));
-    d = df_add(df_add(d, gb), vdt);
-    seed_row_df(cs, c, d, df_fma(vdt, tf_to_df(xc), sb), df_add(vdt, gb), rn, xr, s32, inv_s32, a_nf, a_r, a_rho);
+    seed_row_df<false>(cs, c, d, df_fma(vdt, tf_to_df(xc), sb), df_add(vdt, gb), rn, xr, s32, inv_s32, a_nf, a_r, a_rho);
   }
   return Sums4{a_v.value(), a_nf.value(), a_r.value(), a_rho.value()};
 }
@@ -300,9 +306,15 @@ __device__ bool steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const TM&
         if (!have_u) {
           double u[3];
           if (sweeps == 0) {
-            const Sums3 ui = src_mode
-                                 ? pass_rows_init_mixed_df<B, W, true>(cref, c0, c1, df_of(sh.xref2), s32, inv_s32)
-                                 : pass_rows_init_mixed_df<B, W, false>(cref, c0, c1, df_of(sh.xref2), s32, inv_s32);
+            // the matrix is assembled in the launch's first pass; a step whose rows V left in
+            // place comes here only for its sources' or correctors' sake (never fused) or first
+            const bool rows = step == 0 && pass == 0;
+            const df xr = df_of(sh.xref2);
+            const Sums3 ui =
+                src_mode ? (rows ? pass_rows_init_mixed_df<B, W, true, true>(cref, c0, c1, xr, s32, inv_s32)
+                                 : pass_rows_init_mixed_df<B, W, true, false>(cref, c0, c1, xr, s32, inv_s32))
+                         : (rows ? pass_rows_init_mixed_df<B, W, false, true>(cref, c0, c1, xr, s32, inv_s32)
+                                 : pass_rows_init_mixed_df<B, W, false, false>(cref, c0, c1, xr, s32, inv_s32));
             u[0] = ui.a;
             u[1] = ui.b;
             u[2] = ui.c;

@@ -141,6 +141,36 @@ __global__ void df_vdt_kernel(CaseDev cs, float2* __restrict__ vdt2) {
   if (c < cs.N) st_df(vdt2 + c, df_from_double(__dmul_rn(cs.vdt[c], cs.df_scale)));
 }
 
+// A row's boundary terms per boundary face, in list order (see CaseDev::bg): the products and sums
+// of the assembly in its order, so the rows keep their bits.
+__global__ void boundary_terms_kernel(CaseDev cs, double* __restrict__ g, double* __restrict__ T,
+                                      double* __restrict__ gT, float4* __restrict__ sum2) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= cs.NB) return;
+  auto term = [&](int i, double& gb, double& t) {
+    const int bf = LFM_IDX(cs.b_face[i], cs.NB, 0, kChkBFace);
+    const bool fixed = cs.btype[bf] == LFM_FIXED_VALUE;
+    gb = fixed ? __dmul_rn(__dmul_rn(cs.bDT[bf], cs.bmagSf[bf]), cs.bdelta[bf]) : 0.0;
+    t = fixed ? cs.bval[bf] : 0.0;
+  };
+  double gb, t;
+  term(k, gb, t);
+  g[k] = gb;
+  T[k] = t;
+  gT[k] = __dmul_rn(gb, t);
+  const int c = LFM_IDX(cs.bcell[LFM_IDX(cs.b_face[k], cs.NB, 0, kChkBFace)], cs.N, 0, kChkBFace);
+  if (k != cs.b_start[c]) return;  // the cell's sums stand at its first face
+  double gs = 0.0, ss = 0.0;
+  for (int i = k; i < cs.b_start[c + 1]; ++i) {
+    term(i, gb, t);
+    const double gbs = gb * cs.df_scale;
+    gs += gbs;
+    ss += gbs * t;
+  }
+  const df g2 = df_from_double(gs), s2 = df_from_double(ss);
+  sum2[k] = make_float4(g2.hi, g2.lo, s2.hi, s2.lo);
+}
+
 __global__ void boundary_values_kernel(CaseDev cs, double* Tb) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b < cs.NB) Tb[b] = cs.btype[b] == LFM_FIXED_VALUE ? cs.bval[b] : cs.x[LFM_IDX(cs.bcell[b], cs.N, 0, kChkBFace)];
@@ -451,6 +481,14 @@ cudaError_t launch_df_setup(const CaseDev& cs, cudaStream_t stream) {
   if (cs.Sf && cs.gE2)
     df_ops_kernel<<<(cs.N + 255) / 256, 256, 0, stream>>>(cs, const_cast<float2*>(cs.gE2), const_cast<float2*>(cs.cK2),
                                                           const_cast<float2*>(cs.cL2), const_cast<float2*>(cs.gZ));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_boundary_terms(const CaseDev& cs, cudaStream_t stream) {
+  if (cs.NB == 0) return cudaSuccess;
+  boundary_terms_kernel<<<(cs.NB + 255) / 256, 256, 0, stream>>>(
+      cs, const_cast<double*>(cs.bg), const_cast<double*>(cs.bT), const_cast<double*>(cs.bgT),
+      const_cast<float4*>(cs.bsum2));
   return cudaGetLastError();
 }
 
