@@ -411,7 +411,7 @@ int lfm_debug_check_inject(lfm_ctx *ctx, int32_t site);
  * sorted by owner or a cell above the face limit are reported as LFM_EINVAL by the kernel
  * before it uses any of those indices as an address; x is then left unchanged. Every
  * non-OK return sets the text of lfm_last_error(NULL) on the calling thread.
- * Working memory: one fixed device array of about 4.8 MB inside the library, present on
+ * Working memory: one fixed device array of about 5.8 MB inside the library, present on
  * every GPU that loads it until the process exits; no call allocates, frees or calls an
  * allocating library routine. All calls share that array (each call re-initialises what it
  * needs), so calls whose kernels overlap on one GPU race: order them on one stream. The
