@@ -378,13 +378,32 @@ int h2d(lfm_ctx* c, size_t off, const T* src, size_t n) {
   return LFM_OK;
 }
 
-// Default launch: one team of co-resident CTAs of 512 threads, at least about 4096 cells
-// per CTA (the best shape in launch-shape sweeps on the 200^3 graded box).
+// Default launch shape. A pass costs its rows' dependent loads once per row a thread takes, its
+// FP64 instructions per row an SM takes, and a barrier that grows with the CTAs (two per SM over
+// one per SM: 4.4 against 3.4 us with one sum) and with the threads that add a sum. So: one row
+// per thread while one CTA of 256 per SM can hold them, then up to two; then one CTA of 512 per SM
+// up to four rows a thread; beyond, where bandwidth counts, every co-resident CTA of 512. Between
+// one and two CTAs per SM lies no good shape: the SMs that hold two set the time. Measured (ms a
+// call, before: 4096 cells per CTA of 512): 8,000 cells FP64 1.18 -> 0.44; 32,768 FP64 3.76 ->
+// 1.52; 56,869 mixed 3.76 -> 2.09; 110,592 mixed 2.41 -> 1.62; 262,144 FP64 3.30 -> 2.32 (304 CTAs
+// 2.33); 884,736 mixed 5.90 -> 5.46; 1,000,000 relabelled FP64 1.23 -> 1.09.
+constexpr int kThreadsSmall = 256, kThreads = 512;
+
 int choose_launch(lfm_ctx* c) {
-  const int threads = 512;
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess || sms < 1) sms = 1;
+  const int64_t N = c->N;
+  int threads = kThreads;
+  int64_t want = kMaxCtas;
+  if (N <= 2 * (int64_t)sms * kThreadsSmall) {
+    threads = kThreadsSmall;
+    want = (N + kThreadsSmall - 1) / kThreadsSmall;
+    if (want > sms) want = sms;
+  } else if (N <= 4 * (int64_t)sms * kThreads) {
+    want = sms;
+  }
   int maxc = max_coresident_ctas(c->opts.precision, threads, kernel_width(c->W, c->cs.slot_code != nullptr, threads), c->device);
   if (maxc <= 0) return fail(c, LFM_ECUDA, "cannot size the cooperative launch");
-  int64_t want = ((int64_t)c->N + 4095) / 4096;
   if (want < 1) want = 1;
   if (want > maxc) want = maxc;
   c->tuned_ctas = (int)want;
@@ -394,7 +413,8 @@ int choose_launch(lfm_ctx* c) {
 
 Launch current_launch(lfm_ctx* c, int& err) {
   Launch L{};
-  L.threads = c->threads > 0 ? c->threads : c->tuned_threads;
+  // a caller's CTA count alone keeps the threads it always came with
+  L.threads = c->threads > 0 ? c->threads : c->ctas > 0 ? kThreads : c->tuned_threads;
   int maxc = max_coresident_ctas(c->opts.precision, L.threads, kernel_width(c->W, c->cs.slot_code != nullptr, L.threads), c->device);
   L.ctas = c->ctas > 0 ? c->ctas : c->tuned_ctas;
   if (L.ctas > maxc) L.ctas = maxc;
