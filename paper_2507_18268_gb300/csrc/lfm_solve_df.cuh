@@ -241,10 +241,11 @@ __device__ __forceinline__ df op_corr_df(const CaseDev& cs, int c) {
   return v;
 }
 
-// L2 prefetch of what a row pass loads for row c before its gathers: the slot indices and
+// L2 prefetch of what a row pass loads for row c before its gathers: the slot word or indices and
 // conductances, the field value and V/dt. Issued one trip ahead (c + B), it shortens the
 // dependent chain index -> neighbour value of the next row (row pass 0.32 -> 0.30 ms per
-// step on the 200^3 graded box).
+// step on the 200^3 graded box; one bulk prefetch of the tile per array and CTA instead was slower,
+// 258 against 221 us for 8 M rows of the verification pass, none at all 235).
 template <int W>
 __device__ __forceinline__ void prefetch_row_df(const CaseDev& cs, int c) {
   const size_t N = (size_t)cs.N;
@@ -480,6 +481,68 @@ __device__ __forceinline__ double pass_amul_dot_df(const CaseDev& cs, uint32_t d
   return s.value();
 }
 
+// M with the matrix rows streamed into shared memory by bulk copies, as the FP32 A p
+// (pass_amul_dot_f32_bulk, lfm_solve.cuh): for packed meshes, one row per thread and tile (60
+// bytes per cell), three stages. The same cells per thread in the same order and the same
+// operations as the register form: equal results bit for bit. Needs N a multiple of 4 and the
+// dynamic shared memory of stage_bytes_df; ok = false when a wait ran out (status recorded).
+constexpr int kDfStages = 3;
+template <int W>
+__host__ __device__ constexpr unsigned stage_row_df() {  // bytes per cell: the code word, conductances, diagonal
+  return 4u + 8u * kSlots<W> + 8u;
+}
+template <int B, int W>
+__host__ __device__ constexpr unsigned stage_bytes_df() {
+  return kCoded<W> ? kDfStages * (B * stage_row_df<W>()) + 8u * kDfStages : 0u;
+}
+
+template <int B, int W, class TM>
+__device__ __noinline__ double pass_amul_dot_df_bulk(const CaseDev& cs, int c0, int c1, const float2* __restrict__ p,
+                                                     float2* __restrict__ q, const TM& tm, bool& ok) {
+  constexpr int S = kSlots<W>;
+  constexpr unsigned kStage = B * stage_row_df<W>();
+  const size_t N = (size_t)cs.N;
+  const uint32_t dl = delta_table<W>(cs);
+  const int tid = threadIdx.x;
+  DfAcc acc;
+  auto issue = [&](unsigned char* st, int t0, int n, uint64_t* bar, uint64_t pol) {
+    mbar_arrive_expect_tx(bar, (unsigned)n * stage_row_df<W>());
+#pragma unroll
+    for (int k = 0; k < S; ++k) bulk_g2s(st + 8u * B * k, cs.g2 + (size_t)k * N + t0, 8u * n, bar, pol);
+    bulk_g2s(st + 8u * B * S, cs.diag2 + t0, 8u * n, bar, pol);
+    bulk_g2s(st + 8u * B * (S + 1), cs.slot_code + t0, 4u * n, bar, pol);
+  };
+  auto body = [&](const unsigned char* st, int t0, int nt) {
+    if (tid >= nt) return;
+    const float2* sg = reinterpret_cast<const float2*>(st);
+    const uint32_t word = reinterpret_cast<const uint32_t*>(st + 8u * B * (S + 1))[tid];
+    const int c = t0 + tid;
+    df x[S];
+#pragma unroll
+    for (int k = 0; k < S; ++k) x[k] = ld_df(p + LFM_IDX(c + code_delta(dl, word, k), cs.N, c, kChkSlotCellDf));
+    const df pc = ld_df(p + c);
+    df y = df_mul(ld_df(sg + B * S + tid), pc);
+#pragma unroll
+    for (int k = 0; k < S; ++k) y = df_fma(df_neg(ld_df(sg + B * k + tid)), x[k], y);
+    st_df(q + c, y);
+    acc.add(df_mul(y, pc));
+  };
+  ok = staged_tiles<B, kStage, kDfStages>(c0, c1, tm, issue, body);
+  return acc.value();
+}
+
+template <int B, int W, class TM>
+__device__ __forceinline__ double amul_dot_df(const CaseDev& cs, const CaseDev& cref, int c0, int c1,
+                                              const float2* __restrict__ p, float2* __restrict__ q, const TM& tm,
+                                              bool& ok) {
+  ok = true;
+  if constexpr (kCoded<W>) {
+    if ((cs.N & 3) == 0 && dyn_smem_bytes() >= stage_bytes_df<B, W>())
+      return pass_amul_dot_df_bulk<B, W>(cref, c0, c1, p, q, tm, ok);
+  }
+  return pass_amul_dot_df<B, W>(cs, delta_table<W>(cref), c0, c1, p, q);
+}
+
 // U: e += alpha p (first iteration of a solve: e = alpha p), r -= alpha q, w = rD r; returns
 // this thread's sum|r| and w.r. e, the solve's correction to the field, is added to the
 // triple-float field once per solve (pass_sum_df, pass_store_x), so an iteration moves 8
@@ -594,7 +657,9 @@ __device__ bool steps_df64(const CaseDev& cs, const CaseDev& cref, const TM& tm,
           if (!team_barrier<B>(tm, sh)) return false;
           clk.lap(kPhP);
         }
-        const double s1[1] = {pass_amul_dot_df<B, W>(cs, delta_table<W>(cref), c0, c1, p, q)};
+        bool m_ok;
+        const double s1[1] = {amul_dot_df<B, W>(cs, cref, c0, c1, p, q, tm, m_ok)};
+        if (!m_ok) return false;
         if (!team_allreduce<1, B>(tm, s1, sh, [&](int, double t, int lane) {
               fin_sigma(sh, t, lane);
               if (lane == 0) sh.alpha2 = pair_of(sh.alpha);
