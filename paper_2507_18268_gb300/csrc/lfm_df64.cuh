@@ -144,6 +144,20 @@ __device__ __forceinline__ df tf_diff(tf a, tf b) {
   return fast_two_sum(h.hi, l);
 }
 
+// The same where the leading parts are known to be near each other (tf_near): their difference is
+// then exact (Sterbenz' lemma), its error term zero, and two of the four TwoSums drop out. Bitwise
+// tf_diff: 18 operations instead of 31.
+__device__ __forceinline__ df tf_diff_near(tf a, tf b) {
+  const df s1 = two_sum(a.mid, -b.mid);
+  const df h = two_sum(__fsub_rn(a.hi, b.hi), s1.hi);
+  return fast_two_sum(h.hi, __fadd_rn(h.lo, __fadd_rn(s1.lo, __fsub_rn(a.lo, b.lo))));
+}
+
+// Whether a.hi lies in [b.hi / 2, 2 b.hi], with a margin for the rounding of the test itself: lim
+// is tf_near_limit(b). False for anything non-finite, and across a change of sign.
+__device__ __forceinline__ float tf_near_limit(tf b) { return __fmul_rn(0.49f, fabsf(b.hi)); }
+__device__ __forceinline__ bool tf_near(tf a, tf b, float lim) { return fabsf(__fsub_rn(a.hi, b.hi)) <= lim; }
+
 __device__ __forceinline__ df tf_to_df(tf a) { return fast_two_sum(a.hi, a.mid); }
 
 __device__ __forceinline__ tf tf_from_double(double d) {

@@ -64,9 +64,7 @@ __device__ __forceinline__ void row_flux_df(const CaseDev& cs, int c, const tf& 
 #pragma unroll
       for (int k = 1; k < S; ++k) d = df_add(d, g[k]);  // padding slots hold 0
     }
-    flux = df_mul(g[0], tf_diff(xo[0], xc));
-#pragma unroll
-    for (int k = 1; k < S; ++k) flux = df_fma(g[k], tf_diff(xo[k], xc), flux);
+    flux = flux_sum_df<S>(g, xo, xc);
   } else {
     d = mkdf(0.0f, 0.0f);
     flux = mkdf(0.0f, 0.0f);
@@ -133,7 +131,7 @@ __device__ __noinline__ Sums3 pass_rows_init_mixed_df(const CaseDev& cs, int c0,
     df src = df_fma(vdt, tf_to_df(xo), sb);
     df sa = df_add(vdt, gb);
     df rc = df_add(flux, fb);
-    if (has_old) rc = df_fma(vdt, tf_diff(xo, xc), rc);
+    if (has_old) rc = df_fma(vdt, tf_diff_any(xo, xc), rc);
     if (kSrc && (cs.vSp || cs.vSu)) {
       const double sp = cs.vSp ? cs.vSp[c] * cs.df_scale : 0.0;
       const double su = cs.vSu ? cs.vSu[c] * cs.df_scale : 0.0;
@@ -162,7 +160,7 @@ __device__ __noinline__ double2 pass_true_residual_df(const CaseDev& cs, int c0,
     df gb, sb, fb;
     row_boundary_df(cs, c, xc, gb, sb, fb, word);
     const tf xo = ld_tf(reinterpret_cast<const float2*>(cs.x_old), cs.xolo, c);
-    df rc = df_fma(ldg_df(cs.vdt2 + c), tf_diff(xo, xc), df_add(flux, fb));
+    df rc = df_fma(ldg_df(cs.vdt2 + c), tf_diff_any(xo, xc), df_add(flux, fb));
     if (kSrc && (cs.vSp || cs.vSu)) {
       const double sp = cs.vSp ? cs.vSp[c] * cs.df_scale : 0.0;
       const double su = cs.vSu ? cs.vSu[c] * cs.df_scale : 0.0;
@@ -204,13 +202,22 @@ __device__ __noinline__ Sums4 pass_verify_next_df(const CaseDev& cs, int c0, int
     df d, flux;
     uint32_t word;
     row_flux_df<W, false>(cs, c, xc, d, flux, word);
-    df gb, sb, fb;
-    row_boundary_df(cs, c, xc, gb, sb, fb, word);
     const df vdt = ldg_df(cs.vdt2 + c);
     const tf xo = ld_tf(reinterpret_cast<const float2*>(cs.x_old), cs.xolo, c);
-    const df rn = df_add(flux, fb);  // the next step's first residual
-    a_v.add(df_abs(df_fma(vdt, tf_diff(xo, xc), rn)));
-    seed_row_df<false>(cs, c, d, df_fma(vdt, tf_to_df(xc), sb), df_add(vdt, gb), rn, xr, s32, inv_s32, a_nf, a_r, a_rho);
+    // the next step's first residual, its source and row sum; an inner row adds no boundary terms
+    // (the same values as adding zeros)
+    df rn = flux, src, sa = vdt;
+    if (word >> 31) {
+      df gb, sb, fb;
+      row_boundary_df(cs, c, xc, gb, sb, fb, word);
+      rn = df_add(flux, fb);
+      src = df_fma(vdt, tf_to_df(xc), sb);
+      sa = df_add(vdt, gb);
+    } else {
+      src = df_mul(vdt, tf_to_df(xc));
+    }
+    a_v.add(df_abs(df_fma(vdt, tf_diff_any(xo, xc), rn)));
+    seed_row_df<false>(cs, c, d, src, sa, rn, xr, s32, inv_s32, a_nf, a_r, a_rho);
   }
   return Sums4{a_v.value(), a_nf.value(), a_r.value(), a_rho.value()};
 }
