@@ -354,21 +354,24 @@ int lfm_set_barrier_timeout(lfm_ctx *ctx, uint64_t ns);
 int lfm_debug_skip_arrival(lfm_ctx *ctx, int32_t cta);
 
 /* Test hook: when cta >= 0, the next advance makes CTA `cta` issue no copy for the first tile
- * of its first shared-memory-staged pass (see lfm_debug_stage_rows), so that its wait for
- * those bytes runs out and the advance returns LFM_ETIMEOUT (no fault, no hang: every wait is
- * bounded). One-shot; no effect when the launch stages no rows. */
+ * of its first shared-memory-staged pass, or for its rows of a solve kept on chip (see
+ * lfm_debug_stage_rows), so that its wait for those bytes runs out and the advance returns
+ * LFM_ETIMEOUT (no fault, no hang: every wait is bounded). One-shot; no effect when the launch
+ * brings no rows into shared memory by bulk copies. */
 int lfm_debug_skip_stage_copy(lfm_ctx *ctx, int32_t cta);
 
-/* Test evidence: the number of passes of the last advance (lfm_advance / lfm_advance_async
- * and its finish) that ran with their matrix rows staged in shared memory, counted once per
- * pass on the team's first CTA; 0 when the register form ran throughout. */
+/* Test evidence: the number of matrix products of the last advance (lfm_advance /
+ * lfm_advance_async and its finish) whose matrix rows bulk copies had brought into shared
+ * memory, counted once per product on the team's first CTA; 0 when the register form ran
+ * throughout. */
 int lfm_debug_staged_passes(lfm_ctx *ctx, int64_t *n);
 
-/* Test switch: on != 0 (the default) lets the passes that can stream their matrix rows into
- * shared memory with bulk copies do so (the FP32 A p of the mixed form on orthogonal meshes,
- * in single-case launches, on meshes of six slots per cell with N a multiple of 4); 0 makes
- * them load the rows into registers. Both give the same results bit for bit; the switch exists to test
- * that. */
+/* Test switch: on != 0 (the default) lets single-case launches on meshes of six slots per cell
+ * keep matrix rows in shared memory: the inner solve of the mixed form on orthogonal meshes,
+ * whole (rows loaded once per launch, vectors in registers) where the team's threads take few
+ * enough rows each; else its A p, and the df64 A p on packed meshes, with rows streamed in by
+ * bulk copies (N a multiple of 4). 0 makes every pass load its rows into registers. The results
+ * are the same bit for bit; the switch exists to test that. */
 int lfm_debug_stage_rows(lfm_ctx *ctx, int32_t on);
 
 /* Test switch: on != 0 (the default) lets the kernels read a six-slot mesh's neighbours from

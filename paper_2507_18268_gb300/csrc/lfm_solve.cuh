@@ -1063,6 +1063,23 @@ __device__ __forceinline__ void mixed_outer(TeamShared<B>& sh, const CaseDev& cs
             : (ok && !(sweeps == 0 && cs.min_iter > 0)) || sweeps == kMaxSweeps || iters >= cs.max_iter ? kStop : kGo;
 }
 
+// After U of the inner solve (sum 0 = sum|r|, sum 1 = w.r): whether it goes on after `iters`
+// iterations of the step, k of them this solve's, and beta.
+template <int B>
+__device__ __forceinline__ void fin_inner(TeamShared<B>& sh, int i, double t, int lane, int max_iter, int iters, int k,
+                                          int min_inner) {
+  if (lane != 0) return;
+  if (i == 0) {
+    const double res = t / sh.nf;
+    sh.code = !isfinite(res)                                                      ? kNonFinite
+              : (iters < max_iter && !(res < sh.inner_tol)) || k < min_inner ? kGo
+                                                                                  : kStop;
+  } else {
+    sh.beta32 = (float)(t / sh.rho);
+    sh.rho = t;
+  }
+}
+
 // The inner FP32 CG on A dx = r from its seed (r, p = w; sh.rho, sh.inner_tol): sh.code tells how
 // it ended. False when a barrier failed (the caller leaves).
 template <int B, int W, class TM>
@@ -1088,21 +1105,209 @@ __device__ __forceinline__ bool inner_cg_f32(const CaseDev& cs, const CaseDev& c
     ++k;
     ++iters;
     if (!team_allreduce<2, B>(tm, s2, sh, [&](int i, double t, int lane) {
-          if (lane != 0) return;
-          if (i == 0) {
-            const double res = t / sh.nf;
-            sh.code = !isfinite(res)                                                        ? kNonFinite
-                      : (iters < cs.max_iter && !(res < sh.inner_tol)) || k < min_inner ? kGo
-                                                                                            : kStop;
-          } else {
-            sh.beta32 = (float)(t / sh.rho);
-            sh.rho = t;
-          }
+          fin_inner(sh, i, t, lane, cs.max_iter, iters, k, min_inner);
         }))
       return false;
     clk.lap(kPhU);
     if (sh.code != kGo) return true;
   }
+}
+
+// ---- the inner solve kept on chip -------------------------------------------------------------
+// Where a thread takes at most R rows, nothing of the inner solve but the direction has to pass
+// through memory: a row's matrix (its neighbours, coefficients and diagonal) stays in shared
+// memory for the launch (bulk copies bring it in, on ragged meshes plain loads), r, q, dx, 1/diag
+// and the row's own direction in registers. Other threads need the row's new direction
+// p' = w + beta p only in their products, so the product forms it for each neighbour from w and p
+// (the operation of pass_direction) and no pass and barrier of its own is left: two barriers per
+// iteration instead of three, and of the streaming form's 84 bytes per cell and iteration 8 are
+// written and twelve values gathered. Streamed -> on chip: 5.57 -> 4.92 ms for five steps of the
+// 96^3 box (198 iterations), 2.12 -> 1.87 ms for eight steps of a ragged 57,000-cell box.
+// Every value is formed by the same operations, every sum in the same order as in the streaming
+// form: equal results bit for bit.
+// (Gathering p' this way in the streaming form was slower: there its second gather per slot misses
+// L1 and the matrix rows compete for the loads in flight.)
+template <int B, int W, int R>
+__host__ __device__ constexpr unsigned resident_bytes_f32() {
+  return (unsigned)(R * B) * 4u * stage_planes<W>() + 16u;
+}
+
+// How many rows per thread of B the CTA's range has.
+__host__ __device__ __forceinline__ int rows_per_thread(int N, int ctas, int B) {
+  int chunk = (N + ctas - 1) / ctas;
+  chunk = (chunk + 31) & ~31;
+  return (chunk + B - 1) / B;
+}
+
+// loaded: the rows are in shared memory (the first solve of a launch loads them).
+template <int B, int W, int R, class TM>
+__device__ __forceinline__ bool inner_cg_f32_resident(const CaseDev& cs, const CaseDev& cref, const TM& tm,
+                                                      TeamShared<B>& sh, PhaseClock<B, TM>& clk, int c0, int c1,
+                                                      int min_inner, int& iters, bool& loaded) {
+  constexpr int S = kSlots<W>, kIdx = kCoded<W> ? 1 : S;
+  constexpr int kPlane = R * B;  // a plane holds the CTA's rows in order
+  int32_t* const m_idx = reinterpret_cast<int32_t*>(lfm_dyn_smem);
+  float* const m_coef = reinterpret_cast<float*>(lfm_dyn_smem) + kIdx * kPlane;
+  float* const m_diag = m_coef + S * kPlane;
+  const size_t N = (size_t)cs.N;
+  const uint32_t dl = delta_table<W>(cref);
+  const int first = c0 + (int)threadIdx.x;
+  const bool bulk = (cs.N & 3) == 0;  // 16-byte aligned plane starts and sizes
+  if (!loaded) {
+    if (bulk) {
+      uint64_t* const bar = reinterpret_cast<uint64_t*>(lfm_dyn_smem + (size_t)(R * B) * 4u * stage_planes<W>());
+      if (threadIdx.x == 0) {
+        mbar_init(bar, 1);
+        mbar_init_fence();
+        asm volatile("fence.proxy.async.global;" ::: "memory");  // diag32 was written by ordinary stores
+        if (c1 > c0 && (int)blockIdx.x != g_skip_copy_cta) {
+          const unsigned bytes = (unsigned)(c1 - c0) * 4u;
+          const uint64_t pol = l2_evict_first_policy();
+          unsigned char* const to = lfm_dyn_smem;
+          mbar_arrive_expect_tx(bar, stage_planes<W>() * bytes);
+          for (int k = 0; k < kIdx; ++k) {
+            const void* from = kCoded<W> ? (const void*)(cs.slot_code + c0) : (const void*)(cs.slot_other + k * N + c0);
+            bulk_g2s(to + (size_t)k * (R * B) * 4u, from, bytes, bar, pol);
+          }
+          for (int k = 0; k < S; ++k)
+            bulk_g2s(to + (size_t)(kIdx + k) * (R * B) * 4u, cs.slot_coef32 + k * N + c0, bytes, bar, pol);
+          bulk_g2s(to + (size_t)(kIdx + S) * (R * B) * 4u, cs.diag32 + c0, bytes, bar, pol);
+        }
+      }
+      __syncthreads();
+      const bool got = c1 <= c0 || mbar_wait(bar, 0, &tm.sw->status, tm.timeout_ns);
+      const bool failed = __syncthreads_or(!got);
+      if (threadIdx.x == 0) {
+        if (failed && c1 > c0) mbar_drain(bar, 0, tm.timeout_ns);  // a copy in flight lands before the CTA leaves
+        mbar_inval(bar);
+      }
+      __syncthreads();
+      if (failed) return false;
+    } else {
+      for (int i = threadIdx.x; i < c1 - c0; i += B) {
+        const int c = c0 + i;
+        if constexpr (kCoded<W>) {
+          m_idx[i] = (int32_t)__ldcs(cs.slot_code + c);
+        } else {
+#pragma unroll
+          for (int k = 0; k < S; ++k) m_idx[k * kPlane + i] = __ldcs(cs.slot_other + (size_t)k * N + c);
+        }
+#pragma unroll
+        for (int k = 0; k < S; ++k) m_coef[k * kPlane + i] = __ldcs(cs.slot_coef32 + (size_t)k * N + c);
+        m_diag[i] = cs.diag32[c];
+      }
+      __syncthreads();
+    }
+    loaded = true;
+  }
+  float r[R], rd[R], p[R], q[R], dx[R];
+#pragma unroll
+  for (int j = 0; j < R; ++j) {
+    const int c = first + j * B;
+    if (c >= c1) break;
+    r[j] = cs.r32[c];
+    rd[j] = cs.rD32[c];
+    p[j] = cs.p32[c];
+    dx[j] = 0.0f;
+  }
+  float* pa = cs.p32;  // the direction of the last iteration; the new one goes to the other array
+  float* pb = cs.q32;
+  float* const w = cs.w32;
+  bool go = true;
+  for (int k = 0; go; ++k) {
+    // ---- M (and P): p = w + beta p, q = A p, sigma = p.q ------------------------------------
+    const float beta = sh.beta32;
+    Acc2f sig;
+    if (first < c1) {
+      // two rows at a time where the registers allow (at 64 per thread, R = 6, the second row's
+      // gathers spill), all their gathers issued before any is used; a thread's row past the end of
+      // the range repeats the range's last one and is dropped
+      constexpr int H = R <= 4 ? 2 : 1;
+#pragma unroll
+      for (int j0 = 0; j0 < R; j0 += H) {
+        if (first + j0 * B >= c1) break;
+        float v[H][S];
+        int i_[H];
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+          const int i = min(first + (j0 + h) * B, c1 - 1) - c0, c = c0 + i;
+          i_[h] = i;
+          int o[S];
+          if constexpr (kCoded<W>) {
+            const uint32_t word = (uint32_t)m_idx[i];
+#pragma unroll
+            for (int n = 0; n < S; ++n) o[n] = LFM_IDX(c + code_delta(dl, word, n), cs.N, c, kChkSlotCell);
+          } else {
+#pragma unroll
+            for (int n = 0; n < S; ++n) o[n] = LFM_IDX(m_idx[n * kPlane + i], cs.N, c, kChkSlotCell);
+          }
+          if (k == 0) {
+#pragma unroll
+            for (int n = 0; n < S; ++n) v[h][n] = pa[o[n]];
+          } else {
+#pragma unroll
+            for (int n = 0; n < S; ++n) v[h][n] = fmaf(beta, pa[o[n]], w[o[n]]);
+          }
+        }
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+          const int j = j0 + h;
+          if (first + j * B >= c1) break;
+          if (k > 0) p[j] = fmaf(beta, p[j], rd[j] * r[j]);
+          float y = m_diag[i_[h]] * p[j];
+#pragma unroll
+          for (int n = 0; n < S; ++n) y = fmaf(m_coef[n * kPlane + i_[h]], v[h][n], y);
+          q[j] = y;
+          sig.add_prod(y, p[j]);
+        }
+      }
+      if (k > 0) {
+#pragma unroll
+        for (int j = 0; j < R; ++j)
+          if (first + j * B < c1) pb[first + j * B] = p[j];
+      }
+    }
+    if (k > 0) {
+      float* const t = pa;
+      pa = pb;
+      pb = t;
+    }
+    if (bulk && tm.rank == 0 && threadIdx.x == 0) ++tm.sw->staged;  // read back by the host (a test's evidence)
+    const double s1[1] = {sig.value()};
+    if (!team_allreduce<1, B>(tm, s1, sh, [&](int, double t, int lane) { fin_sigma(sh, t, lane); })) return false;
+    clk.lap(kPhM);
+    if (sh.code != kGo) break;
+    // ---- U -----------------------------------------------------------------------------------
+    const float alpha = sh.alpha32;
+    Acc2f rsum, rho;
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+      const int c = first + j * B;
+      if (c >= c1) break;
+      const float rn = fmaf(-alpha, q[j], r[j]);
+      const float wn = rd[j] * rn;
+      dx[j] = fmaf(alpha, p[j], dx[j]);
+      r[j] = rn;
+      w[c] = wn;
+      rsum.add(fabsf(rn));
+      rho.add_prod(wn, rn);
+    }
+    const double s2[2] = {rsum.value(), rho.value()};
+    ++iters;
+    if (!team_allreduce<2, B>(tm, s2, sh, [&](int i, double t, int lane) {
+          fin_inner(sh, i, t, lane, cs.max_iter, iters, k + 1, min_inner);
+        }))
+      return false;
+    clk.lap(kPhU);
+    go = sh.code == kGo;
+  }
+#pragma unroll
+  for (int j = 0; j < R; ++j) {
+    const int c = first + j * B;
+    if (c >= c1) break;
+    cs.dx32[c] = dx[j];
+  }
+  return true;
 }
 
 template <int B, int W, class TM>

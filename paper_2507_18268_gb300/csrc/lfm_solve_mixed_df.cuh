@@ -269,16 +269,17 @@ __device__ __forceinline__ bool mixed_uses_df(const CaseDev& cs) {
   return cs.x2 != nullptr && cs.Sf == nullptr && cs.df_scale >= 0x1p-100 && cs.df_scale <= 0x1p100;
 }
 
-template <int B, int W, class TM>
+// R: rows per thread of the inner solve kept on chip (0: streamed, see inner_cg_f32_resident).
+template <int B, int W, int R, class TM>
 __device__ bool steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps, TeamShared<B>& sh,
                                int stats_base, int c0, int c1) {
   const int tid = threadIdx.x;
-  float* __restrict__ dx = cs.dx32;
-  float* __restrict__ r = cs.r32;
-  float* __restrict__ w = cs.w32;
-  float* __restrict__ p = cs.p32;
-  float* __restrict__ q = cs.q32;
-  const float* __restrict__ rD = cs.rD32;
+  [[maybe_unused]] float* __restrict__ dx = cs.dx32;
+  [[maybe_unused]] float* __restrict__ r = cs.r32;
+  [[maybe_unused]] float* __restrict__ w = cs.w32;
+  [[maybe_unused]] float* __restrict__ p = cs.p32;
+  [[maybe_unused]] float* __restrict__ q = cs.q32;
+  [[maybe_unused]] const float* __restrict__ rD = cs.rD32;
   const float s32 = (float)cs.df_scale, inv_s32 = (float)(1.0 / cs.df_scale);  // powers of two: exact
 
   PhaseClock<B, TM> clk(cs, tm, sh);
@@ -291,6 +292,7 @@ __device__ bool steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const TM&
   if (seeded && tid == 0)
     for (int k = 0; k < 3; ++k) sh.seed[k] = __ldcg(cs.seed_sums + k);  // normFactor sum, sum|r|, rho
   bool convert = ld_volatile_i32(cs.flags) == 0;  // read by every CTA before the first barrier
+  bool loaded = false;
   for (int step = 0; step < n_steps; ++step) {
     int iters_tot = 0, sweeps_tot = 0, status = 0;
     for (int pass = 0; pass <= cs.n_corr; ++pass) {
@@ -350,8 +352,14 @@ __device__ bool steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const TM&
           break;
         }
         // ---- inner FP32 CG on A dx = r (unscaled) -----------------------------------------
-        if (!inner_cg_f32<B, W>(cs, cref, tm, sh, clk, c0, c1, sweeps == 0 ? cs.min_iter : 0, iters, dx, r, w, p, q, rD))
-          return false;
+        const int min_inner = sweeps == 0 ? cs.min_iter : 0;
+        bool met;
+        if constexpr (R > 0) {
+          met = inner_cg_f32_resident<B, W, R>(cs, cref, tm, sh, clk, c0, c1, min_inner, iters, loaded);
+        } else {
+          met = inner_cg_f32<B, W>(cs, cref, tm, sh, clk, c0, c1, min_inner, iters, dx, r, w, p, q, rD);
+        }
+        if (!met) return false;
         if (sh.code == kSingular) status = LFM_ESINGULAR;
         if (sh.code == kNonFinite) status = LFM_ENONFINITE;
         if (status != 0) break;
@@ -414,13 +422,13 @@ __device__ bool steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const TM&
 }
 
 // The mixed form with df64 outer passes (the case must satisfy mixed_uses_df).
-template <int B, int W, class TM>
+template <int B, int W, int R = 0, class TM>
 __device__ void run_steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps,
                                    TeamShared<B>& sh, int stats_base = 0) {
   if (n_steps <= 0) return;
   int c0, c1;
   cta_range(cs.N, tm.size, tm.rank, c0, c1);
-  steps_mixed_df<B, W>(cs, cref, tm, n_steps, sh, stats_base, c0, c1);
+  steps_mixed_df<B, W, R>(cs, cref, tm, n_steps, sh, stats_base, c0, c1);
   pass_store_x<B>(cref, c0, c1, false);
 }
 

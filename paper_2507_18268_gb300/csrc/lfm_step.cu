@@ -40,9 +40,12 @@ __global__ void __launch_bounds__(B, 1024 / B) step_kernel_mixed(CaseDev cs, Lau
   run_steps_mixed<B, W>(cs, s_cs, tm, n_steps, mode, sh);
 }
 
-// The mixed form with df64 outer passes (orthogonal meshes; the host chooses it).
-template <int B, int W>
-__global__ void __launch_bounds__(B, 1024 / B) step_kernel_mixed_df(CaseDev cs, Launch L, int n_steps, int mode) {
+// The mixed form with df64 outer passes (orthogonal meshes; the host chooses it), its inner solve
+// streamed (R = 0) or kept on chip for up to R rows per thread.
+// The on-chip kernels for small teams (R = 2, 4) run one CTA per SM and take the registers that
+// leaves them; R = 6 shares an SM between two.
+template <int B, int W, int R>
+__global__ void __launch_bounds__(B, R == 2 || R == 4 ? 512 / B : 1024 / B) step_kernel_mixed_df(CaseDev cs, Launch L, int n_steps, int mode) {
   __shared__ TeamShared<B> sh;
   __shared__ CaseDev s_cs;
   if ((int)blockIdx.x == L.skip_cta) return;
@@ -50,7 +53,7 @@ __global__ void __launch_bounds__(B, 1024 / B) step_kernel_mixed_df(CaseDev cs, 
   __syncthreads();
   const Team tm{(int)gridDim.x, (int)blockIdx.x, cs.sync, cs.partials, L.timeout_ns};
   if (threadIdx.x == 0) team_join(tm, sh);
-  run_steps_mixed_df<B, W>(cs, s_cs, tm, n_steps, sh);
+  run_steps_mixed_df<B, W, R>(cs, s_cs, tm, n_steps, sh);
 }
 
 template <int B, int W, bool kGeom>
@@ -333,7 +336,7 @@ constexpr int kMaxCodedThreads = 512;
 
 template <int B, int W>
 void* step_fn_of(int precision) {
-  if (precision == kMixedDf) return (void*)step_kernel_mixed_df<B, W>;
+  if (precision == kMixedDf) return (void*)step_kernel_mixed_df<B, W, 0>;
   if (precision == LFM_MIXED) return (void*)step_kernel_mixed<B, W>;
   if (precision == kDf64Geom) return (void*)step_kernel_df64<B, W, true>;
   if (precision == LFM_DF64) return (void*)step_kernel_df64<B, W, false>;
@@ -345,6 +348,25 @@ void* step_fn_w(int precision, int W) {
   if constexpr (B <= kMaxCodedThreads)
     if (W == (6 | kCodedBit)) return step_fn_of<B, (6 | kCodedBit)>(precision);
   return W == 6 ? step_fn_of<B, 6>(precision) : step_fn_of<B, 0>(precision);
+}
+
+// The mixed kernel whose inner solve stays on chip, for rows per thread up to R: 256 x 2 and 512 x
+// 4 rows per CTA, and for packed slots (98 KB of rows) 512 x 6. The launch takes the first that
+// holds its rows and keeps its CTAs co-resident, and streams otherwise.
+struct Resident {
+  void* fn;
+  unsigned smem;
+  int threads, rows;
+};
+
+template <int W>
+int resident_fns(Resident* out) {
+  int n = 0;
+  out[n++] = {(void*)step_kernel_mixed_df<256, W, 2>, resident_bytes_f32<256, W, 2>(), 256, 2};
+  out[n++] = {(void*)step_kernel_mixed_df<512, W, 4>, resident_bytes_f32<512, W, 4>(), 512, 4};
+  if constexpr (kCoded<W>)
+    out[n++] = {(void*)step_kernel_mixed_df<512, W, 6>, resident_bytes_f32<512, W, 6>(), 512, 6};
+  return n;
 }
 
 void* step_fn_for(int precision, int threads, int W) {
@@ -390,15 +412,32 @@ unsigned step_dyn_smem(int precision, int threads, int W) {
   return 0;
 }
 
-int per_sm_ctas(int precision, int threads, int W) {
-  void* fn = step_fn_for(precision, threads, W);
-  if (!fn) return 0;
-  const unsigned dyn = step_dyn_smem(precision, threads, W);
-  int per_sm = 0;
+// Co-resident CTAs of a kernel per SM of the current device, asked for once per kernel, shape and
+// device (every advance sizes its launch).
+int occupancy_of(void* fn, int threads, unsigned dyn) {
+  struct Known {
+    void* fn;
+    int dev, threads;
+    unsigned dyn;
+    int per_sm;
+  };
+  static std::mutex mu;
+  static std::vector<Known> known;
+  int dev = 0, per_sm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  std::lock_guard<std::mutex> lk(mu);
+  for (const Known& k : known)
+    if (k.fn == fn && k.dev == dev && k.threads == threads && k.dyn == dyn) return k.per_sm;
   if (allow_dyn_smem(fn, dyn) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, dyn) != cudaSuccess)
     return 0;
+  known.push_back(Known{fn, dev, threads, dyn, per_sm});
   return per_sm;
+}
+
+int per_sm_ctas(int precision, int threads, int W) {
+  void* fn = step_fn_for(precision, threads, W);
+  return fn ? occupancy_of(fn, threads, step_dyn_smem(precision, threads, W)) : 0;
 }
 
 }  // namespace
@@ -448,9 +487,23 @@ cudaError_t launch_steps(const CaseDev& cs, const Launch& L, int n_steps, int mo
   const int W = kernel_width(cs.W, cs.slot_code != nullptr, L.threads);
   void* fn = step_fn_for(kind, L.threads, W);
   if (!fn) return cudaErrorInvalidValue;
-  const unsigned dyn = L.stage_rows ? step_dyn_smem(kind, L.threads, W) : 0u;
-  const cudaError_t e = allow_dyn_smem(fn, dyn);
-  if (e != cudaSuccess) return e;
+  unsigned dyn = L.stage_rows ? step_dyn_smem(kind, L.threads, W) : 0u;
+  if (kind == kMixedDf && L.stage_rows && W != 0) {
+    Resident on_chip[3];
+    const int n = W == 6 ? resident_fns<6>(on_chip) : resident_fns<(6 | kCodedBit)>(on_chip);
+    const int rows = rows_per_thread(cs.N, L.ctas, L.threads);
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      sms = 0;
+    for (int i = 0; i < n; ++i) {
+      const Resident& k = on_chip[i];
+      if (k.threads != L.threads || rows > k.rows || L.ctas > occupancy_of(k.fn, k.threads, k.smem) * sms) continue;
+      fn = k.fn;
+      dyn = k.smem;
+      break;
+    }
+  }
   CaseDev a0 = cs;
   a0.precision = prec;
   Launch a1 = L;
