@@ -846,7 +846,7 @@ def _cases_with_meshes(cases):
 
 def batch_record(args, world, rank, local):
     """batch512: 512 independent cases (edge log-uniform 16..96), 10 steps each, in one
-    persistent launch per step (graph replay), FP64, df64 and mixed, against the plain FP64
+    persistent launch for all steps (a captured graph), FP64, df64 and mixed, against the plain FP64
     single-case path run case after case. With N ranks the 512 cases are split over the
     GPUs by the longest-processing-time plan of shard.py (no collective on the data path;
     strong scaling: the batch is the same at every N); times are the maximum over ranks and
@@ -940,7 +940,7 @@ def batch_record(args, world, rank, local):
             "warmup": args.warmup, "ms_per_step": results["fp64"]["ms_total"] / steps, "higher_is_better": True,
             "scaling": "strong" if world > 1 else "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
             "config": {"workload": f"batch{n_cases}: {n_cases} cases, edge log-uniform 16..96 (seed 3), "
-                                   f"{total_cells} cells in total, {steps} steps each, graph-replayed step",
+                                   f"{total_cells} cells in total, {steps} steps each, one graph launch for all",
                        "parallelism": "single GPU" if world == 1 else
                        f"{world} GPUs, cases split by the longest-processing-time plan (no collective)"},
             "clocks": clk,

@@ -554,9 +554,10 @@ int lfm_batch_get_launch(lfm_batch *b, int32_t *ctas, int32_t *threads, int32_t 
 /* Device-side barrier wait limit for batch launches (default 10 s). */
 int lfm_batch_set_barrier_timeout(lfm_batch *b, uint64_t ns);
 
-/* Enqueues n_steps (<= 1024) steps of every member case. use_graph != 0: one step is
- * captured once into a CUDA graph (ticket reset + persistent kernel) and the graph is
- * launched n_steps times; use_graph == 0: one launch runs all n_steps. Members may mix
+/* Enqueues n_steps (<= 1024) steps of every member case. use_graph != 0: the
+ * launch (ticket reset + persistent kernel) is captured once into a CUDA graph that takes the
+ * advance's step count when it is launched; use_graph == 0: it is launched directly. Either way
+ * one launch runs all n_steps, with the same results. Members may mix
  * precisions; when every member runs LFM_FP64, or every member LFM_DF64 (hexahedral slot
  * width), the launch uses a kernel compiled for that precision alone (same results, less
  * code around the iteration loops). */

@@ -1,8 +1,8 @@
 """Batched form: many independent cases per persistent launch, with an autotuner.
 
 A :class:`Batch` owns one ``lfm_batch`` and the :class:`Solver` contexts of its cases. One
-advance runs every member case for n steps; by default one step is captured once into a
-CUDA graph and the graph is replayed per step.
+advance runs every member case for n steps in one launch, by default of a CUDA graph that was
+captured once.
 
 The autotuner picks the launch shape -- threads per CTA and cells per thread for each of the
 three size classes (fewer than 32768 cells, fewer than 262144, larger), which set each

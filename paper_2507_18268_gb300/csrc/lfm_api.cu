@@ -1906,7 +1906,7 @@ int lfm_batch_advance_capped_async(lfm_batch* b, int32_t n_steps, int32_t use_gr
   b->h_hdr->n_jobs = n;
   b->h_hdr->n_tickets = tickets;
   b->h_hdr->ticket = 0;
-  b->h_hdr->pad = 0;
+  b->h_hdr->steps = n_steps;
   BCK(b, cudaMemcpyAsync(b->d_cases, b->h_cases, sizeof(CaseDev) * n, cudaMemcpyHostToDevice, b->stream));
   BCK(b, cudaMemcpyAsync(b->d_job_case, b->h_job_case, sizeof(int32_t) * n, cudaMemcpyHostToDevice, b->stream));
   BCK(b, cudaMemcpyAsync(b->d_job_start, b->h_job_start, sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice, b->stream));
@@ -1939,23 +1939,23 @@ int lfm_batch_advance_capped_async(lfm_batch* b, int32_t n_steps, int32_t use_gr
       b->gexec = nullptr;
       cudaGraph_t graph = nullptr;
       BCK(b, cudaStreamBeginCapture(b->capture_stream, cudaStreamCaptureModeThreadLocal));
-      cudaError_t le = launch_batch_steps(bl, 1, b->capture_stream);
+      cudaError_t le = launch_batch_steps(bl, 0, b->capture_stream);
       cudaError_t ce = cudaStreamEndCapture(b->capture_stream, &graph);
       if (le != cudaSuccess || ce != cudaSuccess) {
         if (graph) cudaGraphDestroy(graph);
-        return bfail(b, LFM_ECUDA, "capturing the batch step failed: %s / %s", cudaGetErrorString(le),
+        return bfail(b, LFM_ECUDA, "capturing the batch launch failed: %s / %s", cudaGetErrorString(le),
                      cudaGetErrorString(ce));
       }
       cudaError_t ie = cudaGraphInstantiate(&b->gexec, graph, 0);
       cudaGraphDestroy(graph);
-      if (ie != cudaSuccess) return bfail(b, LFM_ECUDA, "instantiating the batch step graph failed: %s", cudaGetErrorString(ie));
+      if (ie != cudaSuccess) return bfail(b, LFM_ECUDA, "instantiating the batch graph failed: %s", cudaGetErrorString(ie));
       b->g_threads = b->threads;
       b->g_W = W;
       b->g_ctas = ctas;
       b->g_form = form;
       b->g_stage = b->stage_rows;
     }
-    for (int s = 0; s < n_steps; ++s) BCK(b, cudaGraphLaunch(b->gexec, b->stream));
+    BCK(b, cudaGraphLaunch(b->gexec, b->stream));
   } else {
     BCK(b, launch_batch_steps(bl, n_steps, b->stream));
   }

@@ -194,7 +194,7 @@ struct BatchHeader {
   int32_t n_jobs;
   int32_t n_tickets;
   int32_t ticket;            // next ticket; reset to 0 before every launch
-  int32_t pad;
+  int32_t steps;             // steps of the advance, for a launch that is not told (a captured one)
 };
 
 struct BatchLaunch {
