@@ -1,10 +1,12 @@
 // Host side of the C ABI declared in include/lapfoam.h: mesh validation, the face-to-cell
 // addressing, workspace layout, uploads and the advance calls.
 #include <cmath>
+#include <cstddef>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
 #include <algorithm>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -30,6 +32,11 @@ int fail_free(int code, const char* fmt, ...) {
 }
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
+
+// What a launch brings back to the host in one copy: the barrier words from the status on, then the
+// step records.
+constexpr size_t kBackStats = (sizeof(SyncWords) + 255) / 256 * 256 - offsetof(SyncWords, status);
+constexpr size_t kBackBytes = kBackStats + sizeof(lfm_step_stats) * kStatsCap;
 
 // Byte layout of a case's workspace. Offsets are relative to the workspace base.
 struct Layout {
@@ -70,9 +77,9 @@ Layout make_layout(int64_t N, int64_t F, int64_t NB, int64_t W, int kind, bool s
     o = align_up(o + (bytes ? bytes : 1), 256);
     return at;
   };
-  L.sync = take(sizeof(SyncWords));
-  L.partials = take(sizeof(double) * kMaxCtas * kMaxSums);
+  L.sync = take(sizeof(SyncWords));  // the records follow it: one copy brings both back (kBackBytes)
   L.stats = take(sizeof(lfm_step_stats) * kStatsCap);
+  L.partials = take(sizeof(double) * kMaxCtas * kMaxSums);
   L.flags = take(256);
   if (!shared_mesh) {
     L.slot_other = take(4 * W * N);
@@ -162,6 +169,51 @@ Layout make_layout(int64_t N, int64_t F, int64_t NB, int64_t W, int kind, bool s
   return L;
 }
 
+// Pinned buffers of contexts that are gone, kept for the next ones: cudaFreeHost waits for the
+// device, so a server that releases a finished request's context would wait for the batch in flight
+// (0.4 ms a request). At most kKept are held, all are freed with the last context, and the pool is
+// shared by all threads.
+class BackPool {
+ public:
+  BackPool() { free_.reserve(kKept); }
+  char* take() {
+    {
+      std::lock_guard<std::mutex> lk(mu_);
+      ++live_;
+      if (!free_.empty()) {
+        char* p = free_.back();
+        free_.pop_back();
+        return p;
+      }
+    }
+    void* p = nullptr;
+    if (cudaHostAlloc(&p, kBackBytes, cudaHostAllocPortable) == cudaSuccess) return static_cast<char*>(p);
+    give(nullptr);
+    return nullptr;
+  }
+  void give(char* p) {
+    std::lock_guard<std::mutex> lk(mu_);
+    if (--live_ > 0) {
+      if (!p) return;
+      if (free_.size() < kKept)
+        free_.push_back(p);
+      else
+        cudaFreeHost(p);
+      return;
+    }
+    if (p) cudaFreeHost(p);
+    for (char* q : free_) cudaFreeHost(q);
+    free_.clear();
+  }
+
+ private:
+  static constexpr size_t kKept = 64;  // 3 MB
+  std::mutex mu_;
+  std::vector<char*> free_;
+  int live_ = 0;
+};
+BackPool& g_back = *new BackPool;  // never destroyed: a context may outlive the static objects
+
 struct DeviceGuard {
   int prev = -1;
   explicit DeviceGuard(int dev) {
@@ -233,9 +285,14 @@ struct lfm_ctx {
   int skip_copy_cta = -1;
 
   // async state
-  lfm_step_stats* h_stats = nullptr;  // pinned, kStatsCap records
-  int32_t* h_status = nullptr;        // pinned
-  unsigned long long* h_phase = nullptr;  // pinned, kPhases + 1 (the phase times, then the staged-pass count)
+  char* h_back = nullptr;             // pinned, kBackBytes; the next three point into it
+  lfm_step_stats* h_stats = nullptr;  // kStatsCap records
+  int32_t* h_status = nullptr;
+  unsigned long long* h_phase = nullptr;  // kPhases + 1 (the phase times, then the staged-pass count)
+  cudaEvent_t last = nullptr;         // after the last work that a call left on the stream unwaited for
+  bool touched = false;               // last has been recorded
+  bool settled = true;                // no set-up work (refresh_*) enqueued since the stream was last waited for
+  bool flags_clear = false;           // flags[0] and flags[1] are zero on the device (or will be, in order)
   long long staged_passes = 0;        // passes of the last advance with staged rows (team rank 0)
   double phase_ms[kPhases] = {};      // per phase kind, summed over the last advance
   cudaEvent_t done = nullptr;
@@ -582,14 +639,21 @@ int refresh_vdt(lfm_ctx* c) {
   return LFM_OK;
 }
 
+// Marks the end of work that a call leaves on the context's stream: lfm_destroy waits for it.
+int leave(lfm_ctx* c) {
+  CK(c, cudaEventRecord(c->last, c->stream));
+  c->touched = true;
+  return LFM_OK;
+}
+
 // Rebuilds the face coefficients of the slot arrays (a0) when the mesh or DT changed since
 // they were built (the df64 form keeps its own, see refresh_df).
 int refresh_coef(lfm_ctx* c) {
   if (!c->coef_dirty || c->opts.precision == LFM_DF64) return LFM_OK;
   CK(c, launch_coef_setup(c->cs, c->stream));
-  CK(c, cudaStreamSynchronize(c->stream));
+  c->settled = false;
   c->coef_dirty = false;
-  return LFM_OK;
+  return leave(c);
 }
 
 // Rebuilds the df64 conductances and V/dt (a0 of the df64 form) when the mesh, DT or dt
@@ -599,9 +663,9 @@ int refresh_df(lfm_ctx* c) {
   if (!want || !c->df_dirty) return LFM_OK;
   if (!c->hasdf) return fail(c, LFM_ENOMEM, "the workspace has no df64 buffers");
   CK(c, launch_df_setup(c->cs, c->stream));
-  CK(c, cudaStreamSynchronize(c->stream));  // batches launch on their own stream
+  c->settled = false;
   c->df_dirty = false;
-  return LFM_OK;
+  return leave(c);
 }
 
 // Rebuilds the boundary faces' row terms when the patches, their values, DT, dt or the mesh
@@ -609,9 +673,9 @@ int refresh_df(lfm_ctx* c) {
 int refresh_bnd(lfm_ctx* c) {
   if (!c->bnd_dirty) return LFM_OK;
   CK(c, launch_boundary_terms(c->cs, c->stream));
-  CK(c, cudaStreamSynchronize(c->stream));  // batches launch on their own stream
+  c->settled = false;
   c->bnd_dirty = false;
-  return LFM_OK;
+  return leave(c);
 }
 
 // Rebuilds the case's operator weights (general geometry) when patches, boundary values or
@@ -620,27 +684,30 @@ int refresh_ops(lfm_ctx* c) {
   if (!c->has_geom || !c->ops_dirty) return LFM_OK;
   refresh_case(c);
   CK(c, launch_geom_ops(c->cs, false, c->stream));
-  CK(c, cudaStreamSynchronize(c->stream));  // batches launch on their own stream
+  c->settled = false;
   c->ops_dirty = false;
   c->df_dirty = true;  // the df64 copies of the operators follow them
-  return LFM_OK;
+  return leave(c);
 }
 
 // The FP64 field is about to be written other than by a df64 launch: the triple-float copy
 // the df64 forms carry across launches is stale from then on (see lfm_solve_df.cuh), and so
 // is the mixed form's seed of its next step (flags[1]).
 int invalidate_split(lfm_ctx* c) {
+  if (c->flags_clear) return LFM_OK;  // nothing has set them since
   CK(c, cudaMemsetAsync(c->cs.flags, 0, 2 * sizeof(int32_t), c->stream));
-  return LFM_OK;
+  c->flags_clear = true;
+  return leave(c);
 }
 
 // The case changed (its matrix, source, controls or launch shape): the next step's rows and
 // inner-solve seed that the mixed form's last launch left in place no longer apply
 // (lfm_solve_mixed_df.cuh). Stream-ordered after any launch still pending.
 int invalidate_seed(lfm_ctx* c) {
+  if (c->flags_clear) return LFM_OK;
   DeviceGuard g(c->device);
   CK(c, cudaMemsetAsync(c->cs.flags + 1, 0, sizeof(int32_t), c->stream));
-  return LFM_OK;
+  return leave(c);
 }
 
 int need_uploaded(lfm_ctx* c) {
@@ -675,14 +742,11 @@ int enqueue_chunk(lfm_ctx* c, int steps, int mode) {
   }
   if (L.skip_cta >= 0 && L.ctas < 2) return fail(c, LFM_EINVAL, "the skip-arrival hook needs >= 2 CTAs");
   CK(c, cudaMemsetAsync(c->cs.sync, 0, sizeof(SyncWords), c->stream));
+  if (mode == kModeSteps && c->opts.precision != LFM_FP64) c->flags_clear = false;  // the launch may set them
   CK(c, launch_steps(c->cs, L, steps, mode, c->stream));
   c->skip_cta = -1;
   c->skip_copy_cta = -1;
-  if (steps > 0)
-    CK(c, cudaMemcpyAsync(c->h_stats, c->cs.stats, sizeof(lfm_step_stats) * steps, cudaMemcpyDeviceToHost,
-                          c->stream));
-  CK(c, cudaMemcpyAsync(c->h_status, &c->cs.sync->status, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
-  CK(c, cudaMemcpyAsync(c->h_phase, c->cs.sync->phase_ns, sizeof(unsigned long long) * (kPhases + 1),
+  CK(c, cudaMemcpyAsync(c->h_back, &c->cs.sync->status, kBackStats + sizeof(lfm_step_stats) * (steps > 0 ? steps : 0),
                         cudaMemcpyDeviceToHost, c->stream));
   CK(c, cudaEventRecord(c->done, c->stream));
   return LFM_OK;
@@ -768,13 +832,15 @@ int lfm_create(lfm_ctx** out, int device, void* cuda_stream) {
   c->device = device;
   c->stream = static_cast<cudaStream_t>(cuda_stream);
   DeviceGuard g(device);
-  if (cudaMallocHost(&c->h_stats, sizeof(lfm_step_stats) * kStatsCap) != cudaSuccess ||
-      cudaMallocHost(&c->h_status, sizeof(int32_t)) != cudaSuccess ||
-      cudaMallocHost(&c->h_phase, sizeof(unsigned long long) * (kPhases + 1)) != cudaSuccess ||
-      cudaEventCreateWithFlags(&c->done, cudaEventDisableTiming) != cudaSuccess) {
+  c->h_back = g_back.take();
+  if (!c->h_back || cudaEventCreateWithFlags(&c->done, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&c->last, cudaEventDisableTiming) != cudaSuccess) {
     lfm_destroy(c);
     return fail_free(LFM_ECUDA, "lfm_create: host staging or event allocation failed");
   }
+  c->h_status = reinterpret_cast<int32_t*>(c->h_back);
+  c->h_phase = reinterpret_cast<unsigned long long*>(c->h_back + offsetof(SyncWords, phase_ns) - offsetof(SyncWords, status));
+  c->h_stats = reinterpret_cast<lfm_step_stats*>(c->h_back + kBackStats);
   *out = c;
   return LFM_OK;
 }
@@ -831,6 +897,7 @@ static int upload_mesh_impl(lfm_ctx* c, const lfm_mesh* m, const lfm_geometry* g
   c->NB = m->n_bfaces;
   c->W = W;
   c->packed = 0;
+  c->flags_clear = false;  // a workspace not written yet
   c->has64 = has64;
   c->has32 = has32;
   c->hasdf = hasdf;
@@ -1002,6 +1069,7 @@ int lfm_upload_box(lfm_ctx* c, int32_t nx, int32_t ny, int32_t nz, const double*
   c->NB = NB;
   c->W = W;
   c->packed = 0;
+  c->flags_clear = false;  // a workspace not written yet
   c->has64 = has64;
   c->has32 = has32;
   c->hasdf = hasdf;
@@ -1086,6 +1154,7 @@ int lfm_upload_mesh_shared(lfm_ctx* c, lfm_ctx* src) {
     c->ws_owned = true;
   }
   c->mesh_src = root;
+  c->flags_clear = false;  // a workspace not written yet
   root->n_sharers++;
   c->lay = use;
   c->mean_V = root->mean_V;
@@ -1354,7 +1423,7 @@ int lfm_set_field_device(lfm_ctx* c, const double* T_dev) {
   DeviceGuard g(c->device);
   if ((rc = invalidate_split(c))) return rc;
   CK(c, cudaMemcpyAsync(c->cs.x, T_dev, sizeof(double) * c->N, cudaMemcpyDeviceToDevice, c->stream));
-  return LFM_OK;
+  return leave(c);
 }
 
 int lfm_advance_async(lfm_ctx* c, int32_t n_steps) {
@@ -1568,11 +1637,12 @@ int lfm_destroy(lfm_ctx* c) {
   {
     DeviceGuard g(c->device);
     if (c->pending_steps > 0 && c->done) cudaEventSynchronize(c->done);
+    // a caller may reuse its workspace from here on: nothing on the context's stream still writes it
+    if (c->touched) cudaEventSynchronize(c->last);
     if (c->ws_owned && c->ws) cudaFree(c->ws);
-    if (c->h_stats) cudaFreeHost(c->h_stats);
-    if (c->h_status) cudaFreeHost(c->h_status);
-    if (c->h_phase) cudaFreeHost(c->h_phase);
+    if (c->h_back) g_back.give(c->h_back);
     if (c->done) cudaEventDestroy(c->done);
+    if (c->last) cudaEventDestroy(c->last);
   }
   delete c;
   return LFM_OK;
@@ -1869,6 +1939,12 @@ int lfm_batch_advance_capped_async(lfm_batch* b, int32_t n_steps, int32_t use_gr
       return bfail(b, LFM_ENOMEM, "case %d has no buffers for its precision", b->order[i]);
     if (refresh_coef(c) != LFM_OK || refresh_bnd(c) != LFM_OK || refresh_df(c) != LFM_OK)
       return bfail(b, LFM_ECUDA, "case %d: coefficient set-up failed", b->order[i]);
+    if (!c->settled && c->stream != b->stream) {  // the batch launches on a stream of its own
+      if (cudaStreamSynchronize(c->stream) != cudaSuccess)
+        return bfail(b, LFM_ECUDA, "case %d: coefficient set-up failed", b->order[i]);
+      c->settled = true;
+    }
+    c->flags_clear = false;  // the batch's launch may set them
     b->h_cases[i] = c->cs;
     if (c->W != 6) W = 0;
     if (c->cs.slot_code == nullptr) coded = false;
