@@ -109,6 +109,7 @@ struct TeamShared {
   float2 alpha2, beta2, xref2;  // double-float copies (hi, lo)
   float alpha32, beta32;
   int code, conv;
+  int iters;                // of a solve kept on chip
   int ok;                   // 0: a wait ran out or another CTA failed
   int par;                  // parity of the next barrier
   unsigned target;          // the counter's value after the last barrier passed

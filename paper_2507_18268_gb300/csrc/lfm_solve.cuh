@@ -943,10 +943,275 @@ __device__ __forceinline__ bool assemble_prologue(const CaseDev& cs, const CaseD
   });
 }
 
+// ---- a solve kept on chip ---------------------------------------------------------------------
+// Where a thread takes at most R rows, nothing of a solve but the direction has to pass through
+// memory: a row's matrix (its neighbours, coefficients and diagonal) stays in shared memory for the
+// launch (bulk copies bring it in, on ragged meshes plain loads), r, q, the solution, 1/diag and the
+// row's own direction in registers. Other threads need a row's new direction p' = w + beta p only in
+// their products, so the product forms it for each neighbour from w and p (the operation of
+// pass_direction) and no pass and barrier of its own is left: two barriers per iteration instead of
+// three. Every value is formed by the same operations, every sum in the same order as in the
+// streaming form: equal results bit for bit.
+// (Gathering p' this way in the streaming form was slower: there its second gather per slot misses
+// L1 and the matrix rows compete for the loads in flight.)
+// Measured, us per iteration over ten steps, streamed -> on chip, by cells and rows per thread:
+//   packed slots    8,000 (1)       74,000 (2)      111,000 (2)     262,000 (4)     885,000 (6)
+//     mixed         10.3 -> 8.7     11.1 -> 9.2     12.9 -> 10.4    16.7 -> 11.1    28 -> 24.7
+//     df64          10.3 -> 8.9     11.9 -> 9.8     13.0 -> 11.2    15.7 -> 13.3    does not fit
+//     FP64           9.97 -> 9.75   11.7 -> 10.7    12.8 -> 12.5    16.8 -> 17.0
+//   random order
+//     mixed         10.7 -> 9.3     12.7 -> 11.4    14.2 -> 13.9    19.1 -> 19.9
+//     df64          10.6 -> 9.8     12.5 -> 12.0    14.0 -> 16.0    18.7 -> 23.4
+//     FP64          10.3 -> 10.2    12.6 -> 12.2    14.1 -> 14.4    19.4 -> 19.9
+// (111,000 and more on 512 threads.) The two gathers per slot cost most where they have no order,
+// and in FP64 the five more multiply-adds per row do: the kernels for more than two rows (512
+// threads) serve mixed and df64 on packed slots only.
+struct ChipF32 {
+  using V = float;
+  float *p, *q, *w, *sol;
+  const float *r, *rD, *coef, *diag;
+  struct Sum {
+    Acc2f a;
+    __device__ __forceinline__ void dot(float x, float y) { a.add_prod(x, y); }
+    __device__ __forceinline__ void abs(float x) { a.add(fabsf(x)); }
+    __device__ __forceinline__ double value() const { return a.value(); }
+  };
+  static __device__ __forceinline__ float ld(const float* a, int i) { return a[i]; }
+  static __device__ __forceinline__ void st(float* a, int i, float v) { a[i] = v; }
+  static __device__ __forceinline__ float mul(float a, float b) { return a * b; }
+  static __device__ __forceinline__ float fma(float a, float b, float c) { return fmaf(a, b, c); }
+  static __device__ __forceinline__ float slot(float u, float x, float y) { return fmaf(u, x, y); }  // y + u x
+  static __device__ __forceinline__ float neg(float a) { return -a; }
+  __device__ __forceinline__ float sol0(int) const { return 0.0f; }
+  template <class Sh>
+  static __device__ __forceinline__ float alpha(const Sh& sh) { return sh.alpha32; }
+  template <class Sh>
+  static __device__ __forceinline__ float beta(const Sh& sh) { return sh.beta32; }
+};
+
+struct ChipF64 {
+  using V = double;
+  double *p, *q, *w, *sol;
+  const double *r, *rD, *coef, *diag;
+  struct Sum {
+    double s = 0.0;
+    __device__ __forceinline__ void dot(double x, double y) { s = ::fma(x, y, s); }
+    __device__ __forceinline__ void abs(double x) { s += fabs(x); }
+    __device__ __forceinline__ double value() const { return s; }
+  };
+  static __device__ __forceinline__ double ld(const double* a, int i) { return a[i]; }
+  static __device__ __forceinline__ void st(double* a, int i, double v) { a[i] = v; }
+  static __device__ __forceinline__ double mul(double a, double b) { return a * b; }
+  static __device__ __forceinline__ double fma(double a, double b, double c) { return ::fma(a, b, c); }
+  static __device__ __forceinline__ double slot(double u, double x, double y) { return ::fma(u, x, y); }
+  static __device__ __forceinline__ double neg(double a) { return -a; }
+  __device__ __forceinline__ double sol0(int c) const { return sol[c]; }  // the field itself is updated
+  template <class Sh>
+  static __device__ __forceinline__ double alpha(const Sh& sh) { return sh.alpha; }
+  template <class Sh>
+  static __device__ __forceinline__ double beta(const Sh& sh) { return sh.beta; }
+};
+
+template <int W>
+__host__ __device__ constexpr unsigned chip_row_bytes(unsigned value) {  // neighbours, coefficients, diagonal
+  return 4u * (kCoded<W> ? 1u : (unsigned)kSlots<W>) + value * (kSlots<W> + 1u);
+}
+template <int B, int W, int R>
+__host__ __device__ constexpr unsigned chip_bytes(unsigned value) {
+  return (unsigned)(R * B) * chip_row_bytes<W>(value) + 16u;
+}
+
+// Rows per thread of B of a team's CTAs.
+__host__ __device__ __forceinline__ int rows_per_thread(int N, int ctas, int B) {
+  int chunk = (N + ctas - 1) / ctas;
+  chunk = (chunk + 31) & ~31;
+  return (chunk + B - 1) / B;
+}
+
+// Brings the CTA's matrix rows into shared memory (once per launch). False when a copy's wait ran
+// out (status recorded).
+template <class F, int B, int W, int R, class TM>
+__device__ __noinline__ bool chip_load(const F f, const CaseDev& cs, const TM& tm, int c0, int c1) {
+  using V = typename F::V;
+  constexpr int S = kSlots<W>, kIdx = kCoded<W> ? 1 : S, kPlane = R * B;
+  const size_t N = (size_t)cs.N;
+  int32_t* const m_idx = reinterpret_cast<int32_t*>(lfm_dyn_smem);
+  V* const m_coef = reinterpret_cast<V*>(m_idx + kIdx * kPlane);
+  const int n = c1 - c0;
+  if ((cs.N & 3) != 0) {  // planes do not start on 16 bytes
+    for (int i = threadIdx.x; i < n; i += B) {
+      const int c = c0 + i;
+      if constexpr (kCoded<W>) {
+        m_idx[i] = (int32_t)__ldcs(cs.slot_code + c);
+      } else {
+#pragma unroll
+        for (int k = 0; k < S; ++k) m_idx[k * kPlane + i] = __ldcs(cs.slot_other + (size_t)k * N + c);
+      }
+#pragma unroll
+      for (int k = 0; k < S; ++k) m_coef[k * kPlane + i] = f.coef[(size_t)k * N + c];
+      m_coef[S * kPlane + i] = f.diag[c];
+    }
+    __syncthreads();
+    return true;
+  }
+  uint64_t* const bar = reinterpret_cast<uint64_t*>(lfm_dyn_smem + (size_t)kPlane * chip_row_bytes<W>(sizeof(V)));
+  if (threadIdx.x == 0) {
+    mbar_init(bar, 1);
+    mbar_init_fence();
+    asm volatile("fence.proxy.async.global;" ::: "memory");  // the diagonal was written by ordinary stores
+    if (n > 0 && (int)blockIdx.x != g_skip_copy_cta) {
+      const uint64_t pol = l2_evict_first_policy();
+      mbar_arrive_expect_tx(bar, (unsigned)n * chip_row_bytes<W>(sizeof(V)));
+      for (int k = 0; k < kIdx; ++k) {
+        const void* from = kCoded<W> ? (const void*)(cs.slot_code + c0) : (const void*)(cs.slot_other + k * N + c0);
+        bulk_g2s(m_idx + k * kPlane, from, (unsigned)n * 4u, bar, pol);
+      }
+      for (int k = 0; k < S; ++k)
+        bulk_g2s(m_coef + k * kPlane, f.coef + k * N + c0, (unsigned)(n * sizeof(V)), bar, pol);
+      bulk_g2s(m_coef + S * kPlane, f.diag + c0, (unsigned)(n * sizeof(V)), bar, pol);
+    }
+  }
+  __syncthreads();
+  const bool got = n <= 0 || mbar_wait(bar, 0, &tm.sw->status, tm.timeout_ns);
+  const bool failed = __syncthreads_or(!got);
+  if (threadIdx.x == 0) {
+    if (failed && n > 0) mbar_drain(bar, 0, tm.timeout_ns);  // a copy in flight lands before the CTA leaves
+    mbar_inval(bar);
+  }
+  __syncthreads();
+  return !failed;
+}
+
+// CG from its seed (f.r, f.p = w; the scalars in sh): sh.code tells how it ended. fin_m and fin_u
+// are the fins of the two barriers, fin_u with the iterations done in this solve. False when a
+// barrier failed (the caller leaves).
+template <class F, int B, int W, int R, class TM, class FinM, class FinU>
+__device__ __forceinline__ bool cg_on_chip(const F f, const CaseDev& cs, const CaseDev& cref, const TM& tm,
+                                           TeamShared<B>& sh, PhaseClock<B, TM>& clk, int c0, int c1, bool& loaded,
+                                           FinM&& fin_m, FinU&& fin_u) {
+  using V = typename F::V;
+  constexpr int S = kSlots<W>, kIdx = kCoded<W> ? 1 : S;
+  constexpr int kPlane = R * B;  // a plane holds the CTA's rows in order
+  const int32_t* const m_idx = reinterpret_cast<const int32_t*>(lfm_dyn_smem);
+  const V* const m_coef = reinterpret_cast<const V*>(m_idx + kIdx * kPlane);
+  const V* const m_diag = m_coef + S * kPlane;
+  const uint32_t dl = delta_table<W>(cref);
+  const int first = c0 + (int)threadIdx.x;
+  if (!loaded) {
+    if (!chip_load<F, B, W, R>(f, cref, tm, c0, c1)) return false;
+    loaded = true;
+  }
+  V r[R], rd[R], p[R], q[R], sol[R];
+#pragma unroll
+  for (int j = 0; j < R; ++j) {
+    const int c = first + j * B;
+    if (c >= c1) break;
+    r[j] = F::ld(f.r, c);
+    rd[j] = F::ld(f.rD, c);
+    p[j] = F::ld(f.p, c);
+    sol[j] = f.sol0(c);
+  }
+  V* pa = f.p;  // the direction of the last iteration; the new one goes to the other array
+  V* pb = f.q;
+  bool go = true;
+  for (int k = 0; go; ++k) {
+    const V beta = F::beta(sh);
+    // ---- M (and P): p = w + beta p, q = A p, sigma = p.q ---------------------------------------
+    typename F::Sum sig;
+    if (first < c1) {
+      // two rows at a time where the registers allow (not at 64 per thread, R = 6), all their gathers
+      // issued before any is used; a thread's row past the end of the range repeats the range's
+      // last one and is dropped
+      constexpr int H = R <= 4 ? 2 : 1;
+#pragma unroll
+      for (int j0 = 0; j0 < R; j0 += H) {
+        if (first + j0 * B >= c1) break;
+        V v[H][S];
+        int at[H];
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+          const int i = min(first + (j0 + h) * B, c1 - 1) - c0, c = c0 + i;
+          at[h] = i;
+          int o[S];
+          if constexpr (kCoded<W>) {
+            const uint32_t word = (uint32_t)m_idx[i];
+#pragma unroll
+            for (int n = 0; n < S; ++n) o[n] = LFM_IDX(c + code_delta(dl, word, n), cs.N, c, kChkSlotCell);
+          } else {
+#pragma unroll
+            for (int n = 0; n < S; ++n) o[n] = LFM_IDX(m_idx[n * kPlane + i], cs.N, c, kChkSlotCell);
+          }
+          if (k == 0) {
+#pragma unroll
+            for (int n = 0; n < S; ++n) v[h][n] = F::ld(pa, o[n]);
+          } else {
+#pragma unroll
+            for (int n = 0; n < S; ++n) v[h][n] = F::fma(beta, F::ld(pa, o[n]), F::ld(f.w, o[n]));
+          }
+        }
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+          const int j = j0 + h;
+          if (first + j * B >= c1) break;
+          if (k > 0) p[j] = F::fma(beta, p[j], F::mul(rd[j], r[j]));
+          V y = F::mul(F::ld(m_diag, at[h]), p[j]);
+#pragma unroll
+          for (int n = 0; n < S; ++n) y = F::slot(F::ld(m_coef, n * kPlane + at[h]), v[h][n], y);
+          q[j] = y;
+          sig.dot(y, p[j]);
+        }
+      }
+      if (k > 0) {
+#pragma unroll
+        for (int j = 0; j < R; ++j)
+          if (first + j * B < c1) F::st(pb, first + j * B, p[j]);
+      }
+    }
+    if (k > 0) {
+      V* const t = pa;
+      pa = pb;
+      pb = t;
+    }
+    // passes whose rows bulk copies brought in, read back by the host (a test's evidence)
+    if ((cs.N & 3) == 0 && tm.rank == 0 && threadIdx.x == 0) ++tm.sw->staged;
+    const double s1[1] = {sig.value()};
+    if (!team_allreduce<1, B>(tm, s1, sh, [&](int, double t, int lane) { fin_m(t, lane); })) return false;
+    clk.lap(kPhM);
+    if (sh.code != kGo) break;
+    // ---- U -----------------------------------------------------------------------------------
+    const V alpha = F::alpha(sh), nalpha = F::neg(alpha);
+    typename F::Sum rsum, rho;
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+      const int c = first + j * B;
+      if (c >= c1) break;
+      const V rn = F::fma(nalpha, q[j], r[j]);
+      const V wn = F::mul(rd[j], rn);
+      sol[j] = F::fma(alpha, p[j], sol[j]);
+      r[j] = rn;
+      F::st(f.w, c, wn);
+      rsum.abs(rn);
+      rho.dot(wn, rn);
+    }
+    const double s2[2] = {rsum.value(), rho.value()};
+    if (!team_allreduce<2, B>(tm, s2, sh, [&](int i, double t, int lane) { fin_u(i, t, lane, k + 1); })) return false;
+    clk.lap(kPhU);
+    go = sh.code == kGo;
+  }
+#pragma unroll
+  for (int j = 0; j < R; ++j) {
+    const int c = first + j * B;
+    if (c >= c1) break;
+    F::st(f.sol, c, sol[j]);
+  }
+  return true;
+}
+
 // =======================================================================================
 // FP64 steps (1 + n_corr assemble-and-solve passes per step)
 // =======================================================================================
-template <int B, int W, class TM>
+// R: rows per thread of a solve kept on chip (0: streamed, see cg_on_chip).
+template <int B, int W, int R = 0, class TM>
 __device__ void run_steps_f64(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps, int mode,
                               TeamShared<B>& sh, int stats_base = 0) {
   int c0, c1, f0, f1;
@@ -962,6 +1227,7 @@ __device__ void run_steps_f64(const CaseDev& cs, const CaseDev& cref, const TM& 
 
   PhaseClock<B, TM> clk(cs, tm, sh);
   const bool corr_mode = cs.n_corr > 0 || cs.Sf != nullptr || cs.vSu != nullptr || cs.vSp != nullptr;
+  [[maybe_unused]] bool loaded = false;
   for (int step = 0; step < n_steps; ++step) {
     int iters_tot = 0, solves = 0, status = 0;
     for (int pass = 0; pass <= cs.n_corr; ++pass) {
@@ -993,6 +1259,7 @@ __device__ void run_steps_f64(const CaseDev& cs, const CaseDev& cref, const TM& 
         sh.rho = sh.out[2];
         sh.conv = converged(sh.res, sh.init_res, cs.tol, cs.rel_tol) ? 1 : 0;
         sh.code = cs.min_iter > 0 || !sh.conv ? kGo : kStop;
+        sh.iters = 0;
         if (pass == 0) {
           sh.nf0 = sh.nf;
           sh.init0 = sh.init_res;
@@ -1000,7 +1267,19 @@ __device__ void run_steps_f64(const CaseDev& cs, const CaseDev& cref, const TM& 
       }
       __syncthreads();
       int iters = 0;
-      while (sh.code == kGo) {
+      if constexpr (R > 0) {
+        const ChipF64 f{p, q, w, x, r, rD, cs.slot_coef, cs.diag};
+        if (sh.code == kGo &&
+            !cg_on_chip<ChipF64, B, W, R>(
+                f, cs, cref, tm, sh, clk, c0, c1, loaded, [&](double t, int lane) { fin_sigma(sh, t, lane); },
+                [&](int k, double t, int lane, int done) {
+                  fin_update(sh, k, t, lane, cs.tol, cs.rel_tol, done, cs.max_iter, cs.min_iter);
+                  if (k == 0 && lane == 0) sh.iters = done;
+                }))
+          return;
+        iters = sh.iters;
+      }
+      while (R == 0 && sh.code == kGo) {
         if (iters > 0) {
           // ---- P: search direction -----------------------------------------------
           pass_direction<B, double>(c0, c1, sh.beta, p, w);
@@ -1111,203 +1390,6 @@ __device__ __forceinline__ bool inner_cg_f32(const CaseDev& cs, const CaseDev& c
     clk.lap(kPhU);
     if (sh.code != kGo) return true;
   }
-}
-
-// ---- the inner solve kept on chip -------------------------------------------------------------
-// Where a thread takes at most R rows, nothing of the inner solve but the direction has to pass
-// through memory: a row's matrix (its neighbours, coefficients and diagonal) stays in shared
-// memory for the launch (bulk copies bring it in, on ragged meshes plain loads), r, q, dx, 1/diag
-// and the row's own direction in registers. Other threads need the row's new direction
-// p' = w + beta p only in their products, so the product forms it for each neighbour from w and p
-// (the operation of pass_direction) and no pass and barrier of its own is left: two barriers per
-// iteration instead of three, and of the streaming form's 84 bytes per cell and iteration 8 are
-// written and twelve values gathered. Streamed -> on chip: 5.57 -> 4.92 ms for five steps of the
-// 96^3 box (198 iterations), 2.12 -> 1.87 ms for eight steps of a ragged 57,000-cell box.
-// Every value is formed by the same operations, every sum in the same order as in the streaming
-// form: equal results bit for bit.
-// (Gathering p' this way in the streaming form was slower: there its second gather per slot misses
-// L1 and the matrix rows compete for the loads in flight.)
-template <int B, int W, int R>
-__host__ __device__ constexpr unsigned resident_bytes_f32() {
-  return (unsigned)(R * B) * 4u * stage_planes<W>() + 16u;
-}
-
-// How many rows per thread of B the CTA's range has.
-__host__ __device__ __forceinline__ int rows_per_thread(int N, int ctas, int B) {
-  int chunk = (N + ctas - 1) / ctas;
-  chunk = (chunk + 31) & ~31;
-  return (chunk + B - 1) / B;
-}
-
-// loaded: the rows are in shared memory (the first solve of a launch loads them).
-template <int B, int W, int R, class TM>
-__device__ __forceinline__ bool inner_cg_f32_resident(const CaseDev& cs, const CaseDev& cref, const TM& tm,
-                                                      TeamShared<B>& sh, PhaseClock<B, TM>& clk, int c0, int c1,
-                                                      int min_inner, int& iters, bool& loaded) {
-  constexpr int S = kSlots<W>, kIdx = kCoded<W> ? 1 : S;
-  constexpr int kPlane = R * B;  // a plane holds the CTA's rows in order
-  int32_t* const m_idx = reinterpret_cast<int32_t*>(lfm_dyn_smem);
-  float* const m_coef = reinterpret_cast<float*>(lfm_dyn_smem) + kIdx * kPlane;
-  float* const m_diag = m_coef + S * kPlane;
-  const size_t N = (size_t)cs.N;
-  const uint32_t dl = delta_table<W>(cref);
-  const int first = c0 + (int)threadIdx.x;
-  const bool bulk = (cs.N & 3) == 0;  // 16-byte aligned plane starts and sizes
-  if (!loaded) {
-    if (bulk) {
-      uint64_t* const bar = reinterpret_cast<uint64_t*>(lfm_dyn_smem + (size_t)(R * B) * 4u * stage_planes<W>());
-      if (threadIdx.x == 0) {
-        mbar_init(bar, 1);
-        mbar_init_fence();
-        asm volatile("fence.proxy.async.global;" ::: "memory");  // diag32 was written by ordinary stores
-        if (c1 > c0 && (int)blockIdx.x != g_skip_copy_cta) {
-          const unsigned bytes = (unsigned)(c1 - c0) * 4u;
-          const uint64_t pol = l2_evict_first_policy();
-          unsigned char* const to = lfm_dyn_smem;
-          mbar_arrive_expect_tx(bar, stage_planes<W>() * bytes);
-          for (int k = 0; k < kIdx; ++k) {
-            const void* from = kCoded<W> ? (const void*)(cs.slot_code + c0) : (const void*)(cs.slot_other + k * N + c0);
-            bulk_g2s(to + (size_t)k * (R * B) * 4u, from, bytes, bar, pol);
-          }
-          for (int k = 0; k < S; ++k)
-            bulk_g2s(to + (size_t)(kIdx + k) * (R * B) * 4u, cs.slot_coef32 + k * N + c0, bytes, bar, pol);
-          bulk_g2s(to + (size_t)(kIdx + S) * (R * B) * 4u, cs.diag32 + c0, bytes, bar, pol);
-        }
-      }
-      __syncthreads();
-      const bool got = c1 <= c0 || mbar_wait(bar, 0, &tm.sw->status, tm.timeout_ns);
-      const bool failed = __syncthreads_or(!got);
-      if (threadIdx.x == 0) {
-        if (failed && c1 > c0) mbar_drain(bar, 0, tm.timeout_ns);  // a copy in flight lands before the CTA leaves
-        mbar_inval(bar);
-      }
-      __syncthreads();
-      if (failed) return false;
-    } else {
-      for (int i = threadIdx.x; i < c1 - c0; i += B) {
-        const int c = c0 + i;
-        if constexpr (kCoded<W>) {
-          m_idx[i] = (int32_t)__ldcs(cs.slot_code + c);
-        } else {
-#pragma unroll
-          for (int k = 0; k < S; ++k) m_idx[k * kPlane + i] = __ldcs(cs.slot_other + (size_t)k * N + c);
-        }
-#pragma unroll
-        for (int k = 0; k < S; ++k) m_coef[k * kPlane + i] = __ldcs(cs.slot_coef32 + (size_t)k * N + c);
-        m_diag[i] = cs.diag32[c];
-      }
-      __syncthreads();
-    }
-    loaded = true;
-  }
-  float r[R], rd[R], p[R], q[R], dx[R];
-#pragma unroll
-  for (int j = 0; j < R; ++j) {
-    const int c = first + j * B;
-    if (c >= c1) break;
-    r[j] = cs.r32[c];
-    rd[j] = cs.rD32[c];
-    p[j] = cs.p32[c];
-    dx[j] = 0.0f;
-  }
-  float* pa = cs.p32;  // the direction of the last iteration; the new one goes to the other array
-  float* pb = cs.q32;
-  float* const w = cs.w32;
-  bool go = true;
-  for (int k = 0; go; ++k) {
-    // ---- M (and P): p = w + beta p, q = A p, sigma = p.q ------------------------------------
-    const float beta = sh.beta32;
-    Acc2f sig;
-    if (first < c1) {
-      // two rows at a time where the registers allow (at 64 per thread, R = 6, the second row's
-      // gathers spill), all their gathers issued before any is used; a thread's row past the end of
-      // the range repeats the range's last one and is dropped
-      constexpr int H = R <= 4 ? 2 : 1;
-#pragma unroll
-      for (int j0 = 0; j0 < R; j0 += H) {
-        if (first + j0 * B >= c1) break;
-        float v[H][S];
-        int i_[H];
-#pragma unroll
-        for (int h = 0; h < H; ++h) {
-          const int i = min(first + (j0 + h) * B, c1 - 1) - c0, c = c0 + i;
-          i_[h] = i;
-          int o[S];
-          if constexpr (kCoded<W>) {
-            const uint32_t word = (uint32_t)m_idx[i];
-#pragma unroll
-            for (int n = 0; n < S; ++n) o[n] = LFM_IDX(c + code_delta(dl, word, n), cs.N, c, kChkSlotCell);
-          } else {
-#pragma unroll
-            for (int n = 0; n < S; ++n) o[n] = LFM_IDX(m_idx[n * kPlane + i], cs.N, c, kChkSlotCell);
-          }
-          if (k == 0) {
-#pragma unroll
-            for (int n = 0; n < S; ++n) v[h][n] = pa[o[n]];
-          } else {
-#pragma unroll
-            for (int n = 0; n < S; ++n) v[h][n] = fmaf(beta, pa[o[n]], w[o[n]]);
-          }
-        }
-#pragma unroll
-        for (int h = 0; h < H; ++h) {
-          const int j = j0 + h;
-          if (first + j * B >= c1) break;
-          if (k > 0) p[j] = fmaf(beta, p[j], rd[j] * r[j]);
-          float y = m_diag[i_[h]] * p[j];
-#pragma unroll
-          for (int n = 0; n < S; ++n) y = fmaf(m_coef[n * kPlane + i_[h]], v[h][n], y);
-          q[j] = y;
-          sig.add_prod(y, p[j]);
-        }
-      }
-      if (k > 0) {
-#pragma unroll
-        for (int j = 0; j < R; ++j)
-          if (first + j * B < c1) pb[first + j * B] = p[j];
-      }
-    }
-    if (k > 0) {
-      float* const t = pa;
-      pa = pb;
-      pb = t;
-    }
-    if (bulk && tm.rank == 0 && threadIdx.x == 0) ++tm.sw->staged;  // read back by the host (a test's evidence)
-    const double s1[1] = {sig.value()};
-    if (!team_allreduce<1, B>(tm, s1, sh, [&](int, double t, int lane) { fin_sigma(sh, t, lane); })) return false;
-    clk.lap(kPhM);
-    if (sh.code != kGo) break;
-    // ---- U -----------------------------------------------------------------------------------
-    const float alpha = sh.alpha32;
-    Acc2f rsum, rho;
-#pragma unroll
-    for (int j = 0; j < R; ++j) {
-      const int c = first + j * B;
-      if (c >= c1) break;
-      const float rn = fmaf(-alpha, q[j], r[j]);
-      const float wn = rd[j] * rn;
-      dx[j] = fmaf(alpha, p[j], dx[j]);
-      r[j] = rn;
-      w[c] = wn;
-      rsum.add(fabsf(rn));
-      rho.add_prod(wn, rn);
-    }
-    const double s2[2] = {rsum.value(), rho.value()};
-    ++iters;
-    if (!team_allreduce<2, B>(tm, s2, sh, [&](int i, double t, int lane) {
-          fin_inner(sh, i, t, lane, cs.max_iter, iters, k + 1, min_inner);
-        }))
-      return false;
-    clk.lap(kPhU);
-    go = sh.code == kGo;
-  }
-#pragma unroll
-  for (int j = 0; j < R; ++j) {
-    const int c = first + j * B;
-    if (c >= c1) break;
-    cs.dx32[c] = dx[j];
-  }
-  return true;
 }
 
 template <int B, int W, class TM>

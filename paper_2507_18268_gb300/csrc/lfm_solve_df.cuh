@@ -618,10 +618,36 @@ __device__ __forceinline__ double2 pass_update_df(int c0, int c1, df alpha, floa
   return make_double2(sa.value(), sr.value());
 }
 
+// The df64 solve kept on chip (see cg_on_chip). The conductances are stored, the off-diagonals
+// are their negatives; e starts at zero (e = alpha p + 0 equals the streamed form's e = alpha p).
+struct ChipDf {
+  using V = df;
+  df *p, *q, *w, *sol;
+  const df *r, *rD, *coef, *diag;
+  struct Sum {
+    DfAcc a;
+    __device__ __forceinline__ void dot(df x, df y) { a.add(df_mul(x, y)); }
+    __device__ __forceinline__ void abs(df x) { a.add(df_abs(x)); }
+    __device__ __forceinline__ double value() const { return a.value(); }
+  };
+  static __device__ __forceinline__ df ld(const df* a, int i) { return ld_df(reinterpret_cast<const float2*>(a) + i); }
+  static __device__ __forceinline__ void st(df* a, int i, df v) { st_df(reinterpret_cast<float2*>(a) + i, v); }
+  static __device__ __forceinline__ df mul(df a, df b) { return df_mul(a, b); }
+  static __device__ __forceinline__ df fma(df a, df b, df c) { return df_fma(a, b, c); }
+  static __device__ __forceinline__ df slot(df g, df x, df y) { return df_fma(df_neg(g), x, y); }
+  static __device__ __forceinline__ df neg(df a) { return df_neg(a); }
+  __device__ __forceinline__ df sol0(int) const { return mkdf(0.0f, 0.0f); }
+  template <class Sh>
+  static __device__ __forceinline__ df alpha(const Sh& sh) { return df_of(sh.alpha2); }
+  template <class Sh>
+  static __device__ __forceinline__ df beta(const Sh& sh) { return df_of(sh.beta2); }
+};
+static_assert(sizeof(df) == sizeof(float2), "df arrays are stored as float2");
+
 // The steps of one launch. Returns false when a barrier failed (the caller leaves).
 // `pending` tracks whether e holds a correction not yet added to the field (the same in every
 // CTA: it follows the team-wide iteration counts).
-template <int B, int W, bool kGeom, class TM>
+template <int B, int W, bool kGeom, int R, class TM>
 __device__ bool steps_df64(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps, TeamShared<B>& sh,
                            int stats_base, int c0, int c1, bool& pending) {
   const int tid = threadIdx.x;
@@ -635,6 +661,7 @@ __device__ bool steps_df64(const CaseDev& cs, const CaseDev& cref, const TM& tm,
   PhaseClock<B, TM> clk(cs, tm, sh);
   const bool src_mode = cs.n_corr > 0 || cs.vSu != nullptr || cs.vSp != nullptr || (kGeom && cs.Sf != nullptr);
   bool convert = ld_volatile_i32(cs.flags) == 0;  // read by every CTA before the first barrier
+  [[maybe_unused]] bool loaded = false;
   for (int step = 0; step < n_steps; ++step) {
     int iters_tot = 0, solves = 0, status = 0;
     for (int pass = 0; pass <= cs.n_corr; ++pass) {
@@ -670,6 +697,7 @@ __device__ bool steps_df64(const CaseDev& cs, const CaseDev& cref, const TM& tm,
         sh.rho = sh.out[2];
         sh.conv = converged(sh.res, sh.init_res, cs.tol, cs.rel_tol) ? 1 : 0;
         sh.code = cs.min_iter > 0 || !sh.conv ? kGo : kStop;
+        sh.iters = 0;
         if (pass == 0) {
           sh.nf0 = sh.nf * (1.0 / cs.df_scale);  // a power of two: exact
           sh.init0 = sh.init_res;
@@ -677,7 +705,29 @@ __device__ bool steps_df64(const CaseDev& cs, const CaseDev& cref, const TM& tm,
       }
       __syncthreads();
       int iters = 0;
-      while (sh.code == kGo) {
+      if constexpr (R > 0) {
+        auto df_at = [](const void* a) { return reinterpret_cast<df*>(const_cast<void*>(a)); };
+        const ChipDf f{df_at(p), df_at(q), df_at(w), df_at(e), df_at(r), df_at(rD), df_at(cs.g2), df_at(cs.diag2)};
+        if (sh.code == kGo) {
+          pending = true;  // unless the first product ends the solve: e is then zero, the same field
+          if (!cg_on_chip<ChipDf, B, W, R>(
+                  f, cs, cref, tm, sh, clk, c0, c1, loaded,
+                  [&](double t, int lane) {
+                    fin_sigma(sh, t, lane);
+                    if (lane == 0) sh.alpha2 = pair_of(sh.alpha);
+                  },
+                  [&](int k, double t, int lane, int done) {
+                    fin_update(sh, k, t, lane, cs.tol, cs.rel_tol, done, cs.max_iter, cs.min_iter);
+                    if (k == 0 && lane == 0) sh.iters = done;
+                    if (k == 1 && lane == 0) sh.beta2 = pair_of(sh.beta);
+                  })) {
+            pending = false;  // the solution was not written
+            return false;
+          }
+        }
+        iters = sh.iters;
+      }
+      while (R == 0 && sh.code == kGo) {
         if (iters > 0) {
           pass_direction_df<B>(c0, c1, df_of(sh.beta2), p, w);
           if (!team_barrier<B>(tm, sh)) return false;
@@ -720,15 +770,16 @@ __device__ bool steps_df64(const CaseDev& cs, const CaseDev& cref, const TM& tm,
   return true;
 }
 
-// kGeom: the kernel serves general geometry (the gradient phase is compiled in).
-template <int B, int W, bool kGeom = false, class TM>
+// kGeom: the kernel serves general geometry (the gradient phase is compiled in). R: rows per thread
+// of a solve kept on chip (0: streamed).
+template <int B, int W, bool kGeom = false, int R = 0, class TM>
 __device__ void run_steps_df64(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps, TeamShared<B>& sh,
                                int stats_base = 0) {
   if (n_steps <= 0) return;
   int c0, c1;
   cta_range(cs.N, tm.size, tm.rank, c0, c1);
   bool pending = false;
-  steps_df64<B, W, kGeom>(cs, cref, tm, n_steps, sh, stats_base, c0, c1, pending);
+  steps_df64<B, W, kGeom, R>(cs, cref, tm, n_steps, sh, stats_base, c0, c1, pending);
   // the field and the correction of the CTA's own cells are written by this CTA only, so the
   // FP64 field can be written back without another barrier, also after an early exit.
   pass_store_x<B>(cref, c0, c1, pending);

@@ -269,7 +269,7 @@ __device__ __forceinline__ bool mixed_uses_df(const CaseDev& cs) {
   return cs.x2 != nullptr && cs.Sf == nullptr && cs.df_scale >= 0x1p-100 && cs.df_scale <= 0x1p100;
 }
 
-// R: rows per thread of the inner solve kept on chip (0: streamed, see inner_cg_f32_resident).
+// R: rows per thread of the inner solve kept on chip (0: streamed, see cg_on_chip).
 template <int B, int W, int R, class TM>
 __device__ bool steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps, TeamShared<B>& sh,
                                int stats_base, int c0, int c1) {
@@ -355,7 +355,16 @@ __device__ bool steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const TM&
         const int min_inner = sweeps == 0 ? cs.min_iter : 0;
         bool met;
         if constexpr (R > 0) {
-          met = inner_cg_f32_resident<B, W, R>(cs, cref, tm, sh, clk, c0, c1, min_inner, iters, loaded);
+          const int before = iters;
+          if (tid == 0) sh.iters = before;  // read after the solve's barriers
+          const ChipF32 f{p, q, w, dx, r, rD, cs.slot_coef32, cs.diag32};
+          met = cg_on_chip<ChipF32, B, W, R>(
+              f, cs, cref, tm, sh, clk, c0, c1, loaded, [&](double t, int lane) { fin_sigma(sh, t, lane); },
+              [&](int k, double t, int lane, int done) {
+                fin_inner(sh, k, t, lane, cs.max_iter, before + done, done, min_inner);
+                if (k == 0 && lane == 0) sh.iters = before + done;
+              });
+          iters = sh.iters;
         } else {
           met = inner_cg_f32<B, W>(cs, cref, tm, sh, clk, c0, c1, min_inner, iters, dx, r, w, p, q, rD);
         }

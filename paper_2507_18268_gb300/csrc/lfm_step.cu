@@ -16,8 +16,13 @@ namespace lfm {
 namespace {
 
 // ---- kernels ---------------------------------------------------------------------------
-template <int B, int W>
-__global__ void __launch_bounds__(B, 1024 / B) step_kernel_f64(CaseDev cs, Launch L, int n_steps, int mode) {
+// Register budget of the step kernels: the on-chip ones for small teams (R = 2, 4) run one CTA per SM
+// and take what that leaves them; streaming ones, and R = 6, share an SM between 1024 threads.
+template <int B, int R>
+constexpr int kMinCtas = (R == 2 || R == 4 ? 512 : 1024) / B;
+
+template <int B, int W, int R>
+__global__ void __launch_bounds__(B, kMinCtas<B, R>) step_kernel_f64(CaseDev cs, Launch L, int n_steps, int mode) {
   __shared__ TeamShared<B> sh;
   __shared__ CaseDev s_cs;  // addressable copy for the per-step passes
   if ((int)blockIdx.x == L.skip_cta) return;  // test hook: never arrive
@@ -25,7 +30,7 @@ __global__ void __launch_bounds__(B, 1024 / B) step_kernel_f64(CaseDev cs, Launc
   __syncthreads();
   const Team tm{(int)gridDim.x, (int)blockIdx.x, cs.sync, cs.partials, L.timeout_ns};
   if (threadIdx.x == 0) team_join(tm, sh);
-  run_steps_f64<B, W>(cs, s_cs, tm, n_steps, mode, sh);
+  run_steps_f64<B, W, R>(cs, s_cs, tm, n_steps, mode, sh);
 }
 
 template <int B, int W>
@@ -42,10 +47,8 @@ __global__ void __launch_bounds__(B, 1024 / B) step_kernel_mixed(CaseDev cs, Lau
 
 // The mixed form with df64 outer passes (orthogonal meshes; the host chooses it), its inner solve
 // streamed (R = 0) or kept on chip for up to R rows per thread.
-// The on-chip kernels for small teams (R = 2, 4) run one CTA per SM and take the registers that
-// leaves them; R = 6 shares an SM between two.
 template <int B, int W, int R>
-__global__ void __launch_bounds__(B, R == 2 || R == 4 ? 512 / B : 1024 / B) step_kernel_mixed_df(CaseDev cs, Launch L, int n_steps, int mode) {
+__global__ void __launch_bounds__(B, kMinCtas<B, R>) step_kernel_mixed_df(CaseDev cs, Launch L, int n_steps, int mode) {
   __shared__ TeamShared<B> sh;
   __shared__ CaseDev s_cs;
   if ((int)blockIdx.x == L.skip_cta) return;
@@ -56,8 +59,8 @@ __global__ void __launch_bounds__(B, R == 2 || R == 4 ? 512 / B : 1024 / B) step
   run_steps_mixed_df<B, W, R>(cs, s_cs, tm, n_steps, sh);
 }
 
-template <int B, int W, bool kGeom>
-__global__ void __launch_bounds__(B, 1024 / B) step_kernel_df64(CaseDev cs, Launch L, int n_steps, int mode) {
+template <int B, int W, bool kGeom, int R>
+__global__ void __launch_bounds__(B, kMinCtas<B, R>) step_kernel_df64(CaseDev cs, Launch L, int n_steps, int mode) {
   __shared__ TeamShared<B> sh;
   __shared__ CaseDev s_cs;  // addressable copy for the per-step passes
   if ((int)blockIdx.x == L.skip_cta) return;
@@ -65,7 +68,7 @@ __global__ void __launch_bounds__(B, 1024 / B) step_kernel_df64(CaseDev cs, Laun
   __syncthreads();
   const Team tm{(int)gridDim.x, (int)blockIdx.x, cs.sync, cs.partials, L.timeout_ns};
   if (threadIdx.x == 0) team_join(tm, sh);
-  run_steps_df64<B, W, kGeom>(cs, s_cs, tm, n_steps, sh);
+  run_steps_df64<B, W, kGeom, R>(cs, s_cs, tm, n_steps, sh);
 }
 
 // Set-up (a0): per face g = (DT |Sf|) deltaCoeff (the assembly's products, in its order),
@@ -338,9 +341,9 @@ template <int B, int W>
 void* step_fn_of(int precision) {
   if (precision == kMixedDf) return (void*)step_kernel_mixed_df<B, W, 0>;
   if (precision == LFM_MIXED) return (void*)step_kernel_mixed<B, W>;
-  if (precision == kDf64Geom) return (void*)step_kernel_df64<B, W, true>;
-  if (precision == LFM_DF64) return (void*)step_kernel_df64<B, W, false>;
-  return (void*)step_kernel_f64<B, W>;
+  if (precision == kDf64Geom) return (void*)step_kernel_df64<B, W, true, 0>;
+  if (precision == LFM_DF64) return (void*)step_kernel_df64<B, W, false, 0>;
+  return (void*)step_kernel_f64<B, W, 0>;
 }
 
 template <int B>
@@ -350,22 +353,32 @@ void* step_fn_w(int precision, int W) {
   return W == 6 ? step_fn_of<B, 6>(precision) : step_fn_of<B, 0>(precision);
 }
 
-// The mixed kernel whose inner solve stays on chip, for rows per thread up to R: 256 x 2 and 512 x
-// 4 rows per CTA, and for packed slots (98 KB of rows) 512 x 6. The launch takes the first that
-// holds its rows and keeps its CTAs co-resident, and streams otherwise.
-struct Resident {
+// The kernels whose solves stay on chip (cg_on_chip says where they pay): 256 threads of two rows for
+// every form; on packed slots 512 of four for the mixed and df64 forms, and of six for the mixed
+// form (98 KB of rows, two CTAs per SM). A launch takes the first that holds its rows and keeps its
+// CTAs co-resident, and streams otherwise.
+struct OnChip {
   void* fn;
   unsigned smem;
   int threads, rows;
 };
 
 template <int W>
-int resident_fns(Resident* out) {
+int on_chip_fns(int precision, OnChip* out) {
   int n = 0;
-  out[n++] = {(void*)step_kernel_mixed_df<256, W, 2>, resident_bytes_f32<256, W, 2>(), 256, 2};
-  out[n++] = {(void*)step_kernel_mixed_df<512, W, 4>, resident_bytes_f32<512, W, 4>(), 512, 4};
-  if constexpr (kCoded<W>)
-    out[n++] = {(void*)step_kernel_mixed_df<512, W, 6>, resident_bytes_f32<512, W, 6>(), 512, 6};
+  if (precision == kMixedDf) {
+    out[n++] = {(void*)step_kernel_mixed_df<256, W, 2>, chip_bytes<256, W, 2>(4), 256, 2};
+    if constexpr (kCoded<W>) {
+      out[n++] = {(void*)step_kernel_mixed_df<512, W, 4>, chip_bytes<512, W, 4>(4), 512, 4};
+      out[n++] = {(void*)step_kernel_mixed_df<512, W, 6>, chip_bytes<512, W, 6>(4), 512, 6};
+    }
+  } else if (precision == LFM_FP64) {
+    out[n++] = {(void*)step_kernel_f64<256, W, 2>, chip_bytes<256, W, 2>(8), 256, 2};
+  } else if (precision == LFM_DF64) {
+    out[n++] = {(void*)step_kernel_df64<256, W, false, 2>, chip_bytes<256, W, 2>(8), 256, 2};
+    if constexpr (kCoded<W>)
+      out[n++] = {(void*)step_kernel_df64<512, W, false, 4>, chip_bytes<512, W, 4>(8), 512, 4};
+  }
   return n;
 }
 
@@ -488,16 +501,16 @@ cudaError_t launch_steps(const CaseDev& cs, const Launch& L, int n_steps, int mo
   void* fn = step_fn_for(kind, L.threads, W);
   if (!fn) return cudaErrorInvalidValue;
   unsigned dyn = L.stage_rows ? step_dyn_smem(kind, L.threads, W) : 0u;
-  if (kind == kMixedDf && L.stage_rows && W != 0) {
-    Resident on_chip[3];
-    const int n = W == 6 ? resident_fns<6>(on_chip) : resident_fns<(6 | kCodedBit)>(on_chip);
+  if (mode == kModeSteps && L.stage_rows && W != 0) {
+    OnChip on_chip[3];
+    const int n = W == 6 ? on_chip_fns<6>(kind, on_chip) : on_chip_fns<(6 | kCodedBit)>(kind, on_chip);
     const int rows = rows_per_thread(cs.N, L.ctas, L.threads);
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
       sms = 0;
     for (int i = 0; i < n; ++i) {
-      const Resident& k = on_chip[i];
+      const OnChip& k = on_chip[i];
       if (k.threads != L.threads || rows > k.rows || L.ctas > occupancy_of(k.fn, k.threads, k.smem) * sms) continue;
       fn = k.fn;
       dyn = k.smem;

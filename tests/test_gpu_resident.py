@@ -97,3 +97,39 @@ def test_row_differences_near_and_far(prec, spread):
         s.set_solver(case.tol, 0.0, 1000, 0, prec)
         s.advance(2)
         assert np.max(np.abs(s.field() - To)) <= (1e-10 if prec == B.LFM_DF64 else 1e-5) * np.max(np.abs(To))
+
+
+def run_as(case, prec, on, ctas, threads, cuts=(2, 1)):
+    with Solver.from_case(case) as s:
+        s.set_solver(case.tol, case.rel_tol, case.max_iter, case.min_iter, prec)
+        B.lfm_debug_stage_rows(s.ctx, on)
+        s.set_launch(ctas, threads)
+        st = []
+        for n in cuts:
+            st += s.advance(n)
+        return s.field().copy(), st
+
+
+@pytest.mark.parametrize("prec", [B.LFM_FP64, B.LFM_DF64])
+@pytest.mark.parametrize("permute", [False, True])
+@pytest.mark.parametrize("dims,ctas,threads", SHAPES)
+def test_whole_solve_on_chip_bitwise_equal_to_streamed(dims, ctas, threads, permute, prec):
+    case = case_of(dims, permute)
+    T, st = run_as(case, prec, True, ctas, threads)
+    T0, st0 = run_as(case, prec, False, ctas, threads)
+    assert np.array_equal(T, T0) and st == st0
+    assert max(x["iters"] for x in st) >= 3
+
+
+@pytest.mark.parametrize("prec", [B.LFM_FP64, B.LFM_DF64])
+@pytest.mark.parametrize("kw", [dict(tol=1e-13), dict(tol=1e-3, min_iter=5), dict(tol=1e-12, max_iter=4),
+                                dict(tol=0.0, rel_tol=1e-4), dict(Su=9.0, Sp=-0.3), dict(n_nonorth_corr=2),
+                                dict(DT_uniform=0.0, DTx=None, DTy=None, DTz=None)],
+                         ids=["tight", "min_iter", "max_iter", "rel_tol", "sources", "passes", "no_diffusion"])
+def test_whole_solve_on_chip_options(kw, prec):
+    case = case_of((10, 9, 8)).with_(**kw)
+    for cuts in ((3,), (1, 1, 1)):
+        for launch in ((2, 256), (1, 512)):
+            T, st = run_as(case, prec, True, *launch, cuts)
+            T0, st0 = run_as(case, prec, False, *launch, cuts)
+            assert np.array_equal(T, T0) and st == st0
