@@ -391,11 +391,10 @@ void* step_fn_for(int precision, int threads, int W) {
   }
 }
 
-// Dynamic shared memory of a step kernel: the stages of the bulk-staged A p of the df64 form on packed
-// orthogonal meshes (60 bytes per cell, three stages: 129 -> 112 us per iteration on the 200^3 graded
-// box), and the two of the FP32 A p of the
-// mixed form on orthogonal meshes (the kernel with df64 outer passes, specialised for six
-// slots). The mixed kernel for general meshes runs without them: the shared memory comes out
+// Dynamic shared memory of a step kernel that streams its rows: the stages of the bulk-staged A p of
+// the df64 form on packed orthogonal meshes (60 bytes per cell, three stages: 129 -> 112 us per
+// iteration on the 200^3 graded box), and the two of the FP32 A p of the mixed form on orthogonal
+// meshes (the kernel with df64 outer passes, specialised for six slots). The mixed kernel for general meshes runs without them: the shared memory comes out
 // of the same on-chip array as L1, and its gradient and corrected-row passes, which gather
 // through L1, lost more (skewed200: 0.71 -> 0.86 and 1.97 -> 2.01 ms per step) than its A p
 // gained (0.655 -> 0.638).
@@ -489,6 +488,8 @@ int max_coresident_ctas(int precision, int threads, int W, int device) {
   return n < kMaxCtas / 2 ? n : kMaxCtas / 2;  // the partial sums' table holds two buffers
 }
 
+constexpr int kStageRowsDf = 8;  // the df64 A p stages its rows where a thread takes more than this
+
 cudaError_t launch_steps(const CaseDev& cs, const Launch& L, int n_steps, int mode,
                          cudaStream_t stream) {
   // matrix read-back of a df64 case runs the FP64 assembly (its arrays are the ones read)
@@ -501,6 +502,9 @@ cudaError_t launch_steps(const CaseDev& cs, const Launch& L, int n_steps, int mo
   void* fn = step_fn_for(kind, L.threads, W);
   if (!fn) return cudaErrorInvalidValue;
   unsigned dyn = L.stage_rows ? step_dyn_smem(kind, L.threads, W) : 0u;
+  // df64 A p: us per iteration staged / from registers at 304 CTAs of 512, by rows per thread: 3 (343,000
+  // cells) 21.5 / 18.5; 6 (885,000) 31.3 / 30.1; 10 (1.4 M) 44.2 / 44.5; 27 (4.1 M) 116 / 122
+  if (kind == LFM_DF64 && rows_per_thread(cs.N, L.ctas, L.threads) <= kStageRowsDf) dyn = 0;
   if (mode == kModeSteps && L.stage_rows && W != 0) {
     OnChip on_chip[3];
     const int n = W == 6 ? on_chip_fns<6>(kind, on_chip) : on_chip_fns<(6 | kCodedBit)>(kind, on_chip);

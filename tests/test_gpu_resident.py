@@ -133,3 +133,21 @@ def test_whole_solve_on_chip_options(kw, prec):
             T, st = run_as(case, prec, True, *launch, cuts)
             T0, st0 = run_as(case, prec, False, *launch, cuts)
             assert np.array_equal(T, T0) and st == st0
+
+
+# more than eight rows per thread: the df64 product streams its packed rows through shared memory
+@pytest.mark.parametrize("permute", [False, True])
+@pytest.mark.parametrize("dims,ctas,threads", [((16, 16, 8), 1, 256), ((16, 16, 9), 1, 256), ((24, 16, 12), 1, 256),
+                                               ((20, 20, 13), 2, 256), ((23, 16, 15), 1, 512)])
+def test_df64_streamed_rows_by_rows_per_thread(dims, ctas, threads, permute):
+    case = case_of(dims, permute)
+    out = []
+    for on in (True, False):
+        with Solver.from_case(case) as s:
+            s.set_solver(case.tol, case.rel_tol, case.max_iter, case.min_iter, B.LFM_DF64)
+            B.lfm_debug_stage_rows(s.ctx, on)
+            s.set_launch(ctas, threads)
+            out.append((s.advance(3), s.field().copy(), B.lfm_debug_staged_passes(s.ctx)))
+    assert out[0][0] == out[1][0] and np.array_equal(out[0][1], out[1][1])
+    rows = -(-(case.n_cells // ctas) // threads)
+    assert (out[0][2] > 0) == (not permute and rows > 8 and case.n_cells % 4 == 0) and out[1][2] == 0
