@@ -292,6 +292,7 @@ struct lfm_ctx {
   cudaEvent_t last = nullptr;         // after the last work that a call left on the stream unwaited for
   bool touched = false;               // last has been recorded
   bool settled = true;                // no set-up work (refresh_*) enqueued since the stream was last waited for
+  bool recorded = false;              // a call was recorded into a graph (see recording)
   bool flags_clear = false;           // flags[0] and flags[1] are zero on the device (or will be, in order)
   long long staged_passes = 0;        // passes of the last advance with staged rows (team rank 0)
   double phase_ms[kPhases] = {};      // per phase kind, summed over the last advance
@@ -639,8 +640,21 @@ int refresh_vdt(lfm_ctx* c) {
   return LFM_OK;
 }
 
+// Whether the context's stream records into a graph. What a recorded call does happens at each
+// replay, unseen by the host: from the first one on the context's flags count as unknown.
+bool recording(lfm_ctx* c) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (st != cudaStreamCaptureStatusNone) c->recorded = true;
+  return st != cudaStreamCaptureStatusNone;
+}
+
 // Marks the end of work that a call leaves on the context's stream: lfm_destroy waits for it.
 int leave(lfm_ctx* c) {
+  if (recording(c)) return LFM_OK;
   CK(c, cudaEventRecord(c->last, c->stream));
   c->touched = true;
   return LFM_OK;
@@ -694,7 +708,8 @@ int refresh_ops(lfm_ctx* c) {
 // the df64 forms carry across launches is stale from then on (see lfm_solve_df.cuh), and so
 // is the mixed form's seed of its next step (flags[1]).
 int invalidate_split(lfm_ctx* c) {
-  if (c->flags_clear) return LFM_OK;  // nothing has set them since
+  recording(c);
+  if (c->flags_clear && !c->recorded) return LFM_OK;  // nothing has set them since
   CK(c, cudaMemsetAsync(c->cs.flags, 0, 2 * sizeof(int32_t), c->stream));
   c->flags_clear = true;
   return leave(c);
@@ -704,8 +719,9 @@ int invalidate_split(lfm_ctx* c) {
 // inner-solve seed that the mixed form's last launch left in place no longer apply
 // (lfm_solve_mixed_df.cuh). Stream-ordered after any launch still pending.
 int invalidate_seed(lfm_ctx* c) {
-  if (c->flags_clear) return LFM_OK;
   DeviceGuard g(c->device);
+  recording(c);
+  if (c->flags_clear && !c->recorded) return LFM_OK;
   CK(c, cudaMemsetAsync(c->cs.flags + 1, 0, sizeof(int32_t), c->stream));
   return leave(c);
 }
@@ -741,6 +757,7 @@ int enqueue_chunk(lfm_ctx* c, int steps, int mode) {
     if (L.ctas <= 0) return fail(c, LFM_ECUDA, "no co-resident CTA fits the assembly kernel");
   }
   if (L.skip_cta >= 0 && L.ctas < 2) return fail(c, LFM_EINVAL, "the skip-arrival hook needs >= 2 CTAs");
+  recording(c);
   CK(c, cudaMemsetAsync(c->cs.sync, 0, sizeof(SyncWords), c->stream));
   if (mode == kModeSteps && c->opts.precision != LFM_FP64) c->flags_clear = false;  // the launch may set them
   CK(c, launch_steps(c->cs, L, steps, mode, c->stream));
