@@ -397,6 +397,13 @@ __device__ __forceinline__ void pf_next(const T* v, int c, int c1) {
   if (c + 3 * B < c1) prefetch_l2(v + c + 3 * B);
 }
 
+// The same for a loop that goes backwards.
+template <int B, typename T>
+__device__ __forceinline__ void pf_back(const T* v, int c, int c0) {
+  if (c - 2 * B >= c0) prefetch_l2(v + c - 2 * B);
+  if (c - 3 * B >= c0) prefetch_l2(v + c - 3 * B);
+}
+
 // ---- A v over the slot-major matrix (FP64 or FP32 copy) --------------------------------
 template <typename T>
 struct Slots {
@@ -510,6 +517,60 @@ __device__ __forceinline__ void pass_direction(int c0, int c1, T beta, T* __rest
     p[c + B] = fmadd(beta, p2, w2);
   }
   if (c < c1) p[c] = fmadd(beta, p[c], w[c]);
+}
+
+// Cells from which the streamed solves update the solution in P and not in U (see pass_direction_x):
+// where the vectors do not stay in L2. Below, P and U are bound by their instructions: in batches of
+// up to 1.3 M cells the late form was 2 % slower in mixed, 4 % in df64.
+constexpr int kLateCells = 4000000;
+
+// P of the mixed form: dx += alpha p, the correction's update with the last direction, and
+// p = w + beta p. U used to update dx and read p once more for it: 44 bytes of vectors per cell and
+// iteration against 40 so. Backwards: the pass starts at the rows that U touched last and ends at
+// those that the product reads first, while L2 still holds them. kFirst: dx = alpha p + 0, the same
+// value as from the dx = 0 the solve starts from, without reading it. P and U of an iteration over
+// 33 M cells: 67 + 168 -> 98 + 103 us, a call 17.2 -> 16.2 ms; over 8 M cells 6.80 -> 6.60 ms.
+// (In FP64 the same was slower, 11.39 -> 11.68 ms for 8 M cells: U is bound by its multiply-adds there
+// and hides the loads of the update, which P does not.)
+template <int B, bool kFirst>
+__device__ __forceinline__ void pass_direction_x(int c0, int c1, float alpha, float beta, float* __restrict__ dx,
+                                                 float* __restrict__ p, const float* __restrict__ w) {
+  int c = c0 + (int)threadIdx.x;
+  if (c >= c1) return;
+  c += (c1 - 1 - c) / B * B;  // the thread's last row
+  for (; c >= c0 + B; c -= 2 * B) {
+    const int d = c - B;
+    pf_back<B>(p, c, c0);
+    pf_back<B>(w, c, c0);
+    if (!kFirst) pf_back<B>(dx, c, c0);
+    const float p1 = p[c], p2 = p[d], w1 = w[c], w2 = w[d];
+    const float s1 = kFirst ? 0.0f : dx[c], s2 = kFirst ? 0.0f : dx[d];
+    dx[c] = fmaf(alpha, p1, s1);
+    dx[d] = fmaf(alpha, p2, s2);
+    p[c] = fmaf(beta, p1, w1);
+    p[d] = fmaf(beta, p2, w2);
+  }
+  if (c >= c0) {
+    const float pc = p[c];
+    dx[c] = fmaf(alpha, pc, kFirst ? 0.0f : dx[c]);
+    p[c] = fmaf(beta, pc, w[c]);
+  }
+}
+
+// The correction's last update, after the iteration that ended the solve.
+template <int B, bool kFirst>
+__device__ __forceinline__ void pass_solution(int c0, int c1, float alpha, float* __restrict__ dx,
+                                              const float* __restrict__ p) {
+  int c = c0 + (int)threadIdx.x;
+  for (; c + B < c1; c += 2 * B) {
+    pf_next<B>(p, c, c1);
+    if (!kFirst) pf_next<B>(dx, c, c1);
+    const float p1 = p[c], p2 = p[c + B];
+    const float s1 = kFirst ? 0.0f : dx[c], s2 = kFirst ? 0.0f : dx[c + B];
+    dx[c] = fmaf(alpha, p1, s1);
+    dx[c + B] = fmaf(alpha, p2, s2);
+  }
+  if (c < c1) dx[c] = fmaf(alpha, p[c], kFirst ? 0.0f : dx[c]);
 }
 
 // M (FP64): q = A p; returns this thread's share of p.q.
@@ -756,6 +817,43 @@ __device__ __forceinline__ double2 pass_update_f32(int c0, int c1, float a32, fl
     const float rn = fmaf(-a32, q[c], r[c]);
     const float wn = rD[c] * rn;
     dx[c] = fmaf(a32, p[c], kFirst ? 0.0f : dx[c]);
+    r[c] = rn;
+    w[c] = wn;
+    rsum.add(fabsf(rn));
+    rho_n.add_prod(wn, rn);
+  }
+  return make_double2(rsum.value(), rho_n.value());
+}
+
+// U with dx left to P (FP32): r -= alpha q, w = rD r; returns this thread's sum|r| and w.r, accumulated exactly as
+// FP32 pairs. (dx is updated by the next direction pass, pass_direction_x, or, after the last iteration, by
+// pass_solution.)
+template <int B>
+__device__ __forceinline__ double2 pass_update_late_f32(int c0, int c1, float a32, float* __restrict__ r,
+                                                float* __restrict__ w, const float* __restrict__ q,
+                                                const float* __restrict__ rD) {
+  Acc2f rsum, rho_n;
+  int c = c0 + (int)threadIdx.x;
+  for (; c + B < c1; c += 2 * B) {
+    pf_next<B>(q, c, c1);
+    pf_next<B>(r, c, c1);
+    pf_next<B>(rD, c, c1);
+    const int e = c + B;
+    const float qa = q[c], qb = q[e], ra = r[c], rb = r[e], da = rD[c], db = rD[e];
+    const float rna = fmaf(-a32, qa, ra), rnb = fmaf(-a32, qb, rb);
+    const float wa = da * rna, wb = db * rnb;
+    r[c] = rna;
+    r[e] = rnb;
+    w[c] = wa;
+    w[e] = wb;
+    rsum.add(fabsf(rna));
+    rsum.add(fabsf(rnb));
+    rho_n.add_prod(wa, rna);
+    rho_n.add_prod(wb, rnb);
+  }
+  if (c < c1) {
+    const float rn = fmaf(-a32, q[c], r[c]);
+    const float wn = rD[c] * rn;
     r[c] = rn;
     w[c] = wn;
     rsum.add(fabsf(rn));
@@ -1366,9 +1464,18 @@ __device__ __forceinline__ bool inner_cg_f32(const CaseDev& cs, const CaseDev& c
                                              int c0, int c1, int min_inner, int& iters, float* __restrict__ dx,
                                              float* __restrict__ r, float* __restrict__ w, float* __restrict__ p,
                                              float* __restrict__ q, const float* __restrict__ rD) {
-  for (int k = 0;;) {
+  const bool late = cs.N >= kLateCells;  // dx is updated in P
+  bool due = false;  // the last iteration's dx += alpha p is still to be done
+  int k = 0;
+  do {
     if (k > 0) {
-      pass_direction<B, float>(c0, c1, sh.beta32, p, w);
+      if (!late)
+        pass_direction<B, float>(c0, c1, sh.beta32, p, w);
+      else if (k == 1)
+        pass_direction_x<B, true>(c0, c1, sh.alpha32, sh.beta32, dx, p, w);
+      else
+        pass_direction_x<B, false>(c0, c1, sh.alpha32, sh.beta32, dx, p, w);
+      due = false;
       if (!team_barrier<B>(tm, sh)) return false;
       clk.lap(kPhP);
     }
@@ -1377,9 +1484,11 @@ __device__ __forceinline__ bool inner_cg_f32(const CaseDev& cs, const CaseDev& c
     if (!m_ok) return false;
     if (!team_allreduce<1, B>(tm, s1, sh, [&](int, double t, int lane) { fin_sigma(sh, t, lane); })) return false;
     clk.lap(kPhM);
-    if (sh.code != kGo) return true;
-    const double2 su = k == 0 ? pass_update_f32<B, true>(c0, c1, sh.alpha32, dx, r, w, p, q, rD)
-                              : pass_update_f32<B, false>(c0, c1, sh.alpha32, dx, r, w, p, q, rD);
+    if (sh.code != kGo) break;
+    const double2 su = late     ? pass_update_late_f32<B>(c0, c1, sh.alpha32, r, w, q, rD)
+                       : k == 0 ? pass_update_f32<B, true>(c0, c1, sh.alpha32, dx, r, w, p, q, rD)
+                                : pass_update_f32<B, false>(c0, c1, sh.alpha32, dx, r, w, p, q, rD);
+    due = late;
     const double s2[2] = {su.x, su.y};
     ++k;
     ++iters;
@@ -1388,8 +1497,10 @@ __device__ __forceinline__ bool inner_cg_f32(const CaseDev& cs, const CaseDev& c
         }))
       return false;
     clk.lap(kPhU);
-    if (sh.code != kGo) return true;
-  }
+  } while (sh.code == kGo);
+  if (due && k == 1) pass_solution<B, true>(c0, c1, sh.alpha32, dx, p);
+  if (due && k > 1) pass_solution<B, false>(c0, c1, sh.alpha32, dx, p);
+  return true;
 }
 
 template <int B, int W, class TM>

@@ -484,6 +484,64 @@ __device__ __forceinline__ void pass_direction_df(int c0, int c1, df beta, float
   if (c < c1) st_df(p + c, df_fma(beta, ld_df(p + c), ld_df(w + c)));
 }
 
+// P from kLateCells cells on: e += alpha p, the correction's update with the last direction, and p = w + beta p; backwards, as
+// pass_direction_x (lfm_solve.cuh). It starts with e = alpha p (first). Per iteration of 8 M cells, P and U with the update in U: 31 + 78 us,
+// here 47 + 50; the call 10.89 -> 10.57 ms.
+template <int B>
+__device__ __forceinline__ void pass_direction_x_df(int c0, int c1, df alpha, df beta, float2* __restrict__ e, bool first,
+                                                  float2* __restrict__ p, const float2* __restrict__ w) {
+  int c = c0 + (int)threadIdx.x;
+  if (c >= c1) return;
+  c += (c1 - 1 - c) / B * B;  // the thread's last row
+  auto step_e = [&](int i, df pi) { st_df(e + i, first ? df_mul(alpha, pi) : df_fma(alpha, pi, ld_df(e + i))); };
+  for (; c >= c0 + B; c -= 2 * B) {
+    const int d = c - B;
+    pf_back<B>(p, c, c0);
+    pf_back<B>(w, c, c0);
+    if (!first) pf_back<B>(e, c, c0);
+    const df p1 = ld_df(p + c), p2 = ld_df(p + d), w1 = ld_df(w + c), w2 = ld_df(w + d);
+    if (first) {
+      st_df(e + c, df_mul(alpha, p1));
+      st_df(e + d, df_mul(alpha, p2));
+    } else {
+      const df e1 = ld_df(e + c), e2 = ld_df(e + d);
+      st_df(e + c, df_fma(alpha, p1, e1));
+      st_df(e + d, df_fma(alpha, p2, e2));
+    }
+    st_df(p + c, df_fma(beta, p1, w1));
+    st_df(p + d, df_fma(beta, p2, w2));
+  }
+  if (c >= c0) {
+    const df pc = ld_df(p + c);
+    step_e(c, pc);
+    st_df(p + c, df_fma(beta, pc, ld_df(w + c)));
+  }
+}
+
+// The correction's last update, after the iteration that ended the solve.
+template <int B>
+__device__ __forceinline__ void pass_solution_df(int c0, int c1, df alpha, float2* __restrict__ e, bool first,
+                                                 const float2* __restrict__ p) {
+  int c = c0 + (int)threadIdx.x;
+  for (; c + B < c1; c += 2 * B) {
+    pf_next<B>(p, c, c1);
+    if (!first) pf_next<B>(e, c, c1);
+    const df p1 = ld_df(p + c), p2 = ld_df(p + c + B);
+    if (first) {
+      st_df(e + c, df_mul(alpha, p1));
+      st_df(e + c + B, df_mul(alpha, p2));
+    } else {
+      const df e1 = ld_df(e + c), e2 = ld_df(e + c + B);
+      st_df(e + c, df_fma(alpha, p1, e1));
+      st_df(e + c + B, df_fma(alpha, p2, e2));
+    }
+  }
+  if (c < c1) {
+    const df pc = ld_df(p + c);
+    st_df(e + c, first ? df_mul(alpha, pc) : df_fma(alpha, pc, ld_df(e + c)));
+  }
+}
+
 // M: q = A p; returns this thread's share of p.q.
 template <int B, int W>
 __device__ __forceinline__ double pass_amul_dot_df(const CaseDev& cs, uint32_t dl, int c0, int c1, const float2* __restrict__ p,
@@ -618,6 +676,42 @@ __device__ __forceinline__ double2 pass_update_df(int c0, int c1, df alpha, floa
   return make_double2(sa.value(), sr.value());
 }
 
+// U: r -= alpha q, w = rD r; returns this thread's sum|r| and w.r. (e's update is left to the next
+// direction pass or, after the last iteration, to pass_solution_df.)
+template <int B>
+__device__ __forceinline__ double2 pass_update_late_df(int c0, int c1, df alpha, float2* __restrict__ r,
+                                                  float2* __restrict__ w, const float2* __restrict__ q,
+                                                  const float2* __restrict__ rD) {
+  DfAcc sa, sr;
+  const df nalpha = df_neg(alpha);
+  int c = c0 + (int)threadIdx.x;
+  for (; c + B < c1; c += 2 * B) {
+    const int k = c + B;
+    const df qa = ld_df(q + c), qb = ld_df(q + k);
+    const df ra = ld_df(r + c), rb = ld_df(r + k);
+    const df da = ld_df(rD + c), db = ld_df(rD + k);
+    const df rna = df_fma(nalpha, qa, ra), rnb = df_fma(nalpha, qb, rb);
+    const df wa = df_mul(da, rna), wb = df_mul(db, rnb);
+    st_df(r + c, rna);
+    st_df(r + k, rnb);
+    st_df(w + c, wa);
+    st_df(w + k, wb);
+    sa.add(df_abs(rna));
+    sa.add(df_abs(rnb));
+    sr.add(df_mul(wa, rna));
+    sr.add(df_mul(wb, rnb));
+  }
+  if (c < c1) {
+    const df rn = df_fma(nalpha, ld_df(q + c), ld_df(r + c));
+    const df wn = df_mul(ld_df(rD + c), rn);
+    st_df(r + c, rn);
+    st_df(w + c, wn);
+    sa.add(df_abs(rn));
+    sr.add(df_mul(wn, rn));
+  }
+  return make_double2(sa.value(), sr.value());
+}
+
 // The df64 solve kept on chip (see cg_on_chip). The conductances are stored, the off-diagonals
 // are their negatives; e starts at zero (e = alpha p + 0 equals the streamed form's e = alpha p).
 struct ChipDf {
@@ -727,9 +821,17 @@ __device__ bool steps_df64(const CaseDev& cs, const CaseDev& cref, const TM& tm,
         }
         iters = sh.iters;
       }
+      // e is updated in P (not compiled into the kernels that serve general geometry, the batched ones
+      // among them: the second form's code made batches 2 to 3 % slower)
+      const bool late = R == 0 && !kGeom && cs.N >= kLateCells;
+      bool due = false;  // the last iteration's e += alpha p is still to be done
       while (R == 0 && sh.code == kGo) {
         if (iters > 0) {
-          pass_direction_df<B>(c0, c1, df_of(sh.beta2), p, w);
+          if (late)
+            pass_direction_x_df<B>(c0, c1, df_of(sh.alpha2), df_of(sh.beta2), e, iters == 1, p, w);
+          else
+            pass_direction_df<B>(c0, c1, df_of(sh.beta2), p, w);
+          due = false;
           if (!team_barrier<B>(tm, sh)) return false;
           clk.lap(kPhP);
         }
@@ -743,8 +845,10 @@ __device__ bool steps_df64(const CaseDev& cs, const CaseDev& cref, const TM& tm,
           return false;
         clk.lap(kPhM);
         if (sh.code != kGo) break;
-        const double2 su = pass_update_df<B>(c0, c1, df_of(sh.alpha2), e, iters == 0, r, w, p, q, rD);
-        pending = true;
+        const double2 su = late ? pass_update_late_df<B>(c0, c1, df_of(sh.alpha2), r, w, q, rD)
+                                : pass_update_df<B>(c0, c1, df_of(sh.alpha2), e, iters == 0, r, w, p, q, rD);
+        due = late;
+        pending = pending || !late;
         const double s2[2] = {su.x, su.y};
         ++iters;
         if (!team_allreduce<2, B>(tm, s2, sh, [&](int k, double t, int lane) {
@@ -754,6 +858,8 @@ __device__ bool steps_df64(const CaseDev& cs, const CaseDev& cref, const TM& tm,
           return false;
         clk.lap(kPhU);
       }
+      if (due) pass_solution_df<B>(c0, c1, df_of(sh.alpha2), e, iters == 1, p);
+      if (late && iters > 0) pending = true;
       if (sh.code == kSingular) status = LFM_ESINGULAR;
       if (sh.code == kNonFinite) status = LFM_ENONFINITE;
       iters_tot += iters;
