@@ -200,7 +200,7 @@ cudaError_t launch_batch_collect(const CaseDev* cases, int n_cases, const int32_
 cudaError_t launch_batch_steps(const BatchLaunch& bl, int n_steps, cudaStream_t s) {
   void* fn = batch_fn(bl.launch.threads, bl.W, bl.form);
   if (!fn) return cudaErrorInvalidValue;
-  // the opt-in above 48 KB was made when the launch shape was sized (max_coresident_batch_ctas),
+  // the opt-in for much shared memory was made when the launch shape was sized (max_coresident_batch_ctas),
   // outside any stream capture; this call finds it recorded
   const unsigned dyn = bl.launch.stage_rows ? batch_dyn_smem(bl.launch.threads, bl.W, bl.form) : 0u;
   cudaError_t e = allow_dyn_smem(fn, dyn);

@@ -217,9 +217,10 @@ enum BatchForm { kBatchAny = 0, kBatchFp64 = 1, kBatchDf64 = 2 };
 // Kernel launchers (lfm_step.cu). Return a cudaError_t.
 cudaError_t launch_steps(const CaseDev& cs, const Launch& L, int n_steps, int mode,
                          cudaStream_t stream);
-// Largest co-resident CTA count for the step kernel at `threads` per CTA.
-// Opts a kernel into more than 48 KB of dynamic shared memory (once per kernel and device).
+// Opts a kernel into its dynamic shared memory where that and its static share may exceed 48 KB (once
+// per kernel and device).
 cudaError_t allow_dyn_smem(void* fn, unsigned bytes);
+// Largest co-resident CTA count for the step kernel at `threads` per CTA.
 int max_coresident_ctas(int precision, int threads, int W, int device);
 // Slot width (template argument) of the step kernel a case runs at `threads` per CTA.
 int kernel_width(int W, bool coded, int threads);

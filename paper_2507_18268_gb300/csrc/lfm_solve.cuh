@@ -18,7 +18,8 @@
 //
 // FP64 step (phases separated by team barriers):
 //   A1 sum             sum x for xRef
-//   A2+I rows          diag, source, rD = 1/diag, row sum; from the same loaded row
+//   A2+I rows          diag, rD = 1/diag, row sum (in the launch's first pass, the matrix then
+//                      stands for the launch) and the source; from the same loaded row
 //                      A x, r = b - A x, normFactor, sum|r|, w = rD r, rho; p = w (first
 //                      search direction). The source is needed by no later phase of an
 //                      FP64 step and is stored only for read-back.
@@ -26,6 +27,8 @@
 //   P  p = w + beta p  (skipped on the first iteration)
 //   M  q = A p, sigma = p.q                   -> alpha = rho / sigma
 //   U  x += alpha p, r -= alpha q, w = rD r, sum|r|, rho' = w.r -> beta = rho'/rho
+//   (from kLateCells cells on the FP32 and df64 loops update the solution in P; where a thread takes few rows the loop
+//   keeps them on chip and forms p in M, see cg_on_chip)
 //
 // General (non-orthogonal) meshes (section "Code Porting": the gradient passes): A1 also
 // evaluates the Gauss linear gradient of T per cell, and A2 adds to each row's source the
