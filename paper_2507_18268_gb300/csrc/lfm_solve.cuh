@@ -1069,6 +1069,7 @@ __device__ __forceinline__ bool assemble_prologue(const CaseDev& cs, const CaseD
 // threads) serve mixed and df64 on packed slots only.
 struct ChipF32 {
   using V = float;
+  static constexpr bool kSolInU = false;  // the correction is read by the row's own thread only
   float *p, *q, *w, *sol;
   const float *r, *rD, *coef, *diag;
   struct Sum {
@@ -1092,6 +1093,10 @@ struct ChipF32 {
 
 struct ChipF64 {
   using V = double;
+  // The solution is the field itself, and on general geometry the next pass starts with its gradient,
+  // which gathers the neighbours' T before any barrier: U stores it, so that U's barrier orders it
+  // for every CTA, as in the streamed form.
+  static constexpr bool kSolInU = true;
   double *p, *q, *w, *sol;
   const double *r, *rD, *coef, *diag;
   struct Sum {
@@ -1291,6 +1296,7 @@ __device__ __forceinline__ bool cg_on_chip(const F f, const CaseDev& cs, const C
       sol[j] = F::fma(alpha, p[j], sol[j]);
       r[j] = rn;
       F::st(f.w, c, wn);
+      if constexpr (F::kSolInU) F::st(f.sol, c, sol[j]);
       rsum.abs(rn);
       rho.dot(wn, rn);
     }
@@ -1299,11 +1305,13 @@ __device__ __forceinline__ bool cg_on_chip(const F f, const CaseDev& cs, const C
     clk.lap(kPhU);
     go = sh.code == kGo;
   }
+  if constexpr (!F::kSolInU) {
 #pragma unroll
-  for (int j = 0; j < R; ++j) {
-    const int c = first + j * B;
-    if (c >= c1) break;
-    F::st(f.sol, c, sol[j]);
+    for (int j = 0; j < R; ++j) {
+      const int c = first + j * B;
+      if (c >= c1) break;
+      F::st(f.sol, c, sol[j]);
+    }
   }
   return true;
 }

@@ -716,6 +716,7 @@ __device__ __forceinline__ double2 pass_update_late_df(int c0, int c1, df alpha,
 // are their negatives; e starts at zero (e = alpha p + 0 equals the streamed form's e = alpha p).
 struct ChipDf {
   using V = df;
+  static constexpr bool kSolInU = false;  // e is read by the row's own thread only
   df *p, *q, *w, *sol;
   const df *r, *rD, *coef, *diag;
   struct Sum {
