@@ -321,6 +321,11 @@ __device__ __forceinline__ void mbar_init_fence() {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 
+// Before bulk copies of data that ordinary stores wrote earlier in the launch (a row pass's
+// diagonal): a barrier orders those stores for ordinary loads only, the copy engine reads
+// global memory through another proxy.
+__device__ __forceinline__ void bulk_reads_fence() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
+
 __device__ __forceinline__ void mbar_inval(uint64_t* bar) {
   asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
@@ -402,6 +407,7 @@ __device__ __forceinline__ bool staged_tiles(int c0, int c1, const TM& tm, Issue
   if (tid == 0) {
     for (int s = 0; s < NST; ++s) mbar_init(bar + s, 1);
     mbar_init_fence();
+    bulk_reads_fence();  // once per pass: nothing staged is rewritten during it
     const uint64_t pol = l2_evict_first_policy();
     for (int t = 0; t < NST && t < ntiles; ++t) {
       const int t0 = c0 + t * TC;

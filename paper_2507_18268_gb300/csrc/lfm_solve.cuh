@@ -1164,7 +1164,7 @@ __device__ __noinline__ bool chip_load(const F f, const CaseDev& cs, const TM& t
   if (threadIdx.x == 0) {
     mbar_init(bar, 1);
     mbar_init_fence();
-    asm volatile("fence.proxy.async.global;" ::: "memory");  // the diagonal was written by ordinary stores
+    bulk_reads_fence();
     if (n > 0 && (int)blockIdx.x != g_skip_copy_cta) {
       const uint64_t pol = l2_evict_first_policy();
       mbar_arrive_expect_tx(bar, (unsigned)n * chip_row_bytes<W>(sizeof(V)));
