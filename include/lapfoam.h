@@ -293,7 +293,11 @@ int lfm_set_field_device(lfm_ctx *ctx, const double *T_dev);
 int lfm_advance(lfm_ctx *ctx, int32_t n_steps, lfm_step_stats *out);
 
 /* Enqueues n_steps like lfm_advance without waiting (statistics stay on the device until
- * lfm_finish). At most one pending advance per context. */
+ * lfm_finish). At most one pending advance per context. On a stream that is being captured the
+ * launch is recorded, with a rebuild of the boundary terms, so that a replay reads the patches as
+ * they are then; while other set-up of the case is due (its first advance, or a change of mesh,
+ * diffusivity, time step of a df64 or mixed case, or patches of a general mesh since the last one)
+ * the call returns LFM_ESTATE before any work, and the set-up stays due. */
 int lfm_advance_async(lfm_ctx *ctx, int32_t n_steps);
 
 /* 1 if the pending advance is still running, LFM_OK if done (or none pending). */

@@ -319,6 +319,7 @@ int fail(lfm_ctx* c, int code, const char* fmt, ...) {
 }
 
 int cuda_fail(lfm_ctx* c, cudaError_t e, const char* what) {
+  cudaGetLastError();  // reported here: not once more by the next launch's check
   return fail(c, LFM_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
@@ -640,16 +641,21 @@ int refresh_vdt(lfm_ctx* c) {
   return LFM_OK;
 }
 
-// Whether the context's stream records into a graph. What a recorded call does happens at each
-// replay, unseen by the host: from the first one on the context's flags count as unknown.
-bool recording(lfm_ctx* c) {
+bool capturing(cudaStream_t s) {
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(c->stream, &st) != cudaSuccess) {
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  if (st != cudaStreamCaptureStatusNone) c->recorded = true;
   return st != cudaStreamCaptureStatusNone;
+}
+
+// Whether the context's stream records into a graph. What a recorded call does happens at each
+// replay, unseen by the host: from the first one on the context's flags count as unknown.
+bool recording(lfm_ctx* c) {
+  const bool on = capturing(c->stream);
+  if (on) c->recorded = true;
+  return on;
 }
 
 // Marks the end of work that a call leaves on the context's stream: lfm_destroy waits for it.
@@ -660,10 +666,19 @@ int leave(lfm_ctx* c) {
   return LFM_OK;
 }
 
+// Set-up that is due has to run before the call's own work; on a capturing stream it would only be
+// recorded, and the flag that says it is done would be wrong until a replay. Such a call is refused
+// before any work, the set-up stays due.
+int refuse_setup_in_capture(lfm_ctx* c) {
+  if (!recording(c)) return LFM_OK;
+  return fail(c, LFM_ESTATE, "set-up of the case is due and cannot be recorded: advance once outside the stream capture");
+}
+
 // Rebuilds the face coefficients of the slot arrays (a0) when the mesh or DT changed since
 // they were built (the df64 form keeps its own, see refresh_df).
 int refresh_coef(lfm_ctx* c) {
   if (!c->coef_dirty || c->opts.precision == LFM_DF64) return LFM_OK;
+  if (int rc = refuse_setup_in_capture(c)) return rc;
   CK(c, launch_coef_setup(c->cs, c->stream));
   c->settled = false;
   c->coef_dirty = false;
@@ -676,6 +691,7 @@ int refresh_df(lfm_ctx* c) {
   const bool want = c->opts.precision == LFM_DF64 || (c->opts.precision == LFM_MIXED && c->hasdf && !c->has_geom);
   if (!want || !c->df_dirty) return LFM_OK;
   if (!c->hasdf) return fail(c, LFM_ENOMEM, "the workspace has no df64 buffers");
+  if (int rc = refuse_setup_in_capture(c)) return rc;
   CK(c, launch_df_setup(c->cs, c->stream));
   c->settled = false;
   c->df_dirty = false;
@@ -683,12 +699,19 @@ int refresh_df(lfm_ctx* c) {
 }
 
 // Rebuilds the boundary faces' row terms when the patches, their values, DT, dt or the mesh
-// changed since the last launch (every form's rows read them, matrix read-back too).
-int refresh_bnd(lfm_ctx* c) {
-  if (!c->bnd_dirty) return LFM_OK;
-  CK(c, launch_boundary_terms(c->cs, c->stream));
-  c->settled = false;
+// changed since the last launch (every form's rows read them, matrix read-back too). `on`: the
+// stream of the launch that reads them. A recorded launch brings its own rebuild, so that a replay
+// reads the patches as they are then; outside, a context with recorded launches rebuilds every
+// time, since a replay may have written the terms of another dt.
+int refresh_bnd(lfm_ctx* c, cudaStream_t on) {
+  const bool rec = capturing(on);
+  if (rec) c->recorded = true;
+  if (!c->bnd_dirty && !c->recorded) return LFM_OK;
+  CK(c, launch_boundary_terms(c->cs, on));
+  if (rec) return LFM_OK;
   c->bnd_dirty = false;
+  if (on != c->stream) return LFM_OK;
+  c->settled = false;
   return leave(c);
 }
 
@@ -696,6 +719,7 @@ int refresh_bnd(lfm_ctx* c) {
 // DT changed since the last launch. Enqueued on the context's stream.
 int refresh_ops(lfm_ctx* c) {
   if (!c->has_geom || !c->ops_dirty) return LFM_OK;
+  if (int rc = refuse_setup_in_capture(c)) return rc;
   refresh_case(c);
   CK(c, launch_geom_ops(c->cs, false, c->stream));
   c->settled = false;
@@ -737,10 +761,12 @@ int need_uploaded(lfm_ctx* c) {
 int enqueue_chunk(lfm_ctx* c, int steps, int mode) {
   refresh_case(c);
   if (int rc = refresh_ops(c)) return rc;
-  if (int rc = refresh_bnd(c)) return rc;
   if (mode == kModeSteps) {
     if (int rc = refresh_coef(c)) return rc;
     if (int rc = refresh_df(c)) return rc;
+  }
+  if (int rc = refresh_bnd(c, c->stream)) return rc;
+  if (mode == kModeSteps) {
     const int p = c->opts.precision;
     if (p == LFM_FP64 || (p == LFM_MIXED && !mixed_runs_df(c->cs))) {
       if (int rc = invalidate_split(c)) return rc;
@@ -782,6 +808,7 @@ int take_checks(lfm_ctx* c) {
 // Waits for the enqueued chunk, appends its statistics, maps the device status.
 int collect_chunk(lfm_ctx* c, int steps) {
   CK(c, cudaEventSynchronize(c->done));
+  c->settled = true;
   for (int i = 0; i < steps; ++i) c->stats_acc.push_back(c->h_stats[i]);
   for (int k = 0; k < kPhases; ++k) c->phase_ms[k] += 1e-6 * (double)c->h_phase[k];
   c->staged_passes += (long long)c->h_phase[kPhases];
@@ -1954,7 +1981,8 @@ int lfm_batch_advance_capped_async(lfm_batch* b, int32_t n_steps, int32_t use_gr
     if ((c->opts.precision == LFM_FP64 && !c->has64) || (c->opts.precision == LFM_MIXED && !c->has32) ||
         (c->opts.precision == LFM_DF64 && !(c->hasdf && c->has64)))
       return bfail(b, LFM_ENOMEM, "case %d has no buffers for its precision", b->order[i]);
-    if (refresh_coef(c) != LFM_OK || refresh_bnd(c) != LFM_OK || refresh_df(c) != LFM_OK)
+    const cudaStream_t on = capturing(b->stream) || recording(c) ? b->stream : c->stream;
+    if (refresh_coef(c) != LFM_OK || refresh_df(c) != LFM_OK || refresh_bnd(c, on) != LFM_OK)
       return bfail(b, LFM_ECUDA, "case %d: coefficient set-up failed", b->order[i]);
     if (!c->settled && c->stream != b->stream) {  // the batch launches on a stream of its own
       if (cudaStreamSynchronize(c->stream) != cudaSuccess)
@@ -2384,7 +2412,7 @@ int lfm_dd_advance(lfm_dd* d, int32_t n_steps, lfm_step_stats* out) {
   if (n_steps == 0) return LFM_OK;
   DeviceGuard g(c->device);
   refresh_case(c);
-  if ((rc = refresh_coef(c)) || (rc = refresh_bnd(c))) return ddfail(d, rc, "coefficient set-up of the case failed");
+  if ((rc = refresh_coef(c)) || (rc = refresh_bnd(c, c->stream))) return ddfail(d, rc, "coefficient set-up of the case failed");
   CaseDev cs = c->cs;  // the case's rows, with the decomposition's own barrier words and records
   cs.sync = d->sync;
   cs.partials = d->partials;
