@@ -555,7 +555,9 @@ int lfm_batch_debug_stage_rows(lfm_batch *b, int32_t on);
 /* Current launch shape (ctas = CTAs of the persistent launch). */
 int lfm_batch_get_launch(lfm_batch *b, int32_t *ctas, int32_t *threads, int32_t *cells_per_thread);
 
-/* Device-side barrier wait limit for batch launches (default 10 s). */
+/* Device-side barrier wait limit for batch launches (default 10 s). One launch runs all steps of an
+ * advance: a case's wait for CTAs that other cases still occupy is bounded by the limit times the
+ * steps, every other wait by the limit. */
 int lfm_batch_set_barrier_timeout(lfm_batch *b, uint64_t ns);
 
 /* Enqueues n_steps (<= 1024) steps of every member case. use_graph != 0: the

@@ -63,7 +63,13 @@ __global__ void __launch_bounds__(B, 1024 / B) batch_kernel(const CaseDev* __res
     const int base = case_step[c];
     // a case whose cap is reached runs no step; its team's CTAs go back for tickets at once
     const int run = min(n_steps, case_cap[c] - base);
-    if (run > 0) {
+    // The team meets once before it starts. A team that the launch's CTAs cannot all serve at once waits
+    // here for the jobs before it, which run all steps of the advance: the bound of this wait grows with
+    // the steps, the waits of a staffed team keep theirs. (One barrier without sums per job, 1.6 us.)
+    const uint64_t most = ~0ull / (uint64_t)n_steps;
+    const Team meet{tm.size, tm.rank, tm.sw, tm.partials,
+                    L.timeout_ns < most ? L.timeout_ns * (uint64_t)n_steps : ~0ull};
+    if (run > 0 && team_barrier<B>(meet, sh)) {
       if constexpr (kForm == kBatchFp64) {
         run_steps_f64<B, W>(s_cs, s_cs, tm, run, kModeSteps, sh, base);
       } else if constexpr (kForm == kBatchDf64) {
