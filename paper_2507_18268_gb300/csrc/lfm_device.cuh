@@ -283,12 +283,11 @@ __device__ __forceinline__ bool team_barrier(const Team& tm, TeamShared<B>& sh) 
 
 // Slot k's neighbour distance of a packed slot word (CaseDev::slot_code), from the table at
 // shared-memory address dl. The lanes of a warp mostly hold the same word, and sixteen words
-// sit in different banks, so the lookup never serialises.
+// sit in different banks, so the lookup never serialises. An ordinary shared load: the batched
+// kernel rewrites the table for every job, and the compiler has to see that it is read.
 __device__ __forceinline__ int code_delta(uint32_t dl, uint32_t word, int k) {
   const uint32_t at = (k == 0 ? word << 2 : word >> (4 * k - 2)) & 60u;
-  int d;
-  asm("ld.shared.s32 %0, [%1];" : "=r"(d) : "r"(dl + at));
-  return d;
+  return *static_cast<const int32_t*>(__cvta_shared_to_generic(dl + at));
 }
 
 // ---- bulk copies global -> shared, completed on an mbarrier ------------------------------
