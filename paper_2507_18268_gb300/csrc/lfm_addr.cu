@@ -243,7 +243,9 @@ __device__ __forceinline__ bool table_add(int32_t* t, int32_t d) {
 }
 
 // The distinct neighbour distances of a mesh: per block in shared memory, merged into out
-// (out[kMaxDeltas] != 0: more than fit; blocks that see it stop).
+// (out[kMaxDeltas] != 0: more than fit; blocks that see it stop, and one that finds it out
+// merges nothing: a randomly numbered mesh, where every block does, is given up at once; its
+// upload, 64^3 cells: 3.84 ms without the search, 4.00 when every block merged, 3.88 so).
 __global__ void delta_find_kernel(int32_t N, int32_t W, const int32_t* __restrict__ other, int32_t* __restrict__ out) {
   __shared__ int32_t t[kMaxDeltas];
   if (threadIdx.x < kMaxDeltas) t[threadIdx.x] = kNoDelta;
@@ -252,9 +254,9 @@ __global__ void delta_find_kernel(int32_t N, int32_t W, const int32_t* __restric
   for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < N && fits; c += (int64_t)gridDim.x * blockDim.x) {
     if (*reinterpret_cast<volatile int32_t*>(out + kMaxDeltas) != 0) break;
     for (int k = 0; k < W && fits; ++k) fits = table_add(t, other[(size_t)k * N + c] - (int32_t)c);
+    if (!fits) *reinterpret_cast<volatile int32_t*>(out + kMaxDeltas) = 1;
   }
-  if (!fits) atomicExch(out + kMaxDeltas, 1);
-  __syncthreads();
+  if (__syncthreads_or(!fits)) return;
   if (threadIdx.x < kMaxDeltas && t[threadIdx.x] != kNoDelta && !table_add(out, t[threadIdx.x]))
     atomicExch(out + kMaxDeltas, 1);
 }

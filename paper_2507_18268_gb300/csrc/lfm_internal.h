@@ -264,8 +264,12 @@ cudaError_t build_slot_codes(int32_t N, int32_t W, const int32_t* slot_other, co
 
 // Box meshes built from closed forms (lfm_box.cu).
 int box_slot_width(long long nx, long long ny, long long nz);
+// The neighbour distances of a box of six slots in the order of its slot words; their number, 0 for
+// other boxes.
+int box_deltas(long long nx, long long ny, int W, int32_t* delta);
+// slot_code: the packed slot words, null where the box has none.
 cudaError_t launch_box(long long nx, long long ny, long long nz, int W, const double* xs, const double* ys,
-                       const double* zs, const CaseDev& cs, cudaStream_t stream);
+                       const double* zs, const CaseDev& cs, uint32_t* slot_code, cudaStream_t stream);
 void box_layout_host(long long nx, long long ny, long long nz, int W, const double* xs, const double* ys,
                      const double* zs, int32_t* slot_other, int32_t* slot_face, uint32_t* face_slots,
                      double* V, double* magSf,
