@@ -416,8 +416,13 @@ int lfm_debug_check_inject(lfm_ctx *ctx, int32_t site);
  * Limits: n_cells <= 65536 and n_faces <= 262144, else LFM_EINVAL before any device work;
  * at most 32 internal faces per cell (as lfm_upload_mesh). A face out of range, faces not
  * sorted by owner or a cell above the face limit are reported as LFM_EINVAL by the kernel
- * before it uses any of those indices as an address; x is then left unchanged. Every
- * non-OK return sets the text of lfm_last_error(NULL) on the calling thread.
+ * before it uses any of those indices as an address; x is then left unchanged. The solve is
+ * one cooperative launch of one CTA of 256 threads per 256 cells, at most one CTA per SM, so
+ * on a GPU that other kernels occupy it starts once all of them fit beside those. Its CTAs
+ * meet at barriers; when one wait runs out (2 s; no call that runs undisturbed comes near it)
+ * the kernel stops and the call returns LFM_ETIMEOUT: x then holds an unfinished iterate and
+ * the stats record is not valid beyond its status. Every non-OK return sets the text of
+ * lfm_last_error(NULL) on the calling thread.
  * Working memory: one fixed device array of about 5.8 MB inside the library, present on
  * every GPU that loads it until the process exits; no call allocates, frees or calls an
  * allocating library routine. All calls share that array (each call re-initialises what it
