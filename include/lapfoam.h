@@ -370,6 +370,11 @@ int lfm_debug_skip_stage_copy(lfm_ctx *ctx, int32_t cta);
  * throughout. */
 int lfm_debug_staged_passes(lfm_ctx *ctx, int64_t *n);
 
+/* Test evidence: how the solves of the last advance (its last launch) ran, as the device noted
+ * it: rows receives the rows per thread that the kernel keeping them on chip was compiled for,
+ * 0 when they were streamed (or no step needed an iteration). */
+int lfm_debug_solve_form(lfm_ctx *ctx, int32_t *rows);
+
 /* Test switch: on != 0 (the default) lets single-case launches on meshes of six slots per cell
  * keep matrix rows in shared memory: the inner solve of the mixed form on orthogonal meshes,
  * whole (rows loaded once per launch, vectors in registers) where the team's threads take few

@@ -116,6 +116,7 @@ _SIGS = {
     "lfm_debug_skip_arrival": ([_ctx_p, c_int32], c_int),
     "lfm_debug_stage_rows": ([_ctx_p, c_int32], c_int),
     "lfm_debug_pack_slots": ([_ctx_p, c_int32, POINTER(c_int32)], c_int),
+    "lfm_debug_solve_form": ([_ctx_p, POINTER(c_int32)], c_int),
     "lfm_debug_skip_stage_copy": ([_ctx_p, c_int32], c_int),
     "lfm_debug_staged_passes": ([_ctx_p, POINTER(ctypes.c_int64)], c_int),
     "lfm_pcg_solve_static": ([c_int32, c_int32, c_void_p, c_void_p, c_void_p, c_void_p, c_void_p, c_void_p,
@@ -502,6 +503,13 @@ def lfm_debug_pack_slots(ctx, on: bool) -> int:
     """Distinct neighbour distances of the mesh (0: not packed) after switching its use."""
     n = c_int32(0)
     _check(load().lfm_debug_pack_slots(ctx, 1 if on else 0, ctypes.byref(n)), ctx)
+    return n.value
+
+
+def lfm_debug_solve_form(ctx) -> int:
+    """Rows per thread of the last advance's solves kept on chip (0: streamed)."""
+    n = c_int32(0)
+    _check(load().lfm_debug_solve_form(ctx, ctypes.byref(n)), ctx)
     return n.value
 
 

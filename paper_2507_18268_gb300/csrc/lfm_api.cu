@@ -288,13 +288,14 @@ struct lfm_ctx {
   char* h_back = nullptr;             // pinned, kBackBytes; the next three point into it
   lfm_step_stats* h_stats = nullptr;  // kStatsCap records
   int32_t* h_status = nullptr;
-  unsigned long long* h_phase = nullptr;  // kPhases + 1 (the phase times, then the staged-pass count)
+  unsigned long long* h_phase = nullptr;  // the phase times, then the words of the form that ran (SyncWords)
   cudaEvent_t last = nullptr;         // after the last work that a call left on the stream unwaited for
   bool touched = false;               // last has been recorded
   bool settled = true;                // no set-up work (refresh_*) enqueued since the stream was last waited for
   bool recorded = false;              // a call was recorded into a graph (see recording)
   bool flags_clear = false;           // flags[0] and flags[1] are zero on the device (or will be, in order)
   long long staged_passes = 0;        // passes of the last advance with staged rows (team rank 0)
+  int chip_rows = 0;                  // rows per thread of its solves kept on chip, 0: streamed
   double phase_ms[kPhases] = {};      // per phase kind, summed over the last advance
   cudaEvent_t done = nullptr;
   int pending_steps = 0;
@@ -813,6 +814,7 @@ int collect_chunk(lfm_ctx* c, int steps) {
   for (int i = 0; i < steps; ++i) c->stats_acc.push_back(c->h_stats[i]);
   for (int k = 0; k < kPhases; ++k) c->phase_ms[k] += 1e-6 * (double)c->h_phase[k];
   c->staged_passes += (long long)c->h_phase[kPhases];
+  c->chip_rows = (int)c->h_phase[kPhases + 1];
   int32_t st = *c->h_status;
   if (st != 0) invalidate_seed(c);  // a launch that stopped early left no seed to trust
   if (st == LFM_ETIMEOUT) return fail(c, LFM_ETIMEOUT, "a device barrier wait ran out (kernel stopped)");
@@ -1656,6 +1658,13 @@ int lfm_debug_staged_passes(lfm_ctx* c, int64_t* n) {
   if (!c) return fail_free(LFM_EINVAL, "context is NULL");
   if (!n) return fail(c, LFM_EINVAL, "n is NULL");
   *n = c->staged_passes;
+  return LFM_OK;
+}
+
+int lfm_debug_solve_form(lfm_ctx* c, int32_t* rows) {
+  if (!c) return fail_free(LFM_EINVAL, "context is NULL");
+  if (!rows) return fail(c, LFM_EINVAL, "rows is NULL");
+  *rows = c->chip_rows;
   return LFM_OK;
 }
 

@@ -40,7 +40,8 @@ struct alignas(128) SyncWords {
   int32_t pad3[31];
   unsigned long long phase_ns[8];    // time per phase kind, accumulated by the team's rank 0
   unsigned long long staged;         // passes that ran with rows staged in shared memory (rank 0)
-  unsigned long long pad4[7];
+  unsigned long long chip_rows;      // rows per thread of the launch's solve kept on chip, 0: streamed (rank 0)
+  unsigned long long pad4[6];
 };
 
 // Phase kinds of the step (indices of SyncWords::phase_ns).

@@ -1206,6 +1206,7 @@ __device__ __forceinline__ bool cg_on_chip(const F f, const CaseDev& cs, const C
   if (!loaded) {
     if (!chip_load<F, B, W, R>(f, cref, tm, c0, c1)) return false;
     loaded = true;
+    if (tm.rank == 0 && threadIdx.x == 0) tm.sw->chip_rows = R;  // read back by the host (a test's evidence)
   }
   V r[R], rd[R], p[R], q[R], sol[R];
 #pragma unroll
