@@ -372,8 +372,14 @@ int lfm_debug_staged_passes(lfm_ctx *ctx, int64_t *n);
 
 /* Test evidence: how the solves of the last advance (its last launch) ran, as the device noted
  * it: rows receives the rows per thread that the kernel keeping them on chip was compiled for,
- * 0 when they were streamed (or no step needed an iteration). */
-int lfm_debug_solve_form(lfm_ctx *ctx, int32_t *rows);
+ * 0 when they were streamed (or no step needed an iteration); late (of all its launches) the
+ * number of streamed solves that updated the solution in the direction pass. Either may be NULL. */
+int lfm_debug_solve_form(lfm_ctx *ctx, int32_t *rows, int64_t *late);
+
+/* Test switch: the cells from which streamed mixed solves (df64: half as many) update the solution
+ * in the direction pass instead of the residual's (<= 0 restores the default). The results are the same
+ * bit for bit; the switch exists to test and measure that. */
+int lfm_debug_late_cells(lfm_ctx *ctx, int32_t cells);
 
 /* Test switch: on != 0 (the default) lets single-case launches on meshes of six slots per cell
  * keep matrix rows in shared memory: the inner solve of the mixed form on orthogonal meshes,

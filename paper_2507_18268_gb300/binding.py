@@ -116,7 +116,8 @@ _SIGS = {
     "lfm_debug_skip_arrival": ([_ctx_p, c_int32], c_int),
     "lfm_debug_stage_rows": ([_ctx_p, c_int32], c_int),
     "lfm_debug_pack_slots": ([_ctx_p, c_int32, POINTER(c_int32)], c_int),
-    "lfm_debug_solve_form": ([_ctx_p, POINTER(c_int32)], c_int),
+    "lfm_debug_solve_form": ([_ctx_p, POINTER(c_int32), POINTER(ctypes.c_int64)], c_int),
+    "lfm_debug_late_cells": ([_ctx_p, c_int32], c_int),
     "lfm_debug_skip_stage_copy": ([_ctx_p, c_int32], c_int),
     "lfm_debug_staged_passes": ([_ctx_p, POINTER(ctypes.c_int64)], c_int),
     "lfm_pcg_solve_static": ([c_int32, c_int32, c_void_p, c_void_p, c_void_p, c_void_p, c_void_p, c_void_p,
@@ -509,8 +510,19 @@ def lfm_debug_pack_slots(ctx, on: bool) -> int:
 def lfm_debug_solve_form(ctx) -> int:
     """Rows per thread of the last advance's solves kept on chip (0: streamed)."""
     n = c_int32(0)
-    _check(load().lfm_debug_solve_form(ctx, ctypes.byref(n)), ctx)
+    _check(load().lfm_debug_solve_form(ctx, ctypes.byref(n), None), ctx)
     return n.value
+
+
+def lfm_debug_late_solves(ctx) -> int:
+    """Streamed solves of the last advance that updated the solution in the direction pass."""
+    n = ctypes.c_int64(0)
+    _check(load().lfm_debug_solve_form(ctx, None, ctypes.byref(n)), ctx)
+    return n.value
+
+
+def lfm_debug_late_cells(ctx, cells: int):
+    _check(load().lfm_debug_late_cells(ctx, int(cells)), ctx)
 
 
 def lfm_debug_stage_rows(ctx, on: bool):

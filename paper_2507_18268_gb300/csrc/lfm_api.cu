@@ -282,6 +282,7 @@ struct lfm_ctx {
   uint64_t timeout_ns = 2000000000ull;
   int skip_cta = -1;
   int stage_rows = 1;  // bulk-staged matrix rows where a pass supports them
+  int late_cells = kLateCells;
   int skip_copy_cta = -1;
 
   // async state
@@ -295,6 +296,7 @@ struct lfm_ctx {
   bool recorded = false;              // a call was recorded into a graph (see recording)
   bool flags_clear = false;           // flags[0] and flags[1] are zero on the device (or will be, in order)
   long long staged_passes = 0;        // passes of the last advance with staged rows (team rank 0)
+  long long late_solves = 0;          // its streamed solves that updated the solution in P
   int chip_rows = 0;                  // rows per thread of its solves kept on chip, 0: streamed
   double phase_ms[kPhases] = {};      // per phase kind, summed over the last advance
   cudaEvent_t done = nullptr;
@@ -495,6 +497,7 @@ void refresh_case(lfm_ctx* c) {
   cs.min_iter = c->opts.min_iter;
   cs.precision = c->opts.precision;
   cs.n_corr = c->n_corr;
+  cs.late_cells = c->late_cells;
 }
 
 // Power-of-two scale of the df64 form's system: V/dt near one for a cell of mean volume.
@@ -815,6 +818,7 @@ int collect_chunk(lfm_ctx* c, int steps) {
   for (int k = 0; k < kPhases; ++k) c->phase_ms[k] += 1e-6 * (double)c->h_phase[k];
   c->staged_passes += (long long)c->h_phase[kPhases];
   c->chip_rows = (int)c->h_phase[kPhases + 1];
+  c->late_solves += (long long)c->h_phase[kPhases + 2];
   int32_t st = *c->h_status;
   if (st != 0) invalidate_seed(c);  // a launch that stopped early left no seed to trust
   if (st == LFM_ETIMEOUT) return fail(c, LFM_ETIMEOUT, "a device barrier wait ran out (kernel stopped)");
@@ -1484,7 +1488,7 @@ int lfm_advance_async(lfm_ctx* c, int32_t n_steps) {
   DeviceGuard g(c->device);
   c->stats_acc.clear();
   for (int k = 0; k < kPhases; ++k) c->phase_ms[k] = 0.0;
-  c->staged_passes = 0;
+  c->staged_passes = c->late_solves = 0;
   const int first = n_steps < kStatsCap ? n_steps : kStatsCap;
   if ((rc = enqueue_chunk(c, first, kModeSteps))) return rc;
   c->pending_steps = first;
@@ -1661,10 +1665,16 @@ int lfm_debug_staged_passes(lfm_ctx* c, int64_t* n) {
   return LFM_OK;
 }
 
-int lfm_debug_solve_form(lfm_ctx* c, int32_t* rows) {
+int lfm_debug_solve_form(lfm_ctx* c, int32_t* rows, int64_t* late) {
   if (!c) return fail_free(LFM_EINVAL, "context is NULL");
-  if (!rows) return fail(c, LFM_EINVAL, "rows is NULL");
-  *rows = c->chip_rows;
+  if (rows) *rows = c->chip_rows;
+  if (late) *late = c->late_solves;
+  return LFM_OK;
+}
+
+int lfm_debug_late_cells(lfm_ctx* c, int32_t cells) {
+  if (!c) return fail_free(LFM_EINVAL, "context is NULL");
+  c->late_cells = cells > 0 ? cells : kLateCells;
   return LFM_OK;
 }
 

@@ -19,6 +19,15 @@ constexpr int kMaxSweeps = 5;        // mixed precision: defect-correction sweep
 constexpr int kMaxSlots = 32;        // largest number of internal faces per cell
 constexpr int kMaxDeltas = 16;       // distinct neighbour distances a coded slot row can name
 
+// Cells from which the streamed mixed solves update the solution in P and not in U (see
+// pass_direction_x): where the vectors do not stay in L2. df64 vectors are twice as large, its line
+// lies at half the cells. Below, P and U are bound by their instructions. Time of the update in U over
+// that in P, four steps of a graded box, by millions of cells (runs of one side differ by 0.2 %):
+//          1.0    1.4    2.0    2.5    3.0    3.5    4.1    5.0    6.0    8.0    16.8
+//   mixed  0.995  0.990  0.991  0.993  0.988  0.990  0.992  0.999  1.020  1.025  1.049
+//   df64   0.990  0.984  1.007  1.016  1.018  1.029  1.025  1.023  1.023  1.031  1.034
+constexpr int kLateCells = 5000000;
+
 // Slot width a kernel is compiled for: 0 (the case's, read at run time), 6 (neighbours read
 // from slot_other) or 6 | kCodedBit (neighbours from the packed codes, see CaseDev::slot_code).
 constexpr int kCodedBit = 16;
@@ -41,7 +50,8 @@ struct alignas(128) SyncWords {
   unsigned long long phase_ns[8];    // time per phase kind, accumulated by the team's rank 0
   unsigned long long staged;         // passes that ran with rows staged in shared memory (rank 0)
   unsigned long long chip_rows;      // rows per thread of the launch's solve kept on chip, 0: streamed (rank 0)
-  unsigned long long pad4[6];
+  unsigned long long late;           // streamed solves that updated the solution in P (rank 0)
+  unsigned long long pad4[5];
 };
 
 // Phase kinds of the step (indices of SyncWords::phase_ns).
@@ -54,6 +64,7 @@ struct CaseDev {
   double dt;
   double tol, rel_tol;
   int32_t max_iter, min_iter;
+  int32_t late_cells;        // cells from which streamed mixed solves update the solution in P (kLateCells)
 
   // face-to-cell addressing, slot-major ("ELL"): each cell has W slots, slot k of cell c at
   // index k*N + c. Slots hold the cell's neighbour-side faces (ascending face id), then its

@@ -484,7 +484,7 @@ __device__ __forceinline__ void pass_direction_df(int c0, int c1, df beta, float
   if (c < c1) st_df(p + c, df_fma(beta, ld_df(p + c), ld_df(w + c)));
 }
 
-// P from kLateCells cells on: e += alpha p, the correction's update with the last direction, and p = w + beta p; backwards, as
+// P from CaseDev::late_cells / 2 cells on: e += alpha p, the correction's update with the last direction, and p = w + beta p; backwards, as
 // pass_direction_x (lfm_solve.cuh). It starts with e = alpha p (first). Per iteration of 8 M cells, P and U with the update in U: 31 + 78 us,
 // here 47 + 50; the call 10.89 -> 10.57 ms.
 template <int B>
@@ -824,7 +824,7 @@ __device__ bool steps_df64(const CaseDev& cs, const CaseDev& cref, const TM& tm,
       }
       // e is updated in P (not compiled into the kernels that serve general geometry, the batched ones
       // among them: the second form's code made batches 2 to 3 % slower)
-      const bool late = R == 0 && !kGeom && cs.N >= kLateCells;
+      const bool late = R == 0 && !kGeom && cs.N >= cs.late_cells / 2;
       bool due = false;  // the last iteration's e += alpha p is still to be done
       while (R == 0 && sh.code == kGo) {
         if (iters > 0) {
@@ -859,6 +859,7 @@ __device__ bool steps_df64(const CaseDev& cs, const CaseDev& cref, const TM& tm,
           return false;
         clk.lap(kPhU);
       }
+      if (late && iters > 0 && tm.rank == 0 && tid == 0) ++tm.sw->late;
       if (due) pass_solution_df<B>(c0, c1, df_of(sh.alpha2), e, iters == 1, p);
       if (late && iters > 0) pending = true;
       if (sh.code == kSingular) status = LFM_ESINGULAR;
