@@ -1766,7 +1766,7 @@ struct lfm_batch {
   cudaEvent_t done = nullptr;
   int pending = 0;
   int n_active = 0;
-  // captured one-step graph
+  // captured launch: takes its step count from the header
   cudaGraphExec_t gexec = nullptr;
   int g_threads = 0, g_W = -1, g_ctas = 0, g_form = -1, g_stage = -1;
   int stage_rows = 1;  // bulk-staged matrix rows where a pass supports them

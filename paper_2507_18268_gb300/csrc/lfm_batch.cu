@@ -60,9 +60,8 @@ __global__ void __launch_bounds__(B, 1024 / B) batch_kernel(const CaseDev* __res
     __syncthreads();
     const Team tm{s_job[2], s_job[1], s_cs.sync, s_cs.partials, L.timeout_ns};
     if (threadIdx.x == 0) team_join(tm, sh);
-    const int base = case_step[c];
     // a case whose cap is reached runs no step; its team's CTAs go back for tickets at once
-    const int run = min(n_steps, case_cap[c] - base);
+    const int run = min(n_steps, case_cap[c]);
     // The team meets once before it starts. A team that the launch's CTAs cannot all serve at once waits
     // here for the jobs before it, which run all steps of the advance: the bound of this wait grows with
     // the steps, the waits of a staffed team keep theirs. (One barrier without sums per job, 1.6 us.)
@@ -71,21 +70,19 @@ __global__ void __launch_bounds__(B, 1024 / B) batch_kernel(const CaseDev* __res
                     L.timeout_ns < most ? L.timeout_ns * (uint64_t)n_steps : ~0ull};
     if (run > 0 && team_barrier<B>(meet, sh)) {
       if constexpr (kForm == kBatchFp64) {
-        run_steps_f64<B, W>(s_cs, s_cs, tm, run, kModeSteps, sh, base);
+        run_steps_f64<B, W>(s_cs, s_cs, tm, run, kModeSteps, sh);
       } else if constexpr (kForm == kBatchDf64) {
-        run_steps_df64<B, W, true>(s_cs, s_cs, tm, run, sh, base);
+        run_steps_df64<B, W, true>(s_cs, s_cs, tm, run, sh);
       } else {
         if (s_cs.precision == LFM_MIXED)
-          run_steps_mixed_any<B, W>(s_cs, s_cs, tm, run, kModeSteps, sh, base);
+          run_steps_mixed_any<B, W>(s_cs, s_cs, tm, run, kModeSteps, sh);
         else if (s_cs.precision == LFM_DF64)
-          run_steps_df64<B, W, true>(s_cs, s_cs, tm, run, sh, base);
+          run_steps_df64<B, W, true>(s_cs, s_cs, tm, run, sh);
         else
-          run_steps_f64<B, W>(s_cs, s_cs, tm, run, kModeSteps, sh, base);
+          run_steps_f64<B, W>(s_cs, s_cs, tm, run, kModeSteps, sh);
       }
     }
-    __syncthreads();
-    if (run > 0) team_leave(tm, sh);
-    if (run > 0 && tm.rank == 0 && threadIdx.x == 0) case_step[c] = base + run;
+    if (run > 0 && tm.rank == 0 && threadIdx.x == 0) case_step[c] = run;
     __syncthreads();
   }
 }
@@ -96,7 +93,6 @@ __global__ void batch_prepare_kernel(const CaseDev* __restrict__ cases, int n_ca
   if (i < n_cases) {
     SyncWords* sw = cases[i].sync;
     sw->count = 0;
-    sw->gen = 0;
     sw->status = 0;
     case_step[i] = 0;
     // forms that update the FP64 field directly leave the triple-float one stale

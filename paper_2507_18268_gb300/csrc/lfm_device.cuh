@@ -116,21 +116,14 @@ struct TeamShared {
   unsigned long long phase[kPhases], phase_t;
 };
 
-// Thread 0 of a CTA, when the CTA joins a team (before its first arrival): the counter's value
-// before the team's first barrier, which team_leave or the host left in gen. A CTA that joins
-// a team whose wait has already run out leaves at its first barrier.
+// Thread 0 of a CTA, when the CTA joins a team (before its first arrival): every launch starts with
+// the team's words cleared, and a team runs once per launch. A CTA that joins a team whose wait has
+// already run out leaves at its first barrier.
 template <int B>
 __device__ __forceinline__ void team_join(const Team& tm, TeamShared<B>& sh) {
-  sh.target = *reinterpret_cast<volatile unsigned*>(&tm.sw->gen);
+  sh.target = 0;
   sh.par = 0;
   sh.ok = ld_volatile_i32(&tm.sw->status) != LFM_ETIMEOUT;
-}
-
-// After a team's last barrier of a run: where its next run's counter starts (every CTA of the
-// team has joined by then). Only launches without a host reset in between need it.
-template <int B>
-__device__ __forceinline__ void team_leave(const Team& tm, TeamShared<B>& sh) {
-  if (tm.rank == 0 && threadIdx.x == 0 && sh.ok) *reinterpret_cast<volatile unsigned*>(&tm.sw->gen) = sh.target;
 }
 
 // Spins until *count has reached target (modulo 2^32). False (with the error recorded) when

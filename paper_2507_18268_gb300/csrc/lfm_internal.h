@@ -40,11 +40,8 @@ constexpr int kStaticMaxFaces = 1 << 18;
 
 // Barrier words of one team of CTAs; each field sits on its own 128-byte line.
 struct alignas(128) SyncWords {
-  unsigned int count;                // arrivals, one per CTA and sum of every barrier (only grows)
+  unsigned int count;                // arrivals, one per CTA and sum of every barrier of the launch (only grows)
   unsigned int pad0[31];
-  unsigned int gen;                  // count before the team's next run (see team_leave)
-  unsigned int pad1[31];
-  unsigned int pad2[32];
   int32_t status;                    // first error of the launch (0 = none)
   int32_t pad3[31];
   unsigned long long phase_ns[8];    // time per phase kind, accumulated by the team's rank 0
@@ -214,7 +211,7 @@ struct BatchLaunch {
   const int32_t* job_case;   // [n_jobs] case of job j
   const int32_t* job_start;  // [n_jobs + 1] first ticket of job j
   BatchHeader* hdr;
-  int32_t* case_step;        // [n_cases] steps done in the current advance
+  int32_t* case_step;        // [n_cases] steps run by the current advance
   const int32_t* case_cap;   // [n_cases] at most this many steps of the current advance
   Launch launch;
   int W;

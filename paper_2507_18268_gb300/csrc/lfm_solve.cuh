@@ -1318,7 +1318,7 @@ __device__ __forceinline__ bool cg_on_chip(const F f, const CaseDev& cs, const C
 // R: rows per thread of a solve kept on chip (0: streamed, see cg_on_chip).
 template <int B, int W, int R = 0, class TM>
 __device__ void run_steps_f64(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps, int mode,
-                              TeamShared<B>& sh, int stats_base = 0) {
+                              TeamShared<B>& sh) {
   int c0, c1, f0, f1;
   cta_range(cs.N, tm.size, tm.rank, c0, c1);
   cta_range(cs.F, tm.size, tm.rank, f0, f1);
@@ -1412,7 +1412,7 @@ __device__ void run_steps_f64(const CaseDev& cs, const CaseDev& cref, const TM& 
       solves += iters > 0 ? 1 : 0;
       if (status != 0) break;
     }
-    write_stats(cs, tm, stats_base + step, iters_tot, sh.conv, solves, status, sh.init0, sh.res, sh.nf0);
+    write_stats(cs, tm, step, iters_tot, sh.conv, solves, status, sh.init0, sh.res, sh.nf0);
     clk.flush();
     if (status != 0) {
       if (tm.rank == 0 && tid == 0) set_status(cs.sync, status);
@@ -1513,7 +1513,7 @@ __device__ __forceinline__ bool inner_cg_f32(const CaseDev& cs, const CaseDev& c
 
 template <int B, int W, class TM>
 __device__ void run_steps_mixed(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps, int mode,
-                                TeamShared<B>& sh, int stats_base = 0) {
+                                TeamShared<B>& sh) {
   int c0, c1, f0, f1;
   cta_range(cs.N, tm.size, tm.rank, c0, c1);
   cta_range(cs.F, tm.size, tm.rank, f0, f1);
@@ -1581,7 +1581,7 @@ __device__ void run_steps_mixed(const CaseDev& cs, const CaseDev& cref, const TM
       sweeps_tot += sweeps;
       if (status != 0) break;
     }
-    write_stats(cs, tm, stats_base + step, iters_tot, sh.conv, sweeps_tot, status, sh.init0, sh.res, sh.nf0);
+    write_stats(cs, tm, step, iters_tot, sh.conv, sweeps_tot, status, sh.init0, sh.res, sh.nf0);
     clk.flush();
     if (status != 0) {
       if (tm.rank == 0 && tid == 0) set_status(cs.sync, status);

@@ -744,7 +744,7 @@ static_assert(sizeof(df) == sizeof(float2), "df arrays are stored as float2");
 // CTA: it follows the team-wide iteration counts).
 template <int B, int W, bool kGeom, int R, class TM>
 __device__ bool steps_df64(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps, TeamShared<B>& sh,
-                           int stats_base, int c0, int c1, bool& pending) {
+                           int c0, int c1, bool& pending) {
   const int tid = threadIdx.x;
   float2* __restrict__ e = cs.e2;
   float2* __restrict__ r = reinterpret_cast<float2*>(cs.r);
@@ -868,7 +868,7 @@ __device__ bool steps_df64(const CaseDev& cs, const CaseDev& cref, const TM& tm,
       solves += iters > 0 ? 1 : 0;
       if (status != 0) break;
     }
-    write_stats(cs, tm, stats_base + step, iters_tot, sh.conv, solves, status, sh.init0, sh.res, sh.nf0);
+    write_stats(cs, tm, step, iters_tot, sh.conv, solves, status, sh.init0, sh.res, sh.nf0);
     clk.flush();
     if (status != 0) {
       if (tm.rank == 0 && tid == 0) set_status(cs.sync, status);
@@ -881,13 +881,12 @@ __device__ bool steps_df64(const CaseDev& cs, const CaseDev& cref, const TM& tm,
 // kGeom: the kernel serves general geometry (the gradient phase is compiled in). R: rows per thread
 // of a solve kept on chip (0: streamed).
 template <int B, int W, bool kGeom = false, int R = 0, class TM>
-__device__ void run_steps_df64(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps, TeamShared<B>& sh,
-                               int stats_base = 0) {
+__device__ void run_steps_df64(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps, TeamShared<B>& sh) {
   if (n_steps <= 0) return;
   int c0, c1;
   cta_range(cs.N, tm.size, tm.rank, c0, c1);
   bool pending = false;
-  steps_df64<B, W, kGeom, R>(cs, cref, tm, n_steps, sh, stats_base, c0, c1, pending);
+  steps_df64<B, W, kGeom, R>(cs, cref, tm, n_steps, sh, c0, c1, pending);
   // the field and the correction of the CTA's own cells are written by this CTA only, so the
   // FP64 field can be written back without another barrier, also after an early exit.
   pass_store_x<B>(cref, c0, c1, pending);

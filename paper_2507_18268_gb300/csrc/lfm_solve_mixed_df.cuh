@@ -272,7 +272,7 @@ __device__ __forceinline__ bool mixed_uses_df(const CaseDev& cs) {
 // R: rows per thread of the inner solve kept on chip (0: streamed, see cg_on_chip).
 template <int B, int W, int R, class TM>
 __device__ bool steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps, TeamShared<B>& sh,
-                               int stats_base, int c0, int c1) {
+                               int c0, int c1) {
   const int tid = threadIdx.x;
   [[maybe_unused]] float* __restrict__ dx = cs.dx32;
   [[maybe_unused]] float* __restrict__ r = cs.r32;
@@ -413,7 +413,7 @@ __device__ bool steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const TM&
       sweeps_tot += sweeps;
       if (status != 0) break;
     }
-    write_stats(cs, tm, stats_base + step, iters_tot, sh.conv, sweeps_tot, status, sh.init0, sh.res, sh.nf0);
+    write_stats(cs, tm, step, iters_tot, sh.conv, sweeps_tot, status, sh.init0, sh.res, sh.nf0);
     clk.flush();
     if (status != 0) {
       if (tm.rank == 0 && tid == 0) set_status(cs.sync, status);
@@ -433,22 +433,22 @@ __device__ bool steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const TM&
 // The mixed form with df64 outer passes (the case must satisfy mixed_uses_df).
 template <int B, int W, int R = 0, class TM>
 __device__ void run_steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps,
-                                   TeamShared<B>& sh, int stats_base = 0) {
+                                   TeamShared<B>& sh) {
   if (n_steps <= 0) return;
   int c0, c1;
   cta_range(cs.N, tm.size, tm.rank, c0, c1);
-  steps_mixed_df<B, W, R>(cs, cref, tm, n_steps, sh, stats_base, c0, c1);
+  steps_mixed_df<B, W, R>(cs, cref, tm, n_steps, sh, c0, c1);
   pass_store_x<B>(cref, c0, c1, false);
 }
 
 // The mixed form: df64 outer passes where mixed_uses_df, else FP64 ones (lfm_solve.cuh).
 template <int B, int W, class TM>
 __device__ void run_steps_mixed_any(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps, int mode,
-                                    TeamShared<B>& sh, int stats_base = 0) {
+                                    TeamShared<B>& sh) {
   if (mode != kModeSteps || !mixed_uses_df(cs))
-    run_steps_mixed<B, W>(cs, cref, tm, n_steps, mode, sh, stats_base);
+    run_steps_mixed<B, W>(cs, cref, tm, n_steps, mode, sh);
   else
-    run_steps_mixed_df<B, W>(cs, cref, tm, n_steps, sh, stats_base);
+    run_steps_mixed_df<B, W>(cs, cref, tm, n_steps, sh);
 }
 
 }  // namespace
