@@ -390,8 +390,8 @@ __device__ __forceinline__ void mbar_drain(uint64_t* bar, unsigned parity, uint6
 // issued as soon as every thread is done with tile t. False when a wait ran out or another CTA
 // failed (status recorded): the CTA then lets its copies in flight land (bounded) before the
 // caller leaves.
-template <int TC, unsigned kStage, int NST = 2, class TM, typename Issue, typename Body>
-__device__ __forceinline__ bool staged_tiles(int c0, int c1, const TM& tm, Issue&& issue, Body&& body) {
+template <int TC, unsigned kStage, int NST = 2, typename Issue, typename Body>
+__device__ __forceinline__ bool staged_tiles(int c0, int c1, const Team& tm, Issue&& issue, Body&& body) {
   unsigned char* sm = lfm_dyn_smem;
   uint64_t* bar = reinterpret_cast<uint64_t*>(sm + NST * kStage);
   const int tid = threadIdx.x;

@@ -643,9 +643,9 @@ __device__ __forceinline__ bool use_bulk_f32(const Slots<float>& A) {
   return W > 0 && (A.N & 3) == 0 && dyn_smem_bytes() >= stage_bytes_f32<B, W>();
 }
 
-template <int B, int W, class TM>
+template <int B, int W>
 __device__ __noinline__ double pass_amul_dot_f32_bulk(Slots<float> A, int c0, int c1, const float* __restrict__ p,
-                                                   float* __restrict__ q, const TM& tm, bool& ok) {
+                                                   float* __restrict__ q, const Team& tm, bool& ok) {
   constexpr int TC = 2 * B;
   constexpr int S = W > 0 ? kSlots<W> : 1;
   constexpr int kIdx = kCoded<W> ? 1 : S;  // index planes
@@ -725,9 +725,9 @@ __device__ __noinline__ double pass_amul_dot_f32_bulk(Slots<float> A, int c0, in
 
 // M (FP32) over the bulk-staged rows where the launch gave the shared memory for them, else
 // the register form.
-template <int B, int W, class TM>
+template <int B, int W>
 __device__ __forceinline__ double amul_dot_f32(Slots<float> A, int c0, int c1, const float* __restrict__ p,
-                                               float* __restrict__ q, const TM& tm, bool& ok) {
+                                               float* __restrict__ q, const Team& tm, bool& ok) {
   ok = true;
   if constexpr (W > 0) {
     if (use_bulk_f32<B, W>(A)) return pass_amul_dot_f32_bulk<B, W>(A, c0, c1, p, q, tm, ok);
@@ -946,13 +946,13 @@ __device__ __forceinline__ void pass_correct(int c0, int c1, double* __restrict_
 // kept in shared memory and added to the launch's once per step, by adds that nothing waits
 // for: a load-add-store to global memory here stalled the rank-0 CTA, and with it the team,
 // for an L2 round trip per phase.
-template <int B, class TM>
+template <int B>
 struct PhaseClock {
   const CaseDev& cs;
-  const TM& tm;
+  const Team& tm;
   TeamShared<B>& sh;
   __device__ __forceinline__ bool on() const { return tm.rank == 0 && threadIdx.x == 0; }
-  __device__ __forceinline__ PhaseClock(const CaseDev& c, const TM& t, TeamShared<B>& s) : cs(c), tm(t), sh(s) {
+  __device__ __forceinline__ PhaseClock(const CaseDev& c, const Team& t, TeamShared<B>& s) : cs(c), tm(t), sh(s) {
     if (on()) {
       for (int k = 0; k < kPhases; ++k) sh.phase[k] = 0;
       sh.phase_t = global_timer_ns();
@@ -975,8 +975,7 @@ struct PhaseClock {
   }
 };
 
-template <class TM>
-__device__ __forceinline__ void write_stats(const CaseDev& cs, const TM& tm, int slot, int iters, int conv, int sweeps,
+__device__ __forceinline__ void write_stats(const CaseDev& cs, const Team& tm, int slot, int iters, int conv, int sweeps,
                                             int status, double init_res, double final_res, double nf) {
   if (tm.rank == 0 && threadIdx.x == 0) {
     lfm_step_stats st;
@@ -1028,8 +1027,8 @@ __device__ __forceinline__ void fin_update(TeamShared<B>& sh, int k, double t, i
 // copy of T at the start of the step when save_old, and with general geometry the Gauss
 // gradient in the same phase) and xRef, their team mean. False when a barrier failed (the
 // caller leaves the kernel).
-template <int B, int W, bool kMixed, class TM>
-__device__ __forceinline__ bool assemble_prologue(const CaseDev& cs, const CaseDev& cref, const TM& tm, int c0,
+template <int B, int W, bool kMixed>
+__device__ __forceinline__ bool assemble_prologue(const CaseDev& cs, const CaseDev& cref, const Team& tm, int c0,
                                                   int c1, int f0, int f1, bool write_upper, bool save_old,
                                                   TeamShared<B>& sh) {
   double v[1] = {pass_faces<B, kMixed>(cref, f0, f1, c0, c1, write_upper, save_old)};
@@ -1131,8 +1130,8 @@ __host__ __device__ __forceinline__ int rows_per_thread(int N, int ctas, int B) 
 
 // Brings the CTA's matrix rows into shared memory (once per launch). False when a copy's wait ran
 // out (status recorded).
-template <class F, int B, int W, int R, class TM>
-__device__ __noinline__ bool chip_load(const F f, const CaseDev& cs, const TM& tm, int c0, int c1) {
+template <class F, int B, int W, int R>
+__device__ __noinline__ bool chip_load(const F f, const CaseDev& cs, const Team& tm, int c0, int c1) {
   using V = typename F::V;
   constexpr int S = kSlots<W>, kIdx = kCoded<W> ? 1 : S, kPlane = R * B;
   const size_t N = (size_t)cs.N;
@@ -1186,9 +1185,9 @@ __device__ __noinline__ bool chip_load(const F f, const CaseDev& cs, const TM& t
 // CG from its seed (f.r, f.p = w; the scalars in sh): sh.code tells how it ended. fin_m and fin_u
 // are the fins of the two barriers, fin_u with the iterations done in this solve. False when a
 // barrier failed (the caller leaves).
-template <class F, int B, int W, int R, class TM, class FinM, class FinU>
-__device__ __forceinline__ bool cg_on_chip(const F f, const CaseDev& cs, const CaseDev& cref, const TM& tm,
-                                           TeamShared<B>& sh, PhaseClock<B, TM>& clk, int c0, int c1, bool& loaded,
+template <class F, int B, int W, int R, class FinM, class FinU>
+__device__ __forceinline__ bool cg_on_chip(const F f, const CaseDev& cs, const CaseDev& cref, const Team& tm,
+                                           TeamShared<B>& sh, PhaseClock<B>& clk, int c0, int c1, bool& loaded,
                                            FinM&& fin_m, FinU&& fin_u) {
   using V = typename F::V;
   constexpr int S = kSlots<W>, kIdx = kCoded<W> ? 1 : S;
@@ -1316,8 +1315,8 @@ __device__ __forceinline__ bool cg_on_chip(const F f, const CaseDev& cs, const C
 // FP64 steps (1 + n_corr assemble-and-solve passes per step)
 // =======================================================================================
 // R: rows per thread of a solve kept on chip (0: streamed, see cg_on_chip).
-template <int B, int W, int R = 0, class TM>
-__device__ void run_steps_f64(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps, int mode,
+template <int B, int W, int R = 0>
+__device__ void run_steps_f64(const CaseDev& cs, const CaseDev& cref, const Team& tm, int n_steps, int mode,
                               TeamShared<B>& sh) {
   int c0, c1, f0, f1;
   cta_range(cs.N, tm.size, tm.rank, c0, c1);
@@ -1330,7 +1329,7 @@ __device__ void run_steps_f64(const CaseDev& cs, const CaseDev& cref, const TM& 
   double* __restrict__ q = cs.q;
   const double* __restrict__ rD = cs.rD;
 
-  PhaseClock<B, TM> clk(cs, tm, sh);
+  PhaseClock<B> clk(cs, tm, sh);
   const bool corr_mode = cs.n_corr > 0 || cs.Sf != nullptr || cs.vSu != nullptr || cs.vSp != nullptr;
   [[maybe_unused]] bool loaded = false;
   for (int step = 0; step < n_steps; ++step) {
@@ -1466,8 +1465,8 @@ __device__ __forceinline__ void fin_inner(TeamShared<B>& sh, int i, double t, in
 
 // The inner FP32 CG on A dx = r from its seed (r, p = w; sh.rho, sh.inner_tol): sh.code tells how
 // it ended. False when a barrier failed (the caller leaves).
-template <int B, int W, class TM>
-__device__ __forceinline__ bool inner_cg_f32(const CaseDev& cs, const CaseDev& cref, const TM& tm, TeamShared<B>& sh, PhaseClock<B, TM>& clk,
+template <int B, int W>
+__device__ __forceinline__ bool inner_cg_f32(const CaseDev& cs, const CaseDev& cref, const Team& tm, TeamShared<B>& sh, PhaseClock<B>& clk,
                                              int c0, int c1, int min_inner, int& iters, float* __restrict__ dx,
                                              float* __restrict__ r, float* __restrict__ w, float* __restrict__ p,
                                              float* __restrict__ q, const float* __restrict__ rD) {
@@ -1511,8 +1510,8 @@ __device__ __forceinline__ bool inner_cg_f32(const CaseDev& cs, const CaseDev& c
   return true;
 }
 
-template <int B, int W, class TM>
-__device__ void run_steps_mixed(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps, int mode,
+template <int B, int W>
+__device__ void run_steps_mixed(const CaseDev& cs, const CaseDev& cref, const Team& tm, int n_steps, int mode,
                                 TeamShared<B>& sh) {
   int c0, c1, f0, f1;
   cta_range(cs.N, tm.size, tm.rank, c0, c1);
@@ -1526,7 +1525,7 @@ __device__ void run_steps_mixed(const CaseDev& cs, const CaseDev& cref, const TM
   float* __restrict__ q = cs.q32;
   const float* __restrict__ rD = cs.rD32;
 
-  PhaseClock<B, TM> clk(cs, tm, sh);
+  PhaseClock<B> clk(cs, tm, sh);
   const bool corr_mode = cs.n_corr > 0 || cs.Sf != nullptr || cs.vSu != nullptr || cs.vSp != nullptr;
   for (int step = 0; step < n_steps; ++step) {
     int iters_tot = 0, sweeps_tot = 0, status = 0;

@@ -111,8 +111,7 @@ __device__ __noinline__ double pass_sum_df(const CaseDev& cs, int c0, int c1, bo
 // After the first barrier of a launch that split the FP64 field: every CTA has read the flag,
 // so the team's rank 0 marks the triple-float field current (it persists across launches:
 // the FP64 field is only its rounding, rewritten at the end of every launch).
-template <class TM>
-__device__ __forceinline__ void mark_split(const CaseDev& cs, const TM& tm, bool& convert) {
+__device__ __forceinline__ void mark_split(const CaseDev& cs, const Team& tm, bool& convert) {
   if (convert && tm.rank == 0 && threadIdx.x == 0) *reinterpret_cast<volatile int32_t*>(cs.flags) = 1;
   convert = false;
 }
@@ -580,9 +579,9 @@ __host__ __device__ constexpr unsigned stage_bytes_df() {
   return kCoded<W> ? kDfStages * (B * stage_row_df<W>()) + 8u * kDfStages : 0u;
 }
 
-template <int B, int W, class TM>
+template <int B, int W>
 __device__ __noinline__ double pass_amul_dot_df_bulk(const CaseDev& cs, int c0, int c1, const float2* __restrict__ p,
-                                                     float2* __restrict__ q, const TM& tm, bool& ok) {
+                                                     float2* __restrict__ q, const Team& tm, bool& ok) {
   constexpr int S = kSlots<W>;
   constexpr unsigned kStage = B * stage_row_df<W>();
   const size_t N = (size_t)cs.N;
@@ -615,9 +614,9 @@ __device__ __noinline__ double pass_amul_dot_df_bulk(const CaseDev& cs, int c0, 
   return acc.value();
 }
 
-template <int B, int W, class TM>
+template <int B, int W>
 __device__ __forceinline__ double amul_dot_df(const CaseDev& cs, const CaseDev& cref, int c0, int c1,
-                                              const float2* __restrict__ p, float2* __restrict__ q, const TM& tm,
+                                              const float2* __restrict__ p, float2* __restrict__ q, const Team& tm,
                                               bool& ok) {
   ok = true;
   if constexpr (kCoded<W>) {
@@ -742,8 +741,8 @@ static_assert(sizeof(df) == sizeof(float2), "df arrays are stored as float2");
 // The steps of one launch. Returns false when a barrier failed (the caller leaves).
 // `pending` tracks whether e holds a correction not yet added to the field (the same in every
 // CTA: it follows the team-wide iteration counts).
-template <int B, int W, bool kGeom, int R, class TM>
-__device__ bool steps_df64(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps, TeamShared<B>& sh,
+template <int B, int W, bool kGeom, int R>
+__device__ bool steps_df64(const CaseDev& cs, const CaseDev& cref, const Team& tm, int n_steps, TeamShared<B>& sh,
                            int c0, int c1, bool& pending) {
   const int tid = threadIdx.x;
   float2* __restrict__ e = cs.e2;
@@ -753,7 +752,7 @@ __device__ bool steps_df64(const CaseDev& cs, const CaseDev& cref, const TM& tm,
   float2* __restrict__ q = reinterpret_cast<float2*>(cs.q);
   const float2* __restrict__ rD = cs.rD2;
 
-  PhaseClock<B, TM> clk(cs, tm, sh);
+  PhaseClock<B> clk(cs, tm, sh);
   const bool src_mode = cs.n_corr > 0 || cs.vSu != nullptr || cs.vSp != nullptr || (kGeom && cs.Sf != nullptr);
   bool convert = ld_volatile_i32(cs.flags) == 0;  // read by every CTA before the first barrier
   [[maybe_unused]] bool loaded = false;
@@ -880,8 +879,8 @@ __device__ bool steps_df64(const CaseDev& cs, const CaseDev& cref, const TM& tm,
 
 // kGeom: the kernel serves general geometry (the gradient phase is compiled in). R: rows per thread
 // of a solve kept on chip (0: streamed).
-template <int B, int W, bool kGeom = false, int R = 0, class TM>
-__device__ void run_steps_df64(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps, TeamShared<B>& sh) {
+template <int B, int W, bool kGeom = false, int R = 0>
+__device__ void run_steps_df64(const CaseDev& cs, const CaseDev& cref, const Team& tm, int n_steps, TeamShared<B>& sh) {
   if (n_steps <= 0) return;
   int c0, c1;
   cta_range(cs.N, tm.size, tm.rank, c0, c1);

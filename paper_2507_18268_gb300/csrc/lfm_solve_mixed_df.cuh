@@ -270,8 +270,8 @@ __device__ __forceinline__ bool mixed_uses_df(const CaseDev& cs) {
 }
 
 // R: rows per thread of the inner solve kept on chip (0: streamed, see cg_on_chip).
-template <int B, int W, int R, class TM>
-__device__ bool steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps, TeamShared<B>& sh,
+template <int B, int W, int R>
+__device__ bool steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const Team& tm, int n_steps, TeamShared<B>& sh,
                                int c0, int c1) {
   const int tid = threadIdx.x;
   [[maybe_unused]] float* __restrict__ dx = cs.dx32;
@@ -282,7 +282,7 @@ __device__ bool steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const TM&
   [[maybe_unused]] const float* __restrict__ rD = cs.rD32;
   const float s32 = (float)cs.df_scale, inv_s32 = (float)(1.0 / cs.df_scale);  // powers of two: exact
 
-  PhaseClock<B, TM> clk(cs, tm, sh);
+  PhaseClock<B> clk(cs, tm, sh);
   const bool src_mode = cs.n_corr > 0 || cs.vSu != nullptr || cs.vSp != nullptr;
   const bool fuse = !src_mode;  // verification fused with the next step's T0 (pass V)
   // this step's rows and seed come from the last V pass: of this launch, or of the last
@@ -431,8 +431,8 @@ __device__ bool steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const TM&
 }
 
 // The mixed form with df64 outer passes (the case must satisfy mixed_uses_df).
-template <int B, int W, int R = 0, class TM>
-__device__ void run_steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps,
+template <int B, int W, int R = 0>
+__device__ void run_steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const Team& tm, int n_steps,
                                    TeamShared<B>& sh) {
   if (n_steps <= 0) return;
   int c0, c1;
@@ -442,8 +442,8 @@ __device__ void run_steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const
 }
 
 // The mixed form: df64 outer passes where mixed_uses_df, else FP64 ones (lfm_solve.cuh).
-template <int B, int W, class TM>
-__device__ void run_steps_mixed_any(const CaseDev& cs, const CaseDev& cref, const TM& tm, int n_steps, int mode,
+template <int B, int W>
+__device__ void run_steps_mixed_any(const CaseDev& cs, const CaseDev& cref, const Team& tm, int n_steps, int mode,
                                     TeamShared<B>& sh) {
   if (mode != kModeSteps || !mixed_uses_df(cs))
     run_steps_mixed<B, W>(cs, cref, tm, n_steps, mode, sh);
