@@ -308,6 +308,10 @@ __device__ bool steps_mixed_df(const CaseDev& cs, const CaseDev& cref, const Tea
           return false;
         mark_split(cs, tm, convert);
         clk.lap(kPhAssembly);
+      } else {
+        // no barrier since V's, whose decision (sh.code) every thread has to have read before thread 0
+        // writes this step's first one
+        __syncthreads();
       }
       int iters = 0, sweeps = 0;
       for (;;) {
