@@ -68,7 +68,8 @@ def kernel_hash(family: str = "fp64") -> str:
 
 
 def algorithmic_bytes(N: int, F: int, iters: int, steps: int, precision: int) -> float:
-    """Minimum DRAM bytes of `steps` steps with `iters` PCG iterations in total.
+    """Minimum DRAM bytes of `steps` steps with `iters` PCG iterations in total, on a mesh whose
+    neighbours are read as int32 indices and whose rows every step assembles.
 
     Per PCG iteration (every array touched once per pass, int32 addressing):
       FP64  112 N + 16 F  (p update 32N; A p and p.q 24N + 16F; x, r updates and dots 56N)
@@ -82,6 +83,35 @@ def algorithmic_bytes(N: int, F: int, iters: int, steps: int, precision: int) ->
         per_iter = 56 * N + 12 * F
     per_step = (40 * N + 16 * F) + (48 * N + 16 * F)
     return float(iters) * per_iter + float(steps) * per_step
+
+
+def packed_bytes(N: int, F: int, iters: int, steps: int, form: str, late: bool = False) -> float:
+    """Minimum DRAM bytes of `steps` steps (one solve each, `iters` PCG iterations in total) where
+    the neighbours are one packed word per cell and the matrix is assembled once per launch: each
+    array once per pass that needs it, each face coefficient once, vectors of 8 (fp64, df64) or 4
+    (mixed) bytes.
+
+    Per iteration: p update (w, p in, p out), A p and p.q (word, coefficients, diagonal, p in, q
+    out), updates and dots (x, r, p, q, 1/diag in, x, r, w out): 116 N + 8 F, mixed 60 N + 4 F.
+    late: the p update updates the solution too and the other pass does not: 108 N + 8 F, mixed
+    56 N + 4 F. Per step, less what a solve's first iteration leaves out (its p update, the
+    correction's first read): fp64 sum of T, rows and residual 36 N + 8 F; df64 (12-byte field,
+    with the correction's fold) 48 N + 8 F, late 56 N + 8 F; mixed (correction, verification and
+    next rows in one pass) 76 N + 8 F, late 80 N + 8 F."""
+    if form == "mixed":
+        it, st = ((56, 4), (80, 8)) if late else ((60, 4), (76, 8))
+    elif form == "df64":
+        it, st = ((108, 8), (56, 8)) if late else ((116, 8), (48, 8))
+    else:
+        it, st = (116, 8), (36, 8)
+    return float(iters) * (it[0] * N + it[1] * F) + float(steps) * (st[0] * N + st[1] * F)
+
+
+def launch_bytes(B, solver, N: int, F: int, iters: int, steps: int, form: str) -> float:
+    """The minimum for the form in which the solver's last advance ran."""
+    if B.lfm_debug_pack_slots(solver.ctx, True) > 0:
+        return packed_bytes(N, F, iters, steps, form, B.lfm_debug_late_solves(solver.ctx) > 0)
+    return algorithmic_bytes(N, F, iters, steps, 1 if form == "mixed" else 0)
 
 
 def algorithmic_flops(N: int, F: int, iters: int, steps: int) -> float:
@@ -378,7 +408,7 @@ def main_ours(args, world, rank, local):
     secs_max = reduce_max(secs, world)
     cell_iters_all = reduce_sum(float(N) * iters, world)
     value = cell_iters_all / secs_max
-    alg = algorithmic_bytes(N, F, iters, K, 0)
+    alg = launch_bytes(B, s64, N, F, iters, K, "fp64")
     achieved_gbs = alg / secs / 1e9
     ratio = load_traffic_ratio("graded200_fp64")
     T64 = s64.field()
@@ -399,7 +429,7 @@ def main_ours(args, world, rank, local):
         assert all(x["converged"] for x in dst), "df64 step did not converge"
         dsecs_max = reduce_max(dsecs, world)
         dvalue = reduce_sum(float(N) * diters, world) / dsecs_max
-        dalg = algorithmic_bytes(N, F, diters, K, 0)
+        dalg = launch_bytes(B, sdf, N, F, diters, K, "df64")
         Td = sdf.field()
         dspread = repeat_runs(sdf, B, torch, stream, K, N, Td_start, float(N) * diters / dsecs, args.repeats)
         dratio = load_traffic_ratio("graded200_df64")
@@ -434,7 +464,7 @@ def main_ours(args, world, rank, local):
         assert all(x["converged"] for x in mst), "mixed step did not converge"
         msecs_max = reduce_max(msecs, world)
         mvalue = reduce_sum(float(N) * miters, world) / msecs_max
-        malg = algorithmic_bytes(N, F, miters, K, 1)
+        malg = launch_bytes(B, smx, N, F, miters, K, "mixed")
         Tm = smx.field()
         mspread = repeat_runs(smx, B, torch, stream, K, N, Tm_start, float(N) * miters / msecs, args.repeats)
         mratio = load_traffic_ratio("graded200_mixed")
@@ -579,11 +609,14 @@ SKEWED = ("skewed200: graded200 sheared by x' = x + 0.25 y + 0.15 z (8.0M parall
           "corrector per step (2 assemble-and-solve passes), DT, dt, BCs and PCG controls as graded200")
 
 
-def algorithmic_bytes_corrected(N: int, F: int, iters: int, passes: int) -> float:
+def algorithmic_bytes_corrected(N: int, F: int, iters: int, passes: int, packed: bool = False) -> float:
     """Minimum DRAM bytes of the corrected FP64 step: per PCG iteration as the orthogonal
     step (112 N + 16 F); per assemble-and-solve pass the orthogonal assembly and initial
     residual (88 N + 32 F) plus the Gauss gradient (T, Sf, w in; G out: 32 N + 32 F) and the
-    correction flux (G, k, w, |Sf| in; flux out, read back by the rows: 24 N + 56 F)."""
+    correction flux (G, k, w, |Sf| in; flux out, read back by the rows: 24 N + 56 F). packed: one
+    word per cell instead of 8 bytes per face in each pass that gathers."""
+    if packed:
+        return float(iters) * (116 * N + 8 * F) + float(passes) * ((88 + 32 + 24 + 12) * N + (32 + 32 + 56 - 24) * F)
     return float(iters) * (112 * N + 16 * F) + float(passes) * ((88 + 32 + 24) * N + (32 + 32 + 56) * F)
 
 
@@ -681,7 +714,7 @@ def main_large(args, world, rank, local):
         N = n ** 3
         secs_max = reduce_max(secs, world)
         F = 3 * n * n * (n - 1)
-        alg = algorithmic_bytes(N, F, iters, K, 0 if prec == B.LFM_FP64 else 1)
+        alg = launch_bytes(B, s, N, F, iters, K, name)
         hbm_peak, peak_kind = load_peaks()
         forms[name] = {"value": reduce_sum(float(N) * iters, world) / secs_max, "unit": UNIT,
                        "ms_per_step": 1e3 * secs_max / K, "iters_per_step": iters / K,
@@ -738,7 +771,8 @@ def main_skewed(args, world, rank, local):
     phases = {k: v / K for k, v in s64.phase_times().items()}
     secs_max = reduce_max(secs, world)
     value = reduce_sum(float(N) * iters, world) / secs_max
-    alg = algorithmic_bytes_corrected(N, F, iters, passes)
+    packed = B.lfm_debug_pack_slots(s64.ctx, True) > 0
+    alg = algorithmic_bytes_corrected(N, F, iters, passes, packed)
     sratio = load_traffic_ratio("skewed_fp64")
     T64 = s64.field()
     launch = s64.launch()
@@ -769,7 +803,7 @@ def main_skewed(args, world, rank, local):
         dphases = {k: v / K for k, v in sdf.phase_times().items()}
         sdf.close()
         dsecs_max = reduce_max(dsecs, world)
-        dalg = algorithmic_bytes_corrected(N, F, diters, dpasses)
+        dalg = algorithmic_bytes_corrected(N, F, diters, dpasses, packed)
         df64 = {"value": reduce_sum(float(N) * diters, world) / dsecs_max, "unit": UNIT,
                 "ms_per_step": 1e3 * dsecs_max / K, "iters_per_step": diters / K,
                 "converged": all(x["converged"] for x in dst),
