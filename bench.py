@@ -574,7 +574,7 @@ def main_ours(args, world, rank, local):
                                "fma_per_s": fma_rate, "clocks": fclk,
                                "frac_of_nominal": algorithmic_flops(N, F, iters, K) / secs / 1e12
                                / FP64_NOMINAL_TFLOPS,
-                               "note": "ncu: FP64 pipe 75% busy, DRAM 64% (profiles/step_kernel_f64_graded200.md)"},
+                               "note": "ncu: FP64 pipe 81% busy, DRAM 64% (profiles/step_kernel_f64_graded200.md)"},
         "gpu_launches": 1,
         "clocks": clk,
         "df64": df64,
