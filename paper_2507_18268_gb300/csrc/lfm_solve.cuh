@@ -27,8 +27,8 @@
 //   P  p = w + beta p  (skipped on the first iteration)
 //   M  q = A p, sigma = p.q                   -> alpha = rho / sigma
 //   U  x += alpha p, r -= alpha q, w = rD r, sum|r|, rho' = w.r -> beta = rho'/rho
-//   (large cases, see kLateCells: the FP32 and df64 loops update the solution in P; where a thread takes few rows the loop
-//   keeps them on chip and forms p in M, see cg_on_chip)
+//   (in large cases, see kLateCells, the FP32 and df64 loops update the solution in P; where a
+//   thread takes few rows the loop keeps them on chip and forms p in M, see cg_on_chip)
 //
 // General (non-orthogonal) meshes (section "Code Porting": the gradient passes): A1 also
 // evaluates the Gauss linear gradient of T per cell, and A2 adds to each row's source the

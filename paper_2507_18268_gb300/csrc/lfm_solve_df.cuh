@@ -483,9 +483,10 @@ __device__ __forceinline__ void pass_direction_df(int c0, int c1, df beta, float
   if (c < c1) st_df(p + c, df_fma(beta, ld_df(p + c), ld_df(w + c)));
 }
 
-// P from CaseDev::late_cells / 2 cells on: e += alpha p, the correction's update with the last direction, and p = w + beta p; backwards, as
-// pass_direction_x (lfm_solve.cuh). It starts with e = alpha p (first). Per iteration of 8 M cells, P and U with the update in U: 31 + 78 us,
-// here 47 + 50; the call 10.89 -> 10.57 ms.
+// P from CaseDev::late_cells / 2 cells on: e += alpha p, the correction's update with the last
+// direction, and p = w + beta p; backwards, as pass_direction_x (lfm_solve.cuh). It starts with
+// e = alpha p (first). Per iteration of 8 M cells, P and U with the update in U: 31 + 78 us, here
+// 47 + 50; the call 10.89 -> 10.57 ms.
 template <int B>
 __device__ __forceinline__ void pass_direction_x_df(int c0, int c1, df alpha, df beta, float2* __restrict__ e, bool first,
                                                   float2* __restrict__ p, const float2* __restrict__ w) {
